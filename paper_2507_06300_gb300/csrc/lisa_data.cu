@@ -149,6 +149,23 @@ __global__ void dataset_sums_kernel(const double* __restrict__ lnP, const double
     }
 }
 
+// log10 f of the first and last bin of each adjoint range, as the FP32 and the FP64 table hold it
+// (the adjoint's epilogue searches them for the ranges that touch an interval).
+__global__ void range_bounds_kernel(const DatasetDev* __restrict__ ds, int n_ds, int adj_bins,
+                                    const float* __restrict__ rec32, const double* __restrict__ rec64,
+                                    double2* __restrict__ rx32, double2* __restrict__ rx64) {
+    for (int d = blockIdx.x; d < n_ds; d += gridDim.x) {
+        const DatasetDev& D = ds[d];
+        for (int r = threadIdx.x; r < D.nranges; r += blockDim.x) {
+            const int64_t b0 = D.bin0 + (int64_t)r * adj_bins;
+            const int64_t b1 = min(b0 + adj_bins, D.bin0 + D.npad) - 1;
+            rx64[D.rbase + r] = make_double2(rec64[b0 * kRec], rec64[b1 * kRec]);
+            rx32[D.rbase + r] = make_double2((double)rec32[(b0 >> 1) * kPairRec + (b0 & 1)],
+                                             (double)rec32[(b1 >> 1) * kPairRec + (b1 & 1)]);
+        }
+    }
+}
+
 template <class T>
 lisa_status dev_alloc(T** p, size_t n) {
     if (n == 0) n = 1;
@@ -175,6 +192,9 @@ void release(lisa_data* d) {
     d->d_cta_first = nullptr;
     cudaFree(d->d_adj_units);
     cudaFree(d->d_adj_prefix);
+    cudaFree(d->d_rx32);
+    cudaFree(d->d_rx64);
+    d->d_rx32 = d->d_rx64 = nullptr;
     d->d_adj_units = nullptr;
     d->d_adj_prefix = nullptr;
     d->d_ds = nullptr;
@@ -187,6 +207,21 @@ void release(lisa_data* d) {
     d->d_cross64 = nullptr;
     d->d_cross32 = nullptr;
     d->d_items = nullptr;
+}
+
+// Bins per adjoint range (see kAdjBins): the longest that gives kAdjWarpsPerSm units per SM, or
+// kAdjMinBins.
+int32_t pick_adj_bins(const lisa_data_desc& q, int n_sm) {
+    int32_t bins = kAdjBins;
+    for (; bins > kAdjMinBins; bins >>= 1) {
+        int64_t units = 0;
+        for (int k = 0; k < q.n_datasets; ++k) {
+            const int64_t n = q.bin_offset[k + 1] - q.bin_offset[k], S = q.state_offset[k + 1] - q.state_offset[k];
+            units += (n + bins - 1) / bins * ((S + 31) / 32);
+        }
+        if (units >= (int64_t)kAdjWarpsPerSm * n_sm) break;
+    }
+    return bins;
 }
 
 int pow2ceil(int v) {
@@ -471,7 +506,8 @@ lisa_status lisa_data_create(const lisa_data_desc* desc, lisa_stream_t stream, l
     d->h_state_off.assign(q.state_offset, q.state_offset + D + 1);
     d->h_ds.resize(D);
     std::vector<int32_t> state_ds((size_t)S);
-    int64_t psd_base = 0, pad0 = 0;
+    int64_t psd_base = 0, pad0 = 0, rbase = 0;
+    d->adj_bins = pick_adj_bins(q, d->n_sm);
     for (int k = 0; k < D; ++k) {
         DatasetDev& X = d->h_ds[k];
         X.rbin0 = q.bin_offset[k];
@@ -492,12 +528,18 @@ lisa_status lisa_data_create(const lisa_data_desc* desc, lisa_stream_t stream, l
         psd_base += (int64_t)C * X.ns * X.nbins;
         X.K = 0.0;
         X.Cnu = 0.0;
-        X.nranges = (int32_t)((X.npad + kAdjBins - 1) / kAdjBins);
+        X.nranges = (int32_t)((X.npad + d->adj_bins - 1) / d->adj_bins);
+        X.rbase = (int32_t)rbase;
+        rbase += X.nranges;
         for (int32_t s = X.s0; s < X.s0 + X.ns; ++s) state_ds[s] = k;
     }
     d->n_pad = pad0;
     d->tiling = lisa_tiling{512, 128, 4, 0};
     const int64_t NP = pad0 > 0 ? pad0 : 1;
+    if (rbase > (int64_t)INT32_MAX) {
+        delete d;
+        return LISA_ERR_SHAPE;
+    }
 
     lisa_status st = LISA_SUCCESS;
     double *f = nullptr, *nu = nullptr, *R = nullptr, *lnP = nullptr, *nu_p = nullptr, *X = nullptr;
@@ -518,7 +560,8 @@ lisa_status lisa_data_create(const lisa_data_desc* desc, lisa_stream_t stream, l
         (st = dev_alloc(&d->d_elllo32, (size_t)NP)) || (st = dev_alloc(&nu_p, (size_t)NP)) ||
         (st = dev_alloc(&f, (size_t)N)) ||
         (st = dev_alloc(&nu, (size_t)N)) || (st = dev_alloc(&lnP, (size_t)NP)) ||
-        (st = dev_alloc(&R, (size_t)C * N)))
+        (st = dev_alloc(&R, (size_t)C * N)) || (st = dev_alloc(&d->d_rx32, (size_t)rbase)) ||
+        (st = dev_alloc(&d->d_rx64, (size_t)rbase)))
         return fail(st);
     cudaStream_t sm = (cudaStream_t)stream;
     bool ok = cudaMemcpyAsync(d->d_ds, d->h_ds.data(), D * sizeof(DatasetDev), cudaMemcpyHostToDevice, sm) == cudaSuccess &&
@@ -532,6 +575,8 @@ lisa_status lisa_data_create(const lisa_data_desc* desc, lisa_stream_t stream, l
     prep_kernel<<<blocks, 256, 0, sm>>>(pad0, C, q.tdi_form, q.sgwb_model != 0, f, nu, d->d_P, R, N, d->d_ds, D,
                                         d->d_rec64, d->d_rec32, d->d_xlo32, d->d_elllo32, lnP, nu_p);
     dataset_sums_kernel<<<D, 256, 0, sm>>>(lnP, nu_p, d->d_ds, C);
+    range_bounds_kernel<<<std::min(D, 4 * d->n_sm), 128, 0, sm>>>(d->d_ds, D, d->adj_bins, d->d_rec32, d->d_rec64,
+                                                                  d->d_rx32, d->d_rx64);
     if (cudaGetLastError() != cudaSuccess) return fail(LISA_ERR_CUDA);
     if (d->cov == LISA_COV_FULL) {
         if ((st = dev_alloc(&X, (size_t)3 * N)) || (st = dev_alloc(&d->d_cross64, (size_t)NP * kCross)) ||

@@ -22,7 +22,7 @@
 // Horner evaluation, |x - x_o| <= h/2), which keeps the FP32 partial sums small; the epilogue
 // converts them exactly (FP64 binomial expansion) to moments about the left knot.
 //
-// Determinism: a range rho of kAdjBins bins writes the moments of every interval j it touches
+// Determinism: a range rho of adj_bins bins writes the moments of every interval j it touches
 // to slot rho + j of its (state, spline) row; the intervals a range touches are monotone in rho,
 // so slots never collide, and the epilogue adds them back in a fixed order.
 #include "lisa_math.cuh"
@@ -77,6 +77,15 @@ struct AdjIv {
 
 __device__ __forceinline__ float2 dup2(float v) { return make_float2(v, v); }
 
+// First unit of the calling warp, of nw in the grid (8 CTAs per SM, or one per unit).  Units that the
+// resident warps (3 of the grid's 8 CTAs per SM) can hold at once go to the CTAs before they go to a CTA's
+// warps, so that few of them spread over the SMs; more units go to a CTA's warps in turn, so that every
+// CTA that starts brings its full number of warps (131,072 bins, 2,048 states: 1.11 ms, and 1.35 ms spread).
+__device__ __forceinline__ int64_t first_unit(int64_t n_units, int64_t nw) {
+    const int w = threadIdx.x >> 5;
+    return 8 * n_units <= 3 * nw ? (int64_t)w * gridDim.x + blockIdx.x : (int64_t)blockIdx.x * (blockDim.x >> 5) + w;
+}
+
 // asynchronous global -> shared copies of one thread (completion by cp.async.wait_group)
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
@@ -110,7 +119,7 @@ __global__ void __launch_bounds__(128, 3)
                         const double* __restrict__ theta, const int32_t* __restrict__ sstat,
                         const int32_t* __restrict__ nint, const float* __restrict__ srec, int kmax, int nsp,
                         const int64_t* __restrict__ prefix, double* __restrict__ scal, double* __restrict__ mom,
-                        int S, int32_t* __restrict__ fb) {
+                        int S, int32_t* __restrict__ fb, int adj_bins) {
     constexpr int NSP = C + (HAS_H ? 1 : 0);
     __shared__ float2 s_am[NSP * 4][128];
     __shared__ float2 s_as[6][128];
@@ -120,8 +129,8 @@ __global__ void __launch_bounds__(128, 3)
     const int tid = threadIdx.x;
     const int wid = tid >> 5;
     const int lane = threadIdx.x & 31;
-    const int64_t wg = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int64_t wg = first_unit(n_units, nw);
     const float2 m1 = dup2(-1.f);
     for (int64_t u = wg; u < n_units; u += nw) {
         const AdjUnit U = units[u];
@@ -134,8 +143,8 @@ __global__ void __launch_bounds__(128, 3)
         const float ao2 = (float)(th[0] * th[0]), at2 = (float)(th[1] * th[1]);
         const float Af = HAS_H ? (float)exp10(th[2]) : 0.f;
         const float n1 = (float)th[3], n2 = BROKEN ? (float)th[4] : n1;
-        const int64_t b0 = D.bin0 + (int64_t)U.rho * kAdjBins;        // even
-        const int nb = (int)min((int64_t)kAdjBins, D.bin0 + D.npad - b0);
+        const int64_t b0 = D.bin0 + (int64_t)U.rho * adj_bins;        // even
+        const int nb = (int)min((int64_t)adj_bins, D.bin0 + D.npad - b0);
         const float* tb = rec32 + (b0 >> 1) * kPairRec;
         const int64_t pre = prefix[s];
         const int32_t* nint_s = nint + (int64_t)s * nsp;
@@ -496,11 +505,11 @@ __global__ void __launch_bounds__(128)
                         const double* __restrict__ rec64, const double* __restrict__ theta,
                         const int32_t* __restrict__ sstat, const int32_t* __restrict__ nint,
                         const double* __restrict__ srec, int kmax, int nsp, const int64_t* __restrict__ prefix,
-                        double* __restrict__ scal, double* __restrict__ mom) {
+                        double* __restrict__ scal, double* __restrict__ mom, int adj_bins) {
     constexpr int NSP = C + (HAS_H ? 1 : 0);
     const int lane = threadIdx.x & 31;
-    const int64_t wg = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int64_t wg = first_unit(n_units, nw);
     for (int64_t u = wg; u < n_units; u += nw) {
         const AdjUnit U = units[u];
         const DatasetDev& D = ds[U.ds];
@@ -511,8 +520,8 @@ __global__ void __launch_bounds__(128)
         const double* th = theta + (size_t)s * LISA_N_THETA;
         const double ao2 = th[0] * th[0], at2 = th[1] * th[1], lA = th[2], n1 = th[3];
         const double n2 = BROKEN ? th[4] : n1;
-        const int64_t b0 = D.bin0 + (int64_t)U.rho * kAdjBins;
-        const int nb = (int)min((int64_t)kAdjBins, D.bin0 + D.npad - b0);
+        const int64_t b0 = D.bin0 + (int64_t)U.rho * adj_bins;
+        const int nb = (int)min((int64_t)adj_bins, D.bin0 + D.npad - b0);
         const int64_t pre = prefix[s];
         const double* base[NSP];
         int j[NSP], last[NSP];
@@ -626,8 +635,13 @@ __global__ void __launch_bounds__(MODE == kComp ? 128 : 512)
                          int32_t* __restrict__ fb, int32_t* __restrict__ next_item,
                          const int32_t* __restrict__ nint, const void* __restrict__ srec_v,
                          const float2* __restrict__ hull, int kmax, int nsp, const int64_t* __restrict__ prefix,
-                         double* __restrict__ scal, double* __restrict__ mom) {
+                         double* __restrict__ scal, double* __restrict__ mom, int adj_bins) {
     constexpr int NSP = C + (HAS_H ? 1 : 0);
+    // this pass's ranges: kComp takes kAdjBins bins whatever the adjoint's range size (its lanes'
+    // FP32 template sums then cover the same bins), each holding `sub` of the adjoint's ranges, the
+    // first of which has index rho * sub; kFallback takes the adjoint's ranges
+    const int rbins = MODE == kComp ? kAdjBins : adj_bins;
+    const int sub = rbins / adj_bins;
     // per warp, spline and interval (from the range's first) the 4 moment sums: dynamic shared
     // memory of nwarps * NSP * (kmax + 1) * 4 doubles
     extern __shared__ double s_m[];
@@ -651,9 +665,9 @@ __global__ void __launch_bounds__(MODE == kComp ? 128 : 512)
     const int s = LISA_IDX(list[1 + LISA_IDX(it / R, S)], S), rho = it % R;
     if (MODE == kComp && (sstat[s] & (kUserBits | kRouted)) != kRouted) continue;
     const DatasetDev& D = ds[state_ds[s]];
-    if (rho >= D.nranges) continue;
-    const int64_t b0 = D.bin0 + (int64_t)rho * kAdjBins;
-    const int nb = (int)min((int64_t)kAdjBins, D.bin0 + D.npad - b0);
+    if ((int64_t)rho * sub >= D.nranges) continue;
+    const int64_t b0 = D.bin0 + (int64_t)rho * rbins;
+    const int nb = (int)min((int64_t)rbins, D.bin0 + D.npad - b0);
     const float* tb = rec32 + (b0 >> 1) * kPairRec;
     if (MODE == kComp) {
         const float2 hx = hull[s];
@@ -1057,10 +1071,21 @@ __global__ void __launch_bounds__(MODE == kComp ? 128 : 512)
             v[p] = 0.0;
             for (int w = 0; w < nwarps; ++w) v[p] += sm(w, a, jr, p);
         }
-        double* row = mom_row(mom, pre, s, a, nsp, kmax, D.nranges) + 4 * (int64_t)LISA_IDX(rho + j, D.nranges + kmax + 1);
+        double* row = mom_row(mom, pre, s, a, nsp, kmax, D.nranges);
         if (MODE == kComp) {
-            // the FP32 adjoint's slots carry ln10 (its q's factor)
+            // the FP32 adjoint's slots carry ln10 (its q's factor); the sums go to the slot of the
+            // first of its ranges that holds a bin of the interval
             if (v[0] != 0.0 || v[1] != 0.0 || v[2] != 0.0 || v[3] != 0.0) {
+                int i = 0;
+                if (sub > 1 && j > 0) {
+                    const float left = right_end(a, j - 1);
+                    int hi = nb - 1;
+                    while (i < hi) {
+                        const int mid = (i + hi) >> 1;
+                        if (xbin(mid) >= left) hi = mid; else i = mid + 1;
+                    }
+                }
+                row += 4 * (int64_t)LISA_IDX(rho * sub + i / adj_bins + j, D.nranges + kmax + 1);
                 bool bad = false;
                 for (int p = 0; p < 4; ++p) {
                     row[p] += kLn10 * v[p];
@@ -1069,6 +1094,7 @@ __global__ void __launch_bounds__(MODE == kComp ? 128 : 512)
                 if (bad) fb_flag(fb, S, s);
             }
         } else {
+            row += 4 * (int64_t)LISA_IDX(rho + j, D.nranges + kmax + 1);
             for (int p = 0; p < 4; ++p) row[p] = v[p];
         }
     }
@@ -1076,19 +1102,18 @@ __global__ void __launch_bounds__(MODE == kComp ? 128 : 512)
         const int k = threadIdx.x;
         double v = 0.0;
         for (int w = 0; w < nwarps; ++w) v += s_t[w][k];
+        double* sc = scal + 6 * (pre + (int64_t)rho * sub) + k;
         if (MODE == kComp) {
-            scal[6 * (pre + rho) + k] += v;
-            if (!isfinite(scal[6 * (pre + rho) + k])) fb_flag(fb, S, s);
+            *sc += v;
+            if (!isfinite(*sc)) fb_flag(fb, S, s);
         } else {
-            scal[6 * (pre + rho) + k] = v;
+            *sc = v;
         }
     }
     }
 }
 
 // ---- epilogue: one warp per state, FP64 ----------------------------------------------------------
-constexpr int kEpiRanges = 256;   // adjoint ranges whose bounds the epilogue stages (524,288 bins)
-
 // d s_k / d m_{k+delta}, delta = -2..1, for the Akima slope at knot k (Appendix A rules,
 // including the ends), returned in d[0..3] = delta -2, -1, 0, +1.  mm2..mp1 = m_{k-2}..m_{k+1}.
 template <class T>
@@ -1151,340 +1176,353 @@ __device__ __forceinline__ void akima_slope_grad(int k, int K, T mm2, T mm1, T m
     }
 }
 
-// One state's reverse map (one warp): log L from the range sums, the template components, and
-// per spline the moments gathered over the ranges, re-expanded about the knots (FP32 records:
-// they are about the midpoints) and pushed back through the Akima or natural-cubic construction,
-// in T (double, or float-float on the FP32 pipe).  Returns true, for the caller to redo the
-// state in FP64, where a sum, a moment or a gradient value is not finite (a float-float run
-// whose values left the FP32 exponent range); the FP64 run's return value is not used.
-// sX, sY: the warp's 64-double scratch rows; sRf, sRl: its kEpiRanges-double range-bound rows.
-template <int C, bool HAS_H, bool BROKEN, class T>
-__device__ __noinline__ bool epilogue_state(int s, const int32_t* __restrict__ state_ds,
-                                            const DatasetDev* __restrict__ ds, const int32_t* __restrict__ sstat,
-                                            const double* __restrict__ theta, const int32_t* __restrict__ count,
-                                            const double* __restrict__ kx, const double* __restrict__ kw, int kmax,
-                                            int kind, int nsp, const int64_t* __restrict__ prefix,
-                                            const double* __restrict__ scal, const double* __restrict__ mom,
-                                            const float* __restrict__ rec32, const double* __restrict__ rec64,
-                                            const void* __restrict__ srec_v, int fp32, double* __restrict__ out_logL,
-                                            double* __restrict__ grad, double* sX, double* sY, double* sRf,
-                                            double* sRl) {
+// One spline's reverse map of one state (one warp): the moments gathered over the ranges, re-expanded
+// about the knots (FP32 records: they are about the midpoints) and pushed back through the Akima or
+// natural-cubic construction, in T (double, or float-float on the FP32 pipe); the warp of spline 0
+// also writes log L from the range sums and the template components.  Returns true, for the caller
+// to redo the spline in FP64, where a sum, a moment or a gradient value is not finite (a float-float
+// run whose values left the FP32 exponent range); the FP64 run's return value is not used.
+// sX, sY: the warp's 64-double scratch rows.
+template <class T>
+__device__ __noinline__ bool epilogue_spline(int s, int a, int has_h, int broken, const int32_t* __restrict__ state_ds,
+                                             const DatasetDev* __restrict__ ds, const int32_t* __restrict__ sstat,
+                                             const double* __restrict__ theta, const int32_t* __restrict__ count,
+                                             const double* __restrict__ kx, const double* __restrict__ kw, int kmax,
+                                             int kind, int nsp, const int64_t* __restrict__ prefix,
+                                             const double* __restrict__ scal, const double* __restrict__ mom,
+                                             const double2* __restrict__ rx32, const double2* __restrict__ rx64,
+                                             const void* __restrict__ srec_v, int fp32, double* __restrict__ out_logL,
+                                             double* __restrict__ grad, double* sX, double* sY) {
     constexpr bool kFF = std::is_same<T, spl::F2>::value;
     const int lane = threadIdx.x & 31;
-    const int G = LISA_N_THETA + nsp * (2 * kmax + 2);
-    double* gs = grad + (size_t)s * G;
-    for (int k = lane; k < G; k += 32) gs[k] = 0.0;
+    const int per_spline = 2 * kmax + 2;
+    double* gs = grad + (size_t)s * (LISA_N_THETA + nsp * per_spline);
+    double* ga = gs + LISA_N_THETA + a * per_spline;
+    for (int k = lane; k < per_spline; k += 32) ga[k] = 0.0;
+    if (a == 0 && lane < LISA_N_THETA) gs[lane] = 0.0;
     __syncwarp();
     if (sstat[s] & kUserBits) {
-        if (lane == 0) out_logL[s] = -INFINITY;
+        if (a == 0 && lane == 0) out_logL[s] = -INFINITY;
         return false;
     }
     const DatasetDev& D = ds[state_ds[s]];
     const int nr = D.nranges;
     const int64_t pre = prefix[s];
+    // the range sums: log L's (every warp of the state decides by it) and, for spline 0's warp, the
+    // template terms'
     double v[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    const int nv = a == 0 ? 6 : 1;
     for (int r = lane; r < nr; r += 32)
-        for (int k = 0; k < 6; ++k) v[k] += scal[6 * (pre + r) + k];
-    for (int o = 16; o > 0; o >>= 1)
-        for (int k = 0; k < 6; ++k) v[k] += __shfl_down_sync(kFullMask, v[k], o);
-    for (int k = 0; k < 6; ++k) v[k] = __shfl_sync(kFullMask, v[k], 0);
-    double L = -v[0] - D.Cnu + D.K;
+#pragma unroll
+        for (int k = 0; k < 6; ++k)
+            if (k < nv) v[k] += scal[6 * (pre + r) + k];
+#pragma unroll
+    for (int k = 0; k < 6; ++k)
+        if (k < nv) {
+            for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(kFullMask, v[k], o);
+            v[k] = __shfl_sync(kFullMask, v[k], 0);
+        }
+    const double L = -v[0] - D.Cnu + D.K;
     const bool finite = isfinite(L);
     if (kFF) {
         bool sums_ok = finite;
         for (int k = 1; k < 6; ++k) sums_ok &= isfinite(v[k]);
         if (!sums_ok) return true;
     }
-    if (lane == 0) out_logL[s] = finite ? L : -INFINITY;
+    if (a == 0 && lane == 0) out_logL[s] = finite ? L : -INFINITY;
     if (!finite) return false;   // gradient stays zero
     bool bad = false;            // a non-finite moment or gradient value
-    // range bounds: in shared memory when they fit, else read per range below
-    const bool staged = nr <= kEpiRanges;
-    auto range_x = [&](int rho, double& xf, double& xlb) {
-        const int64_t b0 = D.bin0 + (int64_t)rho * kAdjBins;
-        const int nb = (int)min((int64_t)kAdjBins, D.bin0 + D.npad - b0);
-        if (fp32) {
-            const float* tb = rec32 + (b0 >> 1) * kPairRec;
-            xf = (double)fld(tb, 0, 0);
-            xlb = (double)fld(tb, nb - 1, 0);
-        } else {
-            xf = rec64[b0 * kRec];
-            xlb = rec64[(b0 + nb - 1) * kRec];
-        }
-    };
-    if (staged) {
-        for (int rho = lane; rho < nr; rho += 32) range_x(rho, sRf[LISA_IDX(rho, kEpiRanges)], sRl[LISA_IDX(rho, kEpiRanges)]);
-        __syncwarp();
-    }
-    const double* th = theta + (size_t)s * LISA_N_THETA;
-    if (lane == 0) {
+    const double2* rx = (fp32 ? rx32 : rx64) + D.rbase;   // (first, last) bin's x of each range
+    if (a == 0 && lane == 0) {
+        const double* th = theta + (size_t)s * LISA_N_THETA;
         gs[0] = 2.0 * th[0] * v[1];
         gs[1] = 2.0 * th[1] * v[2];
-        if (HAS_H) {
+        if (has_h) {
             gs[2] = kLn10 * v[3];
-            gs[3] = kLn2 * (BROKEN ? v[4] : v[4] + v[5]);
-            gs[4] = BROKEN ? kLn2 * v[5] : 0.0;
+            gs[3] = kLn2 * (broken ? v[4] : v[4] + v[5]);
+            gs[4] = broken ? kLn2 * v[5] : 0.0;
+        }
+        for (int k = 0; k < LISA_N_THETA; ++k) bad |= !isfinite(gs[k]);
+    }
+    const int64_t sp = (int64_t)s * nsp + a;
+    spl::WarpSpline<T> W;
+    spl::warp_build_spline<T>(W, kx + sp * kmax, kw + sp * (kmax + 2), count[sp], kmax, kind, D.x_lo, D.x_hi, sX, sY);
+    if (W.st) return false;
+    const int K = W.K;
+    const int nint = K - 1;
+    const int nq = K > 32 ? 2 : 1;   // the second lane slot is only used by splines with K > 32
+    const double* row = mom_row(const_cast<double*>(mom), pre, s, a, nsp, kmax, nr);
+    // moments of each interval, gathered over the ranges that touched it (fixed order).  The ranges
+    // that touch an interval are the contiguous span [r0, r1] (bins are sorted): first range whose
+    // last bin reaches its left bound, last one that starts below its right bound, the bounds as the
+    // likelihood kernels' walk sees them.  Each lane finds its own intervals' spans; then the lanes
+    // take (interval, moment) pairs, eight intervals at a time, so that an FP64 add serves 32 sums
+    // (one lane per interval with all four moments left the FP64 pipe adding for 10 of 32 lanes).
+    T M[2][4];
+    int r0[2] = {0, 0}, r1[2] = {-1, -1};
+    double Md[2][4] = {{0.0, 0.0, 0.0, 0.0}, {0.0, 0.0, 0.0, 0.0}};
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        if (q >= nq) break;   // warp-uniform
+        const int jj = lane + 32 * q;
+        if (jj >= nint) continue;
+        double lo_b, hi_b;
+        if (fp32) {
+            const float* r = static_cast<const float*>(srec_v) + (sp * (int64_t)(kmax + 1) + LISA_IDX(jj, kmax + 1)) * kSplineRec32;
+            lo_b = (double)r[6];
+            hi_b = (double)r[0];
+        } else {
+            const double* r = static_cast<const double*>(srec_v) + (sp * (int64_t)(kmax + 1) + LISA_IDX(jj, kmax + 1)) * kSplineRec;
+            lo_b = r[0];
+            hi_b = r[1];
+        }
+        r1[q] = nr - 1;
+        if (jj != 0) {
+            int lo = 0, hi = nr;
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (__ldg(&rx[mid].y) >= lo_b) hi = mid; else lo = mid + 1;
+            }
+            r0[q] = lo;
+        }
+        if (jj != nint - 1) {
+            int lo = 0, hi = nr;
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (__ldg(&rx[mid].x) < hi_b) lo = mid + 1; else hi = mid;
+            }
+            r1[q] = lo - 1;
         }
     }
-    const int per_spline = 2 * kmax + 2;
-    for (int a = 0; a < nsp; ++a) {
-        const int64_t sp = (int64_t)s * nsp + a;
-        spl::WarpSpline<T> W;
-        spl::warp_build_spline<T>(W, kx + sp * kmax, kw + sp * (kmax + 2), count[sp], kmax, kind, D.x_lo, D.x_hi,
-                               sX, sY);
-        if (W.st) continue;
-        const int K = W.K;
-        const int nint = K - 1;
-        const double* row = mom_row(const_cast<double*>(mom), pre, s, a, nsp, kmax, nr);
-        // moments of each interval, gathered over the ranges that touched it (fixed order)
-        double Md[2][4];   // summed in FP64 (the accumulation over ranges)
-        T M[2][4];
+    __syncwarp();
+    for (int g = 0; g < nint; g += 8) {
+        const int jj = g + (lane >> 2);
+        const int q = g >> 5;
+        const int b0 = __shfl_sync(kFullMask, q ? r0[1] : r0[0], jj & 31);
+        const int b1 = __shfl_sync(kFullMask, q ? r1[1] : r1[0], jj & 31);   // -1 past the last interval
+        double sum = 0.0;
+#pragma unroll 4
+        for (int rho = b0; rho <= b1; ++rho)
+            sum += row[4 * (int64_t)LISA_IDX(rho + jj, nr + kmax + 1) + (lane & 3)];
+        const bool mine = ((lane ^ g) & 24) == 0;   // lane is one of g & 31 .. + 7
+        for (int p = 0; p < 4; ++p) {
+            const double m = __shfl_sync(kFullMask, sum, 4 * (lane & 7) + p);
+            if (mine) (q ? Md[1][p] : Md[0][p]) = m;
+        }
+    }
+    for (int q = 0; q < 2; ++q)
+        for (int p = 0; p < 4; ++p) M[q][p] = T(0);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        if (q >= nq) break;   // warp-uniform
+        const int jj = lane + 32 * q;
+        if (jj >= nint) continue;
+        for (int p = 0; p < 4; ++p) {
+            bad |= !isfinite(Md[q][p]);
+            M[q][p] = T(Md[q][p]);
+        }
+        if (fp32) {
+            // moments about the FP32 midpoint xo -> about the left knot x_j:  t = u + mo
+            const float* r = static_cast<const float*>(srec_v) + (sp * (int64_t)(kmax + 1) + LISA_IDX(jj, kmax + 1)) * kSplineRec32;
+            const T mo = spl::from_hilo<T>(r[1], r[8]) - W.x[q];
+            const T C0 = M[q][0], C1 = M[q][1], C2 = M[q][2], C3 = M[q][3];
+            M[q][0] = C0;
+            M[q][1] = C1 + mo * C0;
+            M[q][2] = C2 + mo * (T(2) * C1 + mo * C0);
+            M[q][3] = C3 + mo * (T(3) * C2 + mo * (T(3) * C1 + mo * C0));
+        }
+    }
+    // ---- reverse through the coefficient map
+    T ybar[2], xbar[2], mbar[2], hbar[2], own[2], nxt[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) ybar[q] = xbar[q] = mbar[q] = hbar[q] = own[q] = nxt[q] = T(0);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        if (q >= nq) break;   // warp-uniform
+        const int jj = lane + 32 * q;
+        const bool iv = jj < nint;
+        const T h = W.h[q], ih = W.ih[q], ih2 = ih * ih;
+        const T M0 = M[q][0], M1 = M[q][1], M2 = M[q][2], M3 = M[q][3];
+        ybar[q] = iv ? M0 : T(0);
+        xbar[q] = iv ? -(W.cb[q] * M0 + T(2) * W.cc[q] * M1 + T(3) * W.cd[q] * M2) : T(0);
+        mbar[q] = hbar[q] = own[q] = nxt[q] = T(0);
+        if (!iv) continue;
+        if (K < 4) {
+            mbar[q] = M1;
+        } else if (kind == LISA_SPLINE_NATURAL) {
+            const T Mj = W.d2[q];
+            own[q] = -M1 * h * T(1.0 / 3.0) + T(0.5) * M2 - M3 * ih * T(1.0 / 6.0);   // -> d/dM_j
+            nxt[q] = -M1 * h * T(1.0 / 6.0) + M3 * ih * T(1.0 / 6.0);                // -> d/dM_{j+1}
+            mbar[q] = M1;
+            (void)Mj;
+        } else {
+            own[q] = M1 - T(2) * M2 * ih + M3 * ih2;               // -> d/ds_j
+            nxt[q] = -M2 * ih + M3 * ih2;                         // -> d/ds_{j+1}
+            mbar[q] = T(3) * M2 * ih - T(2) * M3 * ih2;
+            hbar[q] = -(W.cc[q] * M2 + T(2) * W.cd[q] * M3) * ih;
+        }
+    }
+    if (K >= 4 && kind == LISA_SPLINE_NATURAL) {
+        // b = m - h (2 M_j + M_{j+1}) / 6,  d = (M_{j+1} - M_j) / (6 h): h dependence
+        T Mn[2];
+        spl::shift2(W.d2[0], W.d2[1], 1, Mn[0], Mn[1]);
+#pragma unroll
         for (int q = 0; q < 2; ++q) {
             const int jj = lane + 32 * q;
-            for (int p = 0; p < 4; ++p) {
-                Md[q][p] = 0.0;
-                M[q][p] = T(0);
-            }
-            if (jj >= nint) continue;
-            double lo_b, hi_b;   // the interval's bounds as the likelihood kernels' walk sees them
-            if (fp32) {
-                const float* r = static_cast<const float*>(srec_v) + (sp * (int64_t)(kmax + 1) + LISA_IDX(jj, kmax + 1)) * kSplineRec32;
-                lo_b = (double)r[6];
-                hi_b = (double)r[0];
-            } else {
-                const double* r = static_cast<const double*>(srec_v) + (sp * (int64_t)(kmax + 1) + LISA_IDX(jj, kmax + 1)) * kSplineRec;
-                lo_b = r[0];
-                hi_b = r[1];
-            }
-            if (staged) {
-                // the ranges that touch the interval are the contiguous span [r0, r1] (bins are
-                // sorted): first range whose last bin reaches lo_b, last one that starts below hi_b
-                int r0 = 0, r1 = nr - 1;
-                if (jj != 0) {
-                    int lo = 0, hi = nr;
-                    while (lo < hi) {
-                        const int mid = (lo + hi) >> 1;
-                        if (sRl[mid] >= lo_b) hi = mid; else lo = mid + 1;
-                    }
-                    r0 = lo;
-                }
-                if (jj != nint - 1) {
-                    int lo = 0, hi = nr;
-                    while (lo < hi) {
-                        const int mid = (lo + hi) >> 1;
-                        if (sRf[mid] < hi_b) lo = mid + 1; else hi = mid;
-                    }
-                    r1 = lo - 1;
-                }
-                for (int rho = r0; rho <= r1; ++rho)
-                    for (int p = 0; p < 4; ++p) Md[q][p] += row[4 * (int64_t)LISA_IDX(rho + jj, nr + kmax + 1) + p];
-            } else {
-                for (int rho = 0; rho < nr; ++rho) {
-                    double xf, xlb;
-                    range_x(rho, xf, xlb);
-                    const bool touches = (jj == 0 || xlb >= lo_b) && (jj == nint - 1 || xf < hi_b);
-                    if (touches)
-                        for (int p = 0; p < 4; ++p) Md[q][p] += row[4 * (int64_t)LISA_IDX(rho + jj, nr + kmax + 1) + p];
-                }
-            }
-            for (int p = 0; p < 4; ++p) {
-                bad |= !isfinite(Md[q][p]);
-                M[q][p] = T(Md[q][p]);
-            }
-            if (fp32) {
-                // moments about the FP32 midpoint xo -> about the left knot x_j:  t = u + mo
-                const float* r = static_cast<const float*>(srec_v) + (sp * (int64_t)(kmax + 1) + LISA_IDX(jj, kmax + 1)) * kSplineRec32;
-                const T mo = spl::from_hilo<T>(r[1], r[8]) - W.x[q];
-                const T C0 = M[q][0], C1 = M[q][1], C2 = M[q][2], C3 = M[q][3];
-                M[q][0] = C0;
-                M[q][1] = C1 + mo * C0;
-                M[q][2] = C2 + mo * (T(2) * C1 + mo * C0);
-                M[q][3] = C3 + mo * (T(3) * C2 + mo * (T(3) * C1 + mo * C0));
-            }
+            if (jj < nint) hbar[q] = -M[q][1] * (T(2) * W.d2[q] + Mn[q]) * T(1.0 / 6.0) - W.cd[q] * M[q][3] * W.ih[q];
         }
-        // ---- reverse through the coefficient map
-        T ybar[2], xbar[2], mbar[2], hbar[2], own[2], nxt[2];
-        for (int q = 0; q < 2; ++q) {
-            const int jj = lane + 32 * q;
-            const bool iv = jj < nint;
-            const T h = W.h[q], ih = W.ih[q], ih2 = ih * ih;
-            const T M0 = M[q][0], M1 = M[q][1], M2 = M[q][2], M3 = M[q][3];
-            ybar[q] = iv ? M0 : T(0);
-            xbar[q] = iv ? -(W.cb[q] * M0 + T(2) * W.cc[q] * M1 + T(3) * W.cd[q] * M2) : T(0);
-            mbar[q] = hbar[q] = own[q] = nxt[q] = T(0);
-            if (!iv) continue;
-            if (K < 4) {
-                mbar[q] = M1;
-            } else if (kind == LISA_SPLINE_NATURAL) {
-                const T Mj = W.d2[q];
-                own[q] = -M1 * h * T(1.0 / 3.0) + T(0.5) * M2 - M3 * ih * T(1.0 / 6.0);   // -> d/dM_j
-                nxt[q] = -M1 * h * T(1.0 / 6.0) + M3 * ih * T(1.0 / 6.0);                // -> d/dM_{j+1}
-                mbar[q] = M1;
-                (void)Mj;
-            } else {
-                own[q] = M1 - T(2) * M2 * ih + M3 * ih2;               // -> d/ds_j
-                nxt[q] = -M2 * ih + M3 * ih2;                         // -> d/ds_{j+1}
-                mbar[q] = T(3) * M2 * ih - T(2) * M3 * ih2;
-                hbar[q] = -(W.cc[q] * M2 + T(2) * W.cd[q] * M3) * ih;
-            }
-        }
-        if (K >= 4 && kind == LISA_SPLINE_NATURAL) {
-            // b = m - h (2 M_j + M_{j+1}) / 6,  d = (M_{j+1} - M_j) / (6 h): h dependence
-            T Mn[2];
-            spl::shift2(W.d2[0], W.d2[1], 1, Mn[0], Mn[1]);
-            for (int q = 0; q < 2; ++q) {
-                const int jj = lane + 32 * q;
-                if (jj < nint) hbar[q] = -M[q][1] * (T(2) * W.d2[q] + Mn[q]) * T(1.0 / 6.0) - W.cd[q] * M[q][3] * W.ih[q];
-            }
-            // d/dM_k = own_k + nxt_{k-1}; M_0 and M_{K-1} are fixed
-            T nprev[2], Mbar[2];
-            spl::shift2(nxt[0], nxt[1], -1, nprev[0], nprev[1]);
-            T A[2], B[2], Cc[2], R[2];
-            T hm[2];
-            spl::shift2(W.h[0], W.h[1], -1, hm[0], hm[1]);
-            for (int q = 0; q < 2; ++q) {
-                const int k = lane + 32 * q;
-                Mbar[q] = (k >= 1 && k <= K - 2) ? own[q] + nprev[q] : T(0);
-                if (k >= 1 && k <= K - 2) {
-                    A[q] = hm[q];
-                    B[q] = T(2) * (hm[q] + W.h[q]);
-                    Cc[q] = W.h[q];
-                    R[q] = Mbar[q];
-                } else {
-                    A[q] = T(0);
-                    B[q] = T(1);
-                    Cc[q] = T(0);
-                    R[q] = T(0);
-                }
-            }
-            spl::pcr_solve(A, B, Cc, R, K);   // the system is symmetric: lambda = A^-1 Mbar
-            T lam[2], lamn[2], Mnn[2];
-            for (int q = 0; q < 2; ++q) lam[q] = R[q] / B[q];
-            spl::shift2(lam[0], lam[1], 1, lamn[0], lamn[1]);
-            spl::shift2(Mn[0], Mn[1], 1, Mnn[0], Mnn[1]);
-            for (int q = 0; q < 2; ++q) {
-                const int k = lane + 32 * q;
-                const T Mk = W.d2[q];
-                // r_k = 6 (m_k - m_{k-1}):  mbar_k += 6 lam_k - 6 lam_{k+1}
-                if (k >= 1 && k <= K - 2) mbar[q] += T(6) * lam[q];
-                if (k + 1 >= 1 && k + 1 <= K - 2) mbar[q] -= T(6) * lamn[q];
-                // row k:   h_{k-1} M_{k-1} + 2 (h_{k-1} + h_k) M_k + h_k M_{k+1}
-                //   dh_k from row k: 2 M_k + M_{k+1};  from row k+1: M_k + 2 M_{k+1}
-                if (k >= 1 && k <= K - 2) hbar[q] -= lam[q] * (T(2) * Mk + Mn[q]);
-                if (k + 1 >= 1 && k + 1 <= K - 2 && k < nint) hbar[q] -= lamn[q] * (Mk + T(2) * Mn[q]);
-                (void)Mnn;
-            }
-        } else if (K >= 4) {
-            // Akima: d/ds_k = own_k + nxt_{k-1}, then through the slope rule to the interval slopes
-            T nprev[2], sbar[2];
-            spl::shift2(nxt[0], nxt[1], -1, nprev[0], nprev[1]);
-            T mm1[2], mm2[2], mp1[2];
-            spl::shift2(W.m[0], W.m[1], -1, mm1[0], mm1[1]);
-            spl::shift2(W.m[0], W.m[1], -2, mm2[0], mm2[1]);
-            spl::shift2(W.m[0], W.m[1], 1, mp1[0], mp1[1]);
-            T c[4][2];   // contribution of knot k to mbar_{k + delta}, delta = -2..1
-            for (int q = 0; q < 2; ++q) {
-                const int k = lane + 32 * q;
-                sbar[q] = (k < K) ? own[q] + (k >= 1 ? nprev[q] : T(0)) : T(0);
-                T dd[4] = {T(0), T(0), T(0), T(0)};
-                if (k < K) akima_slope_grad(k, K, mm2[q], mm1[q], W.m[q], mp1[q], W.d2[q], dd);
-                for (int t = 0; t < 4; ++t) c[t][q] = sbar[q] * dd[t];
-            }
-            // mbar_i += c_{i+2}[-2] + c_{i+1}[-1] + c_i[0] + c_{i-1}[+1]
-            T f0[2], f1[2], f3[2];
-            spl::shift2(c[0][0], c[0][1], 2, f0[0], f0[1]);
-            spl::shift2(c[1][0], c[1][1], 1, f1[0], f1[1]);
-            spl::shift2(c[3][0], c[3][1], -1, f3[0], f3[1]);
-            for (int q = 0; q < 2; ++q) {
-                const int i = lane + 32 * q;
-                if (i >= nint) continue;
-                T add = c[2][q];
-                if (i + 2 < K) add += f0[q];
-                if (i + 1 < K) add += f1[q];
-                if (i >= 1) add += f3[q];
-                mbar[q] += add;
-            }
-        }
-        // m_j = (y_{j+1} - y_j) / h_j ;  h_j = x_{j+1} - x_j
-        T gmy[2], gmyp[2], ghp[2];
-        for (int q = 0; q < 2; ++q) {
-            const int jj = lane + 32 * q;
-            gmy[q] = (jj < nint) ? mbar[q] * W.ih[q] : T(0);
-            if (jj < nint) hbar[q] -= W.m[q] * gmy[q];
-            else hbar[q] = T(0);
-        }
-        spl::shift2(gmy[0], gmy[1], -1, gmyp[0], gmyp[1]);
-        spl::shift2(hbar[0], hbar[1], -1, ghp[0], ghp[1]);
+        // d/dM_k = own_k + nxt_{k-1}; M_0 and M_{K-1} are fixed
+        T nprev[2], Mbar[2];
+        spl::shift2(nxt[0], nxt[1], -1, nprev[0], nprev[1]);
+        T A[2], B[2], Cc[2], R[2];
+        T hm[2];
+        spl::shift2(W.h[0], W.h[1], -1, hm[0], hm[1]);
+#pragma unroll
         for (int q = 0; q < 2; ++q) {
             const int k = lane + 32 * q;
-            if (k >= K) {
-                ybar[q] = xbar[q] = T(0);
-                continue;
+            Mbar[q] = (k >= 1 && k <= K - 2) ? own[q] + nprev[q] : T(0);
+            if (k >= 1 && k <= K - 2) {
+                A[q] = hm[q];
+                B[q] = T(2) * (hm[q] + W.h[q]);
+                Cc[q] = W.h[q];
+                R[q] = Mbar[q];
+            } else {
+                A[q] = T(0);
+                B[q] = T(1);
+                Cc[q] = T(0);
+                R[q] = T(0);
             }
-            ybar[q] += -gmy[q] + (k >= 1 ? gmyp[q] : T(0));
-            xbar[q] += -hbar[q] + (k >= 1 ? ghp[q] : T(0));
         }
-        // scatter: sorted knot k -> caller slots
-        double* ga = gs + LISA_N_THETA + a * per_spline;
-        const T y0 = spl::bcast(ybar[0], ybar[1], 0);
-        const T yK = spl::bcast(ybar[0], ybar[1], K - 1);
-        if (lane == 0) {
-            ga[0] = spl::to_double(y0);
-            ga[kmax + 1] = spl::to_double(yK);
-            bad |= !isfinite(ga[0]) || !isfinite(ga[kmax + 1]);
+        spl::pcr_solve(A, B, Cc, R, K);   // the system is symmetric: lambda = A^-1 Mbar
+        T lam[2], lamn[2], Mnn[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) lam[q] = R[q] / B[q];
+        spl::shift2(lam[0], lam[1], 1, lamn[0], lamn[1]);
+        spl::shift2(Mn[0], Mn[1], 1, Mnn[0], Mnn[1]);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int k = lane + 32 * q;
+            const T Mk = W.d2[q];
+            // r_k = 6 (m_k - m_{k-1}):  mbar_k += 6 lam_k - 6 lam_{k+1}
+            if (k >= 1 && k <= K - 2) mbar[q] += T(6) * lam[q];
+            if (k + 1 >= 1 && k + 1 <= K - 2) mbar[q] -= T(6) * lamn[q];
+            // row k:   h_{k-1} M_{k-1} + 2 (h_{k-1} + h_k) M_k + h_k M_{k+1}
+            //   dh_k from row k: 2 M_k + M_{k+1};  from row k+1: M_k + 2 M_{k+1}
+            if (k >= 1 && k <= K - 2) hbar[q] -= lam[q] * (T(2) * Mk + Mn[q]);
+            if (k + 1 >= 1 && k + 1 <= K - 2 && k < nint) hbar[q] -= lamn[q] * (Mk + T(2) * Mn[q]);
+            (void)Mnn;
         }
-        const int k_in = K - 2;
-        for (int half = 0; half < 2; ++half) {
-            const int i = lane + 32 * half;          // caller's in-between knot index
-            const int r = half ? W.rb : W.ra;        // its sorted position (1..K-2)
-            const int rs = (i < k_in) ? r : 0;
-            const T gy = spl::shfl(rs < 32 ? ybar[0] : ybar[1], rs & 31);
-            const T gx = spl::shfl(rs < 32 ? xbar[0] : xbar[1], rs & 31);
-            if (i < k_in) {
-                ga[1 + LISA_IDX(i, kmax)] = spl::to_double(gy);
-                ga[kmax + 2 + LISA_IDX(i, kmax)] = spl::to_double(gx);
-                bad |= !isfinite(ga[1 + i]) || !isfinite(ga[kmax + 2 + i]);
-            }
+    } else if (K >= 4) {
+        // Akima: d/ds_k = own_k + nxt_{k-1}, then through the slope rule to the interval slopes
+        T nprev[2], sbar[2];
+        spl::shift2(nxt[0], nxt[1], -1, nprev[0], nprev[1]);
+        T mm1[2], mm2[2], mp1[2];
+        spl::shift2(W.m[0], W.m[1], -1, mm1[0], mm1[1]);
+        spl::shift2(W.m[0], W.m[1], -2, mm2[0], mm2[1]);
+        spl::shift2(W.m[0], W.m[1], 1, mp1[0], mp1[1]);
+        T c[4][2];   // contribution of knot k to mbar_{k + delta}, delta = -2..1
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int k = lane + 32 * q;
+            sbar[q] = (k < K) ? own[q] + (k >= 1 ? nprev[q] : T(0)) : T(0);
+            T dd[4] = {T(0), T(0), T(0), T(0)};
+            if (k < K) akima_slope_grad(k, K, mm2[q], mm1[q], W.m[q], mp1[q], W.d2[q], dd);
+            for (int t = 0; t < 4; ++t) c[t][q] = sbar[q] * dd[t];
+        }
+        // mbar_i += c_{i+2}[-2] + c_{i+1}[-1] + c_i[0] + c_{i-1}[+1]
+        T f0[2], f1[2], f3[2];
+        spl::shift2(c[0][0], c[0][1], 2, f0[0], f0[1]);
+        spl::shift2(c[1][0], c[1][1], 1, f1[0], f1[1]);
+        spl::shift2(c[3][0], c[3][1], -1, f3[0], f3[1]);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int i = lane + 32 * q;
+            if (i >= nint) continue;
+            T add = c[2][q];
+            if (i + 2 < K) add += f0[q];
+            if (i + 1 < K) add += f1[q];
+            if (i >= 1) add += f3[q];
+            mbar[q] += add;
         }
     }
-    // (the template components were written by lane 0, which checks them)
-    if (lane == 0)
-        for (int k = 0; k < LISA_N_THETA; ++k) bad |= !isfinite(gs[k]);
+    // m_j = (y_{j+1} - y_j) / h_j ;  h_j = x_{j+1} - x_j
+    T gmy[2], gmyp[2], ghp[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const int jj = lane + 32 * q;
+        gmy[q] = (jj < nint) ? mbar[q] * W.ih[q] : T(0);
+        if (jj < nint) hbar[q] -= W.m[q] * gmy[q];
+        else hbar[q] = T(0);
+    }
+    spl::shift2(gmy[0], gmy[1], -1, gmyp[0], gmyp[1]);
+    spl::shift2(hbar[0], hbar[1], -1, ghp[0], ghp[1]);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const int k = lane + 32 * q;
+        if (k >= K) {
+            ybar[q] = xbar[q] = T(0);
+            continue;
+        }
+        ybar[q] += -gmy[q] + (k >= 1 ? gmyp[q] : T(0));
+        xbar[q] += -hbar[q] + (k >= 1 ? ghp[q] : T(0));
+    }
+    // scatter: sorted knot k -> caller slots
+    const T y0 = spl::bcast(ybar[0], ybar[1], 0);
+    const T yK = spl::bcast(ybar[0], ybar[1], K - 1);
+    if (lane == 0) {
+        ga[0] = spl::to_double(y0);
+        ga[kmax + 1] = spl::to_double(yK);
+        bad |= !isfinite(ga[0]) || !isfinite(ga[kmax + 1]);
+    }
+    const int k_in = K - 2;
+    for (int half = 0; half < 2; ++half) {
+        const int i = lane + 32 * half;          // caller's in-between knot index
+        const int r = half ? W.rb : W.ra;        // its sorted position (1..K-2)
+        const int rs = (i < k_in) ? r : 0;
+        const T gy = spl::shfl(rs < 32 ? ybar[0] : ybar[1], rs & 31);
+        const T gx = spl::shfl(rs < 32 ? xbar[0] : xbar[1], rs & 31);
+        if (i < k_in) {
+            ga[1 + LISA_IDX(i, kmax)] = spl::to_double(gy);
+            ga[kmax + 2 + LISA_IDX(i, kmax)] = spl::to_double(gx);
+            bad |= !isfinite(ga[1 + i]) || !isfinite(ga[kmax + 2 + i]);
+        }
+    }
     return __any_sync(kFullMask, bad);
 }
 
-// One warp per state.  The FP32 call runs the reverse map in float-float and redoes in FP64 the
-// states its adjoint passes flagged (fb[s]: sums beyond the FP32 range, recomputed by the
-// fallback pass) and those whose float-float values are not finite; the FP64 call runs FP64.
-// 4 CTAs of 128 threads per SM (128 registers) keep 2,432 states resident at once.
-template <int C, bool HAS_H, bool BROKEN>
+// One warp per (state, spline).  The FP32 call runs the reverse map in float-float and redoes in
+// FP64 the states its adjoint passes flagged (fb[s]: sums beyond the FP32 range, recomputed by the
+// fallback pass) and the splines whose float-float values are not finite; the FP64 call runs FP64.
+// Each warp's chain of dependent steps (sort, build, gather, reverse map) is what a launch of few
+// states waits for, so a state's splines run side by side, and the two knot slots of a lane are
+// unrolled (in registers; as loops they lived in local memory).  Against one warp per state and one
+// lane per interval's four moments: 128 states x 3 splines 59 -> 28 us, 400 x 4 112 -> 33 us, 2,048 x 4
+// 192 -> 129 us, 400 x 4 natural cubics in FP64 261 -> 120 us (all bound by the FP64 pipe or the chain).
+// 4 CTAs of 128 threads per SM (at most 128 registers) keep 2,432 warps resident.
 __global__ void __launch_bounds__(128, 4)
-    adjoint_epilogue_kernel(int S, const int32_t* __restrict__ state_ds, const DatasetDev* __restrict__ ds,
-                            const int32_t* __restrict__ sstat, const double* __restrict__ theta,
-                            const int32_t* __restrict__ count, const double* __restrict__ kx,
-                            const double* __restrict__ kw, int kmax, int kind, int nsp,
+    adjoint_epilogue_kernel(int S, int has_h, int broken, const int32_t* __restrict__ state_ds,
+                            const DatasetDev* __restrict__ ds, const int32_t* __restrict__ sstat,
+                            const double* __restrict__ theta, const int32_t* __restrict__ count,
+                            const double* __restrict__ kx, const double* __restrict__ kw, int kmax, int kind, int nsp,
                             const int64_t* __restrict__ prefix, const double* __restrict__ scal,
-                            const double* __restrict__ mom, const float* __restrict__ rec32,
-                            const double* __restrict__ rec64, const void* __restrict__ srec_v, int fp32,
+                            const double* __restrict__ mom, const double2* __restrict__ rx32,
+                            const double2* __restrict__ rx64, const void* __restrict__ srec_v, int fp32,
                             double* __restrict__ out_logL, double* __restrict__ grad,
                             const int32_t* __restrict__ fb) {
     __shared__ double sX[4][64];
     __shared__ double sY[4][64];
-    // first and last bin's x of each adjoint range of the warp's dataset (the same for all its
-    // states and splines), for datasets of up to kEpiRanges ranges
-    __shared__ double sRf[4][kEpiRanges], sRl[4][kEpiRanges];
     const int warp = threadIdx.x >> 5;
-    const int s = blockIdx.x * 4 + warp;
-    if (s >= S) return;
+    const int64_t u = (int64_t)blockIdx.x * 4 + warp;
+    if (u >= (int64_t)S * nsp) return;
+    const int s = (int)(u / nsp), a = (int)(u % nsp);
     bool redo = !fp32 || fb[s] != 0;
     if (!redo)
-        redo = epilogue_state<C, HAS_H, BROKEN, spl::F2>(s, state_ds, ds, sstat, theta, count, kx, kw, kmax, kind,
-                                                         nsp, prefix, scal, mom, rec32, rec64, srec_v, fp32,
-                                                         out_logL, grad, sX[warp], sY[warp], sRf[warp], sRl[warp]);
+        redo = epilogue_spline<spl::F2>(s, a, has_h, broken, state_ds, ds, sstat, theta, count, kx, kw, kmax, kind, nsp,
+                                        prefix, scal, mom, rx32, rx64, srec_v, fp32, out_logL, grad, sX[warp],
+                                        sY[warp]);
     if (redo)
-        epilogue_state<C, HAS_H, BROKEN, double>(s, state_ds, ds, sstat, theta, count, kx, kw, kmax, kind, nsp,
-                                                 prefix, scal, mom, rec32, rec64, srec_v, fp32, out_logL, grad,
-                                                 sX[warp], sY[warp], sRf[warp], sRl[warp]);
+        epilogue_spline<double>(s, a, has_h, broken, state_ds, ds, sstat, theta, count, kx, kw, kmax, kind, nsp, prefix,
+                                scal, mom, rx32, rx64, srec_v, fp32, out_logL, grad, sX[warp], sY[warp]);
 }
 
 // Whether every dataset meets the EXACT_T condition of adjoint_fp32_kernel.
@@ -1500,11 +1538,11 @@ inline bool adj_exact_t(const lisa_data* d) {
     return true;
 }
 
-// The most adjoint ranges of any dataset (the per-(state, range) grids' second dimension).
-inline int adj_max_ranges(const lisa_data* d) {
-    int m = 1;
-    for (const auto& Dh : d->h_ds) m = std::max(m, (int)Dh.nranges);
-    return m;
+// The most ranges of `bins` bins of any dataset (the per-(state, range) items of a pass).
+inline int adj_max_ranges(const lisa_data* d, int bins) {
+    int64_t m = 1;
+    for (const auto& Dh : d->h_ds) m = std::max(m, (Dh.npad + bins - 1) / bins);
+    return (int)m;
 }
 
 // Dynamic shared memory of adjoint_range_kernel with nwarps warps.
@@ -1527,10 +1565,10 @@ cudaError_t launch_adjoint(const lisa_data* d, bool fp32, const lisa_params* par
                            double* out, double* grad, cudaStream_t sm) {
     double* scal = gw.scal;
     double* mom = gw.mom;
-    const int grid = d->n_sm * 8;
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(d->n_sm * 8, d->n_adj_units));
     const bool prof = prof_active(d, sm);
     const int S = (int)d->n_states;
-    const int R = adj_max_ranges(d);
+    const int Rc = adj_max_ranges(d, kAdjBins), Rf = adj_max_ranges(d, d->adj_bins);
     prof_mark(d, prof, 0, sm);
     if (fp32 && cudaMemsetAsync(gw.fb, 0, sizeof(int32_t) * (2 * (size_t)S + 3), sm) != cudaSuccess)
         return cudaErrorInvalidValue;
@@ -1538,11 +1576,13 @@ cudaError_t launch_adjoint(const lisa_data* d, bool fp32, const lisa_params* par
         if (fp32 && adj_exact_t(d))
             adjoint_fp32_kernel<C, H, B, true><<<grid, 128, 0, sm>>>(
                 d->d_adj_units, d->n_adj_units, d->d_ds, d->d_rec32, d->d_xlo32, params->theta_dev, sstat, nint,
-                static_cast<const float*>(srec), kn->kmax, d->nsp, d->d_adj_prefix, scal, mom, S, gw.fb);
+                static_cast<const float*>(srec), kn->kmax, d->nsp, d->d_adj_prefix, scal, mom, S, gw.fb,
+                d->adj_bins);
         else if (fp32)
             adjoint_fp32_kernel<C, H, B, false><<<grid, 128, 0, sm>>>(
                 d->d_adj_units, d->n_adj_units, d->d_ds, d->d_rec32, d->d_xlo32, params->theta_dev, sstat, nint,
-                static_cast<const float*>(srec), kn->kmax, d->nsp, d->d_adj_prefix, scal, mom, S, gw.fb);
+                static_cast<const float*>(srec), kn->kmax, d->nsp, d->d_adj_prefix, scal, mom, S, gw.fb,
+                d->adj_bins);
         prof_mark(d, prof, 1, sm);
         if (fp32) {
             // the bins of ill-conditioned intervals (routed states), masked above: the route
@@ -1557,7 +1597,8 @@ cudaError_t launch_adjoint(const lisa_data* d, bool fp32, const lisa_params* par
                 return cudaErrorInvalidValue;
             adjoint_range_kernel<C, H, B, kComp><<<d->n_sm * std::max(occ, 1), 128, smc, sm>>>(
                 S, d->d_state_ds, d->d_ds, d->d_rec32, d->d_xlo32, d->d_elllo32, params->theta_dev, sstat, gw.route,
-                R, gw.fb, gw.fb + 2 * S + 1, nint, srec, gw.hull, kn->kmax, d->nsp, d->d_adj_prefix, scal, mom);
+                Rc, gw.fb, gw.fb + 2 * S + 1, nint, srec, gw.hull, kn->kmax, d->nsp, d->d_adj_prefix, scal, mom,
+                d->adj_bins);
             // the states whose FP32 sums left the FP32 range (flagged by both passes above): all
             // their bins again, FP64 sums, on a resident grid of 16-warp CTAs
             const size_t smf = range_smem(d, kn->kmax, 16);
@@ -1569,23 +1610,23 @@ cudaError_t launch_adjoint(const lisa_data* d, bool fp32, const lisa_params* par
                 return cudaErrorInvalidValue;
             adjoint_range_kernel<C, H, B, kFallback><<<d->n_sm * std::max(occ, 1), 512, smf, sm>>>(
                 S, d->d_state_ds, d->d_ds, d->d_rec32, d->d_xlo32, d->d_elllo32, params->theta_dev, sstat,
-                gw.fb + S, R, gw.fb, gw.fb + 2 * S + 2, nint, srec, nullptr, kn->kmax, d->nsp, d->d_adj_prefix, scal,
-                mom);
+                gw.fb + S, Rf, gw.fb, gw.fb + 2 * S + 2, nint, srec, nullptr, kn->kmax, d->nsp, d->d_adj_prefix, scal,
+                mom, d->adj_bins);
         } else
             adjoint_fp64_kernel<C, H, B><<<grid, 128, 0, sm>>>(d->d_adj_units, d->n_adj_units, d->d_ds, d->d_rec64,
                                                                params->theta_dev, sstat, nint,
                                                                static_cast<const double*>(srec), kn->kmax, d->nsp,
-                                                               d->d_adj_prefix, scal, mom);
+                                                               d->d_adj_prefix, scal, mom, d->adj_bins);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     } else {
         prof_mark(d, prof, 1, sm);
     }
     prof_mark(d, prof, 2, sm);
-    const unsigned eb = (unsigned)((d->n_states + 3) / 4);
-    adjoint_epilogue_kernel<C, H, B><<<eb, 128, 0, sm>>>(
-        S, d->d_state_ds, d->d_ds, sstat, params->theta_dev, kn->count_dev, kn->x_dev, kn->w_dev, kn->kmax, kn->kind,
-        d->nsp, d->d_adj_prefix, scal, mom, d->d_rec32, d->d_rec64, srec, fp32 ? 1 : 0, out, grad, gw.fb);
+    const unsigned eb = (unsigned)((d->n_states * d->nsp + 3) / 4);
+    adjoint_epilogue_kernel<<<eb, 128, 0, sm>>>(
+        S, H ? 1 : 0, B ? 1 : 0, d->d_state_ds, d->d_ds, sstat, params->theta_dev, kn->count_dev, kn->x_dev, kn->w_dev, kn->kmax, kn->kind,
+        d->nsp, d->d_adj_prefix, scal, mom, d->d_rx32, d->d_rx64, srec, fp32 ? 1 : 0, out, grad, gw.fb);
     const cudaError_t e = cudaGetLastError();
     prof_mark(d, prof, 3, sm);
     if (prof) d->prof_valid = true;

@@ -73,7 +73,17 @@ constexpr unsigned kWaitLimit = 1u << 20;   // bounded spin on an mbarrier (then
 constexpr int kErrTimeout = 1;              // workspace error word: a bounded wait gave up
 constexpr int kMaxTileBins = 2048;          // 2 staged tiles x 48 B/bin must fit in 227 KB
 constexpr int kMaxTileBinsFull = 1024;      // dense covariance: 2 staged tiles x 64 B/bin
-constexpr int kAdjBins = 2048;              // bins per (state, range) in the adjoint
+// Bins per (state, range) of the adjoint: kAdjBins, halved down to kAdjMinBins for data objects whose
+// units (range x 32 states, one warp each) would not fill the GPU.  A unit walks its bins one after
+// the other, so with few units the walk's length is the kernel's time: A, E, 2,000 bins, 128 states has
+// 4 units of 2,000 bins (461 us) or 64 of 128 bins (121 us).  kAdjMinBins is the number of bins between two
+// flushes of the FP32 chunk sums, so the chunk sums are the same for every range size.  The line:
+// kAdjWarpsPerSm warps per SM is the occupancy of the FP32 kernel (3 CTAs of 4 warps); with that many
+// units longer ranges are better (fewer interval searches and moment slots: 131,072 bins, 2,048 states
+// took 1.66 ms at 2,048-bin ranges and 1.80 ms at 1,024).
+constexpr int kAdjBins = 2048;
+constexpr int kAdjMinBins = 128;
+constexpr int kAdjWarpsPerSm = 12;
 // Work balance of the fused kernel: an item (a tile of bins x a chunk of states) costs
 // (bins + kKnotBinsPerDecade x its width in log10 f) per state.  The second term stands for the
 // interval advances: knots are drawn uniformly in log10 f, so the low-frequency tiles (few bins,
@@ -96,7 +106,7 @@ struct WorkItem {
 };
 static_assert(sizeof(WorkItem) == 32, "WorkItem layout");
 
-// One unit of the adjoint: a range of kAdjBins bins of one dataset and up to 32 of its states
+// One unit of the adjoint: a range of adj_bins bins of one dataset and up to 32 of its states
 // (one warp, lanes = states).
 struct AdjUnit {
     int32_t ds, rho, s0, ns;
@@ -110,7 +120,8 @@ struct DatasetDev {
     int64_t psd_base;        // first element of the dataset's states in a model-PSD output
     int32_t s0, ns;          // state range
     int32_t ntiles;          // tiles of tile_bins bins
-    int32_t nranges;         // adjoint ranges of kAdjBins bins
+    int32_t nranges;         // adjoint ranges of adj_bins bins
+    int32_t rbase;           // first range in the range-bound tables
     double x_lo, x_hi;       // edge knot positions
     double xb_min, xb_max;   // log10 f of the first and last bin
     double f_ref;
@@ -155,6 +166,11 @@ struct lisa_data {
     int64_t n_adj_units = 0;
     int64_t* d_adj_prefix = nullptr; // [n_states] adjoint ranges of all earlier states
     int64_t adj_ranges = 0;          // sum over states of their dataset's ranges
+    int32_t adj_bins = lisa::kAdjBins;   // bins per range: kAdjBins / 2^k, at least kAdjMinBins
+    // log10 f of the first and last bin of every range (all datasets): of the FP32 table's x and
+    // of the FP64 table's
+    double2* d_rx32 = nullptr;
+    double2* d_rx64 = nullptr;
     int64_t n_items = 0;
     int64_t n_partials = 0;          // sum over datasets of states x tiles
     // per-kernel timing of lisa_psd_loglike (lisa_data_set_profiling): events around the main,

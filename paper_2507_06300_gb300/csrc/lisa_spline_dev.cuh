@@ -108,6 +108,7 @@ __device__ __forceinline__ void pcr_solve(T (&A)[2], T (&B)[2], T (&Cc)[2], T (&
         shift2(B[0], B[1], dd, Bp[0], Bp[1]);
         shift2(Cc[0], Cc[1], dd, Cp[0], Cp[1]);
         shift2(Rr[0], Rr[1], dd, Rp[0], Rp[1]);
+#pragma unroll
         for (int q = 0; q < 2; ++q) {
             const int j = lane + 32 * q;
             const bool lo_ok = j - dd >= 0 && j - dd < K;
@@ -264,13 +265,16 @@ __device__ __forceinline__ void warp_build_spline(WarpSpline<T>& W, const double
     shift2(xd[0], xd[1], 1, xn[0], xn[1]);
     shift2(yd[0], yd[1], 1, yn[0], yn[1]);
     T* ih = W.ih;
+#pragma unroll
     for (int q = 0; q < 2; ++q) {
         x[q] = T(xd[q]);
         y[q] = T(yd[q]);
     }
     h[1] = ih[1] = T(1);
     m[1] = T(0);
-    for (int q = 0; q < (K > 32 ? 2 : 1); ++q) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        if (q >= (K > 32 ? 2 : 1)) break;   // warp-uniform
         const int j = lane + 32 * q;
         if (j < K - 1) {
             h[q] = T(xn[q] - xd[q]);
@@ -290,7 +294,9 @@ __device__ __forceinline__ void warp_build_spline(WarpSpline<T>& W, const double
     const int nq = K > 32 ? 2 : 1;   // the second lane slot is only used by splines with K > 32
     if (K < 4) {
         // Sec. III.A: fewer than two in-between knots -> linear interpolant
-        for (int q = 0; q < nq; ++q) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            if (q >= nq) break;   // warp-uniform
             ca[q] = y[q];
             cb[q] = m[q];
             cc[q] = T(0);
@@ -304,6 +310,7 @@ __device__ __forceinline__ void warp_build_spline(WarpSpline<T>& W, const double
         shift2(h[0], h[1], -1, hm[0], hm[1]);
         shift2(m[0], m[1], -1, mm[0], mm[1]);
         T A[2], B[2], Cc[2], Rr[2];
+#pragma unroll
         for (int q = 0; q < 2; ++q) {
             const int j = lane + 32 * q;
             if (j >= 1 && j <= K - 2) {
@@ -320,9 +327,13 @@ __device__ __forceinline__ void warp_build_spline(WarpSpline<T>& W, const double
         }
         pcr_solve(A, B, Cc, Rr, K);
         T Mn[2];
-        for (int q = 0; q < nq; ++q) W.d2[q] = Rr[q] / B[q];
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+            if (q < nq) W.d2[q] = Rr[q] / B[q];
         shift2(W.d2[0], W.d2[1], 1, Mn[0], Mn[1]);
-        for (int q = 0; q < nq; ++q) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            if (q >= nq) break;   // warp-uniform
             const T M = W.d2[q];
             ca[q] = y[q];
             cb[q] = m[q] - h[q] * (T(2) * M + Mn[q]) * T(1.0 / 6.0);
@@ -338,12 +349,16 @@ __device__ __forceinline__ void warp_build_spline(WarpSpline<T>& W, const double
         const T m_0 = bcast(m[0], m[1], 0), m_1 = bcast(m[0], m[1], 1);
         const T m_Km2 = bcast(m[0], m[1], K - 2), m_Km3 = bcast(m[0], m[1], K - 3);
         T sn[2];
-        for (int q = 0; q < nq; ++q) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            if (q >= nq) break;   // warp-uniform
             const int j = lane + 32 * q;
             W.d2[q] = (j < K) ? akima_slope(j, K, mm2[q], mm1[q], m[q], mp1[q], m_0, m_1, m_Km2, m_Km3) : T(0);
         }
         shift2(W.d2[0], W.d2[1], 1, sn[0], sn[1]);
-        for (int q = 0; q < nq; ++q) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            if (q >= nq) break;   // warp-uniform
             const T sl = W.d2[q];
             ca[q] = y[q];
             cb[q] = sl;
