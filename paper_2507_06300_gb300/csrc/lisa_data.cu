@@ -238,37 +238,79 @@ int pow2ceil(int v) {
 // each CTA a contiguous, cost-balanced block of it, so a CTA mostly walks consecutive tiles of
 // the same states; otherwise the items are assigned longest-first (knot-aware cost) to the
 // least-loaded CTA and each CTA's share is laid out contiguously.
+//
+// Problems with few items (kMinItemsPerSm per SM or fewer) split each item into nseg segments, down to
+// one FP32 chunk (64 bins) per thread: A, E, 2,000 bins, 128 states has 4 items of 512 bins (127 us in
+// the fused kernel) or 32 of 64 bins (45 us).  The line: kMinItemsPerSm CTAs of 128 threads already
+// give every scheduler of the GPU its warps; more items only repeat the interval search.  A split
+// keeps the forward workspace within LISA_NOALLOC_SCRATCH_BYTES, so the allocation-free entry
+// point takes every problem that it takes unsplit.
 lisa_status rebuild_work(lisa_data* d) {
     const lisa_tiling& t = d->tiling;
     std::vector<WorkItem> items;
-    int64_t pbase = 0;
+    auto lanes = [&](const DatasetDev& D) { return std::max(1, std::min(t.states_per_cta, pow2ceil(D.ns))); };
+    // layout for a number of segments: items, partial slots, units of the compensated kernel
+    auto lay_out = [&](int nseg) {
+        int64_t n_items = 0;
+        d->nseg = nseg;
+        d->rt_bins = std::max(kSegBins, t.tile_bins / nseg / 32 * 32);
+        d->stage_bins = 0;
+        d->n_partials = d->n_units = 0;
+        for (DatasetDev& D : d->h_ds) {
+            const int32_t ntiles = (int32_t)((D.npad + t.tile_bins - 1) / t.tile_bins);
+            D.nslots = ntiles * nseg;
+            D.nrt = (int32_t)((D.npad + d->rt_bins - 1) / d->rt_bins);
+            D.pbase = d->n_partials;
+            d->n_partials += (int64_t)D.ns * D.nslots;
+            d->n_units += (int64_t)D.ns * D.nrt;
+            if (D.ns == 0 || D.npad == 0) continue;
+            const int sc = lanes(D), R = kThreads32 / sc;
+            n_items += (int64_t)ntiles * nseg * ((D.ns + sc - 1) / sc);
+            // one row: the item's bins are contiguous and staged alone; more rows: the whole tile
+            // (and, for later segments, the pair block before them)
+            d->stage_bins = std::max(d->stage_bins, R == 1 && nseg > 1
+                                                        ? std::min(t.tile_bins, seg_bins(t.tile_bins, 1, nseg) + 2)
+                                                        : t.tile_bins);
+        }
+        if (d->stage_bins == 0) d->stage_bins = t.tile_bins;
+        return n_items;
+    };
+    int max_seg = 1;   // segments of one chunk in the longest run
+    for (const DatasetDev& D : d->h_ds)
+        if (D.ns > 0)
+            max_seg = std::max(max_seg, (seg_bins(t.tile_bins, kThreads32 / lanes(D), 1) + kSegBins - 1) / kSegBins);
+    int64_t n_items = lay_out(1);
+    const size_t ws1 = ws_fwd_bytes(d);
+    for (int nseg = 2; n_items <= (int64_t)kMinItemsPerSm * d->n_sm && nseg < 2 * max_seg; nseg *= 2) {
+        n_items = lay_out(nseg);
+        if (ws_fwd_bytes(d) > std::max((size_t)LISA_NOALLOC_SCRATCH_BYTES / 2, ws1)) {
+            lay_out(nseg / 2);
+            break;
+        }
+    }
+    items.reserve((size_t)n_items);
     for (int k = 0; k < d->n_datasets; ++k) {
-        DatasetDev& D = d->h_ds[k];
-        D.ntiles = (int32_t)((D.npad + t.tile_bins - 1) / t.tile_bins);
-        D.pbase = pbase;
-        pbase += (int64_t)D.ns * D.ntiles;
+        const DatasetDev& D = d->h_ds[k];
         if (D.ns == 0 || D.npad == 0) continue;
-        int sc = std::min(t.states_per_cta, pow2ceil(D.ns));
-        sc = std::max(sc, 1);
+        const int sc = lanes(D);
         for (int32_t s = 0; s < D.ns; s += sc) {
-            for (int32_t tile = 0; tile < D.ntiles; ++tile) {
-                int64_t b0 = D.bin0 + (int64_t)tile * t.tile_bins;
-                int32_t nb = (int32_t)std::min<int64_t>(t.tile_bins, D.bin0 + D.npad - b0);
-                WorkItem w;
+            for (int32_t slot = 0; slot < D.nslots; ++slot) {
+                const int64_t b0 = D.bin0 + (int64_t)(slot / d->nseg) * t.tile_bins;
+                WorkItem w = {};
                 w.bin0 = b0;
-                w.nb = nb;
+                w.nb = (int16_t)std::min<int64_t>(t.tile_bins, D.bin0 + D.npad - b0);
                 w.s0 = D.s0 + s;
-                w.ns = std::min(sc, D.ns - s);
-                w.sc = sc;
-                w.tile = tile;
+                w.ns = (int16_t)std::min(sc, D.ns - s);
+                w.sc = (int16_t)sc;
+                w.slot = slot;
+                w.seg = (int16_t)(slot % d->nseg);
                 w.ds = k;
                 items.push_back(w);
             }
         }
     }
-    d->n_partials = pbase;
     const int occ = t.ctas_per_sm > 0 ? t.ctas_per_sm : fused_ctas_per_sm(d, t);
-    const int grid = std::max(1, d->n_sm * std::max(occ, 1));
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(d->n_sm * std::max(occ, 1), (int64_t)items.size()));
     // contiguous blocks pay off when a CTA has many items and each thread takes few bins from an
     // item (small state chunks: the per-item interval search dominates); with a few items per CTA
     // or wide items, cutting a handful of tiles by cost balances poorly, and a longest-first
@@ -291,7 +333,7 @@ lisa_status rebuild_work(lisa_data* d) {
         const DatasetDev& D = d->h_ds[w.ds];
         const int64_t a = w.bin0 - D.bin0, e = a + w.nb;
         const double dx = D.nbins > 0 ? x_at(w.ds, e) - x_at(w.ds, a) : 0.0;
-        return ((double)w.nb + kKnotBinsPerDecade * dx) * (double)w.ns;
+        return ((double)w.nb + kKnotBinsPerDecade * dx) * (double)w.ns;   // (a tile's segments alike)
     };
     std::vector<int32_t> cta_first((size_t)grid + 1, 0);
     if (d->fblocks) {
@@ -334,7 +376,7 @@ lisa_status rebuild_work(lisa_data* d) {
             const WorkItem &x = items[a], &y = items[b];
             if (x.ds != y.ds) return x.ds < y.ds;
             if (x.s0 != y.s0) return x.s0 < y.s0;
-            return x.tile < y.tile;
+            return x.slot < y.slot;
         });
         std::vector<WorkItem> sorted(items.size());
         for (size_t q = 0; q < items.size(); ++q) {
@@ -359,7 +401,7 @@ lisa_status rebuild_work(lisa_data* d) {
         cudaMemcpy(d->d_cta_first, cta_first.data(), cta_first.size() * sizeof(int32_t), cudaMemcpyHostToDevice) !=
             cudaSuccess)
         return LISA_ERR_CUDA;
-    // device copy of the dataset table (ntiles / pbase changed)
+    // device copy of the dataset table (slots changed)
     if (cudaMemcpy(d->d_ds, d->h_ds.data(), d->h_ds.size() * sizeof(DatasetDev),
                    cudaMemcpyHostToDevice) != cudaSuccess)
         return LISA_ERR_CUDA;
@@ -522,7 +564,7 @@ lisa_status lisa_data_create(const lisa_data_desc* desc, lisa_stream_t stream, l
         X.xb_min = X.nbins ? std::log10(q.freq[X.rbin0]) : 0.0;
         X.xb_max = X.nbins ? std::log10(q.freq[X.rbin0 + X.nbins - 1]) : 0.0;
         X.f_ref = q.f_ref[k];
-        X.ntiles = 0;
+        X.nslots = X.nrt = 0;
         X.pbase = 0;
         X.psd_base = psd_base;
         psd_base += (int64_t)C * X.ns * X.nbins;

@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(kThreads)
                      const double* __restrict__ cross64, const double* __restrict__ theta,
                      const int32_t* __restrict__ sstat, const int32_t* __restrict__ nint,
                      const double* __restrict__ srec, int kmax, int nsp, const DatasetDev* __restrict__ ds,
-                     double* __restrict__ partial) {
+                     double* __restrict__ partial, int tile_bins, int nseg) {
     constexpr int NSP = 3 + (HAS_H ? 1 : 0) + 3;
     constexpr int ZB = 3 + (HAS_H ? 1 : 0);   // first correlation spline
     __shared__ double red[kThreads];
@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(kThreads)
         const bool active = ls < w.ns && sstat[s] == 0;
         double acc = 0.0;
         if (active) {
-            const int lo = (r * w.nb) / R, hi = ((r + 1) * w.nb) / R;
+            const int lo = item_lo(w, r, R, tile_bins, nseg), hi = item_lo(w, r + 1, R, tile_bins, nseg);
             if (lo < hi) {
                 const double* th = theta + (size_t)s * LISA_N_THETA;
                 const double ao2 = th[0] * th[0], at2 = th[1] * th[1], lA = th[2], n1 = th[3];
@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(kThreads)
             double sum = 0.0;
             for (int q = 0; q < R; ++q) sum += red[ls + q * sc];
             const DatasetDev& D = ds[w.ds];
-            partial[D.pbase + (int64_t)(s - D.s0) * D.ntiles + w.tile] = sum;
+            partial[D.pbase + (int64_t)(s - D.s0) * D.nslots + w.slot] = sum;
         }
         __syncthreads();
     }
@@ -255,7 +255,8 @@ __global__ void __launch_bounds__(kFullThreads, 4)
                      const double* __restrict__ theta,
                      const int32_t* __restrict__ sstat, const float* __restrict__ kxr,
                      const float* __restrict__ srec, int kmax, int nsp, const DatasetDev* __restrict__ ds,
-                     double* __restrict__ partial, int* __restrict__ err, int tile_bins, unsigned wait_limit) {
+                     double* __restrict__ partial, int* __restrict__ err, int tile_bins, int nseg,
+                     unsigned wait_limit) {
     constexpr int NSP = 3 + (HAS_H ? 1 : 0) + 3;
     constexpr int ZB = 3 + (HAS_H ? 1 : 0);
     constexpr float kL2 = 3.32192809488736234787f;   // log2(10): the records' coefficients carry it
@@ -303,9 +304,16 @@ __global__ void __launch_bounds__(kFullThreads, 4)
         const int r = tid / sc;
         const int s = w.s0 + ls;
         const bool active = ok && ls < w.ns && (sstat[s] & kUserBits) == 0;
-        const int lo = (r * w.nb) / R, hi = ((r + 1) * w.nb) / R;
+        int lo = (r * w.nb) / R, hi = ((r + 1) * w.nb) / R;
+        int run = (w.nb + R - 1) / R;                          // the longest of the CTA
+        if (nseg > 1) {                                        // this item's segment of the run
+            const int len = seg_bins(tile_bins, R, nseg);
+            lo += w.seg * len;
+            hi = min(hi, lo + len);
+            run = min(run, len);
+        }
         const bool run_bins = active && lo < hi;
-        const int nch = ((w.nb + R - 1) / R + kFullChunk - 1) / kFullChunk;   // uniform over the CTA
+        const int nch = (run + kFullChunk - 1) / kFullChunk;   // uniform over the CTA
         s_far[tid] = 0.0;
         ff accf = {0.f, 0.f};
         const StateParams p = prm[run_bins ? s : w.s0];
@@ -539,7 +547,7 @@ __global__ void __launch_bounds__(kFullThreads, 4)
             double sum = red[ls];
             for (int q = 1; q < R; ++q) sum += red[ls + q * sc];
             const DatasetDev& D = ds[w.ds];
-            partial[D.pbase + (int64_t)(s - D.s0) * D.ntiles + w.tile] = sum;
+            partial[D.pbase + (int64_t)(s - D.s0) * D.nslots + w.slot] = sum;
         }
         __syncthreads();   // the buffer read in this iteration is refilled in the next one
     }
@@ -564,7 +572,8 @@ cudaError_t launch_full(const lisa_data* d, bool fp32, const double* theta, cons
         if (grid > d->n_items) grid = d->n_items;
         kern<<<(unsigned)(grid < 1 ? 1 : grid), kFullThreads, smem, sm>>>(
             d->d_items, (int)d->n_items, d->d_rec32, d->d_cross32, d->d_xlo32, d->d_elllo32, prm, theta, sstat, kxr,
-            static_cast<const float*>(srec), kmax, d->nsp, d->d_ds, partial, err, d->tiling.tile_bins, d->wait_limit);
+            static_cast<const float*>(srec), kmax, d->nsp, d->d_ds, partial, err, d->tiling.tile_bins, d->nseg,
+            d->wait_limit);
         return cudaGetLastError();
     }
     auto kern = full_fp64_kernel<H, B>;
@@ -576,7 +585,7 @@ cudaError_t launch_full(const lisa_data* d, bool fp32, const double* theta, cons
     kern<<<(unsigned)(grid < 1 ? 1 : grid), kThreads, 0, sm>>>(d->d_items, (int)d->n_items, d->d_rec64,
                                                                 d->d_cross64, theta, sstat, nint,
                                                                 static_cast<const double*>(srec), kmax, d->nsp,
-                                                                d->d_ds, partial);
+                                                                d->d_ds, partial, d->tiling.tile_bins, d->nseg);
     return cudaGetLastError();
 }
 

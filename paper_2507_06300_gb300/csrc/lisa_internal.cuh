@@ -90,21 +90,34 @@ constexpr int kAdjWarpsPerSm = 12;
 // wide in log10 f) hold most of them, and each advance stalls its warp on record loads.
 constexpr double kKnotBinsPerDecade = 2500.0;
 constexpr int kXsStride = 32;               // bins between the host copies of log10 f
+constexpr int kMinItemsPerSm = 2;            // fewer items per SM than this are split into segments
 constexpr int kBlockItemsPerCta = 16;       // contiguous blocks need this many items per CTA
 constexpr double kBlockThreadBins = 128.0;  // and fewer bins per thread and item than this
 
 // One unit of work of the fused kernels: a tile of bins of one dataset and a chunk of its
 // states.  Threads map to (state lane, bin sub-range): lane = tid % sc, range = tid / sc.
+// A small problem's items are split further, into segments of every thread's run of bins: segment
+// seg takes the seg_bins(...) bins of each run from seg times that, a multiple of the FP32 chunk
+// (kSegBins), so that the chunk sums are those of the unsplit item.
 struct WorkItem {
-    int64_t bin0;   // first bin (global index)
-    int32_t nb;     // bins in the tile
+    int64_t bin0;   // first bin of the tile (global index)
     int32_t s0;     // first state (global index)
-    int32_t ns;     // states in the chunk (<= sc)
-    int32_t sc;     // state lanes of this dataset's items (power of two, <= kMaxStatesPerItem)
-    int32_t tile;   // tile index within the dataset
+    int32_t slot;   // partial slot within the state's row: tile index * nseg + seg
     int32_t ds;     // dataset index
+    int16_t nb;     // bins in the tile
+    int16_t ns;     // states in the chunk (<= sc)
+    int16_t sc;     // state lanes of this dataset's items (power of two, <= kMaxStatesPerItem)
+    int16_t seg;    // segment of the runs
+    int32_t pad;
 };
 static_assert(sizeof(WorkItem) == 32, "WorkItem layout");
+
+constexpr int kSegBins = 64;   // bins of an FP32 chunk sum of the fused kernel (a multiple of the dense one's)
+// Bins of a thread's run in one segment: the run of a full tile with R rows, cut into nseg.
+__host__ __device__ inline int seg_bins(int tile_bins, int R, int nseg) {
+    const int run = 2 * ((tile_bins / 2 + R - 1) / R);
+    return ((run + nseg - 1) / nseg + kSegBins - 1) / kSegBins * kSegBins;
+}
 
 // One unit of the adjoint: a range of adj_bins bins of one dataset and up to 32 of its states
 // (one warp, lanes = states).
@@ -116,10 +129,11 @@ struct DatasetDev {
     int64_t bin0, nbins;     // bin range: bin0 in padded indexing, nbins real bins
     int64_t npad;            // nbins rounded up to even (bins [bin0, bin0 + npad) in the tables)
     int64_t rbin0;           // first bin in the caller's (unpadded) arrays
-    int64_t pbase;           // first partial slot of the dataset (partials are [tile][state])
+    int64_t pbase;           // first partial slot of the dataset (partials are [state][slot])
     int64_t psd_base;        // first element of the dataset's states in a model-PSD output
     int32_t s0, ns;          // state range
-    int32_t ntiles;          // tiles of tile_bins bins
+    int32_t nslots;          // partial slots per state: tiles of tile_bins bins, times nseg
+    int32_t nrt;             // tiles of the compensated kernel (rt_bins bins)
     int32_t nranges;         // adjoint ranges of adj_bins bins
     int32_t rbase;           // first range in the range-bound tables
     double x_lo, x_hi;       // edge knot positions
@@ -172,7 +186,11 @@ struct lisa_data {
     double2* d_rx32 = nullptr;
     double2* d_rx64 = nullptr;
     int64_t n_items = 0;
-    int64_t n_partials = 0;          // sum over datasets of states x tiles
+    int64_t n_partials = 0;          // sum over datasets of states x slots
+    int64_t n_units = 0;             // sum over datasets of states x tiles of the compensated kernel
+    int32_t nseg = 1;                // segments per work item
+    int32_t stage_bins = 0;          // bins per staging buffer of the fused kernels
+    int32_t rt_bins = 0;             // bins per unit of the compensated kernel
     // per-kernel timing of lisa_psd_loglike (lisa_data_set_profiling): events around the main,
     // compensated and finalize kernels of the most recent uncaptured call
     cudaEvent_t prof_ev[4] = {nullptr, nullptr, nullptr, nullptr};
@@ -236,19 +254,20 @@ struct RobustEntry {
     uint32_t u0;        // first unit
     int32_t nt;         // live tiles (>= 1)
     int64_t b0;         // first bin of tile t0 (padded global index)
-    uint32_t p0;        // partial slot of (s, t0); tile t0 + k has slot p0 + k
-    int32_t nb_last;    // bins in tile t0 + nt - 1 (all earlier tiles hold tile_bins)
+    uint32_t pad;
+    int32_t nb_last;    // bins in tile t0 + nt - 1 (all earlier tiles hold rt_bins)
 };
 static_assert(sizeof(RobustEntry) == 32, "two int4");
 
 // Forward workspace: error flag (int32 at 0) and work-list counter (uint64 at 8) in the first
-// 256 bytes | FP64 partial sums [state][tile] of the fused kernel | StateParams [S] |
+// 256 bytes | FP64 partial sums [state][slot] of the fused kernel | StateParams [S] |
 // RobustEntry [S] | int32 entry of each state in the work list (-1: none) [S] | FP64 sums of the
 // compensated kernel, one per (state, tile) unit of the work list [up to states x tiles].  The
 // two kinds of partial sums live apart, so the two kernels may run at the same time; the
 // finalize kernel adds both in a fixed order.
 constexpr size_t kWsCounterOff = 8;
 inline size_t ws_partials_bytes(const lisa_data* d) { return align256(sizeof(double) * (size_t)d->n_partials); }
+inline size_t ws_rpart_bytes(const lisa_data* d) { return align256(sizeof(double) * (size_t)d->n_units); }
 inline size_t ws_prm_bytes(const lisa_data* d) { return align256(sizeof(StateParams) * (size_t)d->n_states); }
 inline size_t ws_rlist_bytes(const lisa_data* d) { return align256(sizeof(RobustEntry) * (size_t)d->n_states); }
 inline size_t ws_rent_bytes(const lisa_data* d) { return align256(sizeof(int32_t) * (size_t)d->n_states); }
@@ -262,7 +281,7 @@ inline WsLayout ws_layout(const lisa_data* d) {
     L.off_rlist = L.off_prm + ws_prm_bytes(d);
     L.off_rent = L.off_rlist + ws_rlist_bytes(d);
     L.off_rpart = L.off_rent + ws_rent_bytes(d);
-    L.bytes = L.off_rpart + ws_partials_bytes(d);
+    L.bytes = L.off_rpart + ws_rpart_bytes(d);
     return L;
 }
 inline size_t ws_fwd_bytes(const lisa_data* d) { return ws_layout(d).bytes; }

@@ -192,7 +192,7 @@ __device__ __forceinline__ float bin_x(const float* __restrict__ rec32, int64_t 
 __global__ void state_prep_kernel(int S, const double* __restrict__ theta, StateParams* __restrict__ prm,
                                   const int32_t* __restrict__ sstat, const float2* __restrict__ hull,
                                   const int32_t* __restrict__ state_ds, const DatasetDev* __restrict__ ds,
-                                  const float* __restrict__ rec32, int tile_bins,
+                                  const float* __restrict__ rec32, int rt_bins,
                                   unsigned long long* __restrict__ rcount, RobustEntry* __restrict__ rlist,
                                   int32_t* __restrict__ rent) {
     const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -222,7 +222,7 @@ __global__ void state_prep_kernel(int S, const double* __restrict__ theta, State
     if (!(__ldg(sstat + s) & kRouted)) return;   // the same word in every lane
     const DatasetDev& D = ds[__ldg(state_ds + s)];
     const float2 h = __ldg(hull + s);
-    const int nt = D.ntiles;
+    const int nt = D.nrt;
     const int64_t bend = D.bin0 + D.npad;
     // ta = first tile whose last bin has x >= h.x, tb = first tile whose first bin has x >= h.y;
     // the live tiles are [ta, tb).  Both searches run together, 32 samples per round.
@@ -231,8 +231,8 @@ __global__ void state_prep_kernel(int S, const double* __restrict__ theta, State
         const int sa = (ahi - alo + 31) >> 5, sb = (bhi - blo + 31) >> 5;
         const int tA = alo + lane * sa, tB = blo + lane * sb;
         bool pa = true, pb = true;
-        if (alo < ahi && tA < ahi) pa = bin_x(rec32, min(D.bin0 + (int64_t)(tA + 1) * tile_bins, bend) - 1) >= h.x;
-        if (blo < bhi && tB < bhi) pb = bin_x(rec32, D.bin0 + (int64_t)tB * tile_bins) >= h.y;
+        if (alo < ahi && tA < ahi) pa = bin_x(rec32, min(D.bin0 + (int64_t)(tA + 1) * rt_bins, bend) - 1) >= h.x;
+        if (blo < bhi && tB < bhi) pb = bin_x(rec32, D.bin0 + (int64_t)tB * rt_bins) >= h.y;
         const unsigned ma = __ballot_sync(0xffffffffu, pa), mb = __ballot_sync(0xffffffffu, pb);
         if (alo < ahi) search_narrow(alo, ahi, sa, ma);
         if (blo < bhi) search_narrow(blo, bhi, sb, mb);
@@ -244,9 +244,9 @@ __global__ void state_prep_kernel(int S, const double* __restrict__ theta, State
         e.t0 = alo;
         e.u0 = (uint32_t)(old & 0xffffffffull);
         e.nt = blo - alo;
-        e.b0 = D.bin0 + (int64_t)alo * tile_bins;
-        e.p0 = (uint32_t)(D.pbase + (int64_t)(s - D.s0) * nt + alo);
-        e.nb_last = (int32_t)min((int64_t)tile_bins, D.npad - (int64_t)(blo - 1) * tile_bins);
+        e.b0 = D.bin0 + (int64_t)alo * rt_bins;
+        e.pad = 0;
+        e.nb_last = (int32_t)min((int64_t)rt_bins, D.npad - (int64_t)(blo - 1) * rt_bins);
         rlist[old >> 32] = e;
         rent[s] = (int32_t)(old >> 32);
     }
@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(kThreads32, G == 8 ? 4 : (G == 4 ? 5 : 6))
                         const StateParams* __restrict__ prm, const int32_t* __restrict__ sstat,
                         const float* __restrict__ kxr, const float* __restrict__ srec, int kmax, int nsp,
                         const DatasetDev* __restrict__ ds, double* __restrict__ partial, int* __restrict__ err,
-                        int tile_bins, unsigned wait_limit, int skip_copies) {
+                        int tile_bins, int stage_bins, int nseg, unsigned wait_limit, int skip_copies) {
     constexpr int NSP = C + (HAS_H ? 1 : 0);
     constexpr int U = G / 2;                  // pair blocks per iteration of the knot-free loop
     constexpr int kChunkPairs = 32;           // pair blocks per FP32 partial sum (64 bins)
@@ -374,7 +374,7 @@ __global__ void __launch_bounds__(kThreads32, G == 8 ? 4 : (G == 4 ? 5 : 6))
     __shared__ unsigned s_hm[kThreads32];     // bit a: spline a ill-conditioned; kLocated: set up
     const int tid = threadIdx.x;
     const int lane = tid & 31;
-    const size_t stage_floats = (size_t)tile_bins * kRec;
+    const size_t stage_floats = (size_t)stage_bins * kRec;
     // the compensated kernel, launched next as a programmatic dependent, may place its CTAs as
     // soon as this grid's CTAs leave SMs (it does not read what this kernel writes)
     asm volatile("griddepcontrol.launch_dependents;");
@@ -387,12 +387,27 @@ __global__ void __launch_bounds__(kThreads32, G == 8 ? 4 : (G == 4 ? 5 : 6))
     const int step = cta_first ? 1 : (int)gridDim.x;
     const int i_begin = cta_first ? cta_first[blockIdx.x] : (int)blockIdx.x;
     const int i_end = cta_first ? cta_first[blockIdx.x + 1] : n_items;
+    // pair blocks [a, b) of the tile that an item's table holds: its segment where a thread's run is
+    // the whole tile (one row), with the block before it (see locate's call), else the tile
+    auto staged = [&](const WorkItem& w, int& a, int& b) {
+        a = 0;
+        b = w.nb >> 1;
+        if (w.sc == kThreads32 && nseg > 1) {
+            const int len = seg_bins(tile_bins, 1, nseg) >> 1;
+            a = min(b, w.seg * len);
+            b = min(b, a + len);
+            a -= a < b && w.seg > 0;
+        }
+    };
     auto stage = [&](int q, int item) {   // one bulk copy of item's bin table into buffer q
         const WorkItem w = items[item];
-        const unsigned bytes = (unsigned)w.nb * kRec * sizeof(float);
+        int a, b;
+        staged(w, a, b);
+        const unsigned bytes = (unsigned)(b - a) * kPairRec * sizeof(float);
         mbar_expect_tx(&full[q], bytes);
-        bulk_copy_g2s(reinterpret_cast<float*>(smem) + q * stage_floats, rec32 + (w.bin0 >> 1) * kPairRec, bytes,
-                      &full[q]);
+        if (bytes > 0)
+            bulk_copy_g2s(reinterpret_cast<float*>(smem) + q * stage_floats, rec32 + ((w.bin0 >> 1) + a) * kPairRec,
+                          bytes, &full[q]);
     };
     if (tid == 0) {
         s_fail = 0;
@@ -431,12 +446,15 @@ __global__ void __launch_bounds__(kThreads32, G == 8 ? 4 : (G == 4 ? 5 : 6))
             s_fail = 1;
             atomicOr(err, kErrTimeout);
         }
-        const float* tb = reinterpret_cast<const float*>(smem) + b * stage_floats;
+        // the staged part starts at pair block st_a of the tile; tb is where block 0 would lie
+        int st_a, st_b;
+        staged(w, st_a, st_b);
+        const float* tb = reinterpret_cast<const float*>(smem) + b * stage_floats - st_a * kPairRec;
         const float4* tb4 = reinterpret_cast<const float4*>(tb);
         bool carry = false;
         if (k > 0) {
             const WorkItem pw = items[it - step];
-            carry = w.ds == pw.ds && w.s0 == pw.s0 && w.tile == pw.tile + 1;
+            carry = w.ds == pw.ds && w.s0 == pw.s0 && w.slot == pw.slot + 1;
         }
         const int sc = w.sc;
         const int R = kThreads32 / sc;
@@ -449,7 +467,12 @@ __global__ void __launch_bounds__(kThreads32, G == 8 ? 4 : (G == 4 ? 5 : 6))
         ff accf = {0.f, 0.f};
         if (active) {
             const int np = w.nb >> 1;                          // pair blocks in the tile
-            const int plo = (r * np) / R, phi = ((r + 1) * np) / R;
+            int plo = (r * np) / R, phi = ((r + 1) * np) / R;
+            if (nseg > 1) {                                    // this item's segment of the run
+                const int len = seg_bins(tile_bins, R, nseg) >> 1;
+                plo += w.seg * len;
+                phi = min(phi, plo + len);
+            }
             if (plo < phi) {
                 const float4 q0 = __ldg(reinterpret_cast<const float4*>(prm + s));
                 const float ao2 = q0.x, at2 = q0.y, Af = HAS_H ? q0.z : 0.f, n1 = q0.w;
@@ -532,7 +555,9 @@ __global__ void __launch_bounds__(kThreads32, G == 8 ? 4 : (G == 4 ? 5 : 6))
                 // intervals carry over from this thread's previous item when it held the
                 // preceding tile of the same states (a thread whose row was empty there keeps
                 // those of an earlier tile, which lie to the left: advancing finds the new ones)
-                if (!(carry && (s_hm[tid] & kLocated))) locate(fld(tb, 2 * plo, 0));
+                // a later segment of a run finds them at the bin before its first one, as the unsplit
+                // run would arrive there: a knot between the two bins then takes the same path
+                if (!(carry && (s_hm[tid] & kLocated))) locate(fld(tb, 2 * plo - (w.seg > 0 ? 1 : 0), 0));
                 int ip = plo;
                 while (ip < phi) {
                     const int pc0 = ip;
@@ -599,7 +624,7 @@ __global__ void __launch_bounds__(kThreads32, G == 8 ? 4 : (G == 4 ? 5 : 6))
         const DatasetDev& D = ds[w.ds];
         if (R == 1) {
             if (active)
-                partial[D.pbase + (int64_t)(s - D.s0) * D.ntiles + LISA_IDX(w.tile, D.ntiles)] =
+                partial[D.pbase + (int64_t)(s - D.s0) * D.nslots + LISA_IDX(w.slot, D.nslots)] =
                     (double)accf.hi + (double)accf.lo;
         } else {
             red[tid] = make_float2(accf.hi, accf.lo);
@@ -607,7 +632,7 @@ __global__ void __launch_bounds__(kThreads32, G == 8 ? 4 : (G == 4 ? 5 : 6))
             if (r == 0 && active) {
                 ff sum = {red[ls].x, red[ls].y};
                 for (int q = 1; q < R; ++q) sum = ff_add(sum, ff{red[ls + q * sc].x, red[ls + q * sc].y});
-                partial[D.pbase + (int64_t)(s - D.s0) * D.ntiles + LISA_IDX(w.tile, D.ntiles)] =
+                partial[D.pbase + (int64_t)(s - D.s0) * D.nslots + LISA_IDX(w.slot, D.nslots)] =
                     (double)sum.hi + (double)sum.lo;
             }
             __syncthreads();   // red is rewritten by the next item
@@ -961,7 +986,7 @@ __global__ void __launch_bounds__(kThreads)
     loglike_fp64_kernel(const WorkItem* __restrict__ items, int n_items, const double* __restrict__ rec64,
                         const double* __restrict__ theta, const int32_t* __restrict__ sstat,
                         const int32_t* __restrict__ nint, const double* __restrict__ srec, int kmax, int nsp,
-                        const DatasetDev* __restrict__ ds, double* __restrict__ partial) {
+                        const DatasetDev* __restrict__ ds, double* __restrict__ partial, int tile_bins, int nseg) {
     constexpr int NSP = C + (HAS_H ? 1 : 0);
     __shared__ double red[kThreads];
     const int tid = threadIdx.x;
@@ -975,7 +1000,7 @@ __global__ void __launch_bounds__(kThreads)
         const bool active = ls < w.ns && sstat[s] == 0;
         double acc = 0.0;
         if (active) {
-            const int lo = (r * w.nb) / R, hi = ((r + 1) * w.nb) / R;
+            const int lo = item_lo(w, r, R, tile_bins, nseg), hi = item_lo(w, r + 1, R, tile_bins, nseg);
             if (lo < hi) {
                 const double* th = theta + (size_t)s * LISA_N_THETA;
                 const double ao2 = th[0] * th[0], at2 = th[1] * th[1], lA = th[2], n1 = th[3];
@@ -1026,7 +1051,7 @@ __global__ void __launch_bounds__(kThreads)
             double sum = 0.0;
             for (int q = 0; q < R; ++q) sum += red[ls + q * sc];
             const DatasetDev& D = ds[w.ds];
-            partial[D.pbase + (int64_t)(s - D.s0) * D.ntiles + w.tile] = sum;
+            partial[D.pbase + (int64_t)(s - D.s0) * D.nslots + w.slot] = sum;
         }
         __syncthreads();
     }
@@ -1047,9 +1072,9 @@ __global__ void finalize_kernel(int S, const int32_t* __restrict__ state_ds, con
         return;
     }
     const DatasetDev& D = ds[state_ds[s]];
-    const double* p = partial + D.pbase + (int64_t)(s - D.s0) * D.ntiles;
+    const double* p = partial + D.pbase + (int64_t)(s - D.s0) * D.nslots;
     double sum = 0.0;
-    for (int t = lane; t < D.ntiles; t += 32) sum += p[t];
+    for (int t = lane; t < D.nslots; t += 32) sum += p[t];
     // FP32 mode: the compensated kernel's sums of this state's units, if it has any
     const int e = fp32 ? rent[s] : -1;
     if (e >= 0) {
@@ -1126,12 +1151,13 @@ cudaError_t launch_fp32_g(const lisa_data* d, const StateParams* prm, const int3
                           int kmax,
                           double* partial, double* rpart, int* err, cudaStream_t sm, bool prof) {
     auto kern = loglike_fp32_kernel<C, H, B, G>;
-    const size_t smem = 2 * (size_t)d->tiling.tile_bins * kRec * sizeof(float);
+    const size_t smem = 2 * (size_t)d->stage_bins * kRec * sizeof(float);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     kern<<<d->fgrid, kThreads32, smem, sm>>>(d->d_items, (int)d->n_items, d->d_cta_first,
                                               d->d_rec32, prm, sstat, kxr, srec, kmax, d->nsp, d->d_ds, partial, err,
-                                              d->tiling.tile_bins, d->wait_limit, d->test_skip_copies);
+                                              d->tiling.tile_bins, d->stage_bins, d->nseg, d->wait_limit,
+                                              d->test_skip_copies);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     prof_mark(d, prof, 1, sm);
@@ -1152,7 +1178,7 @@ cudaError_t launch_fp32_g(const lisa_data* d, const StateParams* prm, const int3
     attr[0].val.programmaticStreamSerializationAllowed = prof ? 0 : 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, rk, rcount, rlist, d->tiling.tile_bins, (const float*)d->d_rec32,
+    e = cudaLaunchKernelEx(&cfg, rk, rcount, rlist, d->rt_bins, (const float*)d->d_rec32,
                            (const float*)d->d_xlo32, (const float*)d->d_elllo32, prm, nint, srec, kmax, d->nsp, rpart,
                            err, d->wait_limit);
     if (e == cudaSuccess) e = cudaGetLastError();
@@ -1173,9 +1199,9 @@ int robust_occupancy() {
 }
 
 template <int C, bool H, bool B, int G>
-int occupancy_g(const lisa_tiling& t) {
+int occupancy_g(int stage_bins) {
     auto kern = loglike_fp32_kernel<C, H, B, G>;
-    const size_t smem = 2 * (size_t)t.tile_bins * kRec * sizeof(float);
+    const size_t smem = 2 * (size_t)stage_bins * kRec * sizeof(float);
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
         cudaGetLastError();
         return 1;
@@ -1189,19 +1215,19 @@ int occupancy_g(const lisa_tiling& t) {
 }
 
 template <int C, bool H, bool B>
-int occupancy_m(const lisa_tiling& t) {
+int occupancy_m(const lisa_tiling& t, int stage_bins) {
     switch (t.group) {
-        case 2: return occupancy_g<C, H, B, 2>(t);
-        case 8: return occupancy_g<C, H, B, 8>(t);
-        default: return occupancy_g<C, H, B, 4>(t);
+        case 2: return occupancy_g<C, H, B, 2>(stage_bins);
+        case 8: return occupancy_g<C, H, B, 8>(stage_bins);
+        default: return occupancy_g<C, H, B, 4>(stage_bins);
     }
 }
 
 template <int C>
-int occupancy_c(int sgwb, const lisa_tiling& t) {
-    if (sgwb == 0) return occupancy_m<C, false, false>(t);
-    if (sgwb == 1) return occupancy_m<C, true, false>(t);
-    return occupancy_m<C, true, true>(t);
+int occupancy_c(int sgwb, const lisa_tiling& t, int stage_bins) {
+    if (sgwb == 0) return occupancy_m<C, false, false>(t, stage_bins);
+    if (sgwb == 1) return occupancy_m<C, true, false>(t, stage_bins);
+    return occupancy_m<C, true, true>(t, stage_bins);
 }
 
 template <int C, bool H, bool B>
@@ -1225,7 +1251,7 @@ cudaError_t launch_fp64(const lisa_data* d, const double* theta, const int32_t* 
     auto kern = loglike_fp64_kernel<C, H, B>;
     const int grid = grid_for(kern, d, 0, kThreads);
     kern<<<grid, kThreads, 0, sm>>>(d->d_items, (int)d->n_items, d->d_rec64, theta, sstat, nint, srec, kmax,
-                                    d->nsp, d->d_ds, partial);
+                                    d->nsp, d->d_ds, partial, d->tiling.tile_bins, d->nseg);
     const cudaError_t e = cudaGetLastError();
     prof_mark(d, prof, 1, sm);
     prof_mark(d, prof, 2, sm);   // no compensated kernel in FP64 mode
@@ -1258,7 +1284,7 @@ cudaError_t dispatch_model(const lisa_data* d, bool fp32, const double* theta, c
 }  // namespace
 
 int fused_ctas_per_sm(const lisa_data* d, const lisa_tiling& t) {
-    return d->C == 3 ? occupancy_c<3>(d->sgwb_model, t) : occupancy_c<2>(d->sgwb_model, t);
+    return d->C == 3 ? occupancy_c<3>(d->sgwb_model, t, d->stage_bins) : occupancy_c<2>(d->sgwb_model, t, d->stage_bins);
 }
 
 template <int C>
@@ -1299,7 +1325,7 @@ lisa_status lisa_psd_loglike(const lisa_data* d, const lisa_params* params, cons
     if (buf_bytes < L.bytes || (reinterpret_cast<uintptr_t>(buf) & 255)) return LISA_ERR_WORKSPACE;
     if (ws_bytes < ws_fwd_bytes(d) || (reinterpret_cast<uintptr_t>(ws) & 255)) return LISA_ERR_WORKSPACE;
     // the compensated kernel's unit counter holds up to 2^32 - 1 (state, tile) units
-    if (fp32 && d->n_partials > (int64_t)0xffffffffLL) return LISA_ERR_SHAPE;
+    if (fp32 && d->n_units > (int64_t)0xffffffffLL) return LISA_ERR_SHAPE;
     if (d->n_states == 0) return LISA_SUCCESS;
     cudaStream_t sm = (cudaStream_t)stream;
     const char* base = static_cast<const char*>(buf);
@@ -1324,7 +1350,7 @@ lisa_status lisa_psd_loglike(const lisa_data* d, const lisa_params* params, cons
     if (fp32) {
         const int64_t threads = 32 * (int64_t)S;
         state_prep_kernel<<<(unsigned)((threads + 127) / 128), 128, 0, sm>>>(
-            S, params->theta_dev, prm, sstat, hull, d->d_state_ds, d->d_ds, d->d_rec32, d->tiling.tile_bins, rcount,
+            S, params->theta_dev, prm, sstat, hull, d->d_state_ds, d->d_ds, d->d_rec32, d->rt_bins, rcount,
             rlist, rent);
         if (cudaGetLastError() != cudaSuccess) return LISA_ERR_CUDA;
     }
