@@ -350,7 +350,7 @@ constexpr int kStages = 2;
 constexpr int kWarps32 = kThreads32 / 32;
 
 template <int C, bool HAS_H, bool BROKEN, int G>
-__global__ void __launch_bounds__(kThreads32, G == 8 ? 4 : (G == 4 ? 5 : 6))
+__global__ void __launch_bounds__(kThreads32, G == 2 ? 5 : 4)
     loglike_fp32_kernel(const WorkItem* __restrict__ items, int n_items, const int32_t* __restrict__ cta_first,
                         const float* __restrict__ rec32,
                         const StateParams* __restrict__ prm, const int32_t* __restrict__ sstat,
@@ -599,8 +599,37 @@ __global__ void __launch_bounds__(kThreads32, G == 8 ? 4 : (G == 4 ? 5 : 6))
                         for (; ip < pcend; ++ip, blk += kPairRec / 4) {
                             const float4 q0 = blk[0];
                             if (q0.y >= xmin) {
-                                acc2.x += scalar_bin(2 * ip);
-                                acc2.x += scalar_bin(2 * ip + 1);
+                                // the next record of every spline that passes a knot by the second
+                                // bin, all loads in flight at once (one spline after the other, each
+                                // load waited for, cost 1.4 % of the paper-scale step: 299 -> 295 us)
+                                float4 NA[NSP], NB[NSP];
+                                unsigned have = 0u;
+#pragma unroll
+                                for (int a = 0; a < NSP; ++a)
+                                    if (q0.y >= s_xr[a][tid]) {
+                                        const float4* q = rec(a, min(s_jj[a][tid] + 1, kmax));
+                                        NA[a] = __ldg(q);
+                                        NB[a] = __ldg(q + 1);
+                                        have |= 1u << a;
+                                    }
+#pragma unroll 1
+                                for (int e = 0; e < 2; ++e) {
+                                    const float x = e ? q0.y : q0.x;
+                                    if (x >= xmin) {
+#pragma unroll
+                                        for (int a = 0; a < NSP; ++a)
+                                            if (x >= s_xr[a][tid]) {
+                                                if ((have >> a) & 1u) {
+                                                    have &= ~(1u << a);
+                                                    install(a, min(s_jj[a][tid] + 1, kmax), NA[a], NB[a]);
+                                                }
+                                                advance(a, x);
+                                            }
+                                        xmin = nearest();
+                                    }
+                                    acc2.x += keep2.x * bin_term32p<C, HAS_H, BROKEN>(tb, 2 * ip + e, iv2, ao2, at2, n1,
+                                                                                      n2, Af);
+                                }
                             } else {
                                 acc2 = __ffma2_rn(keep2, pair_term32<C, HAS_H, BROKEN>(q0, blk, iv2, ao2_2, at2_2, n1,
                                                                                        n2, Af2, mx),
