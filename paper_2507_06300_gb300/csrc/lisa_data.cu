@@ -194,6 +194,8 @@ void release(lisa_data* d) {
     cudaFree(d->d_adj_prefix);
     cudaFree(d->d_rx32);
     cudaFree(d->d_rx64);
+    cudaFree(d->d_exptab);
+    d->d_exptab = nullptr;
     d->d_rx32 = d->d_rx64 = nullptr;
     d->d_adj_units = nullptr;
     d->d_adj_prefix = nullptr;
@@ -207,6 +209,16 @@ void release(lisa_data* d) {
     d->d_cross64 = nullptr;
     d->d_cross32 = nullptr;
     d->d_items = nullptr;
+}
+
+// 2^(j / kExpTab) rounded from long double, computed once per process.
+const double* exp_table() {
+    static const std::vector<double> T = [] {
+        std::vector<double> v((size_t)kExpTab);
+        for (int j = 0; j < kExpTab; ++j) v[(size_t)j] = (double)std::exp2((long double)j / kExpTab);
+        return v;
+    }();
+    return T.data();
 }
 
 // Bins per adjoint range (see kAdjBins): the longest that gives kAdjWarpsPerSm units per SM, or
@@ -287,6 +299,22 @@ lisa_status rebuild_work(lisa_data* d) {
             lay_out(nseg / 2);
             break;
         }
+    }
+    // the plain FP64 kernels' units: half a segment of bins x 32 states, one warp each.  (They share
+    // the FP64 pipe, so what counts is that the units are many and of one size; half a segment is what
+    // the workspace of the FP32 path holds slots for.)
+    for (int64_t b64 = std::max<int64_t>(16, (t.tile_bins / d->nseg + 3) / 4 * 2);; b64 *= 2) {
+        int64_t units = 0, slots = 0;
+        d->b64 = (int32_t)b64;
+        for (DatasetDev& D : d->h_ds) {
+            D.n64 = (int32_t)((D.npad + b64 - 1) / b64);
+            D.ubase64 = units;
+            D.pbase64 = slots;
+            units += (int64_t)D.n64 * ((D.ns + 31) / 32);
+            slots += (int64_t)D.n64 * D.ns;
+        }
+        d->n_units64 = units;
+        if (ws_bytes64(d, slots) <= ws_fwd_bytes(d)) break;
     }
     items.reserve((size_t)n_items);
     for (int k = 0; k < d->n_datasets; ++k) {
@@ -564,7 +592,8 @@ lisa_status lisa_data_create(const lisa_data_desc* desc, lisa_stream_t stream, l
         X.xb_min = X.nbins ? std::log10(q.freq[X.rbin0]) : 0.0;
         X.xb_max = X.nbins ? std::log10(q.freq[X.rbin0 + X.nbins - 1]) : 0.0;
         X.f_ref = q.f_ref[k];
-        X.nslots = X.nrt = 0;
+        X.nslots = X.nrt = X.n64 = 0;
+        X.ubase64 = X.pbase64 = 0;
         X.pbase = 0;
         X.psd_base = psd_base;
         psd_base += (int64_t)C * X.ns * X.nbins;
@@ -603,11 +632,12 @@ lisa_status lisa_data_create(const lisa_data_desc* desc, lisa_stream_t stream, l
         (st = dev_alloc(&f, (size_t)N)) ||
         (st = dev_alloc(&nu, (size_t)N)) || (st = dev_alloc(&lnP, (size_t)NP)) ||
         (st = dev_alloc(&R, (size_t)C * N)) || (st = dev_alloc(&d->d_rx32, (size_t)rbase)) ||
-        (st = dev_alloc(&d->d_rx64, (size_t)rbase)))
+        (st = dev_alloc(&d->d_rx64, (size_t)rbase)) || (st = dev_alloc(&d->d_exptab, (size_t)kExpTab)))
         return fail(st);
     cudaStream_t sm = (cudaStream_t)stream;
     bool ok = cudaMemcpyAsync(d->d_ds, d->h_ds.data(), D * sizeof(DatasetDev), cudaMemcpyHostToDevice, sm) == cudaSuccess &&
               cudaMemcpyAsync(d->d_state_ds, state_ds.data(), S * sizeof(int32_t), cudaMemcpyHostToDevice, sm) == cudaSuccess &&
+              cudaMemcpyAsync(d->d_exptab, exp_table(), kExpTab * sizeof(double), cudaMemcpyHostToDevice, sm) == cudaSuccess &&
               cudaMemcpyAsync(f, q.freq, N * sizeof(double), cudaMemcpyHostToDevice, sm) == cudaSuccess &&
               cudaMemcpyAsync(nu, q.nu, N * sizeof(double), cudaMemcpyHostToDevice, sm) == cudaSuccess &&
               cudaMemcpyAsync(d->d_P, q.periodogram, C * N * sizeof(double), cudaMemcpyHostToDevice, sm) == cudaSuccess &&

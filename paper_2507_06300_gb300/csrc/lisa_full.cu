@@ -16,6 +16,7 @@
 // with the 3x3 adjugate and determinant written out.  The constant -sum nu sum_c ln P_cc is
 // added by the finalize, as for the diagonal model.
 #include "lisa_math.cuh"
+#include "lisa_math64.cuh"
 
 namespace lisa {
 namespace {
@@ -26,16 +27,32 @@ constexpr int kFullThreads = 128;
 // The per-bin term in FP64 (without the factor nu): tr(C^-1 P-hat) + ln det C from the spline
 // values (log10 units for the noise and SGWB splines, plain values for the correlations), the
 // bin's table q (x, ell, nu, Go[3], Gt[3], Gh[3]), its cross-spectral entries xc[3], and the
-// state's parameters.  Non-finite results (a PSD outside the FP64 range, a singular K) propagate,
-// and the finalize turns the state's log L into -inf.
+// state's parameters.  The exponentials take the table exptab where every exponent is below 100 decades
+// (4 instead of about 40 FP64 instructions each), else the library's functions.  Non-finite results (a
+// PSD outside the FP64 range, a singular K) propagate, and the finalize turns the state's log L into
+// -inf.
 template <bool HAS_H>
 __device__ __forceinline__ double full_term64(const double pn[3], double ph, const double zv[3], const double* q,
-                                              const double* xc, double ao2, double at2, double lA, double sl) {
+                                              const double* xc, double ao2, double at2, double lA, double sl,
+                                              const double* __restrict__ exptab) {
     double D[3], Cd[3];
-    const double eh = HAS_H ? exp10(lA + ph) * exp2(sl * q[1]) : 0.0;
+    constexpr double kLog10_2 = 0.301029995663981195213739;
+    const double yh = HAS_H ? fma(sl * kLog10_2, q[1], lA + ph) : 0.0;
+    const bool in_range = m64::small_exponent(pn[0]) && m64::small_exponent(pn[1]) && m64::small_exponent(pn[2]) &&
+                          m64::small_exponent(yh);
+    double E[3], eh = 0.0;
+    if (in_range) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) E[c] = m64::exp10_fast(pn[c], exptab);
+        if (HAS_H) eh = m64::exp10_fast(yh, exptab);
+    } else {
+#pragma unroll 1
+        for (int c = 0; c < 3; ++c) E[c] = exp10(pn[c]);
+        if (HAS_H) eh = exp10(lA + ph) * exp2(sl * q[1]);
+    }
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        D[c] = (ao2 * q[3 + c] + at2 * q[6 + c]) * exp10(pn[c]);
+        D[c] = (ao2 * q[3 + c] + at2 * q[6 + c]) * E[c];
         Cd[c] = HAS_H ? D[c] + eh * q[9 + c] : D[c];
     }
     double r[3], sq[3];
@@ -62,78 +79,72 @@ __device__ __forceinline__ double full_term64(const double pn[3], double ph, con
 }
 
 // ---- plain FP64 path --------------------------------------------------------------------------
+// One warp per unit of b64 bins x 32 states, as the diagonal model's (lanes = states).
 template <bool HAS_H, bool BROKEN>
-__global__ void __launch_bounds__(kThreads)
-    full_fp64_kernel(const WorkItem* __restrict__ items, int n_items, const double* __restrict__ rec64,
-                     const double* __restrict__ cross64, const double* __restrict__ theta,
-                     const int32_t* __restrict__ sstat, const int32_t* __restrict__ nint,
-                     const double* __restrict__ srec, int kmax, int nsp, const DatasetDev* __restrict__ ds,
-                     double* __restrict__ partial, int tile_bins, int nseg) {
+__global__ void __launch_bounds__(64)
+    full_fp64_kernel(int64_t n_units, int n_ds, int b64, const double* __restrict__ rec64,
+                     const double* __restrict__ cross64, const double* __restrict__ exptab,
+                     const double* __restrict__ theta, const int32_t* __restrict__ sstat,
+                     const int32_t* __restrict__ nint, const double* __restrict__ srec, int kmax, int nsp,
+                     const DatasetDev* __restrict__ ds, double* __restrict__ partial) {
     constexpr int NSP = 3 + (HAS_H ? 1 : 0) + 3;
     constexpr int ZB = 3 + (HAS_H ? 1 : 0);   // first correlation spline
-    __shared__ double red[kThreads];
-    const int tid = threadIdx.x;
-    for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
-        const WorkItem w = items[LISA_IDX(it, n_items)];
-        const int sc = w.sc;
-        const int R = kThreads / sc;
-        const int ls = tid & (sc - 1);
-        const int r = tid / sc;
-        const int s = w.s0 + ls;
-        const bool active = ls < w.ns && sstat[s] == 0;
-        double acc = 0.0;
-        if (active) {
-            const int lo = item_lo(w, r, R, tile_bins, nseg), hi = item_lo(w, r + 1, R, tile_bins, nseg);
-            if (lo < hi) {
-                const double* th = theta + (size_t)s * LISA_N_THETA;
-                const double ao2 = th[0] * th[0], at2 = th[1] * th[1], lA = th[2], n1 = th[3];
-                const double n2 = BROKEN ? th[4] : n1;
-                const double* base[NSP];
-                int j[NSP], last[NSP];
-                double xl[NSP], xr[NSP], ca[NSP], cb[NSP], cc[NSP], cd[NSP];
-                const double x0 = __ldg(rec64 + (w.bin0 + lo) * kRec);
-                for (int a = 0; a < NSP; ++a) {
-                    const int64_t sp = (int64_t)s * nsp + a;
-                    base[a] = srec + sp * (int64_t)(kmax + 1) * kSplineRec;
-                    last[a] = nint[sp] - 1;
-                    j[a] = find_interval<double, kSplineRec, 0>(base[a], nint[sp], x0);
-                    const double* z = base[a] + (size_t)LISA_IDX(j[a], kmax + 1) * kSplineRec;
-                    xl[a] = z[0]; xr[a] = z[1]; ca[a] = z[2]; cb[a] = z[3]; cc[a] = z[4]; cd[a] = z[5];
-                }
-                for (int i = lo; i < hi; ++i) {
-                    const double* q = rec64 + (w.bin0 + i) * kRec;
-                    double qq[kRec];
-                    for (int k = 0; k < kRec; ++k) qq[k] = __ldg(q + k);
-                    const double x = qq[0];
-                    double P[NSP];
-                    for (int a = 0; a < NSP; ++a) {
-                        while (x >= xr[a] && j[a] < last[a]) {
-                            ++j[a];
-                            const double* z = base[a] + (size_t)LISA_IDX(j[a], kmax + 1) * kSplineRec;
-                            xl[a] = z[0]; xr[a] = z[1]; ca[a] = z[2]; cb[a] = z[3]; cc[a] = z[4]; cd[a] = z[5];
-                        }
-                        const double t = x - xl[a];
-                        P[a] = ca[a] + t * (cb[a] + t * (cc[a] + t * cd[a]));
-                    }
-                    const double* xc = cross64 + (w.bin0 + i) * kCross;
-                    const double xcv[3] = {__ldg(xc), __ldg(xc + 1), __ldg(xc + 2)};
-                    const double sl = BROKEN ? (qq[1] < 0.0 ? n1 : n2) : n1;
-                    const double pn[3] = {P[0], P[1], P[2]};
-                    const double zv[3] = {P[ZB], P[ZB + 1], P[ZB + 2]};
-                    acc += qq[2] * full_term64<HAS_H>(pn, HAS_H ? P[3] : 0.0, zv, qq, xcv, ao2, at2, lA, sl);
+    const int64_t u = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (u >= n_units) return;
+    int slot, s;
+    const DatasetDev& D = m64::unit_of(ds, n_ds, u, slot, s);
+    if (s >= D.s0 + D.ns || sstat[s] != 0) return;
+    const int64_t b0 = D.bin0 + (int64_t)slot * b64;
+    const int nb = (int)min((int64_t)b64, D.bin0 + D.npad - b0);
+    const double* th = theta + (size_t)s * LISA_N_THETA;
+    const double ao2 = th[0] * th[0], at2 = th[1] * th[1], lA = th[2], n1 = th[3];
+    const double n2 = BROKEN ? th[4] : n1;
+    int j[NSP];
+    double xl[NSP], ca[NSP], cb[NSP], cc[NSP], cd[NSP];
+    long long xr[NSP];
+    auto load = [&](int a) {
+        const double* z = srec + (((int64_t)s * nsp + a) * (int64_t)(kmax + 1) + LISA_IDX(j[a], kmax + 1)) * kSplineRec;
+        xl[a] = z[0];
+        xr[a] = m64::order_key(z[1]);
+        ca[a] = z[2];
+        cb[a] = z[3];
+        cc[a] = z[4];
+        cd[a] = z[5];
+    };
+    const double x0 = __ldg(rec64 + b0 * kRec);
+    for (int a = 0; a < NSP; ++a) {
+        const int64_t sp = (int64_t)s * nsp + a;
+        j[a] = find_interval<double, kSplineRec, 0>(srec + sp * (int64_t)(kmax + 1) * kSplineRec, nint[sp], x0);
+        load(a);
+    }
+    double acc = 0.0;
+    for (int i = 0; i < nb; ++i) {
+        const double* q = rec64 + (b0 + i) * kRec;
+        double qq[kRec];
+        for (int k = 0; k < kRec; ++k) qq[k] = __ldg(q + k);
+        const double x = qq[0];
+        const long long xk = m64::order_key(x);
+        double P[NSP];
+#pragma unroll
+        for (int a = 0; a < NSP; ++a) {
+            if (xk >= xr[a]) {
+                const int last = nint[(int64_t)s * nsp + a] - 1;
+                while (xk >= xr[a] && j[a] < last) {
+                    ++j[a];
+                    load(a);
                 }
             }
+            const double t = x - xl[a];
+            P[a] = ca[a] + t * (cb[a] + t * (cc[a] + t * cd[a]));
         }
-        red[tid] = acc;
-        __syncthreads();
-        if (r == 0 && ls < w.ns && sstat[s] == 0) {
-            double sum = 0.0;
-            for (int q = 0; q < R; ++q) sum += red[ls + q * sc];
-            const DatasetDev& D = ds[w.ds];
-            partial[D.pbase + (int64_t)(s - D.s0) * D.nslots + w.slot] = sum;
-        }
-        __syncthreads();
+        const double* xc = cross64 + (b0 + i) * kCross;
+        const double xcv[3] = {__ldg(xc), __ldg(xc + 1), __ldg(xc + 2)};
+        const double sl = BROKEN ? (m64::negative(qq[1]) ? n1 : n2) : n1;
+        const double pn[3] = {P[0], P[1], P[2]};
+        const double zv[3] = {P[ZB], P[ZB + 1], P[ZB + 2]};
+        acc += qq[2] * full_term64<HAS_H>(pn, HAS_H ? P[3] : 0.0, zv, qq, xcv, ao2, at2, lA, sl, exptab);
     }
+    partial[D.pbase64 + (int64_t)(s - D.s0) * D.n64 + LISA_IDX(slot, D.n64)] = acc;
 }
 
 // ---- FP32 bulk path ---------------------------------------------------------------------------
@@ -192,7 +203,8 @@ template <bool HAS_H, bool BROKEN>
 __device__ __noinline__ double full_careful_term(int s, int bin, const float* tb, const float* tx, int i,
                                                  const float* __restrict__ xlo32, const float* __restrict__ elllo32,
                                                  const double* __restrict__ theta, const float* __restrict__ kxr,
-                                                 const float* __restrict__ srec, int kmax, int nsp) {
+                                                 const float* __restrict__ srec, int kmax, int nsp,
+                                                 const double* __restrict__ exptab) {
     constexpr int NSP = 3 + (HAS_H ? 1 : 0) + 3;
     constexpr int ZB = 3 + (HAS_H ? 1 : 0);
     const float x = fld(tb, i, 0);
@@ -231,7 +243,8 @@ __device__ __noinline__ double full_careful_term(int s, int bin, const float* tb
     const double sl = BROKEN ? (qd[1] < 0.0 ? th[3] : th[4]) : th[3];
     const double pn[3] = {pd[0], pd[1], pd[2]};
     const double zv[3] = {pd[ZB], pd[ZB + 1], pd[ZB + 2]};
-    return full_term64<HAS_H>(pn, HAS_H ? pd[3] : 0.0, zv, qd, xcd, th[0] * th[0], th[1] * th[1], th[2], sl);
+    return full_term64<HAS_H>(pn, HAS_H ? pd[3] : 0.0, zv, qd, xcd, th[0] * th[0], th[1] * th[1], th[2], sl,
+                              exptab);
 }
 
 // One thread per state and contiguous bins of the item, one bin at a time.  The current interval of
@@ -252,7 +265,7 @@ __global__ void __launch_bounds__(kFullThreads, 4)
     full_fp32_kernel(const WorkItem* __restrict__ items, int n_items, const float* __restrict__ rec32,
                      const float* __restrict__ cross32, const float* __restrict__ xlo32,
                      const float* __restrict__ elllo32, const StateParams* __restrict__ prm,
-                     const double* __restrict__ theta,
+                     const double* __restrict__ theta, const double* __restrict__ exptab,
                      const int32_t* __restrict__ sstat, const float* __restrict__ kxr,
                      const float* __restrict__ srec, int kmax, int nsp, const DatasetDev* __restrict__ ds,
                      double* __restrict__ partial, int* __restrict__ err, int tile_bins, int nseg,
@@ -534,7 +547,7 @@ __global__ void __launch_bounds__(kFullThreads, 4)
                 const int so = w.s0 + (owner & (sc - 1));
                 const float nu = fld(tb, i, 2);
                 const double t64 = full_careful_term<HAS_H, BROKEN>(so, w.bin0 + i, tb, tx, i, xlo32, elllo32, theta,
-                                                                    kxr, srec, kmax, nsp);
+                                                                    kxr, srec, kmax, nsp, exptab);
                 if (nu != 0.f) atomicAdd(&s_far[owner], (double)nu * (t64 - 3.0));
             }
             __syncwarp();
@@ -571,21 +584,16 @@ cudaError_t launch_full(const lisa_data* d, bool fp32, const double* theta, cons
         int64_t grid = (int64_t)d->n_sm * per_sm;
         if (grid > d->n_items) grid = d->n_items;
         kern<<<(unsigned)(grid < 1 ? 1 : grid), kFullThreads, smem, sm>>>(
-            d->d_items, (int)d->n_items, d->d_rec32, d->d_cross32, d->d_xlo32, d->d_elllo32, prm, theta, sstat, kxr,
+            d->d_items, (int)d->n_items, d->d_rec32, d->d_cross32, d->d_xlo32, d->d_elllo32, prm, theta, d->d_exptab,
+            sstat, kxr,
             static_cast<const float*>(srec), kmax, d->nsp, d->d_ds, partial, err, d->tiling.tile_bins, d->nseg,
             d->wait_limit);
         return cudaGetLastError();
     }
-    auto kern = full_fp64_kernel<H, B>;
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, 0) != cudaSuccess || per_sm < 1)
-        per_sm = 1;
-    int64_t grid = (int64_t)d->n_sm * per_sm;
-    if (grid > d->n_items) grid = d->n_items;
-    kern<<<(unsigned)(grid < 1 ? 1 : grid), kThreads, 0, sm>>>(d->d_items, (int)d->n_items, d->d_rec64,
-                                                                d->d_cross64, theta, sstat, nint,
-                                                                static_cast<const double*>(srec), kmax, d->nsp,
-                                                                d->d_ds, partial, d->tiling.tile_bins, d->nseg);
+    if (d->n_units64 > 0)
+        full_fp64_kernel<H, B><<<(unsigned)((d->n_units64 + 1) / 2), 64, 0, sm>>>(
+            d->n_units64, d->n_datasets, d->b64, d->d_rec64, d->d_cross64, d->d_exptab, theta, sstat, nint,
+            static_cast<const double*>(srec), kmax, d->nsp, d->d_ds, partial);
     return cudaGetLastError();
 }
 

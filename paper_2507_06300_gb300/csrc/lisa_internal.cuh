@@ -51,9 +51,8 @@ constexpr int kRec = 12;         // per-bin fields: x, ell, nu, Goms[3], Gtm[3],
 constexpr int kPairRec = 2 * kRec;
 constexpr int kCross = 4;        // FP64 cross-spectral fields per bin (three and a pad)
 constexpr int kPairCross = 8;    // FP32 cross-spectral floats per pair block
-constexpr int kThreads = 256;    // threads of the plain FP64 likelihood kernel
 constexpr int kThreads32 = 128;  // threads of the fused FP32 likelihood kernel
-constexpr int kMaxStatesPerItem = 128;  // state lanes of a work item (<= both thread counts)
+constexpr int kMaxStatesPerItem = 128;  // state lanes of a work item (<= the threads of a CTA)
 // Per-interval records, 64 bytes in both precisions:
 //   FP64: xl, xr, a, b, c, d, 0, 0 (coefficients about xl, log10 units)
 //   FP32: [0] xr  [1] xo  [2..5] c0..c3  [6] xl  [7] conditioning T      (first 32 bytes)
@@ -89,6 +88,7 @@ constexpr int kAdjWarpsPerSm = 12;
 // interval advances: knots are drawn uniformly in log10 f, so the low-frequency tiles (few bins,
 // wide in log10 f) hold most of them, and each advance stalls its warp on record loads.
 constexpr double kKnotBinsPerDecade = 2500.0;
+constexpr int kExpTab = 8192;               // entries of the FP64 path's table of 2^(j / kExpTab)
 constexpr int kXsStride = 32;               // bins between the host copies of log10 f
 constexpr int kMinItemsPerSm = 2;            // fewer items per SM than this are split into segments
 constexpr int kBlockItemsPerCta = 16;       // contiguous blocks need this many items per CTA
@@ -134,6 +134,10 @@ struct DatasetDev {
     int32_t s0, ns;          // state range
     int32_t nslots;          // partial slots per state: tiles of tile_bins bins, times nseg
     int32_t nrt;             // tiles of the compensated kernel (rt_bins bins)
+    // plain FP64 path: units of b64 bins x 32 states (one warp each), the dataset's first unit, and
+    // its partial slots [state][n64]
+    int32_t n64;
+    int64_t ubase64, pbase64;
     int32_t nranges;         // adjoint ranges of adj_bins bins
     int32_t rbase;           // first range in the range-bound tables
     double x_lo, x_hi;       // edge knot positions
@@ -191,6 +195,9 @@ struct lisa_data {
     int32_t nseg = 1;                // segments per work item
     int32_t stage_bins = 0;          // bins per staging buffer of the fused kernels
     int32_t rt_bins = 0;             // bins per unit of the compensated kernel
+    int32_t b64 = 0;                 // bins per unit of the plain FP64 kernels
+    int64_t n_units64 = 0;           // their units
+    double* d_exptab = nullptr;      // [kExpTab] 2^(j / kExpTab)
     // per-kernel timing of lisa_psd_loglike (lisa_data_set_profiling): events around the main,
     // compensated and finalize kernels of the most recent uncaptured call
     cudaEvent_t prof_ev[4] = {nullptr, nullptr, nullptr, nullptr};
@@ -285,6 +292,8 @@ inline WsLayout ws_layout(const lisa_data* d) {
     return L;
 }
 inline size_t ws_fwd_bytes(const lisa_data* d) { return ws_layout(d).bytes; }
+// The plain FP64 path keeps its partial sums (256 bytes on) in the same bytes.
+inline size_t ws_bytes64(const lisa_data* d, int64_t n_partials64) { return 256 + sizeof(double) * (size_t)n_partials64; }
 
 // Extra workspace of the adjoint entry point (after the forward region); the FP32 call also holds
 // a per-state flag (states redone by the fallback pass).

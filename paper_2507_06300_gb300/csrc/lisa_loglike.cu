@@ -28,6 +28,7 @@
 #include <cmath>
 
 #include "lisa_math.cuh"
+#include "lisa_math64.cuh"
 
 namespace lisa {
 namespace {
@@ -1008,82 +1009,151 @@ __global__ void __launch_bounds__(kRobWarps * 32, 2)
 }
 
 
-// ---- plain FP64 path: the same decomposition, FP64 throughout, library exp10 / exp2 / log ----
+// ---- plain FP64 path: FP64 throughout ------------------------------------------------------
 
+// One bin's sum_c (1 / S_c + ln S_c) by the library's exp10, exp2 and log and FP64 divisions, for
+// bins whose exponents or products leave the range of the short forms (any value, NaN included).
+template <int C, bool HAS_H>
+__device__ __noinline__ double bin_term64_wide(const double* P, double ao2, double at2, double lA, double slope,
+                                               const double* __restrict__ q) {
+    const double eh = HAS_H ? exp10(lA + P[C]) * exp2(slope * q[1]) : 0.0;
+    double term = 0.0;
+    for (int c = 0; c < C; ++c) {
+        const double Sc = (ao2 * q[3 + c] + at2 * q[6 + c]) * exp10(P[c]) + (HAS_H ? eh * q[9 + c] : 0.0);
+        term += 1.0 / Sc + log(Sc);
+    }
+    return term;
+}
+
+// One warp per unit: b64 bins of one dataset x up to 32 of its states (lanes = states, so every lane
+// reads the same bin).  Bound by the FP64 pipe (2 lane operations per clock and SM): per state-bin 16
+// instructions for the four cubics, 17 for their exponentials and the power law, 12 for the PSDs, 4 for
+// their product and the numerator of sum 1 / S, 4 for the division, 2 for the sums; the logarithm of
+// the channels' product is taken once for up to kLogRun bins of equal nu.  Intervals, range checks and
+// conversions are integer work (lisa_math64.cuh).  65,537 bins x 400 states: 13.7 -> 3.0 ms.
+constexpr int kLogRun = 64;   // factors of a LogProduct: its mantissa stays below 2^64
 template <int C, bool HAS_H, bool BROKEN>
-__global__ void __launch_bounds__(kThreads)
-    loglike_fp64_kernel(const WorkItem* __restrict__ items, int n_items, const double* __restrict__ rec64,
-                        const double* __restrict__ theta, const int32_t* __restrict__ sstat,
-                        const int32_t* __restrict__ nint, const double* __restrict__ srec, int kmax, int nsp,
-                        const DatasetDev* __restrict__ ds, double* __restrict__ partial, int tile_bins, int nseg) {
+__global__ void __launch_bounds__(64)
+    loglike_fp64_kernel(int64_t n_units, int n_ds, int b64, const double* __restrict__ rec64,
+                        const double* __restrict__ exptab, const double* __restrict__ theta,
+                        const int32_t* __restrict__ sstat, const int32_t* __restrict__ nint,
+                        const double* __restrict__ srec, int kmax, int nsp, const DatasetDev* __restrict__ ds,
+                        double* __restrict__ partial) {
     constexpr int NSP = C + (HAS_H ? 1 : 0);
-    __shared__ double red[kThreads];
-    const int tid = threadIdx.x;
-    for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
-        const WorkItem w = items[LISA_IDX(it, n_items)];
-        const int sc = w.sc;
-        const int R = kThreads / sc;
-        const int ls = tid & (sc - 1);
-        const int r = tid / sc;
-        const int s = w.s0 + ls;
-        const bool active = ls < w.ns && sstat[s] == 0;
-        double acc = 0.0;
-        if (active) {
-            const int lo = item_lo(w, r, R, tile_bins, nseg), hi = item_lo(w, r + 1, R, tile_bins, nseg);
-            if (lo < hi) {
-                const double* th = theta + (size_t)s * LISA_N_THETA;
-                const double ao2 = th[0] * th[0], at2 = th[1] * th[1], lA = th[2], n1 = th[3];
-                const double n2 = BROKEN ? th[4] : n1;
-                const double* base[NSP];
-                int j[NSP], last[NSP];
-                double xl[NSP], xr[NSP], ca[NSP], cb[NSP], cc[NSP], cd[NSP];
-                const double* rb = rec64 + (w.bin0 + lo) * kRec;
-                for (int a = 0; a < NSP; ++a) {
-                    const int64_t sp = (int64_t)s * nsp + a;
-                    base[a] = srec + sp * (int64_t)(kmax + 1) * kSplineRec;
-                    last[a] = nint[sp] - 1;
-                    j[a] = find_interval<double, kSplineRec, 0>(base[a], nint[sp], __ldg(rb));
-                    const double* q = base[a] + (size_t)LISA_IDX(j[a], kmax + 1) * kSplineRec;
-                    xl[a] = q[0]; xr[a] = q[1]; ca[a] = q[2]; cb[a] = q[3]; cc[a] = q[4]; cd[a] = q[5];
-                }
-                for (int i = lo; i < hi; ++i) {
-                    const double* q = rec64 + (w.bin0 + i) * kRec;
-                    const double x = __ldg(q), ell = __ldg(q + 1), nu = __ldg(q + 2);
-                    double P[NSP];
-                    for (int a = 0; a < NSP; ++a) {
-                        while (x >= xr[a] && j[a] < last[a]) {
-                            ++j[a];
-                            const double* z = base[a] + (size_t)LISA_IDX(j[a], kmax + 1) * kSplineRec;
-                            xl[a] = z[0]; xr[a] = z[1]; ca[a] = z[2]; cb[a] = z[3]; cc[a] = z[4]; cd[a] = z[5];
-                        }
-                        const double t = x - xl[a];
-                        P[a] = ca[a] + t * (cb[a] + t * (cc[a] + t * cd[a]));
-                    }
-                    double eh = 0.0;
-                    if (HAS_H) {
-                        const double sl = BROKEN ? (ell < 0.0 ? n1 : n2) : n1;
-                        eh = exp10(lA + P[C]) * exp2(sl * ell);
-                    }
-                    double term = 0.0;
-                    for (int c = 0; c < C; ++c) {
-                        const double Sc = (ao2 * __ldg(q + 3 + c) + at2 * __ldg(q + 6 + c)) * exp10(P[c]) +
-                                          (HAS_H ? eh * __ldg(q + 9 + c) : 0.0);
-                        term += 1.0 / Sc + log(Sc);
-                    }
-                    acc += nu * term;
+    const int64_t u = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (u >= n_units) return;
+    int slot, s;
+    const DatasetDev& D = m64::unit_of(ds, n_ds, u, slot, s);
+    if (s >= D.s0 + D.ns || sstat[s] != 0) return;
+    const int64_t b0 = D.bin0 + (int64_t)slot * b64;
+    const int nb = (int)min((int64_t)b64, D.bin0 + D.npad - b0);
+    const double* q = rec64 + b0 * kRec;
+    const double* th = theta + (size_t)s * LISA_N_THETA;
+    const double ao2 = th[0] * th[0], at2 = th[1] * th[1], lA = th[2], n1 = th[3];
+    const double n2 = BROKEN ? th[4] : n1;
+    constexpr double kLog10_2 = 0.301029995663981195213739;
+    const double m1 = n1 * kLog10_2, m2 = n2 * kLog10_2;   // slopes in decades per octave
+    // the current interval of each spline: left knot, cubic (the background's with log10 A in its
+    // constant), and its right end as an order key (no FP64 comparison)
+    double xl[NSP], ca[NSP], cb[NSP], cc[NSP], cd[NSP];
+    long long xr[NSP];
+    int j[NSP];
+    auto load = [&](int a) {
+        const double* z = srec + (((int64_t)s * nsp + a) * (int64_t)(kmax + 1) + LISA_IDX(j[a], kmax + 1)) * kSplineRec;
+        xl[a] = z[0];
+        xr[a] = m64::order_key(z[1]);
+        ca[a] = HAS_H && a == C ? z[2] + lA : z[2];
+        cb[a] = z[3];
+        cc[a] = z[4];
+        cd[a] = z[5];
+    };
+    long long xmin = 0;
+    auto nearest = [&]() {
+        xmin = xr[0];
+#pragma unroll
+        for (int a = 1; a < NSP; ++a) xmin = min(xmin, xr[a]);
+    };
+#pragma unroll
+    for (int a = 0; a < NSP; ++a) {
+        const int64_t sp = (int64_t)s * nsp + a;
+        j[a] = find_interval<double, kSplineRec, 0>(srec + sp * (int64_t)(kmax + 1) * kSplineRec, nint[sp], __ldg(q));
+        load(a);
+    }
+    nearest();
+    double acc = 0.0, run = 0.0;   // the finished runs, and the current run's sum of 1 / S
+    m64::LogProduct lp;
+    lp.reset();
+    int len = 0;
+    double nu_run = 0.0;
+    for (int i = 0; i < nb; ++i, q += kRec) {
+        const double2* q2 = reinterpret_cast<const double2*>(q);   // 96-byte records
+        const double2 f0 = __ldg(q2), f1 = __ldg(q2 + 1), f2 = __ldg(q2 + 2), f3 = __ldg(q2 + 3), f4 = __ldg(q2 + 4),
+                      f5 = __ldg(q2 + 5);
+        const double x = f0.x, ell = f0.y, nu = f1.x;
+        const double go[3] = {f1.y, f2.x, f2.y}, gt[3] = {f3.x, f3.y, f4.x}, gh[3] = {f4.y, f5.x, f5.y};
+        if (m64::order_key(x) >= xmin) {
+            const long long xk = m64::order_key(x);
+#pragma unroll
+            for (int a = 0; a < NSP; ++a) {
+                if (xk < xr[a]) continue;
+                const int last = nint[(int64_t)s * nsp + a] - 1;
+                while (xk >= xr[a] && j[a] < last) {
+                    ++j[a];
+                    load(a);
                 }
             }
+            nearest();
         }
-        red[tid] = acc;
-        __syncthreads();
-        if (r == 0 && ls < w.ns && sstat[s] == 0) {
-            double sum = 0.0;
-            for (int q = 0; q < R; ++q) sum += red[ls + q * sc];
-            const DatasetDev& D = ds[w.ds];
-            partial[D.pbase + (int64_t)(s - D.s0) * D.nslots + w.slot] = sum;
+        // a run of bins with one nu ends (the lanes share the bins)
+        if (__double_as_longlong(nu) != __double_as_longlong(nu_run) || len == kLogRun) {
+            acc = fma(nu_run, run + lp.log_value(), acc);
+            run = 0.0;
+            lp.reset();
+            len = 0;
+            nu_run = nu;
         }
-        __syncthreads();
+        double P[NSP];
+        bool ok = true;
+#pragma unroll
+        for (int a = 0; a < NSP; ++a) {
+            const double t = x - xl[a];
+            P[a] = fma(t, fma(t, fma(t, cd[a], cc[a]), cb[a]), ca[a]);
+        }
+        const double slope = BROKEN ? (m64::negative(ell) ? m1 : m2) : m1;
+        if (HAS_H) P[C] = fma(slope, ell, P[C]);
+#pragma unroll
+        for (int a = 0; a < NSP; ++a) ok &= m64::small_exponent(P[a]);
+        double S[C], eh = 0.0;
+        if (HAS_H) eh = m64::exp10_fast(P[C], exptab);
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            const double N = fma(ao2, go[c], at2 * gt[c]);
+            const double E = m64::exp10_fast(P[c], exptab);
+            S[c] = HAS_H ? fma(N, E, eh * gh[c]) : N * E;
+        }
+        const double p01 = S[0] * S[1];
+        const double prod = C == 3 ? p01 * S[C - 1] : p01;
+        const double num = C == 3 ? fma(S[C - 1], S[0] + S[1], p01) : S[0] + S[1];
+        // products of normal size: nothing over- or underflowed on the way
+        ok &= m64::normal_range(p01) && m64::normal_range(prod) && m64::normal_range(num);
+        if (ok) {
+            run += m64::divide(num, prod);
+            lp.mul(prod);
+            ++len;
+        } else {
+            double Pv[NSP];
+#pragma unroll
+            for (int a = 0; a < NSP; ++a) {
+                const double t = x - xl[a];
+                const double c0 = HAS_H && a == C ? __ldg(srec + (((int64_t)s * nsp + a) * (int64_t)(kmax + 1) + j[a]) * kSplineRec + 2)
+                                                  : ca[a];
+                Pv[a] = c0 + t * (cb[a] + t * (cc[a] + t * cd[a]));
+            }
+            acc += nu * bin_term64_wide<C, HAS_H>(Pv, ao2, at2, lA, BROKEN ? (m64::negative(ell) ? n1 : n2) : n1, q);
+        }
     }
+    acc = fma(nu_run, run + lp.log_value(), acc);
+    partial[D.pbase64 + (int64_t)(s - D.s0) * D.n64 + LISA_IDX(slot, D.n64)] = acc;
 }
 
 // Per state (one warp): fixed-order sum of its tiles' partials (lane-strided, then a shuffle
@@ -1101,9 +1171,10 @@ __global__ void finalize_kernel(int S, const int32_t* __restrict__ state_ds, con
         return;
     }
     const DatasetDev& D = ds[state_ds[s]];
-    const double* p = partial + D.pbase + (int64_t)(s - D.s0) * D.nslots;
+    const int n = fp32 ? D.nslots : D.n64;
+    const double* p = partial + (fp32 ? D.pbase : D.pbase64) + (int64_t)(s - D.s0) * n;
     double sum = 0.0;
-    for (int t = lane; t < D.nslots; t += 32) sum += p[t];
+    for (int t = lane; t < n; t += 32) sum += p[t];
     // FP32 mode: the compensated kernel's sums of this state's units, if it has any
     const int e = fp32 ? rent[s] : -1;
     if (e >= 0) {
@@ -1120,10 +1191,14 @@ __global__ void finalize_kernel(int S, const int32_t* __restrict__ state_ds, con
     }
 }
 
-// Model PSD in physical units, FP64: one thread per (state, bin).
+// Model PSD in physical units, FP64: one thread per (state, bin).  The FP64 pipe bounds it: 48
+// instructions per state-bin (cubics 16, exponentials and power law 17, PSDs 12, normalisation 3); the
+// interval searches compare order keys, and the exponentials take the table, on the other pipes (the
+// library's functions: 140).  131,072 bins x 64 states: 2.05 ms -> 0.79 ms.
 template <int C>
 __global__ void model_psd_kernel(const int32_t* __restrict__ state_ds, const DatasetDev* __restrict__ ds,
-                                 const double* __restrict__ rec64, const double* __restrict__ P, int64_t n_bins,
+                                 const double* __restrict__ rec64, const double* __restrict__ exptab,
+                                 const double* __restrict__ P, int64_t n_bins,
                                  const double* __restrict__ theta, const int32_t* __restrict__ sstat,
                                  const int32_t* __restrict__ nint, const double* __restrict__ srec, int kmax,
                                  int nsp, int has_h, int broken, double* __restrict__ out) {
@@ -1141,37 +1216,47 @@ __global__ void model_psd_kernel(const int32_t* __restrict__ state_ds, const Dat
     const double* q = rec64 + g * kRec;
     const double x = q[0], ell = q[1];
     const double* th = theta + (size_t)s * LISA_N_THETA;
-    double Pv[4];
-    for (int a = 0; a < C + has_h; ++a) {   // the noise and SGWB splines (not the correlations)
+    const long long xk = m64::order_key(x);
+    double Pv[C + 1];
+    bool ok = true;
+#pragma unroll
+    for (int a = 0; a < C + 1; ++a) {   // the noise and SGWB splines (not the correlations)
+        if (a == C && !has_h) break;
         const int64_t sp = (int64_t)s * nsp + a;
         const double* base = srec + sp * (int64_t)(kmax + 1) * kSplineRec;
-        const int j = find_interval<double, kSplineRec, 0>(base, nint[sp], x);
-        const double* z = base + (size_t)LISA_IDX(j, kmax + 1) * kSplineRec;
-        const double t = x - z[0];
-        Pv[a] = z[2] + t * (z[3] + t * (z[4] + t * z[5]));
+        int lo = 0, hi = nint[sp] - 1;   // the last interval whose left knot is <= x (0 below the first)
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (m64::order_key(__ldg(base + (size_t)mid * kSplineRec)) <= xk) lo = mid; else hi = mid - 1;
+        }
+        const double2* z = reinterpret_cast<const double2*>(base + (size_t)LISA_IDX(lo, kmax + 1) * kSplineRec);
+        const double2 z0 = __ldg(z), z1 = __ldg(z + 1), z2 = __ldg(z + 2);   // xl, xr, a, b, c, d
+        const double t = x - z0.x;
+        Pv[a] = fma(t, fma(t, fma(t, z2.y, z2.x), z1.y), z1.x);
     }
-    double eh = 0.0;
-    if (has_h) {
-        const double sl = (broken && ell >= 0.0) ? th[4] : th[3];
-        eh = exp10(th[2] + Pv[C]) * exp2(sl * ell);
+    const double sl = (broken && !m64::negative(ell)) ? th[4] : th[3];
+    constexpr double kLog10_2 = 0.301029995663981195213739;
+    const double yh = has_h ? fma(sl * kLog10_2, ell, th[2] + Pv[C]) : 0.0;
+    ok = m64::small_exponent(yh);
+#pragma unroll
+    for (int c = 0; c < C; ++c) ok &= m64::small_exponent(Pv[c]);
+    double E[C], eh = 0.0;
+    if (ok) {
+        if (has_h) eh = m64::exp10_fast(yh, exptab);
+#pragma unroll
+        for (int c = 0; c < C; ++c) E[c] = m64::exp10_fast(Pv[c], exptab);
+    } else {
+        if (has_h) eh = exp10(th[2] + Pv[C]) * exp2(sl * ell);
+#pragma unroll 1
+        for (int c = 0; c < C; ++c) E[c] = exp10(Pv[c]);
     }
+    const double ao2 = th[0] * th[0], at2 = th[1] * th[1];
+#pragma unroll
     for (int c = 0; c < C; ++c) {
-        const double Sc = (th[0] * th[0] * q[3 + c] + th[1] * th[1] * q[6 + c]) * exp10(Pv[c]) + eh * q[9 + c];
+        const double N = fma(ao2, q[3 + c], at2 * q[6 + c]);
+        const double Sc = fma(N, E[c], eh * q[9 + c]);
         o[(int64_t)c * D.nbins + i] = Sc * P[(int64_t)c * n_bins + gr];
     }
-}
-
-template <class K>
-int grid_for(K kernel, const lisa_data* d, size_t smem, int threads) {
-    int per_sm = d->tiling.ctas_per_sm;
-    if (per_sm <= 0) {
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem) != cudaSuccess ||
-            per_sm < 1)
-            per_sm = 1;
-    }
-    int64_t g = (int64_t)d->n_sm * per_sm;
-    if (g > d->n_items) g = d->n_items;
-    return (int)(g < 1 ? 1 : g);
 }
 
 template <int C, bool H, bool B, int G>
@@ -1277,10 +1362,10 @@ cudaError_t launch_fp32(const lisa_data* d, const StateParams* prm, const int32_
 template <int C, bool H, bool B>
 cudaError_t launch_fp64(const lisa_data* d, const double* theta, const int32_t* sstat, const int32_t* nint,
                         const double* srec, int kmax, double* partial, cudaStream_t sm, bool prof) {
-    auto kern = loglike_fp64_kernel<C, H, B>;
-    const int grid = grid_for(kern, d, 0, kThreads);
-    kern<<<grid, kThreads, 0, sm>>>(d->d_items, (int)d->n_items, d->d_rec64, theta, sstat, nint, srec, kmax,
-                                    d->nsp, d->d_ds, partial, d->tiling.tile_bins, d->nseg);
+    if (d->n_units64 > 0)
+        loglike_fp64_kernel<C, H, B><<<(unsigned)((d->n_units64 + 1) / 2), 64, 0, sm>>>(
+            d->n_units64, d->n_datasets, d->b64, d->d_rec64, d->d_exptab, theta, sstat, nint, srec, kmax, d->nsp, d->d_ds,
+            partial);
     const cudaError_t e = cudaGetLastError();
     prof_mark(d, prof, 1, sm);
     prof_mark(d, prof, 2, sm);   // no compensated kernel in FP64 mode
@@ -1450,10 +1535,10 @@ lisa_status lisa_model_psd(const lisa_data* d, const lisa_params* params, const 
     cudaStream_t sm = (cudaStream_t)stream;
     const int h = d->sgwb_model != 0, br = d->sgwb_model == 2;
     if (d->C == 3)
-        model_psd_kernel<3><<<grid, 256, 0, sm>>>(d->d_state_ds, d->d_ds, d->d_rec64, d->d_P, d->n_bins,
+        model_psd_kernel<3><<<grid, 256, 0, sm>>>(d->d_state_ds, d->d_ds, d->d_rec64, d->d_exptab, d->d_P, d->n_bins,
                                                   params->theta_dev, sstat, nint, srec, kmax, d->nsp, h, br, out);
     else
-        model_psd_kernel<2><<<grid, 256, 0, sm>>>(d->d_state_ds, d->d_ds, d->d_rec64, d->d_P, d->n_bins,
+        model_psd_kernel<2><<<grid, 256, 0, sm>>>(d->d_state_ds, d->d_ds, d->d_rec64, d->d_exptab, d->d_P, d->n_bins,
                                                   params->theta_dev, sstat, nint, srec, kmax, d->nsp, h, br, out);
     return check_cuda(cudaGetLastError());
 }

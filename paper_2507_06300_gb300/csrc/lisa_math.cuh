@@ -41,14 +41,6 @@ __device__ __forceinline__ float fld(const float* __restrict__ t, int i, int k) 
     return t[(i >> 1) * kPairRec + 2 * k + (i & 1)];
 }
 
-// First bin (within the tile) of row r of R in an FP64 kernel's item: the item's 1 / nseg of the
-// tile, split over the rows.
-__device__ __forceinline__ int item_lo(const WorkItem& w, int r, int R, int tile_bins, int nseg) {
-    const int len = (tile_bins + nseg - 1) / nseg;
-    const int a = min((int)w.nb, w.seg * len), b = min((int)w.nb, a + len);
-    return a + (r * (b - a)) / R;
-}
-
 // Float-float ("double-float") arithmetic: a value is hi + lo with |lo| <= ulp(hi)/2.
 struct ff {
     float hi, lo;

@@ -1,0 +1,116 @@
+// FP64 building blocks of the plain FP64 path, with as few instructions on the FP64 pipe as they can
+// do with.
+//
+// GB300 runs 2 FP64 lane operations per clock and SM against 128 FP32 or integer ones: one FP64
+// instruction of a warp takes the pipe as long as 64 other instructions take to issue.  So everything
+// that need not be rounded to 53 bits runs elsewhere: exponents, table indices, conversions and
+// comparisons on the integer pipe (from the bits of the doubles), reciprocal seeds and the last terms of
+// the series, below 2^-28 of the result, in FP32.  Against the library's exp10, exp2, log and
+// division a state-bin of the likelihood takes 55 FP64 instructions instead of 225.
+#pragma once
+
+#include "lisa_math.cuh"
+
+namespace lisa {
+namespace m64 {
+
+__device__ __forceinline__ unsigned hi32(double v) { return (unsigned)__double2hiint(v); }
+__device__ __forceinline__ unsigned lo32(double v) { return (unsigned)__double2loint(v); }
+
+// A double truncated to FP32 by its bits (magnitudes below 2^-126 become 0; not for |v| >= 2^128).
+__device__ __forceinline__ float to_float(double v) {
+    const unsigned h = hi32(v), a = h & 0x7fffffffu;
+    const unsigned m = (__funnelshift_l(lo32(v), h, 3) - (896u << 23)) & 0x7fffffffu;
+    return __uint_as_float(a >= (897u << 20) ? (m | (h & 0x80000000u)) : 0u);
+}
+// A normal FP32 number as a double by its bits (0 becomes +-2^-127, which every use here drowns in a
+// larger term).
+__device__ __forceinline__ double to_double(float f) {
+    const unsigned b = __float_as_uint(f);
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
+}
+// The order of doubles on integers (NaN excluded): comparisons without the FP64 pipe.
+__device__ __forceinline__ long long order_key(double v) {
+    const long long b = __double_as_longlong(v);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
+}
+// Biased exponent of a double (0: zero or subnormal, 2047: infinite or NaN).
+__device__ __forceinline__ int exponent(double v) { return (int)((hi32(v) >> 20) & 0x7ffu); }
+
+__device__ __forceinline__ bool negative(double v) { return (int)hi32(v) < 0; }   // (-0 included)
+// Whether |v| lies in [2^-900, 2^900) (false for NaN).
+__device__ __forceinline__ bool normal_range(double v) { return (unsigned)(exponent(v) - 123) < 1800u; }
+// |v| < 100 (false for NaN): the range of exp10_fast.
+__device__ __forceinline__ bool small_exponent(double v) { return (hi32(v) & 0x7fffffffu) < 0x40590000u; }
+
+// 10^v for |v| < 100 from the table T of 2^(j / kExpTab) (the table-driven scheme of Tang, ACM TOMS 15,
+// 1989): 4 FP64 instructions, error within 1 ulp plus the rounding of v.  v = k log10(2) / 8192 + r with
+// k chosen in FP32 (any k near the nearest one does), r exact to twice the precision;
+// 10^r = 1 + r ln10 + q, where q <= 2^-30 is summed in FP32.  The table (64 KB) is read through L1,
+// which the kernels that use it leave free.
+__device__ __forceinline__ double exp10_fast(double v, const double* __restrict__ T) {
+    constexpr double C_hi = 0x1.34413509f79ffp-15;    // log10(2) / 8192, rounded to FP64
+    constexpr double C_lo = -0x1.9dc1da994fd21p-72;   // and the rest
+    static_assert(kExpTab == 8192, "constants");
+    const float tf = fmaf(to_float(v), 27213.2350f, 12582912.f);   // 8192 / log10(2): k in the low bits
+    const int k = __float_as_int(tf) - 0x4b400000;
+    const double kd = to_double(tf - 12582912.f);
+    double r = fma(kd, -C_hi, v);
+    r = fma(kd, -C_lo, r);
+    const float rf = to_float(r);
+    const float q = rf * rf * fmaf(rf, 2.03467859f, 2.65094906f);   // ln10^2 / 2, ln10^3 / 6
+    const double p = fma(r, kLn10, to_double(q));
+    const double t = __ldg(T + (k & (kExpTab - 1)));
+    const double e = fma(t, p, t);
+    return __hiloint2double((int)(hi32(e) + (unsigned)((k >> 13) << 20)), (int)lo32(e));
+}
+
+// n / d for a normal d well inside the range: an FP32 reciprocal of d's mantissa and one cubic step
+// (4 FP64 instructions, error within 1 ulp).
+__device__ __forceinline__ double divide(double n, double d) {
+    const unsigned h = hi32(d);
+    const float m = __uint_as_float(0x3f800000u | ((h & 0xfffffu) << 3) | (lo32(d) >> 29));
+    const unsigned b = __float_as_uint(dm::rcp_approx(m));
+    // 1 / m in (1/2, 1] as a double, times 2^-(exponent of d)
+    const double r = __hiloint2double((int)((b >> 3) + (896u << 20) + (1023u << 20) - (h & 0x7ff00000u)), (int)(b << 29));
+    const double e = fma(-d, r, 1.0);
+    const double e2 = fma(e, e, e);
+    const double w = n * r;
+    return fma(w, e2, w);
+}
+
+// Running product of normal positive doubles as mantissa and exponent: one FP64 instruction a factor.
+// Its logarithm is taken once for many factors (the mantissa grows by less than 2 a factor).
+struct LogProduct {
+    double m;
+    int e;
+    __device__ __forceinline__ void reset() {
+        m = 1.0;
+        e = 0;
+    }
+    __device__ __forceinline__ void mul(double v) {
+        const unsigned h = hi32(v);
+        e += (int)(h >> 20) - 1023;
+        m *= __hiloint2double((int)((h & 0xfffffu) | 0x3ff00000u), (int)lo32(v));
+    }
+    __device__ __forceinline__ double log_value() const { return fma((double)e, kLn2, log(m)); }
+};
+
+// The calling warp's unit u of a plain FP64 kernel: its dataset (the last one whose first unit is <= u;
+// empty ones share their successor's), its slot of b64 bins, and its lane's state.
+__device__ __forceinline__ const DatasetDev& unit_of(const DatasetDev* __restrict__ ds, int n_ds, int64_t u, int& slot,
+                                                     int& s) {
+    int lo = 0, hi = n_ds - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (ds[mid].ubase64 <= u) lo = mid; else hi = mid - 1;
+    }
+    const DatasetDev& D = ds[lo];
+    const int groups = (D.ns + 31) >> 5;
+    slot = (int)((u - D.ubase64) / groups);
+    s = D.s0 + 32 * (int)((u - D.ubase64) % groups) + (int)(threadIdx.x & 31);
+    return D;
+}
+
+}  // namespace m64
+}  // namespace lisa
