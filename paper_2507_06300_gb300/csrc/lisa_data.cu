@@ -684,6 +684,7 @@ lisa_status lisa_data_create(const lisa_data_desc* desc, lisa_stream_t stream, l
             for (int32_t r = 0; r < X.nranges; ++r)
                 for (int32_t g = 0; g < X.ns; g += 32) units.push_back(AdjUnit{k, r, X.s0 + g, std::min(32, X.ns - g)});
         }
+        if (units.size() > (size_t)INT32_MAX) return fail(LISA_ERR_SHAPE);   // the launch's grid
         d->adj_ranges = acc;
         d->n_adj_units = (int64_t)units.size();
         if ((st = dev_alloc(&d->d_adj_units, units.size())) || (st = dev_alloc(&d->d_adj_prefix, prefix.size())))

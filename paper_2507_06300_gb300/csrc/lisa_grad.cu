@@ -531,188 +531,185 @@ __device__ __noinline__ void adjoint_bin64_wide(const double* P, double ao2, dou
 
 // Per state-bin 108 FP64 instructions (about 340 with the library's functions and a division per
 // channel): the forward pass as loglike_fp64_kernel's, 9 for the channels' reciprocals from one of their
-// product, 21 for the template sums and signals, 24 for the moments.  16,384 bins x 400 states with the
-// epilogue: 5.8 -> 2.06 ms.
+// product, 21 for the template sums and signals, 24 for the moments.  One unit and warp per CTA: the
+// units of a small problem spread over all SMs and start as registers come free (four units to a CTA,
+// their CTAs half empty: 1.85 against 1.53 ms).  16,384 bins x 400 states with the epilogue: 5.8 -> 1.68 ms.
 constexpr int kLogRun = 64;   // factors of a LogProduct: its mantissa stays below 2^64
 template <int C, bool HAS_H, bool BROKEN>
-__global__ void __launch_bounds__(128)
-    adjoint_fp64_kernel(const AdjUnit* __restrict__ units, int64_t n_units, const DatasetDev* __restrict__ ds,
+__global__ void __launch_bounds__(32)
+    adjoint_fp64_kernel(const AdjUnit* __restrict__ units, const DatasetDev* __restrict__ ds,
                         const double* __restrict__ rec64, const double* __restrict__ exptab,
                         const double* __restrict__ theta, const int32_t* __restrict__ sstat,
                         const int32_t* __restrict__ nint, const double* __restrict__ srec, int kmax, int nsp,
                         const int64_t* __restrict__ prefix, double* __restrict__ scal, double* __restrict__ mom,
                         int adj_bins) {
     constexpr int NSP = C + (HAS_H ? 1 : 0);
-    const int lane = threadIdx.x & 31;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int64_t wg = first_unit(n_units, nw);
-    for (int64_t u = wg; u < n_units; u += nw) {
-        const AdjUnit U = units[u];
-        const DatasetDev& D = ds[U.ds];
-        const int s = U.s0 + lane;
-        if (lane >= U.ns || (sstat[s] & kUserBits)) continue;
-        const double* th = theta + (size_t)s * LISA_N_THETA;
-        const double ao2 = th[0] * th[0], at2 = th[1] * th[1], lA = th[2], n1 = th[3];
-        const double n2 = BROKEN ? th[4] : n1;
-        constexpr double kLog10_2 = 0.301029995663981195213739;
-        const double m1 = n1 * kLog10_2, m2 = n2 * kLog10_2;   // slopes in decades per octave
-        const int64_t b0 = D.bin0 + (int64_t)U.rho * adj_bins;
-        const int nb = (int)min((int64_t)adj_bins, D.bin0 + D.npad - b0);
-        const int64_t pre = prefix[s];
-        int j[NSP];
-        double xl[NSP], ca[NSP], cb[NSP], cc[NSP], cd[NSP];
-        long long xr[NSP];
-        double m[NSP][4];
-        auto load = [&](int a) {
-            const double* z = srec + (((int64_t)s * nsp + a) * (int64_t)(kmax + 1) + LISA_IDX(j[a], kmax + 1)) * kSplineRec;
-            xl[a] = z[0];
-            xr[a] = m64::order_key(z[1]);
-            ca[a] = HAS_H && a == C ? z[2] + lA : z[2];
-            cb[a] = z[3];
-            cc[a] = z[4];
-            cd[a] = z[5];
-        };
-        auto store = [&](int a) {
-            double* row = mom_row(mom, pre, s, a, nsp, kmax, D.nranges) + 4 * (int64_t)LISA_IDX(U.rho + j[a], D.nranges + kmax + 1);
+    const int lane = threadIdx.x;
+    const AdjUnit U = units[blockIdx.x];
+    const DatasetDev& D = ds[U.ds];
+    const int s = U.s0 + lane;
+    if (lane >= U.ns || (sstat[s] & kUserBits)) return;
+    const double* th = theta + (size_t)s * LISA_N_THETA;
+    const double ao2 = th[0] * th[0], at2 = th[1] * th[1], lA = th[2], n1 = th[3];
+    const double n2 = BROKEN ? th[4] : n1;
+    constexpr double kLog10_2 = 0.301029995663981195213739;
+    const double m1 = n1 * kLog10_2, m2 = n2 * kLog10_2;   // slopes in decades per octave
+    const int64_t b0 = D.bin0 + (int64_t)U.rho * adj_bins;
+    const int nb = (int)min((int64_t)adj_bins, D.bin0 + D.npad - b0);
+    const int64_t pre = prefix[s];
+    int j[NSP];
+    double xl[NSP], ca[NSP], cb[NSP], cc[NSP], cd[NSP];
+    long long xr[NSP];
+    double m[NSP][4];
+    auto load = [&](int a) {
+        const double* z = srec + (((int64_t)s * nsp + a) * (int64_t)(kmax + 1) + LISA_IDX(j[a], kmax + 1)) * kSplineRec;
+        xl[a] = z[0];
+        xr[a] = m64::order_key(z[1]);
+        ca[a] = HAS_H && a == C ? z[2] + lA : z[2];
+        cb[a] = z[3];
+        cc[a] = z[4];
+        cd[a] = z[5];
+    };
+    auto store = [&](int a) {
+        double* row = mom_row(mom, pre, s, a, nsp, kmax, D.nranges) + 4 * (int64_t)LISA_IDX(U.rho + j[a], D.nranges + kmax + 1);
 #pragma unroll
-            for (int p = 0; p < 4; ++p) {
-                row[p] = kLn10 * m[a][p];   // q carries ln10 only here
-                m[a][p] = 0.0;
+        for (int p = 0; p < 4; ++p) {
+            row[p] = kLn10 * m[a][p];   // q carries ln10 only here
+            m[a][p] = 0.0;
+        }
+    };
+    long long xmin = 0;
+    auto nearest = [&]() {
+        xmin = xr[0];
+#pragma unroll
+        for (int a = 1; a < NSP; ++a) xmin = min(xmin, xr[a]);
+    };
+    const double* q = rec64 + b0 * kRec;
+#pragma unroll
+    for (int a = 0; a < NSP; ++a) {
+        const int64_t sp = (int64_t)s * nsp + a;
+        j[a] = find_interval<double, kSplineRec, 0>(srec + sp * (int64_t)(kmax + 1) * kSplineRec, nint[sp], __ldg(q));
+        load(a);
+#pragma unroll
+        for (int p = 0; p < 4; ++p) m[a][p] = 0.0;
+    }
+    nearest();
+    double acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    // the current run of bins with one nu: sum of (sum_c 1 / S_c - C), product of the S_c, length
+    double run = 0.0, nu_run = 0.0;
+    m64::LogProduct lp;
+    lp.reset();
+    int len = 0;
+    for (int i = 0; i < nb; ++i, q += kRec) {
+        const double2* q2 = reinterpret_cast<const double2*>(q);   // 96-byte records
+        const double2 f0 = __ldg(q2), f1 = __ldg(q2 + 1), f2 = __ldg(q2 + 2), f3 = __ldg(q2 + 3), f4 = __ldg(q2 + 4),
+                      f5 = __ldg(q2 + 5);
+        const double x = f0.x, ell = f0.y, nu = f1.x;
+        const double go[3] = {f1.y, f2.x, f2.y}, gt[3] = {f3.x, f3.y, f4.x}, gh[3] = {f4.y, f5.x, f5.y};
+        const long long xk = m64::order_key(x);
+        if (xk >= xmin) {
+#pragma unroll
+            for (int a = 0; a < NSP; ++a) {
+                if (xk < xr[a]) continue;
+                const int last = nint[(int64_t)s * nsp + a] - 1;
+                while (xk >= xr[a] && j[a] < last) {
+                    store(a);
+                    ++j[a];
+                    load(a);
+                }
             }
-        };
-        long long xmin = 0;
-        auto nearest = [&]() {
-            xmin = xr[0];
-#pragma unroll
-            for (int a = 1; a < NSP; ++a) xmin = min(xmin, xr[a]);
-        };
-        const double* q = rec64 + b0 * kRec;
+            nearest();
+        }
+        if (__double_as_longlong(nu) != __double_as_longlong(nu_run) || len == kLogRun) {
+            acc[0] = fma(nu_run, run + lp.log_value(), acc[0]);
+            run = 0.0;
+            lp.reset();
+            len = 0;
+            nu_run = nu;
+        }
+        double P[NSP], t[NSP];
+        bool ok = true;
 #pragma unroll
         for (int a = 0; a < NSP; ++a) {
-            const int64_t sp = (int64_t)s * nsp + a;
-            j[a] = find_interval<double, kSplineRec, 0>(srec + sp * (int64_t)(kmax + 1) * kSplineRec, nint[sp], __ldg(q));
-            load(a);
-#pragma unroll
-            for (int p = 0; p < 4; ++p) m[a][p] = 0.0;
+            t[a] = x - xl[a];
+            P[a] = fma(t[a], fma(t[a], fma(t[a], cd[a], cc[a]), cb[a]), ca[a]);
         }
-        nearest();
-        double acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-        // the current run of bins with one nu: sum of (sum_c 1 / S_c - C), product of the S_c, length
-        double run = 0.0, nu_run = 0.0;
-        m64::LogProduct lp;
-        lp.reset();
-        int len = 0;
-        for (int i = 0; i < nb; ++i, q += kRec) {
-            const double2* q2 = reinterpret_cast<const double2*>(q);   // 96-byte records
-            const double2 f0 = __ldg(q2), f1 = __ldg(q2 + 1), f2 = __ldg(q2 + 2), f3 = __ldg(q2 + 3), f4 = __ldg(q2 + 4),
-                          f5 = __ldg(q2 + 5);
-            const double x = f0.x, ell = f0.y, nu = f1.x;
-            const double go[3] = {f1.y, f2.x, f2.y}, gt[3] = {f3.x, f3.y, f4.x}, gh[3] = {f4.y, f5.x, f5.y};
-            const long long xk = m64::order_key(x);
-            if (xk >= xmin) {
+        if (HAS_H) P[C] = fma(BROKEN ? (m64::negative(ell) ? m1 : m2) : m1, ell, P[C]);
 #pragma unroll
-                for (int a = 0; a < NSP; ++a) {
-                    if (xk < xr[a]) continue;
-                    const int last = nint[(int64_t)s * nsp + a] - 1;
-                    while (xk >= xr[a] && j[a] < last) {
-                        store(a);
-                        ++j[a];
-                        load(a);
-                    }
-                }
-                nearest();
-            }
-            if (__double_as_longlong(nu) != __double_as_longlong(nu_run) || len == kLogRun) {
-                acc[0] = fma(nu_run, run + lp.log_value(), acc[0]);
-                run = 0.0;
-                lp.reset();
-                len = 0;
-                nu_run = nu;
-            }
-            double P[NSP], t[NSP];
-            bool ok = true;
+        for (int a = 0; a < NSP; ++a) ok &= m64::small_exponent(P[a]);
+        double S[C], E[C], N[C], Eh[C], r[C], qv[NSP];
+        double eh = 0.0;
+        if (HAS_H) eh = m64::exp10_fast(P[C], exptab);
 #pragma unroll
-            for (int a = 0; a < NSP; ++a) {
-                t[a] = x - xl[a];
-                P[a] = fma(t[a], fma(t[a], fma(t[a], cd[a], cc[a]), cb[a]), ca[a]);
+        for (int c = 0; c < C; ++c) {
+            N[c] = fma(ao2, go[c], at2 * gt[c]);
+            E[c] = m64::exp10_fast(P[c], exptab);
+            Eh[c] = HAS_H ? eh * gh[c] : 0.0;
+            S[c] = HAS_H ? fma(N[c], E[c], Eh[c]) : N[c] * E[c];
+        }
+        const double p01 = S[0] * S[1];
+        const double prod = C == 3 ? p01 * S[C - 1] : p01;
+        ok &= m64::normal_range(p01) && m64::normal_range(prod) && m64::normal_range(S[0]) && m64::normal_range(S[1]) &&
+              m64::normal_range(S[C - 1]);
+        if (ok) {
+            const double rp = m64::divide(1.0, prod);
+            if (C == 3) {
+                const double rp2 = rp * S[C - 1];
+                r[C - 1] = rp * p01;
+                r[0] = rp2 * S[1];
+                r[1] = rp2 * S[0];
+            } else {
+                r[0] = rp * S[1];
+                r[1] = rp * S[0];
             }
-            if (HAS_H) P[C] = fma(BROKEN ? (m64::negative(ell) ? m1 : m2) : m1, ell, P[C]);
-#pragma unroll
-            for (int a = 0; a < NSP; ++a) ok &= m64::small_exponent(P[a]);
-            double S[C], E[C], N[C], Eh[C], r[C], qv[NSP];
-            double eh = 0.0;
-            if (HAS_H) eh = m64::exp10_fast(P[C], exptab);
+            double H = 0.0;
 #pragma unroll
             for (int c = 0; c < C; ++c) {
-                N[c] = fma(ao2, go[c], at2 * gt[c]);
-                E[c] = m64::exp10_fast(P[c], exptab);
-                Eh[c] = HAS_H ? eh * gh[c] : 0.0;
-                S[c] = HAS_H ? fma(N[c], E[c], Eh[c]) : N[c] * E[c];
+                const double g = fma(nu, r[c], -nu) * r[c];   // nu (1 - S) / S^2
+                const double gE = g * E[c];
+                run += r[c];
+                acc[1] = fma(gE, go[c], acc[1]);
+                acc[2] = fma(gE, gt[c], acc[2]);
+                qv[c] = gE * N[c];
+                if (HAS_H) H = c == 0 ? g * Eh[c] : fma(g, Eh[c], H);
             }
-            const double p01 = S[0] * S[1];
-            const double prod = C == 3 ? p01 * S[C - 1] : p01;
-            ok &= m64::normal_range(p01) && m64::normal_range(prod) && m64::normal_range(S[0]) && m64::normal_range(S[1]) &&
-                  m64::normal_range(S[C - 1]);
-            if (ok) {
-                const double rp = m64::divide(1.0, prod);
-                if (C == 3) {
-                    const double rp2 = rp * S[C - 1];
-                    r[C - 1] = rp * p01;
-                    r[0] = rp2 * S[1];
-                    r[1] = rp2 * S[0];
-                } else {
-                    r[0] = rp * S[1];
-                    r[1] = rp * S[0];
-                }
-                double H = 0.0;
-#pragma unroll
-                for (int c = 0; c < C; ++c) {
-                    const double g = fma(nu, r[c], -nu) * r[c];   // nu (1 - S) / S^2
-                    const double gE = g * E[c];
-                    run += r[c];
-                    acc[1] = fma(gE, go[c], acc[1]);
-                    acc[2] = fma(gE, gt[c], acc[2]);
-                    qv[c] = gE * N[c];
-                    if (HAS_H) H = c == 0 ? g * Eh[c] : fma(g, Eh[c], H);
-                }
-                if (HAS_H) qv[C] = H;
-                run -= (double)C;
-                lp.mul(prod);
-                ++len;
-            } else {
-                double Pv[NSP], out[4 + NSP];
-#pragma unroll
-                for (int a = 0; a < NSP; ++a) {
-                    const double c0 = HAS_H && a == C ? __ldg(srec + (((int64_t)s * nsp + a) * (int64_t)(kmax + 1) + j[a]) * kSplineRec + 2)
-                                                      : ca[a];
-                    Pv[a] = c0 + t[a] * (cb[a] + t[a] * (cc[a] + t[a] * cd[a]));
-                }
-                adjoint_bin64_wide<C, HAS_H>(Pv, ao2, at2, lA, BROKEN ? (m64::negative(ell) ? n1 : n2) : n1, q, out);
-                acc[0] += nu * (out[0] - (double)C);
-                acc[1] += out[1];
-                acc[2] += out[2];
-#pragma unroll
-                for (int a = 0; a < NSP; ++a) qv[a] = out[4 + a];
-            }
-            if (HAS_H) {
-                acc[3] += qv[C];
-                if (BROKEN && !m64::negative(ell)) acc[5] = fma(ell, qv[C], acc[5]); else acc[4] = fma(ell, qv[C], acc[4]);
-            }
+            if (HAS_H) qv[C] = H;
+            run -= (double)C;
+            lp.mul(prod);
+            ++len;
+        } else {
+            double Pv[NSP], out[4 + NSP];
 #pragma unroll
             for (int a = 0; a < NSP; ++a) {
-                const double qt = qv[a] * t[a], qt2 = qt * t[a];
-                m[a][0] += qv[a];
-                m[a][1] += qt;
-                m[a][2] += qt2;
-                m[a][3] = fma(qt2, t[a], m[a][3]);
+                const double c0 = HAS_H && a == C ? __ldg(srec + (((int64_t)s * nsp + a) * (int64_t)(kmax + 1) + j[a]) * kSplineRec + 2)
+                                                  : ca[a];
+                Pv[a] = c0 + t[a] * (cb[a] + t[a] * (cc[a] + t[a] * cd[a]));
             }
-        }
-        acc[0] = fma(nu_run, run + lp.log_value(), acc[0]);
+            adjoint_bin64_wide<C, HAS_H>(Pv, ao2, at2, lA, BROKEN ? (m64::negative(ell) ? n1 : n2) : n1, q, out);
+            acc[0] += nu * (out[0] - (double)C);
+            acc[1] += out[1];
+            acc[2] += out[2];
 #pragma unroll
-        for (int a = 0; a < NSP; ++a) store(a);
-        double* sc = scal + 6 * (pre + U.rho);
-        for (int k = 0; k < 6; ++k) sc[k] = acc[k];
+            for (int a = 0; a < NSP; ++a) qv[a] = out[4 + a];
+        }
+        if (HAS_H) {
+            acc[3] += qv[C];
+            if (BROKEN && !m64::negative(ell)) acc[5] = fma(ell, qv[C], acc[5]); else acc[4] = fma(ell, qv[C], acc[4]);
+        }
+#pragma unroll
+        for (int a = 0; a < NSP; ++a) {
+            const double qt = qv[a] * t[a], qt2 = qt * t[a];
+            m[a][0] += qv[a];
+            m[a][1] += qt;
+            m[a][2] += qt2;
+            m[a][3] = fma(qt2, t[a], m[a][3]);
+        }
     }
+    acc[0] = fma(nu_run, run + lp.log_value(), acc[0]);
+#pragma unroll
+    for (int a = 0; a < NSP; ++a) store(a);
+    double* sc = scal + 6 * (pre + U.rho);
+    for (int k = 0; k < 6; ++k) sc[k] = acc[k];
 }
 
 // ---- the FP32 gradient's two per-state passes: one CTA per (state, range) item --------------
@@ -1728,7 +1725,7 @@ cudaError_t launch_adjoint(const lisa_data* d, bool fp32, const lisa_params* par
                 gw.fb + S, Rf, gw.fb, gw.fb + 2 * S + 2, nint, srec, nullptr, kn->kmax, d->nsp, d->d_adj_prefix, scal,
                 mom, d->adj_bins);
         } else
-            adjoint_fp64_kernel<C, H, B><<<grid, 128, 0, sm>>>(d->d_adj_units, d->n_adj_units, d->d_ds, d->d_rec64,
+            adjoint_fp64_kernel<C, H, B><<<(unsigned)d->n_adj_units, 32, 0, sm>>>(d->d_adj_units, d->d_ds, d->d_rec64,
                                                                d->d_exptab, params->theta_dev, sstat, nint,
                                                                static_cast<const double*>(srec), kn->kmax, d->nsp,
                                                                d->d_adj_prefix, scal, mom, d->adj_bins);
