@@ -256,7 +256,10 @@ int pow2ceil(int v) {
 // the fused kernel) or 32 of 64 bins (45 us).  The line: kMinItemsPerSm CTAs of 128 threads already
 // give every scheduler of the GPU its warps; more items only repeat the interval search.  A split
 // keeps the forward workspace within LISA_NOALLOC_SCRATCH_BYTES, so the allocation-free entry
-// point takes every problem that it takes unsplit.
+// point takes every problem that it takes unsplit (a larger one may grow: to 10 MB of partial sums at
+// most, since only problems of few items are split).  The dense covariance splits earlier
+// (kMinItemsPerSmFull): its warps' times differ widely (careful bins in FP64), and a unit's time, 0.7 ms
+// for 512 bins, is the launch's tail (131,072 bins x 1,024 states: 2.5 -> 2.0 ms).
 lisa_status rebuild_work(lisa_data* d) {
     const lisa_tiling& t = d->tiling;
     std::vector<WorkItem> items;
@@ -293,9 +296,10 @@ lisa_status rebuild_work(lisa_data* d) {
             max_seg = std::max(max_seg, (seg_bins(t.tile_bins, kThreads32 / lanes(D), 1) + kSegBins - 1) / kSegBins);
     int64_t n_items = lay_out(1);
     const size_t ws1 = ws_fwd_bytes(d);
-    for (int nseg = 2; n_items <= (int64_t)kMinItemsPerSm * d->n_sm && nseg < 2 * max_seg; nseg *= 2) {
+    const int64_t enough = (int64_t)(d->cov == LISA_COV_FULL ? kMinItemsPerSmFull : kMinItemsPerSm) * d->n_sm;
+    for (int nseg = 2; n_items <= enough && nseg < 2 * max_seg; nseg *= 2) {
         n_items = lay_out(nseg);
-        if (ws_fwd_bytes(d) > std::max((size_t)LISA_NOALLOC_SCRATCH_BYTES / 2, ws1)) {
+        if (ws1 <= LISA_NOALLOC_SCRATCH_BYTES && ws_fwd_bytes(d) > LISA_NOALLOC_SCRATCH_BYTES) {
             lay_out(nseg / 2);
             break;
         }
@@ -364,7 +368,11 @@ lisa_status rebuild_work(lisa_data* d) {
         return ((double)w.nb + kKnotBinsPerDecade * dx) * (double)w.ns;   // (a tile's segments alike)
     };
     std::vector<int32_t> cta_first((size_t)grid + 1, 0);
-    if (d->fblocks) {
+    if (d->cov == LISA_COV_FULL) {
+        // the dense kernels take the items in order: the low-frequency tiles, which hold most knots and
+        // ill-conditioned intervals, first
+        std::stable_sort(items.begin(), items.end(), [](const WorkItem& a, const WorkItem& b) { return a.slot < b.slot; });
+    } else if (d->fblocks) {
         // contiguous blocks of the (dataset, chunk, tile)-ordered list, cut so that every CTA gets
         // the same cost (item boundaries at cost midpoints)
         std::vector<double> pre(items.size() + 1, 0.0);

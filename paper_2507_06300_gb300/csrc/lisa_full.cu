@@ -22,7 +22,8 @@ namespace lisa {
 namespace {
 using namespace dm;
 
-constexpr int kFullThreads = 128;
+constexpr int kFullThreads = 128;   // threads of a work item (lanes x rows)
+constexpr int kFullPiece = 64;      // bins per staged piece of a one-warp CTA (a multiple of kFullChunk)
 
 // The per-bin term in FP64 (without the factor nu): tr(C^-1 P-hat) + ln det C from the spline
 // values (log10 units for the noise and SGWB splines, plain values for the correlations), the
@@ -169,24 +170,26 @@ __device__ __forceinline__ bool bar_wait(uint64_t* bar, unsigned parity, unsigne
         if (bar_try(bar, parity)) return true;
     return false;
 }
-// the item's two tables (the pair-block bin table and the cross-spectral table) by two bulk
-// copies completing on one mbarrier
-__device__ __forceinline__ void stage_item(float* dst, const float* rec32, const float* cross32, const WorkItem& w,
-                                           int tile_bins, uint64_t* bar) {
-    const unsigned b1 = (unsigned)w.nb * kRec * sizeof(float);
-    const unsigned b2 = (unsigned)(w.nb >> 1) * kPairCross * sizeof(float);
+// bins [a, b) (even) of the item's two tables (the pair-block bin table and the cross-spectral table,
+// which starts cross_at floats into the buffer) by two bulk copies completing on one mbarrier
+__device__ __forceinline__ void stage_bins(float* dst, const float* rec32, const float* cross32, const WorkItem& w,
+                                           int a, int b, int cross_at, uint64_t* bar) {
+    const unsigned b1 = (unsigned)(b - a) * kRec * sizeof(float);
+    const unsigned b2 = (unsigned)((b - a) >> 1) * kPairCross * sizeof(float);
+    const int64_t p0 = (w.bin0 + a) >> 1;
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(b1 + b2)
                  : "memory");
+    if (b1 == 0) return;
     asm volatile(
         "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
             smem_u32(dst)),
-        "l"(rec32 + (w.bin0 >> 1) * kPairRec), "r"(b1), "r"(smem_u32(bar))
+        "l"(rec32 + p0 * kPairRec), "r"(b1), "r"(smem_u32(bar))
         : "memory");
     asm volatile(
         "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-            smem_u32(dst + (size_t)tile_bins * kRec)),
-        "l"(cross32 + (w.bin0 >> 1) * kPairCross), "r"(b2), "r"(smem_u32(bar))
+            smem_u32(dst + cross_at)),
+        "l"(cross32 + p0 * kPairCross), "r"(b2), "r"(smem_u32(bar))
         : "memory");
 }
 
@@ -260,8 +263,16 @@ __device__ __noinline__ double full_careful_term(int s, int bin, const float* tb
 // evaluates its queued bins in FP64, one bin per lane, so that they cost full lanes rather than a
 // divergent branch in the bin loop (and no CTA barrier: the warps of a CTA drift freely within an
 // item).  Each warp's queue holds a chunk's worth of bins of its 32 threads and cannot overflow.
-template <bool HAS_H, bool BROKEN>
-__global__ void __launch_bounds__(kFullThreads, 4)
+//
+// W = 1 (every dataset has more than 64 states, so that a warp's 32 states walk the same bins): a CTA is
+// one of an item's four warps and stages its bins itself, kFullPiece at a time, double-buffered.  There
+// is no CTA barrier (a warp whose lanes meet ill-conditioned intervals or knots runs much longer than
+// its neighbours), shared memory does not depend on the tile (at 512-bin tiles the two staged tiles
+// left 2 CTAs per SM: 8 warps against 16), and items start as SMs come free.  131,072 bins x 1,024
+// states at the default tiling: 5.2 -> 2.5 ms.  W = 4 (fewer states: a state's bins are split over rows,
+// combined in shared memory): a CTA per item on a resident grid, whole tiles staged.
+template <bool HAS_H, bool BROKEN, int W>
+__global__ void __launch_bounds__(32 * W, 16 / W)
     full_fp32_kernel(const WorkItem* __restrict__ items, int n_items, const float* __restrict__ rec32,
                      const float* __restrict__ cross32, const float* __restrict__ xlo32,
                      const float* __restrict__ elllo32, const StateParams* __restrict__ prm,
@@ -275,48 +286,69 @@ __global__ void __launch_bounds__(kFullThreads, 4)
     constexpr float kL2 = 3.32192809488736234787f;   // log2(10): the records' coefficients carry it
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) uint64_t bars[2];
-    __shared__ float s_xr[NSP][kFullThreads];
-    __shared__ int s_jj[NSP][kFullThreads];
-    __shared__ double red[kFullThreads];
-    __shared__ double s_far[kFullThreads];                 // FP64 sums of the queued bins, per thread
-    __shared__ uint32_t s_q[kFullThreads / 32][32 * kFullChunk];   // per-warp careful queue: thread << 16 | bin
-    __shared__ int s_nq[kFullThreads / 32];
+    constexpr int T = 32 * W;
+    __shared__ float s_xr[NSP][T];
+    __shared__ int s_jj[NSP][T];
+    __shared__ double red[T];
+    __shared__ double s_far[T];                 // FP64 sums of the queued bins, per thread
+    __shared__ uint32_t s_q[W][32 * kFullChunk];           // per-warp careful queue: thread << 16 | bin
+    __shared__ int s_nq[W];
     __shared__ int s_fail;   // a bounded wait ran out: stage nothing more (a late copy may still land)
     const int tid = threadIdx.x;
     const int wid = tid >> 5, lane = tid & 31;
-    const size_t stage_floats = (size_t)tile_bins * kRec + (size_t)(tile_bins >> 1) * kPairCross;
+    const int vtid = W == 1 ? (int)(blockIdx.x & 3u) * 32 + lane : tid;   // the thread of the item
+    const int buf_bins = W == 1 ? kFullPiece : tile_bins;
+    const int cross_at = buf_bins * kRec;                                 // the cross table within a buffer
+    const int stage_floats = cross_at + (buf_bins >> 1) * kPairCross;
     float* sb[2] = {reinterpret_cast<float*>(smem), reinterpret_cast<float*>(smem) + stage_floats};
+    const int it0 = W == 1 ? (int)(blockIdx.x >> 2) : (int)blockIdx.x;
+    const int step = W == 1 ? n_items : (int)gridDim.x;   // W = 1: one item
+    // the bins of an item that its threads' runs cover: its segment where a run is the whole tile
+    auto extent = [&](const WorkItem& w, int& a, int& b) {
+        a = 0;
+        b = w.nb;
+        if (nseg > 1 && w.sc == kFullThreads) {
+            const int len = seg_bins(tile_bins, 1, nseg);
+            a = min(b, w.seg * len);
+            b = min(b, a + len);
+        }
+    };
+    auto stage = [&](int q, const WorkItem& w, int a, int b) {
+        stage_bins(sb[q], rec32, cross32, w, a, b, cross_at, &bars[q]);
+    };
+    if (W == 1) {   // a warp past the item's states
+        const WorkItem w = items[it0];
+        if (((vtid & ~31) & (w.sc - 1)) >= w.ns) return;
+    }
     if (tid == 0) {
         s_fail = 0;
-        for (int q = 0; q < kFullThreads / 32; ++q) s_nq[q] = 0;
+        for (int q = 0; q < W; ++q) s_nq[q] = 0;
         bar_init(&bars[0]);
         bar_init(&bars[1]);
-        if ((int)blockIdx.x < n_items) stage_item(sb[0], rec32, cross32, items[blockIdx.x], tile_bins, &bars[0]);
+        if (it0 < n_items) {
+            const WorkItem w = items[it0];
+            int a, b;
+            extent(w, a, b);
+            stage(0, w, W == 1 ? a : 0, W == 1 ? min(b, a + kFullPiece) : w.nb);
+        }
     }
     __syncthreads();
     // per spline: the current interval's cubic (xo, c0..c3) and whether it is well conditioned
     float cxo[NSP], c0[NSP], c1[NSP], c2[NSP], c3[NSP];
     unsigned hm = 0;
-    int k = 0;
-    for (int it = blockIdx.x; it < n_items; it += gridDim.x, ++k) {
-        const int b = k & 1;
-        const int nxt = it + gridDim.x;
-        if (nxt < n_items && tid == 0 && !s_fail)
-            stage_item(sb[b ^ 1], rec32, cross32, items[nxt], tile_bins, &bars[b ^ 1]);
+    int k = 0;   // staged pieces so far
+    for (int it = it0; it < n_items; it += step) {
         const WorkItem w = items[LISA_IDX(it, n_items)];
-        const bool ok = bar_wait(&bars[b], (unsigned)(k >> 1) & 1u, wait_limit);
-        if (!ok) {
-            s_fail = 1;   // read by thread 0 after the next barrier
-            atomicOr(err, kErrTimeout);
-        }
-        const float* tb = sb[b];
-        const float* tx = sb[b] + (size_t)tile_bins * kRec;   // cross-spectral pair blocks
+        int e_a, e_b;
+        extent(w, e_a, e_b);
+        const int len = W == 1 ? kFullPiece : tile_bins;
+        const int p_a = W == 1 ? e_a : 0, p_b = W == 1 ? e_b : (int)w.nb;
         const int sc = w.sc;
         const int R = kFullThreads / sc;
-        const int ls = tid & (sc - 1);
-        const int r = tid / sc;
+        const int ls = vtid & (sc - 1);
+        const int r = vtid / sc;
         const int s = w.s0 + ls;
-        const bool active = ok && ls < w.ns && (sstat[s] & kUserBits) == 0;
+        const bool mine = ls < w.ns && (sstat[s] & kUserBits) == 0;
         int lo = (r * w.nb) / R, hi = ((r + 1) * w.nb) / R;
         int run = (w.nb + R - 1) / R;                          // the longest of the CTA
         if (nseg > 1) {                                        // this item's segment of the run
@@ -325,11 +357,12 @@ __global__ void __launch_bounds__(kFullThreads, 4)
             hi = min(hi, lo + len);
             run = min(run, len);
         }
-        const bool run_bins = active && lo < hi;
-        const int nch = (run + kFullChunk - 1) / kFullChunk;   // uniform over the CTA
         s_far[tid] = 0.0;
         ff accf = {0.f, 0.f};
-        const StateParams p = prm[run_bins ? s : w.s0];
+        bool located = false;
+        float xmin = 0.f;
+        bool all_ok = true;
+        const StateParams p = prm[mine && lo < hi ? s : w.s0];
         const float ao2 = p.ao2, at2 = p.at2, Af = HAS_H ? p.Af : 0.f;
         auto rec = [&](int a, int j) {
             return srec + (((int64_t)s * nsp + a) * (int64_t)(kmax + 1) + LISA_IDX(j, kmax + 1)) * kSplineRec32;
@@ -346,8 +379,37 @@ __global__ void __launch_bounds__(kFullThreads, 4)
             c3[a] = B.y;
             hm = B.w <= (float)kRobustT ? (hm & ~(1u << a)) : (hm | (1u << a));
         };
-        float xmin = 0.f;
-        if (run_bins) {
+        int* nq = &s_nq[wid];
+        // the item's staged pieces (W = 4: one, the tile)
+        for (int pa = p_a; pa == p_a || pa < p_b; pa += len, ++k) {
+        const int b = k & 1;
+        if (tid == 0 && !s_fail) {   // the next piece, of this item or the next one
+            if (pa + len < p_b) {
+                stage(b ^ 1, w, pa + len, min(p_b, pa + 2 * len));
+            } else if (it + step < n_items) {
+                const WorkItem nx = items[it + step];
+                stage(b ^ 1, nx, 0, nx.nb);
+            }
+        }
+        const bool ok = bar_wait(&bars[b], (unsigned)(k >> 1) & 1u, wait_limit);
+        if (!ok) {
+            s_fail = 1;   // read by thread 0 after the next barrier
+            atomicOr(err, kErrTimeout);
+            if (W == 1) bar_wait(&bars[b], (unsigned)(k >> 1) & 1u, wait_limit);   // this CTA's copy, once more
+        }
+        all_ok &= ok;
+        // bin i of the tile is entry i - off of the staged tables; chunk indices run over the item's
+        // bins, ch0 is the piece's first
+        const int off = W == 1 ? pa : 0;
+        const float* tb = sb[b] - (off >> 1) * kPairRec;
+        const float* tx = sb[b] + cross_at - (off >> 1) * kPairCross;   // cross-spectral pair blocks
+        const bool run_bins = mine && all_ok && lo < hi;
+        const int ch0 = W == 1 ? (pa - p_a) / kFullChunk : 0;
+        // (uniform over the warp; over the CTA for W = 4)
+        const int nch = W == 1 ? (min(p_b, pa + len) - p_a + kFullChunk - 1) / kFullChunk
+                               : (run + kFullChunk - 1) / kFullChunk;
+        if (run_bins && !located) {
+            located = true;
             // intervals at the first bin: the count of right ends <= x in the right-end table
             const float x = fld(tb, lo, 0);
             const int kxs = kxr_stride(kmax);
@@ -366,8 +428,7 @@ __global__ void __launch_bounds__(kFullThreads, 4)
 #pragma unroll
             for (int a = 1; a < NSP; ++a) xmin = fminf(xmin, s_xr[a][tid]);
         }
-        int* nq = &s_nq[wid];
-        for (int ch = 0; ch < nch; ++ch) {
+        for (int ch = ch0; ch < nch; ++ch) {
             if (run_bins) {
                 float acc = 0.f;
                 const int iend = min(hi, lo + (ch + 1) * kFullChunk);
@@ -544,7 +605,7 @@ __global__ void __launch_bounds__(kFullThreads, 4)
             for (int e = lane; e < nqv; e += 32) {
                 const uint32_t ent = s_q[wid][e];
                 const int owner = (int)(ent >> 16), i = (int)(ent & 0xffffu);
-                const int so = w.s0 + (owner & (sc - 1));
+                const int so = w.s0 + ((W == 1 ? (int)(blockIdx.x & 3u) * 32 + owner : owner) & (sc - 1));
                 const float nu = fld(tb, i, 2);
                 const double t64 = full_careful_term<HAS_H, BROKEN>(so, w.bin0 + i, tb, tx, i, xlo32, elllo32, theta,
                                                                     kxr, srec, kmax, nsp, exptab);
@@ -554,15 +615,23 @@ __global__ void __launch_bounds__(kFullThreads, 4)
             if (lane == 0) *nq = 0;
             __syncwarp();
         }
-        red[tid] = ((double)accf.hi + (double)accf.lo) + s_far[tid];
-        __syncthreads();
-        if (r == 0 && active) {
-            double sum = red[ls];
-            for (int q = 1; q < R; ++q) sum += red[ls + q * sc];
-            const DatasetDev& D = ds[w.ds];
-            partial[D.pbase + (int64_t)(s - D.s0) * D.nslots + w.slot] = sum;
+        if (W == 1) __syncwarp();   // every lane is done with the buffer that the next piece refills
         }
-        __syncthreads();   // the buffer read in this iteration is refilled in the next one
+        const bool active = mine && all_ok;
+        const DatasetDev& D = ds[w.ds];
+        double* out = partial + D.pbase + (int64_t)(s - D.s0) * D.nslots + w.slot;
+        if (W == 1) {   // one row
+            if (active) *out = ((double)accf.hi + (double)accf.lo) + s_far[tid];
+        } else {
+            red[tid] = ((double)accf.hi + (double)accf.lo) + s_far[tid];
+            __syncthreads();
+            if (r == 0 && active) {
+                double sum = red[ls];
+                for (int q = 1; q < R; ++q) sum += red[ls + q * sc];
+                *out = sum;
+            }
+            __syncthreads();   // the buffer read in this iteration is refilled in the next one
+        }
     }
 }
 
@@ -571,10 +640,19 @@ cudaError_t launch_full(const lisa_data* d, bool fp32, const double* theta, cons
                         const int32_t* sstat, const int32_t* nint, const float* kxr, const void* srec, int kmax,
                         double* partial, int* err, cudaStream_t sm) {
     if (fp32) {
-        auto kern = full_fp32_kernel<H, B>;
-        const size_t stage = (size_t)d->tiling.tile_bins * kRec * sizeof(float) +
-                             (size_t)(d->tiling.tile_bins >> 1) * kPairCross * sizeof(float);
-        const size_t smem = 2 * stage;
+        bool rows = false;   // some dataset's items split a state's bins over rows
+        for (const auto& D : d->h_ds) rows |= D.ns > 0 && D.ns <= kFullThreads / 2;
+        rows |= d->tiling.states_per_cta < kFullThreads;
+        const int buf_bins = rows ? d->tiling.tile_bins : kFullPiece;
+        const size_t smem = 2 * ((size_t)buf_bins * kRec + (size_t)(buf_bins >> 1) * kPairCross) * sizeof(float);
+        if (!rows) {
+            full_fp32_kernel<H, B, 1><<<(unsigned)d->n_items * 4u, 32, smem, sm>>>(
+                d->d_items, (int)d->n_items, d->d_rec32, d->d_cross32, d->d_xlo32, d->d_elllo32, prm, theta, d->d_exptab,
+                sstat, kxr, static_cast<const float*>(srec), kmax, d->nsp, d->d_ds, partial, err, d->tiling.tile_bins,
+                d->nseg, d->wait_limit);
+            return cudaGetLastError();
+        }
+        auto kern = full_fp32_kernel<H, B, 4>;
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         int per_sm = 0;
@@ -585,8 +663,7 @@ cudaError_t launch_full(const lisa_data* d, bool fp32, const double* theta, cons
         if (grid > d->n_items) grid = d->n_items;
         kern<<<(unsigned)(grid < 1 ? 1 : grid), kFullThreads, smem, sm>>>(
             d->d_items, (int)d->n_items, d->d_rec32, d->d_cross32, d->d_xlo32, d->d_elllo32, prm, theta, d->d_exptab,
-            sstat, kxr,
-            static_cast<const float*>(srec), kmax, d->nsp, d->d_ds, partial, err, d->tiling.tile_bins, d->nseg,
+            sstat, kxr, static_cast<const float*>(srec), kmax, d->nsp, d->d_ds, partial, err, d->tiling.tile_bins, d->nseg,
             d->wait_limit);
         return cudaGetLastError();
     }

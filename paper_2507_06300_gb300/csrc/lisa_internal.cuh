@@ -91,6 +91,7 @@ constexpr double kKnotBinsPerDecade = 2500.0;
 constexpr int kExpTab = 8192;               // entries of the FP64 path's table of 2^(j / kExpTab)
 constexpr int kXsStride = 32;               // bins between the host copies of log10 f
 constexpr int kMinItemsPerSm = 2;            // fewer items per SM than this are split into segments
+constexpr int kMinItemsPerSmFull = 32;       // the same for the dense covariance
 constexpr int kBlockItemsPerCta = 16;       // contiguous blocks need this many items per CTA
 constexpr double kBlockThreadBins = 128.0;  // and fewer bins per thread and item than this
 
