@@ -1,34 +1,108 @@
 // Data preparation (Sec. III.C): synthetic frequency-domain data and the averaged periodogram,
-// the inputs of lisa_data_create.  Both are streaming kernels bound by HBM bandwidth.
+// the inputs of lisa_data_create.  Both are streaming kernels; HBM bounds them only because their FP64
+// arithmetic runs on the integer pipes (lisa_soft64.cuh).
 #include <cmath>
 
 #include "lisa_internal.cuh"
+#include "lisa_soft64.cuh"
 
 namespace lisa {
 namespace {
 
-// d = sqrt(S / 2) (z0 + i z1), grid-stride over (channel, sample), 16-byte loads and stores.
-__global__ void fd_synth_kernel(const double* __restrict__ S, const double2* __restrict__ z, int64_t n,
-                                double2* __restrict__ d) {
+// a v by the integer pipes, or by the FP64 instruction where a factor or the product is not normal.
+__device__ __forceinline__ double times(double a, int ea, uint64_t A, bool a_ok, double v) {
+    uint64_t r;
+    const bool ok = soft64::mul(ea, A, (uint64_t)__double_as_longlong(v), r);
+    if (ok && a_ok) return __longlong_as_double((long long)r);
+    return a * v;
+}
+
+// d = sqrt(S / 2) (z0 + i z1), grid-stride over (channel, sample), 16-byte loads and stores.  The FP64
+// pipe took 11 instructions a sample for the square root and the products (2.1 TB/s); about 150
+// integer instructions run on pipes 32 to 64 times as wide.  25.2 M samples: 522 us -> 232 us (4.3 TB/s).
+__global__ void __launch_bounds__(256) fd_synth_kernel(const double* __restrict__ S, const double2* __restrict__ z,
+                                                       int64_t n, double2* __restrict__ d) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const double a = sqrt(0.5 * __ldg(S + i));
+        const double s = __ldg(S + i);
         const double2 v = __ldg(z + i);
-        d[i] = make_double2(a * v.x, a * v.y);
+        uint64_t ab;
+        double a;
+        if (soft64::sqrt_half((uint64_t)__double_as_longlong(s), ab)) {
+            a = __longlong_as_double((long long)ab);
+        } else {
+            a = sqrt(0.5 * s);
+            ab = (uint64_t)__double_as_longlong(a);
+        }
+        const bool a_ok = soft64::is_normal(ab) && !(ab >> 63);
+        const uint64_t A = ((ab & soft64::kMant) | soft64::kOne) << 11;
+        const int ea = soft64::exp_of(ab);
+        d[i] = make_double2(times(a, ea, A, a_ok, v.x), times(a, ea, A, a_ok, v.y));
     }
 }
 
+// A lane's sum of squares: fixed point on the integer pipes (SOFT), or FP64 multiply-adds.
+template <bool SOFT>
+struct LaneSum {
+    static constexpr int kBatch = SOFT ? 4 : 1;   // samples added at once
+    double fp;   // SOFT: of batches with an infinity or a NaN only
+    soft64::SquareSum q;
+    __device__ __forceinline__ void reset() {
+        fp = 0.0;
+        if (SOFT) q.reset();
+    }
+    // Adds kBatch samples (absent ones as zeros, which add nothing).
+    __device__ __forceinline__ void add(const double2* v) {
+        if (!SOFT) {
+#pragma unroll
+            for (int u = 0; u < kBatch; ++u) fp = fma(v[u].x, v[u].x, fma(v[u].y, v[u].y, fp));
+            return;
+        }
+        uint64_t b[2 * kBatch];
+        int e = 0;
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+            b[2 * u] = (uint64_t)__double_as_longlong(v[u].x);
+            b[2 * u + 1] = (uint64_t)__double_as_longlong(v[u].y);
+            e = max(e, max(soft64::exp_of(b[2 * u]), soft64::exp_of(b[2 * u + 1])));
+        }
+        if (e > q.E) {
+            if (e == 2047) {   // an infinity or a NaN: the sum is one too
+#pragma unroll
+                for (int u = 0; u < kBatch; ++u) fp = fma(v[u].x, v[u].x, fma(v[u].y, v[u].y, fp));
+                return;
+            }
+            q.raise(e);
+        }
+#pragma unroll
+        for (int u = 0; u < 2 * kBatch; ++u) q.add(b[u]);
+    }
+    __device__ __forceinline__ double value() const {
+        if (!SOFT) return fp;
+        // the 96-bit sum rounded to FP64, scaled by 2^(2 (E - 1023) - 62) in two exact halves
+        const double m = fma((double)q.top, 18446744073709551616.0, (double)q.acc);
+        const int k = 2 * (q.E - 1023) - 62, k1 = k >> 1, k2 = k - k1;
+        const double s1 = __longlong_as_double((long long)(k1 + 1023) << 52);
+        const double s2 = __longlong_as_double((long long)(k2 + 1023) << 52);
+        if (q.E == 0) return fp;
+        // (beyond 2^+-800 the halves or the result may leave the normal range)
+        return ((unsigned)(q.E - 223) < 1600u ? m * s1 * s2 : scalbn(m, k)) + fp;
+    }
+};
+
 // Averaged periodogram: a group of G lanes per bin (G divides 32), lanes striding over the bin's
 // samples with 16-byte loads; the group's partial sums are combined by a butterfly of shuffles (a
-// fixed order for a given G).  GB300's FP64 pipe, not HBM, bounds this kernel: per complex sample
-// the work is two FP64 FMAs, and each bin adds log2(G) shuffle-adds per channel plus an epilogue
-// (a division, the bin centre) that occupy FP64 issue slots for the whole warp.  G = 4 keeps the
-// useful share of those slots near 85 % for 64-sample bins while each group still reads 64
-// contiguous bytes.
-template <int C, int G>
-__global__ void avg_periodogram_kernel(const double2* __restrict__ d, int64_t n_freq, double f0, double df,
-                                       const int64_t* __restrict__ off, int64_t n_bins, double* __restrict__ P,
-                                       double* __restrict__ f_out, double* __restrict__ nu_out, int n_ch) {
+// fixed order for a given G), and with G >= 4 its lanes share the epilogue: lane c divides channel
+// c's sum, lane 3 writes the bin's centre and nu.  With FP64 multiply-adds the FP64 pipe bounded this
+// kernel (two of them per complex sample, 81 us for 25.2 M samples at its rate against 60 us of HBM
+// time); the lanes' sums of squares run on the integer pipes (about 40 instructions a sample, exact to
+// 2^-61 of the sum) where a bin has enough samples to pay for the conversion of the sums, which is the
+// rule's line at 12 samples per bin.  25.2 M samples in 64-sample bins: 125 us -> 92 us.
+template <int C, int G, bool SOFT>
+__global__ void __launch_bounds__(256)
+    avg_periodogram_kernel(const double2* __restrict__ d, int64_t n_freq, double f0, double df,
+                           const int64_t* __restrict__ off, int64_t n_bins, double* __restrict__ P,
+                           double* __restrict__ f_out, double* __restrict__ nu_out, int n_ch) {
     const int lane = threadIdx.x & (G - 1);
     const int64_t g0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
     const int64_t ng = ((int64_t)gridDim.x * blockDim.x) / G;
@@ -43,23 +117,39 @@ __global__ void avg_periodogram_kernel(const double2* __restrict__ d, int64_t n_
         }
         double acc[C];
 #pragma unroll
-        for (int c = 0; c < C; ++c) acc[c] = 0.0;
-#pragma unroll 4
-        for (int64_t k = b0 + lane; k < b1; k += G) {
+        for (int c = 0; c < C; ++c) {
+            acc[c] = 0.0;
+            if (c >= n_ch) continue;
+            LaneSum<SOFT> sum;
+            sum.reset();
+            const double2* dc = d + (int64_t)c * n_freq;
+            constexpr int kBatch = LaneSum<SOFT>::kBatch;
+#pragma unroll(SOFT ? 1 : 4)
+            for (int64_t k = b0 + lane; k < b1; k += kBatch * G) {
+                double2 v[kBatch];
 #pragma unroll
-            for (int c = 0; c < C; ++c) {
-                if (c < n_ch) {
-                    const double2 v = __ldg(d + (int64_t)c * n_freq + k);
-                    acc[c] = fma(v.x, v.x, fma(v.y, v.y, acc[c]));
-                }
+                for (int u = 0; u < kBatch; ++u)
+                    v[u] = k + u * G < b1 ? __ldg(dc + k + u * G) : make_double2(0.0, 0.0);
+                sum.add(v);
             }
+            acc[c] = sum.value();
         }
 #pragma unroll
         for (int o = G / 2; o > 0; o >>= 1)
 #pragma unroll
             for (int c = 0; c < C; ++c) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o, G);
-        if (live && lane == 0) {
-            const int64_t n = b1 - b0;
+        const int64_t n = b1 - b0;
+        if (G >= 4) {
+            double v = acc[0];
+#pragma unroll
+            for (int c = 1; c < C; ++c)
+                if (lane == c) v = acc[c];
+            if (live && lane < n_ch) P[(int64_t)lane * n_bins + i] = n > 0 ? v / (double)n : NAN;
+            if (live && lane == 3) {
+                f_out[i] = f0 + df * (0.5 * (double)(b0 + b1 - 1));
+                nu_out[i] = (double)n;
+            }
+        } else if (live && lane == 0) {
 #pragma unroll
             for (int c = 0; c < C; ++c)
                 if (c < n_ch) P[(int64_t)c * n_bins + i] = n > 0 ? acc[c] / (double)n : NAN;
@@ -69,7 +159,7 @@ __global__ void avg_periodogram_kernel(const double2* __restrict__ d, int64_t n_
     }
 }
 
-template <int C, int G>
+template <int C, int G, bool SOFT>
 cudaError_t launch_avg(const double2* d, int64_t n_freq, double f0, double df, const int64_t* off, int64_t n_bins,
                        double* P, double* f, double* nu, int n_ch, cudaStream_t sm) {
     int dev = 0, n_sm = 1;
@@ -79,7 +169,7 @@ cudaError_t launch_avg(const double2* d, int64_t n_freq, double f0, double df, c
     const int64_t want = (n_bins * G + threads - 1) / threads;
     const int64_t cap = (int64_t)n_sm * 8;   // persistent: 8 blocks of 256 threads per SM
     const unsigned grid = (unsigned)(want < cap ? (want < 1 ? 1 : want) : cap);
-    avg_periodogram_kernel<C, G><<<grid, threads, 0, sm>>>(d, n_freq, f0, df, off, n_bins, P, f, nu, n_ch);
+    avg_periodogram_kernel<C, G, SOFT><<<grid, threads, 0, sm>>>(d, n_freq, f0, df, off, n_bins, P, f, nu, n_ch);
     return cudaGetLastError();
 }
 
@@ -121,11 +211,11 @@ extern "C" lisa_status lisa_averaged_periodogram(const double* d, int32_t n_chan
     const double width = (double)n_freq / (double)n_bins;
     cudaError_t e;
     if (width >= 256.0)
-        e = launch_avg<3, 8>(dd, n_freq, f0, df, off, n_bins, P, f, nu, n_channels, sm);
+        e = launch_avg<3, 8, true>(dd, n_freq, f0, df, off, n_bins, P, f, nu, n_channels, sm);
     else if (width >= 12.0)
-        e = launch_avg<3, 4>(dd, n_freq, f0, df, off, n_bins, P, f, nu, n_channels, sm);
+        e = launch_avg<3, 4, true>(dd, n_freq, f0, df, off, n_bins, P, f, nu, n_channels, sm);
     else
-        e = launch_avg<3, 1>(dd, n_freq, f0, df, off, n_bins, P, f, nu, n_channels, sm);
+        e = launch_avg<3, 1, false>(dd, n_freq, f0, df, off, n_bins, P, f, nu, n_channels, sm);
     return check_cuda(e);
 }
 
