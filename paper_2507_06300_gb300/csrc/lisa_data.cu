@@ -304,6 +304,8 @@ lisa_status rebuild_work(lisa_data* d) {
             break;
         }
     }
+    d->chunk_items = d->nseg > 1 && seg_bins(t.tile_bins, 1, d->nseg) == kSegBins;
+    for (const DatasetDev& D : d->h_ds) d->chunk_items &= D.ns == 0 || lanes(D) == kThreads32;
     // the plain FP64 kernels' units: half a segment of bins x 32 states, one warp each.  (They share
     // the FP64 pipe, so what counts is that the units are many and of one size; half a segment is what
     // the workspace of the FP32 path holds slots for.)

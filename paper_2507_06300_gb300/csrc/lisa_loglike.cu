@@ -348,6 +348,7 @@ __device__ __forceinline__ float2 pair_term32(const float4 q0, const float4* __r
 // Items with one state per thread write their partial sums directly; items that split a state's
 // bins over several threads (rows) combine the rows in shared memory between two barriers.
 constexpr int kStages = 2;
+constexpr int kChunkPairs = 32;   // pair blocks per FP32 partial sum (64 bins)
 constexpr int kWarps32 = kThreads32 / 32;
 
 template <int C, bool HAS_H, bool BROKEN, int G>
@@ -360,7 +361,6 @@ __global__ void __launch_bounds__(kThreads32, G == 2 ? 5 : 4)
                         int tile_bins, int stage_bins, int nseg, unsigned wait_limit, int skip_copies) {
     constexpr int NSP = C + (HAS_H ? 1 : 0);
     constexpr int U = G / 2;                  // pair blocks per iteration of the knot-free loop
-    constexpr int kChunkPairs = 32;           // pair blocks per FP32 partial sum (64 bins)
     constexpr unsigned kLocated = 1u << 31;   // s_hm: this thread's intervals have been located
     constexpr unsigned kSplineBits = (1u << NSP) - 1u;
     extern __shared__ __align__(128) unsigned char smem[];
@@ -685,6 +685,233 @@ __global__ void __launch_bounds__(kThreads32, G == 2 ? 5 : 4)
     }
 }
 
+// ---- the fused likelihood of small problems ----------------------------------------------------
+// For items of a single FP32 chunk (64 bins; the segments of a problem too small to fill the GPU).
+// There a chunk's 32 pair blocks, one after the other in one warp, were the kernel's time, above all the
+// lowest-frequency chunk's: most of a short record's knots lie in it, and each block that holds a knot
+// of any of the warp's 32 states costs about 600 instructions (A, E, 2,000 bins, 128 states: 41 us with
+// its knots, 10 us without).  Here a CTA takes one chunk of 32 states and its four warps evaluate eight
+// pair blocks each; then one warp adds the terms in the order, and with the operations, of the fused
+// kernel (the same bits): 16 us.  Plain loads stage the 3 KB of the table.
+constexpr int kChunkWarps = 4;
+
+template <int C, bool HAS_H, bool BROKEN>
+__global__ void __launch_bounds__(32 * kChunkWarps)
+    loglike_chunk_kernel(const WorkItem* __restrict__ items, const float* __restrict__ rec32,
+                         const StateParams* __restrict__ prm, const int32_t* __restrict__ sstat,
+                         const float* __restrict__ kxr, const float* __restrict__ srec, int kmax, int nsp,
+                         const DatasetDev* __restrict__ ds, double* __restrict__ partial) {
+    constexpr int NSP = C + (HAS_H ? 1 : 0);
+    constexpr int kOwn = kChunkPairs / kChunkWarps;                       // pair blocks per warp
+    __shared__ __align__(16) float s_tab[(kChunkPairs + 1) * kPairRec];   // the chunk, and the block before it
+    __shared__ float4 s_val[kChunkPairs][32];                             // (v, log2 prod) of both bins
+    __shared__ unsigned char s_flag[kChunkPairs][32];                     // bit 0, 1: bin kept; bit 2: reaches a knot
+    __shared__ float s_mx[kChunkWarps][32];
+    asm volatile("griddepcontrol.launch_dependents;");
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const WorkItem w = items[blockIdx.x >> 2];
+    const int ls = 32 * (int)(blockIdx.x & 3u) + lane;
+    if ((ls & ~31) >= w.ns) return;   // no states: the whole CTA
+    const int p_lo = min(w.nb >> 1, w.seg * kChunkPairs), p_hi = min(w.nb >> 1, p_lo + kChunkPairs);
+    const int prev = w.seg > 0 && p_lo < p_hi ? 1 : 0;   // the block before the chunk is staged too
+    {
+        const float4* src = reinterpret_cast<const float4*>(rec32 + ((w.bin0 >> 1) + p_lo - prev) * kPairRec);
+        const int n = (p_hi - p_lo + prev) * (kPairRec / 4);
+        for (int e = threadIdx.x; e < n; e += blockDim.x) reinterpret_cast<float4*>(s_tab)[e] = __ldg(src + e);
+    }
+    const int s = w.s0 + ls;
+    const bool active = ls < w.ns && (sstat[s] & kUserBits) == 0;
+    const DatasetDev& D = ds[w.ds];
+    __syncthreads();
+    const float* tb = s_tab + prev * kPairRec;   // pair block 0 of the chunk
+    const int np = p_hi - p_lo;
+    float ao2 = 0.f, at2 = 0.f, Af = 0.f, n1 = 0.f, n2 = 0.f;
+    if (active) {
+        const float4 q0 = __ldg(reinterpret_cast<const float4*>(prm + s));
+        ao2 = q0.x;
+        at2 = q0.y;
+        Af = HAS_H ? q0.z : 0.f;
+        n1 = q0.w;
+        n2 = BROKEN ? __ldg(&prm[s].n2) : n1;
+    }
+    // this thread's current intervals (an ill-conditioned one as the zero cubic, its bins masked)
+    Iv32 iv[NSP];
+    float xr[NSP], xmin = INFINITY;
+    int jj[NSP];
+    unsigned hm = 0u;
+    auto rec = [&](int a, int j) {
+        return reinterpret_cast<const float4*>(
+            srec + (((int64_t)s * nsp + a) * (int64_t)(kmax + 1) + LISA_IDX(j, kmax + 1)) * kSplineRec32);
+    };
+    auto install = [&](int a, int j, float4 A, float4 B) {
+        xr[a] = A.x;
+        jj[a] = j;
+        if (B.w <= (float)kRobustT) {
+            iv[a] = Iv32{A.y, A.z, A.w, B.x, B.y};
+            hm &= ~(1u << a);
+        } else {
+            iv[a] = Iv32{0.f, 0.f, 0.f, 0.f, 0.f};
+            hm |= 1u << a;
+        }
+    };
+    auto nearest = [&]() {
+        xmin = xr[0];
+#pragma unroll
+        for (int a = 1; a < NSP; ++a) xmin = fminf(xmin, xr[a]);
+    };
+    auto locate = [&](float x) {
+        const int kxs = kxr_stride(kmax);
+        hm = 0u;
+#pragma unroll
+        for (int a = 0; a < NSP; ++a) {
+            const float4* kq = reinterpret_cast<const float4*>(kxr + ((int64_t)s * nsp + a) * kxs);
+            int j = 0;
+#pragma unroll 4
+            for (int q = 0; q < kxs / 4; ++q) {
+                const float4 v = __ldg(kq + q);
+                j += (v.x <= x) + (v.y <= x) + (v.z <= x) + (v.w <= x);
+            }
+            j = min(j, kmax);
+            install(a, j, __ldg(rec(a, j)), __ldg(rec(a, j) + 1));
+        }
+        nearest();
+    };
+    // to the intervals that hold x: the next records of all splines that pass a knot at once
+    auto advance_to = [&](float x) {
+        if (x < xmin) return;
+        float4 A[NSP], B[NSP];
+        unsigned need = 0u;
+#pragma unroll
+        for (int a = 0; a < NSP; ++a)
+            if (x >= xr[a]) {
+                const float4* q = rec(a, min(jj[a] + 1, kmax));
+                A[a] = __ldg(q);
+                B[a] = __ldg(q + 1);
+                need |= 1u << a;
+            }
+#pragma unroll
+        for (int a = 0; a < NSP; ++a)
+            if ((need >> a) & 1u) {
+                int j = min(jj[a] + 1, kmax);
+                while (x >= A[a].x && j < kmax) {
+                    ++j;
+                    A[a] = __ldg(rec(a, j));
+                    B[a] = __ldg(rec(a, j) + 1);
+                }
+                install(a, j, A[a], B[a]);
+            }
+        nearest();
+    };
+    // v = sum_c 1/S_c - C and lg = log2 prod_c S_c of bin i; guarded: per channel when the product leaves
+    // [1e-30, 1e30], as term_from_S
+    auto parts = [&](int i, bool guarded, float& v, float& lg) {
+        const float x = fld(tb, i, 0), ell = fld(tb, i, 1);
+        float S[C], p[NSP];
+#pragma unroll
+        for (int a = 0; a < NSP; ++a) {
+            const float t = x - iv[a].xo;
+            p[a] = fmaf(fmaf(fmaf(iv[a].c3, t, iv[a].c2), t, iv[a].c1), t, iv[a].c0);
+        }
+        float eh = 0.f;
+        if (HAS_H) eh = Af * ex2_approx(fmaf(BROKEN ? (ell < 0.f ? n1 : n2) : n1, ell, p[C]));
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            const float nc = fmaf(ao2, fld(tb, i, 3 + c), at2 * fld(tb, i, 6 + c));
+            const float e = ex2_approx(p[c]);
+            S[c] = HAS_H ? fmaf(e, nc, eh * fld(tb, i, 9 + c)) : e * nc;
+        }
+        const float p01 = S[0] * S[1];
+        const float prod = C == 3 ? p01 * S[C - 1] : p01;
+        const float num = C == 3 ? fmaf(S[C - 1], S[0] + S[1], p01) : S[0] + S[1];
+        v = fmaf(num, rcp_approx(prod), -(float)C);
+        lg = lg2_approx(prod);
+        if (guarded && !(prod > 1e-30f && prod < 1e30f && num < 1e30f)) {
+            v = -(float)C;
+            lg = 0.f;
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                v += rcp_approx(S[c]);
+                lg += lg2_approx(S[c]);
+            }
+        }
+    };
+    const int q_lo = warp * kOwn, q_hi = min(np, q_lo + kOwn);
+    float mx = -INFINITY, xmin0 = INFINITY;
+    float keep0 = 1.f;   // at the chunk's start (warp 0)
+    if (active && q_lo < q_hi) {
+        // where the fused kernel's walk would be before this warp's first bin
+        locate(fld(tb, 2 * q_lo - (q_lo > 0 || prev ? 1 : 0), 0));
+        xmin0 = xmin;
+        keep0 = hm ? 0.f : 1.f;
+#pragma unroll 1
+        for (int q = q_lo; q < q_hi; ++q) {
+            const float x0 = fld(tb, 2 * q, 0), x1 = fld(tb, 2 * q + 1, 0);
+            const bool cross = x1 >= xmin;
+            float4 o;
+            if (cross) advance_to(x0);
+            unsigned f = (hm ? 0u : 1u) | (cross ? 4u : 0u);
+            parts(2 * q, cross, o.x, o.z);
+            if (cross) advance_to(x1);
+            f |= hm ? 0u : 2u;
+            parts(2 * q + 1, cross, o.y, o.w);
+            if (!cross) mx = fmax3(mx, o.z, o.w);
+            s_val[q][lane] = o;
+            s_flag[q][lane] = (unsigned char)f;
+        }
+    }
+    s_mx[warp][lane] = mx;
+    __syncthreads();
+    if (warp > 0) return;
+    // the fused kernel's sums over the chunk: in a chunk without a knot of any of the warp's states the
+    // nu-weighted sums of v and log2 prod run apart, else term by term
+    if (!active) return;
+    float acc_hi = 0.f, acc_lo = 0.f;
+    if (np > 0) {
+        float2 acc2 = make_float2(0.f, 0.f);
+        const float x_last = fld(tb, 2 * np - 1, 0);
+        if (!__any_sync(__activemask(), x_last >= xmin0)) {
+            float2 accv = make_float2(0.f, 0.f), accl = make_float2(0.f, 0.f);
+            for (int q = 0; q < np; ++q) {
+                const float4 o = s_val[q][lane];
+                const float2 nu = make_float2(fld(tb, 2 * q, 2), fld(tb, 2 * q + 1, 2));
+                accv = __ffma2_rn(nu, make_float2(o.x, o.y), accv);
+                accl = __ffma2_rn(nu, make_float2(o.z, o.w), accl);
+            }
+            acc2 = __fmul2_rn(make_float2(keep0, keep0),
+                              __ffma2_rn(make_float2((float)kLn2, (float)kLn2), accl, accv));
+        } else {
+            for (int q = 0; q < np; ++q) {
+                const float4 o = s_val[q][lane];
+                const unsigned f = s_flag[q][lane];
+                const float tx = fld(tb, 2 * q, 2) * fmaf((float)kLn2, o.z, o.x);
+                const float ty = fld(tb, 2 * q + 1, 2) * fmaf((float)kLn2, o.w, o.y);
+                const float kx = f & 1u ? 1.f : 0.f, ky = f & 2u ? 1.f : 0.f;
+                const bool cross = f & 4u;
+                acc2.x = fmaf(kx, tx, acc2.x);
+                const float r = fmaf(ky, ty, cross ? acc2.x : acc2.y);
+                if (cross) acc2.x = r; else acc2.y = r;
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < kChunkWarps; ++q) mx = fmaxf(mx, s_mx[q][lane]);
+        if (!(mx <= kPairLg2Max && fabsf(acc2.x + acc2.y) < INFINITY)) {
+            // redone bin by bin on the guarded path, as the fused kernel does
+            locate(fld(tb, 0, 0));
+            acc2 = make_float2(0.f, 0.f);
+#pragma unroll 1
+            for (int i = 0; i < 2 * np; ++i) {
+                advance_to(fld(tb, i, 0));
+                float v, lg;
+                parts(i, true, v, lg);
+                acc2.x += (hm ? 0.f : 1.f) * (fld(tb, i, 2) * fmaf((float)kLn2, lg, v));
+            }
+        }
+        const ff sum = ff_add(ff{0.f, 0.f}, two_sum(acc2.x, acc2.y));
+        acc_hi = sum.hi;
+        acc_lo = sum.lo;
+    }
+    partial[D.pbase + (int64_t)(s - D.s0) * D.nslots + LISA_IDX(w.slot, D.nslots)] = (double)acc_hi + (double)acc_lo;
+}
 
 // ---- compensated path: the ill-conditioned intervals of the states the setup routed ------
 struct IvR {
@@ -1268,7 +1495,11 @@ cudaError_t launch_fp32_g(const lisa_data* d, const StateParams* prm, const int3
     const size_t smem = 2 * (size_t)d->stage_bins * kRec * sizeof(float);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<d->fgrid, kThreads32, smem, sm>>>(d->d_items, (int)d->n_items, d->d_cta_first,
+    if (d->chunk_items && !d->test_skip_copies)   // (the test of the timeout path needs the bulk copies)
+        loglike_chunk_kernel<C, H, B><<<(unsigned)d->n_items * 4u, 32 * kChunkWarps, 0, sm>>>(
+            d->d_items, d->d_rec32, prm, sstat, kxr, srec, kmax, d->nsp, d->d_ds, partial);
+    else
+        kern<<<d->fgrid, kThreads32, smem, sm>>>(d->d_items, (int)d->n_items, d->d_cta_first,
                                               d->d_rec32, prm, sstat, kxr, srec, kmax, d->nsp, d->d_ds, partial, err,
                                               d->tiling.tile_bins, d->stage_bins, d->nseg, d->wait_limit,
                                               d->test_skip_copies);
