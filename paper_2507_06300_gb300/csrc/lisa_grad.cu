@@ -133,6 +133,9 @@ __global__ void __launch_bounds__(128, 3)
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const int64_t wg = first_unit(n_units, nw);
     const float2 m1 = dup2(-1.f);
+    // the compensated pass, launched next as a programmatic dependent, may start on the SMs that this
+    // grid's CTAs leave (it waits for this grid before it touches what this kernel writes)
+    asm volatile("griddepcontrol.launch_dependents;");
     for (int64_t u = wg; u < n_units; u += nw) {
         const AdjUnit U = units[u];
         const DatasetDev& D = ds[U.ds];
@@ -767,6 +770,9 @@ __global__ void __launch_bounds__(MODE == kComp ? 128 : 512)
     // from the counter (a state's heavy ranges are contiguous in the list); the exits below are
     // CTA-uniform
     __shared__ int s_item;
+    asm volatile("griddepcontrol.launch_dependents;");
+    // kFallback reads what the passes before it wrote; kComp only adds to it, after its own work
+    if (MODE == kFallback) asm volatile("griddepcontrol.wait;" ::: "memory");
     const int n_items = list[0] * R;
     for (;;) {
     if (threadIdx.x == 0) s_item = atomicAdd(next_item, 1);
@@ -1172,6 +1178,7 @@ __global__ void __launch_bounds__(MODE == kComp ? 128 : 512)
         const double v = wsum(MODE == kComp ? (double)ltf[k] : ts[k]);
         if (lane == 0) s_t[warp][k] = v;
     }
+    if (MODE == kComp) asm volatile("griddepcontrol.wait;" ::: "memory");
     __syncthreads();
     // the warps' sums in order, to the slots
     for (int e = threadIdx.x; e < NSP * nsl; e += blockDim.x) {
@@ -1223,6 +1230,8 @@ __global__ void __launch_bounds__(MODE == kComp ? 128 : 512)
         }
     }
     }
+    // (not complete before the adjoint kernel is: the passes after this one wait for it alone)
+    if (MODE == kComp) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // ---- epilogue: one warp per state, FP64 ----------------------------------------------------------
@@ -1623,6 +1632,7 @@ __global__ void __launch_bounds__(128, 4)
                             const int32_t* __restrict__ fb) {
     __shared__ double sX[4][64];
     __shared__ double sY[4][64];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int warp = threadIdx.x >> 5;
     const int64_t u = (int64_t)blockIdx.x * 4 + warp;
     if (u >= (int64_t)S * nsp) return;
@@ -1682,6 +1692,7 @@ cudaError_t launch_adjoint(const lisa_data* d, bool fp32, const lisa_params* par
     const int S = (int)d->n_states;
     const int Rc = adj_max_ranges(d, kAdjBins), Rf = adj_max_ranges(d, d->adj_bins);
     prof_mark(d, prof, 0, sm);
+    cudaError_t e = cudaSuccess;
     if (fp32 && cudaMemsetAsync(gw.fb, 0, sizeof(int32_t) * (2 * (size_t)S + 3), sm) != cudaSuccess)
         return cudaErrorInvalidValue;
     if (d->n_adj_units > 0) {
@@ -1707,9 +1718,10 @@ cudaError_t launch_adjoint(const lisa_data* d, bool fp32, const lisa_params* par
             if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, adjoint_range_kernel<C, H, B, kComp>, 128, smc) !=
                 cudaSuccess)
                 return cudaErrorInvalidValue;
-            adjoint_range_kernel<C, H, B, kComp><<<d->n_sm * std::max(occ, 1), 128, smc, sm>>>(
-                S, d->d_state_ds, d->d_ds, d->d_rec32, d->d_xlo32, d->d_elllo32, params->theta_dev, sstat, gw.route,
-                Rc, gw.fb, gw.fb + 2 * S + 1, nint, srec, gw.hull, kn->kmax, d->nsp, d->d_adj_prefix, scal, mom,
+            e = launch_dependent(
+                adjoint_range_kernel<C, H, B, kComp>, d->n_sm * std::max(occ, 1), 128, smc, sm, !prof, S,
+                d->d_state_ds, d->d_ds, d->d_rec32, d->d_xlo32, d->d_elllo32, params->theta_dev, sstat, gw.route, Rc,
+                gw.fb, gw.fb + 2 * S + 1, nint, srec, gw.hull, kn->kmax, d->nsp, d->d_adj_prefix, scal, mom,
                 d->adj_bins);
             // the states whose FP32 sums left the FP32 range (flagged by both passes above): all
             // their bins again, FP64 sums, on a resident grid of 16-warp CTAs
@@ -1720,26 +1732,29 @@ cudaError_t launch_adjoint(const lisa_data* d, bool fp32, const lisa_params* par
             if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, adjoint_range_kernel<C, H, B, kFallback>, 512,
                                                               smf) != cudaSuccess)
                 return cudaErrorInvalidValue;
-            adjoint_range_kernel<C, H, B, kFallback><<<d->n_sm * std::max(occ, 1), 512, smf, sm>>>(
-                S, d->d_state_ds, d->d_ds, d->d_rec32, d->d_xlo32, d->d_elllo32, params->theta_dev, sstat,
-                gw.fb + S, Rf, gw.fb, gw.fb + 2 * S + 2, nint, srec, nullptr, kn->kmax, d->nsp, d->d_adj_prefix, scal,
+            if (e != cudaSuccess) return e;
+            e = launch_dependent(
+                adjoint_range_kernel<C, H, B, kFallback>, d->n_sm * std::max(occ, 1), 512, smf, sm, !prof, S,
+                d->d_state_ds, d->d_ds, d->d_rec32, d->d_xlo32, d->d_elllo32, params->theta_dev, sstat, gw.fb + S, Rf,
+                gw.fb, gw.fb + 2 * S + 2, nint, srec, (const float2*)nullptr, kn->kmax, d->nsp, d->d_adj_prefix, scal,
                 mom, d->adj_bins);
         } else
             adjoint_fp64_kernel<C, H, B><<<(unsigned)d->n_adj_units, 32, 0, sm>>>(d->d_adj_units, d->d_ds, d->d_rec64,
                                                                d->d_exptab, params->theta_dev, sstat, nint,
                                                                static_cast<const double*>(srec), kn->kmax, d->nsp,
                                                                d->d_adj_prefix, scal, mom, d->adj_bins);
-        cudaError_t e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     } else {
         prof_mark(d, prof, 1, sm);
     }
     prof_mark(d, prof, 2, sm);
     const unsigned eb = (unsigned)((d->n_states * d->nsp + 3) / 4);
-    adjoint_epilogue_kernel<<<eb, 128, 0, sm>>>(
-        S, H ? 1 : 0, B ? 1 : 0, d->d_state_ds, d->d_ds, sstat, params->theta_dev, kn->count_dev, kn->x_dev, kn->w_dev, kn->kmax, kn->kind,
-        d->nsp, d->d_adj_prefix, scal, mom, d->d_rx32, d->d_rx64, srec, fp32 ? 1 : 0, out, grad, gw.fb);
-    const cudaError_t e = cudaGetLastError();
+    e = launch_dependent(
+        adjoint_epilogue_kernel, eb, 128, 0, sm, !prof && d->n_adj_units > 0, S, H ? 1 : 0, B ? 1 : 0, d->d_state_ds,
+        d->d_ds, sstat, params->theta_dev, kn->count_dev, kn->x_dev, kn->w_dev, kn->kmax, kn->kind, d->nsp,
+        d->d_adj_prefix, scal, mom, d->d_rx32, d->d_rx64, srec, fp32 ? 1 : 0, out, grad, gw.fb);
+    if (e == cudaSuccess) e = cudaGetLastError();
     prof_mark(d, prof, 3, sm);
     if (prof) d->prof_valid = true;
     return e;

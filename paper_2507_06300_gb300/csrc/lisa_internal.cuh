@@ -323,4 +323,23 @@ inline void prof_mark(const lisa_data* d, bool on, int k, cudaStream_t sm) {
 }
 lisa_status check_cuda(cudaError_t e);
 
+// Launches kern as a programmatic dependent of the kernel before it in the stream (when dep; else the
+// ordinary way): its CTAs may start before that one has ended, and it waits itself
+// (griddepcontrol.wait) where it needs the results.
+template <class... P, class... A>
+cudaError_t launch_dependent(void (*kern)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t sm, bool dep,
+                             A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = sm;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = dep ? 1 : 0;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, (P)args...);
+}
+
 }  // namespace lisa

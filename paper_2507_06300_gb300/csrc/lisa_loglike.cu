@@ -1227,6 +1227,7 @@ __global__ void __launch_bounds__(kRobWarps * 32, 2)
                           const float* __restrict__ elllo32, const StateParams* __restrict__ prm,
                           const int32_t* __restrict__ nint, const float* __restrict__ srec, int kmax, int nsp,
                           double* __restrict__ rpart, int* __restrict__ err, unsigned wait_limit) {
+    asm volatile("griddepcontrol.launch_dependents;");   // the finalize kernel (it waits for this one's end)
     robust_units<C, HAS_H, BROKEN>(rcount, rlist, tile_bins, rec32, xlo32, elllo32, prm, nint, srec, kmax, nsp, rpart,
                                    err, wait_limit);
     // launched as a programmatic dependent of the fused kernel, so that its CTAs can start on SMs
@@ -1390,6 +1391,8 @@ __global__ void finalize_kernel(int S, const int32_t* __restrict__ state_ds, con
                                 const int32_t* __restrict__ rent, const RobustEntry* __restrict__ rlist,
                                 const double* __restrict__ rpart, const int* __restrict__ err, int fp32,
                                 double* __restrict__ out) {
+    // launched as a programmatic dependent of the likelihood's last kernel, whose end it waits for
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int s = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (s >= S) return;   // uniform per warp
@@ -1718,9 +1721,9 @@ lisa_status lisa_psd_loglike(const lisa_data* d, const lisa_params* params, cons
         prof_mark(d, prof, 2, sm);
     }
     if (e != cudaSuccess) return LISA_ERR_CUDA;
-    finalize_kernel<<<(S + 7) / 8, 256, 0, sm>>>(S, d->d_state_ds, d->d_ds, sstat, partial, rent, rlist, rpart, err,
-                                                 fp32 ? 1 : 0, out);
-    e = cudaGetLastError();
+    e = launch_dependent(finalize_kernel, (unsigned)((S + 7) / 8), 256, 0, sm, !prof && d->n_items > 0, S, d->d_state_ds, d->d_ds, sstat,
+                         partial, rent, rlist, rpart, err, fp32 ? 1 : 0, out);
+    if (e == cudaSuccess) e = cudaGetLastError();
     prof_mark(d, prof, 3, sm);
     if (prof) d->prof_valid = true;
     return check_cuda(e);
