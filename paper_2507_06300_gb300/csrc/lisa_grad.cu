@@ -1390,19 +1390,20 @@ __device__ __noinline__ bool epilogue_spline(int s, int a, int has_h, int broken
         double lo_b, hi_b;
         if (fp32) {
             const float* r = static_cast<const float*>(srec_v) + (sp * (int64_t)(kmax + 1) + LISA_IDX(jj, kmax + 1)) * kSplineRec32;
-            lo_b = (double)r[6];
-            hi_b = (double)r[0];
+            lo_b = spl::widen(r[6]);
+            hi_b = spl::widen(r[0]);
         } else {
             const double* r = static_cast<const double*>(srec_v) + (sp * (int64_t)(kmax + 1) + LISA_IDX(jj, kmax + 1)) * kSplineRec;
             lo_b = r[0];
             hi_b = r[1];
         }
+        const long long lo_k = m64::order_key(lo_b), hi_k = m64::order_key(hi_b);   // integer comparisons
         r1[q] = nr - 1;
         if (jj != 0) {
             int lo = 0, hi = nr;
             while (lo < hi) {
                 const int mid = (lo + hi) >> 1;
-                if (__ldg(&rx[mid].y) >= lo_b) hi = mid; else lo = mid + 1;
+                if (m64::order_key(__ldg(&rx[mid].y)) >= lo_k) hi = mid; else lo = mid + 1;
             }
             r0[q] = lo;
         }
@@ -1410,7 +1411,7 @@ __device__ __noinline__ bool epilogue_spline(int s, int a, int has_h, int broken
             int lo = 0, hi = nr;
             while (lo < hi) {
                 const int mid = (lo + hi) >> 1;
-                if (__ldg(&rx[mid].x) < hi_b) lo = mid + 1; else hi = mid;
+                if (m64::order_key(__ldg(&rx[mid].x)) < hi_k) lo = mid + 1; else hi = mid;
             }
             r1[q] = lo - 1;
         }
@@ -1439,8 +1440,8 @@ __device__ __noinline__ bool epilogue_spline(int s, int a, int has_h, int broken
         const int jj = lane + 32 * q;
         if (jj >= nint) continue;
         for (int p = 0; p < 4; ++p) {
-            bad |= !isfinite(Md[q][p]);
-            M[q][p] = T(Md[q][p]);
+            bad |= m64::exponent(Md[q][p]) == 2047;
+            M[q][p] = spl::from_double<T>(Md[q][p]);
         }
         if (fp32) {
             // moments about the FP32 midpoint xo -> about the left knot x_j:  t = u + mo
@@ -1593,7 +1594,7 @@ __device__ __noinline__ bool epilogue_spline(int s, int a, int has_h, int broken
     if (lane == 0) {
         ga[0] = spl::to_double(y0);
         ga[kmax + 1] = spl::to_double(yK);
-        bad |= !isfinite(ga[0]) || !isfinite(ga[kmax + 1]);
+        bad |= m64::exponent(ga[0]) == 2047 || m64::exponent(ga[kmax + 1]) == 2047;
     }
     const int k_in = K - 2;
     for (int half = 0; half < 2; ++half) {
@@ -1605,7 +1606,7 @@ __device__ __noinline__ bool epilogue_spline(int s, int a, int has_h, int broken
         if (i < k_in) {
             ga[1 + LISA_IDX(i, kmax)] = spl::to_double(gy);
             ga[kmax + 2 + LISA_IDX(i, kmax)] = spl::to_double(gx);
-            bad |= !isfinite(ga[1 + i]) || !isfinite(ga[kmax + 2 + i]);
+            bad |= m64::exponent(ga[1 + i]) == 2047 || m64::exponent(ga[kmax + 2 + i]) == 2047;
         }
     }
     return __any_sync(kFullMask, bad);

@@ -7,6 +7,7 @@
 #pragma once
 
 #include "lisa_math.cuh"
+#include "lisa_math64.cuh"
 
 namespace lisa {
 namespace spl {
@@ -52,8 +53,37 @@ __device__ __forceinline__ bool operator==(F2 a, F2 b) { return a.hi == b.hi && 
 __device__ __forceinline__ F2 fabs(F2 a) { return a.hi < 0.f || (a.hi == 0.f && a.lo < 0.f) ? -a : a; }
 __device__ __forceinline__ double fabs(double v) { return ::fabs(v); }   // (not hidden by the above)
 
+// An FP32 number as a double, exactly, by its bits (a conversion takes the FP64 pipe: 64 issue slots;
+// subnormals take it).
+__device__ __forceinline__ double widen(float f) {
+    const unsigned b = __float_as_uint(f), a = b & 0x7fffffffu;
+    if (a - 0x00800000u >= 0x7f000000u) return (double)f;   // 0, subnormal, infinite, NaN
+    return __hiloint2double((int)((b & 0x80000000u) | ((a >> 3) + (896u << 20))), (int)(b << 29));
+}
 __device__ __forceinline__ double to_double(double v) { return v; }
-__device__ __forceinline__ double to_double(F2 v) { return (double)v.hi + (double)v.lo; }
+__device__ __forceinline__ double to_double(F2 v) { return widen(v.hi) + widen(v.lo); }
+// A double in T.  As a float-float it is F2(double)'s value, bit for bit, split on the integer pipes (the
+// conversions and the difference take four FP64-pipe slots; 2,048 states x 4 splines x 8 knots with
+// their gradient: 1,317 -> 1,295 us, mostly in the epilogue):
+// hi is rounded to nearest even, lo the remainder, an integer below 2^29 times 2^(e - 52), rounded.
+template <class T>
+__device__ __forceinline__ T from_double(double v);
+template <>
+__device__ __forceinline__ double from_double<double>(double v) { return v; }
+template <>
+__device__ __forceinline__ F2 from_double<F2>(double v) {
+    const unsigned h = m64::hi32(v), l = m64::lo32(v);
+    const int e = (int)((h >> 20) & 0x7ffu) - 1023;
+    if ((unsigned)(e + 70) >= 190u)   // |v| outside [2^-70, 2^120): zero above all
+        return v == 0.0 ? F2(0.f, 0.f) : F2(v);
+    const unsigned m = ((h & 0xfffffu) << 3) | (l >> 29), rem = l & 0x1fffffffu;
+    const unsigned up = rem > 0x10000000u || (rem == 0x10000000u && (m & 1u)) ? 1u : 0u;
+    const unsigned sign = h & 0x80000000u;
+    const float hi = __uint_as_float(sign | ((((unsigned)(e + 127)) << 23 | m) + up));
+    const int r = (int)rem - (int)(up << 29);
+    const float scale = __uint_as_float(sign | ((unsigned)(e - 52 + 127) << 23));
+    return F2(hi, (float)r * scale);
+}
 __device__ __forceinline__ double sign_of(double v) { return v > 0.0 ? 1.0 : (v < 0.0 ? -1.0 : 0.0); }
 __device__ __forceinline__ F2 sign_of(F2 v) {
     const float h = v.hi != 0.f ? v.hi : v.lo;
@@ -188,32 +218,32 @@ __device__ __forceinline__ void warp_build_spline(WarpSpline<T>& W, const double
     int ra = 0, rb = 0;
     if (!st) {
         bool bx = false, bw = false;
+        // (comparisons on the integer pipes)
+        auto finite = [](double v) { return m64::exponent(v) != 2047; };
+        const long long klo = m64::order_key(xlo), khi = m64::order_key(xhi);
+        auto inside = [&](double v) { return finite(v) && m64::order_key(v) > klo && m64::order_key(v) < khi; };
         if (lane < k) {
             xa = px[LISA_IDX(lane, kmax)];
             wa = pw[1 + LISA_IDX(lane, kmax)];
-            bx |= !(isfinite(xa) && xa > xlo && xa < xhi);
-            bw |= !isfinite(wa);
+            bx |= !inside(xa);
+            bw |= !finite(wa);
         }
         if (lane + 32 < k) {
             xb = px[LISA_IDX(lane + 32, kmax)];
             wb = pw[1 + LISA_IDX(lane + 32, kmax)];
-            bx |= !(isfinite(xb) && xb > xlo && xb < xhi);
-            bw |= !isfinite(wb);
+            bx |= !inside(xb);
+            bw |= !finite(wb);
         }
         w0 = pw[0];
         wn = pw[kmax + 1];
-        bw |= !isfinite(w0) || !isfinite(wn);
+        bw |= !finite(w0) || !finite(wn);
         if (__any_sync(kFull, bx)) st |= LISA_STATE_BAD_POSITION;
         if (__any_sync(kFull, bw)) st |= LISA_STATE_BAD_AMPLITUDE;
     }
     if (!st) {
         // rank sort (stable) with duplicate detection, on integer keys that order like the
         // (finite) doubles, so the comparisons run on the integer pipes
-        auto key = [](double v) {
-            const long long b = __double_as_longlong(v);
-            return b >= 0 ? b : b ^ 0x7fffffffffffffffLL;
-        };
-        const long long ka = key(xa), kb = key(xb);
+        const long long ka = m64::order_key(xa), kb = m64::order_key(xb);
         bool dup = false;
         for (int i = 0; i < k; ++i) {
             const long long ki = __shfl_sync(kFull, i < 32 ? ka : kb, i & 31);
@@ -267,8 +297,8 @@ __device__ __forceinline__ void warp_build_spline(WarpSpline<T>& W, const double
     T* ih = W.ih;
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
-        x[q] = T(xd[q]);
-        y[q] = T(yd[q]);
+        x[q] = from_double<T>(xd[q]);
+        y[q] = from_double<T>(yd[q]);
     }
     h[1] = ih[1] = T(1);
     m[1] = T(0);
@@ -277,9 +307,9 @@ __device__ __forceinline__ void warp_build_spline(WarpSpline<T>& W, const double
         if (q >= (K > 32 ? 2 : 1)) break;   // warp-uniform
         const int j = lane + 32 * q;
         if (j < K - 1) {
-            h[q] = T(xn[q] - xd[q]);
+            h[q] = from_double<T>(xn[q] - xd[q]);
             ih[q] = T(1) / h[q];
-            m[q] = T(yn[q] - yd[q]) * ih[q];
+            m[q] = from_double<T>(yn[q] - yd[q]) * ih[q];
         } else {
             h[q] = ih[q] = T(1);
             m[q] = T(0);
