@@ -192,9 +192,7 @@ void release(lisa_data* d) {
     d->d_cta_first = nullptr;
     cudaFree(d->d_adj_units);
     cudaFree(d->d_adj_prefix);
-    cudaFree(d->d_rx32);
-    cudaFree(d->d_rx64);
-    cudaFree(d->d_exptab);
+    cudaFree(d->d_exptab);   // with the range-bound tables behind it
     d->d_exptab = nullptr;
     d->d_rx32 = d->d_rx64 = nullptr;
     d->d_adj_units = nullptr;
@@ -641,9 +639,10 @@ lisa_status lisa_data_create(const lisa_data_desc* desc, lisa_stream_t stream, l
         (st = dev_alloc(&d->d_elllo32, (size_t)NP)) || (st = dev_alloc(&nu_p, (size_t)NP)) ||
         (st = dev_alloc(&f, (size_t)N)) ||
         (st = dev_alloc(&nu, (size_t)N)) || (st = dev_alloc(&lnP, (size_t)NP)) ||
-        (st = dev_alloc(&R, (size_t)C * N)) || (st = dev_alloc(&d->d_rx32, (size_t)rbase)) ||
-        (st = dev_alloc(&d->d_rx64, (size_t)rbase)) || (st = dev_alloc(&d->d_exptab, (size_t)kExpTab)))
+        (st = dev_alloc(&R, (size_t)C * N)) || (st = dev_alloc(&d->d_exptab, (size_t)kExpTab + 4 * (size_t)rbase)))
         return fail(st);
+    d->d_rx32 = reinterpret_cast<double2*>(d->d_exptab + kExpTab);
+    d->d_rx64 = d->d_rx32 + rbase;
     cudaStream_t sm = (cudaStream_t)stream;
     bool ok = cudaMemcpyAsync(d->d_ds, d->h_ds.data(), D * sizeof(DatasetDev), cudaMemcpyHostToDevice, sm) == cudaSuccess &&
               cudaMemcpyAsync(d->d_state_ds, state_ds.data(), S * sizeof(int32_t), cudaMemcpyHostToDevice, sm) == cudaSuccess &&

@@ -67,6 +67,12 @@ __device__ __forceinline__ void fb_flag(int32_t* fb, int S, int s) {
     if (atomicExch(fb + s, 1) == 0) fb[S + 1 + atomicAdd(fb + S, 1)] = s;
 }
 
+// A = 10^log10A in FP32 (the library's exp10, about 40 FP64 instructions for every unit, where the table
+// does not reach).
+__device__ __forceinline__ float amplitude(double v, const double* __restrict__ exptab) {
+    return (float)(m64::small_exponent(v) ? m64::exp10_fast(v, exptab) : exp10(v));
+}
+
 // ---- FP32 adjoint: one warp per (dataset, range, up to 32 states) -----------------------------
 // The current interval of a spline: right end and index, and -x_o, -x_o's low part and the cubic's
 // coefficients duplicated in register pairs for the packed (two bins per instruction) path.
@@ -120,7 +126,7 @@ __global__ void __launch_bounds__(128, 3)
                         const double* __restrict__ theta, const int32_t* __restrict__ sstat,
                         const int32_t* __restrict__ nint, const float* __restrict__ srec, int kmax, int nsp,
                         const int64_t* __restrict__ prefix, double* __restrict__ scal, double* __restrict__ mom,
-                        int S, int32_t* __restrict__ fb, int adj_bins) {
+                        int S, int32_t* __restrict__ fb, int adj_bins, const double* __restrict__ exptab) {
     constexpr int NSP = C + (HAS_H ? 1 : 0);
     __shared__ float2 s_am[NSP * 4][128];
     __shared__ float2 s_as[6][128];
@@ -145,7 +151,7 @@ __global__ void __launch_bounds__(128, 3)
         if (!((amask >> lane) & 1u)) continue;
         const double* th = theta + (size_t)s * LISA_N_THETA;
         const float ao2 = (float)(th[0] * th[0]), at2 = (float)(th[1] * th[1]);
-        const float Af = HAS_H ? (float)exp10(th[2]) : 0.f;
+        const float Af = HAS_H ? amplitude(th[2], exptab) : 0.f;
         const float n1 = (float)th[3], n2 = BROKEN ? (float)th[4] : n1;
         const int64_t b0 = D.bin0 + (int64_t)U.rho * adj_bins;        // even
         const int nb = (int)min((int64_t)adj_bins, D.bin0 + D.npad - b0);
@@ -216,8 +222,10 @@ __global__ void __launch_bounds__(128, 3)
             double* row = mom_row(mom, pre, s, a, nsp, kmax, D.nranges) + 4 * (int64_t)LISA_IDX(U.rho + iv[a].j, D.nranges + kmax + 1);
 #pragma unroll
             for (int p = 0; p < 4; ++p) {
+                // one FP64 instruction a moment (16 with conversions and the factor, at every knot:
+                // gradient of A, E, 2,000 bins, 128 states 160 -> 137 us)
                 const float2 v = s_am[4 * a + p][tid];
-                row[p] = kLn10 * ((double)v.x + (double)v.y);   // q carries ln10 only here
+                row[p] = spl::widen(v.x) + spl::widen(v.y);   // (ln10, q's factor, comes in the epilogue)
                 bad |= !isfinite(v.x);
                 s_am[4 * a + p][tid] = make_float2(0.f, 0.f);
             }
@@ -577,7 +585,7 @@ __global__ void __launch_bounds__(32)
         double* row = mom_row(mom, pre, s, a, nsp, kmax, D.nranges) + 4 * (int64_t)LISA_IDX(U.rho + j[a], D.nranges + kmax + 1);
 #pragma unroll
         for (int p = 0; p < 4; ++p) {
-            row[p] = kLn10 * m[a][p];   // q carries ln10 only here
+            row[p] = m[a][p];   // (ln10, q's factor, comes in the epilogue)
             m[a][p] = 0.0;
         }
     };
@@ -725,7 +733,7 @@ __global__ void __launch_bounds__(32)
 // Mode kFallback: the states the FP32 epilogue flagged (their FP32 sums left the FP32 range), all
 // their bins: spline values in float-float from the FP32 records, the PSDs, 1 / S-hat and the
 // sums in FP64; the sums overwrite the slots (every interval from the range's first bin to its
-// last), in the FP32 adjoint's convention (moments about the records' midpoints, ln10 in q).
+// last), in the FP32 adjoint's convention (moments about the records' midpoints, q without ln10).
 // A resident grid runs the (state, range) items of a compact list (kComp: the setup's route
 // list; kFallback: the flag area's list), each CTA fetching its next item from a counter.
 // The CTA's warps (4 for kComp, 16 for kFallback) split the range's bins, their lanes 32
@@ -750,7 +758,8 @@ __global__ void __launch_bounds__(MODE == kComp ? 128 : 512)
                          int32_t* __restrict__ fb, int32_t* __restrict__ next_item,
                          const int32_t* __restrict__ nint, const void* __restrict__ srec_v,
                          const float2* __restrict__ hull, int kmax, int nsp, const int64_t* __restrict__ prefix,
-                         double* __restrict__ scal, double* __restrict__ mom, int adj_bins) {
+                         double* __restrict__ scal, double* __restrict__ mom, int adj_bins,
+                         const double* __restrict__ exptab) {
     constexpr int NSP = C + (HAS_H ? 1 : 0);
     // this pass's ranges: kComp takes kAdjBins bins whatever the adjoint's range size (its lanes'
     // FP32 template sums then cover the same bins), each holding `sub` of the adjoint's ranges, the
@@ -795,7 +804,7 @@ __global__ void __launch_bounds__(MODE == kComp ? 128 : 512)
     const int64_t pre = prefix[s];
     // the state's parameters as the FP32 adjoint derives them
     const float ao2 = (float)(th[0] * th[0]), at2 = (float)(th[1] * th[1]);
-    const float Af = (MODE == kComp && HAS_H) ? (float)exp10(th[2]) : 0.f;
+    const float Af = (MODE == kComp && HAS_H) ? amplitude(th[2], exptab) : 0.f;
     const float n1 = (float)th[3], n2 = BROKEN ? (float)th[4] : n1;
     // kFallback: the SGWB slopes and log2 A in float-float
     const ff sl1 = ff_from_double(th[3]), sl2 = ff_from_double(BROKEN ? th[4] : th[3]);
@@ -1081,7 +1090,7 @@ __global__ void __launch_bounds__(MODE == kComp ? 128 : 512)
                     To = fma(gr, (double)(rEN * go), To);
                     Tt = fma(gr, (double)(rEN * gt), Tt);
                     if (HAS_H) H = fma(gr, (double)(eHs * rp), H);
-                    qd[c] = (kLn10 * gr) * (double)rE;
+                    qd[c] = gr * (double)rE;
                 }
                 const double elld = (double)ell.hi + (double)ell.lo;
                 tc[0] = nu * (rs + kLn2 * ((double)ks + (double)l2s) - (double)C);
@@ -1092,7 +1101,7 @@ __global__ void __launch_bounds__(MODE == kComp ? 128 : 512)
                     tc[5] = elld * H;
                 else
                     tc[4] = elld * H;
-                if (HAS_H) qd[C] = kLn10 * H;
+                if (HAS_H) qd[C] = H;
             }
         }
         if (MODE == kFallback)
@@ -1192,8 +1201,8 @@ __global__ void __launch_bounds__(MODE == kComp ? 128 : 512)
         }
         double* row = mom_row(mom, pre, s, a, nsp, kmax, D.nranges);
         if (MODE == kComp) {
-            // the FP32 adjoint's slots carry ln10 (its q's factor); the sums go to the slot of the
-            // first of its ranges that holds a bin of the interval
+            // the sums go to the slot of the first of the adjoint's ranges that holds a bin of the
+            // interval
             if (v[0] != 0.0 || v[1] != 0.0 || v[2] != 0.0 || v[3] != 0.0) {
                 int i = 0;
                 if (sub > 1 && j > 0) {
@@ -1207,7 +1216,7 @@ __global__ void __launch_bounds__(MODE == kComp ? 128 : 512)
                 row += 4 * (int64_t)LISA_IDX(rho * sub + i / adj_bins + j, D.nranges + kmax + 1);
                 bool bad = false;
                 for (int p = 0; p < 4; ++p) {
-                    row[p] += kLn10 * v[p];
+                    row[p] += v[p];
                     bad |= !isfinite(row[p]);
                 }
                 if (bad) fb_flag(fb, S, s);
@@ -1440,8 +1449,9 @@ __device__ __noinline__ bool epilogue_spline(int s, int a, int has_h, int broken
         const int jj = lane + 32 * q;
         if (jj >= nint) continue;
         for (int p = 0; p < 4; ++p) {
-            bad |= m64::exponent(Md[q][p]) == 2047;
-            M[q][p] = spl::from_double<T>(Md[q][p]);
+            const double v10 = kLn10 * Md[q][p];   // q's factor ln10
+            bad |= m64::exponent(v10) == 2047;
+            M[q][p] = spl::from_double<T>(v10);
         }
         if (fp32) {
             // moments about the FP32 midpoint xo -> about the left knot x_j:  t = u + mo
@@ -1701,12 +1711,12 @@ cudaError_t launch_adjoint(const lisa_data* d, bool fp32, const lisa_params* par
             adjoint_fp32_kernel<C, H, B, true><<<grid, 128, 0, sm>>>(
                 d->d_adj_units, d->n_adj_units, d->d_ds, d->d_rec32, d->d_xlo32, params->theta_dev, sstat, nint,
                 static_cast<const float*>(srec), kn->kmax, d->nsp, d->d_adj_prefix, scal, mom, S, gw.fb,
-                d->adj_bins);
+                d->adj_bins, d->d_exptab);
         else if (fp32)
             adjoint_fp32_kernel<C, H, B, false><<<grid, 128, 0, sm>>>(
                 d->d_adj_units, d->n_adj_units, d->d_ds, d->d_rec32, d->d_xlo32, params->theta_dev, sstat, nint,
                 static_cast<const float*>(srec), kn->kmax, d->nsp, d->d_adj_prefix, scal, mom, S, gw.fb,
-                d->adj_bins);
+                d->adj_bins, d->d_exptab);
         prof_mark(d, prof, 1, sm);
         if (fp32) {
             // the bins of ill-conditioned intervals (routed states), masked above: the route
@@ -1723,7 +1733,7 @@ cudaError_t launch_adjoint(const lisa_data* d, bool fp32, const lisa_params* par
                 adjoint_range_kernel<C, H, B, kComp>, d->n_sm * std::max(occ, 1), 128, smc, sm, !prof, S,
                 d->d_state_ds, d->d_ds, d->d_rec32, d->d_xlo32, d->d_elllo32, params->theta_dev, sstat, gw.route, Rc,
                 gw.fb, gw.fb + 2 * S + 1, nint, srec, gw.hull, kn->kmax, d->nsp, d->d_adj_prefix, scal, mom,
-                d->adj_bins);
+                d->adj_bins, d->d_exptab);
             // the states whose FP32 sums left the FP32 range (flagged by both passes above): all
             // their bins again, FP64 sums, on a resident grid of 16-warp CTAs
             const size_t smf = range_smem(d, kn->kmax, 16);
@@ -1738,7 +1748,7 @@ cudaError_t launch_adjoint(const lisa_data* d, bool fp32, const lisa_params* par
                 adjoint_range_kernel<C, H, B, kFallback>, d->n_sm * std::max(occ, 1), 512, smf, sm, !prof, S,
                 d->d_state_ds, d->d_ds, d->d_rec32, d->d_xlo32, d->d_elllo32, params->theta_dev, sstat, gw.fb + S, Rf,
                 gw.fb, gw.fb + 2 * S + 2, nint, srec, (const float2*)nullptr, kn->kmax, d->nsp, d->d_adj_prefix, scal,
-                mom, d->adj_bins);
+                mom, d->adj_bins, d->d_exptab);
         } else
             adjoint_fp64_kernel<C, H, B><<<(unsigned)d->n_adj_units, 32, 0, sm>>>(d->d_adj_units, d->d_ds, d->d_rec64,
                                                                d->d_exptab, params->theta_dev, sstat, nint,
