@@ -598,6 +598,21 @@ __global__ void __launch_bounds__(kThreads32, G == 2 ? 5 : 4)
                         // others stay packed
 #pragma unroll 1
                         for (; ip < pcend; ++ip, blk += kPairRec / 4) {
+                            // U blocks at once where no lane reaches a knot in them (the same operations
+                            // in the same order)
+                            if (ip + U <= pcend &&
+                                !__any_sync(__activemask(), blk[(U - 1) * (kPairRec / 4)].y >= xmin)) {
+#pragma unroll
+                                for (int u = 0; u < U; ++u) {
+                                    const float4* pb = blk + u * (kPairRec / 4);
+                                    acc2 = __ffma2_rn(keep2, pair_term32<C, HAS_H, BROKEN>(pb[0], pb, iv2, ao2_2, at2_2, n1,
+                                                                                           n2, Af2, mx),
+                                                      acc2);
+                                }
+                                ip += U - 1;
+                                blk += (U - 1) * (kPairRec / 4);
+                                continue;
+                            }
                             const float4 q0 = blk[0];
                             if (q0.y >= xmin) {
                                 // the next record of every spline that passes a knot by the second
