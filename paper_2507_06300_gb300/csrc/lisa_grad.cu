@@ -162,16 +162,18 @@ __global__ void __launch_bounds__(128, 3)
         unsigned hm = 0;   // splines whose current interval is ill-conditioned (T > kRobustT)
         bool bad = false;  // a sum beyond the FP32 range: the state goes to the fallback list
         auto base = [&](int a) { return srec + ((int64_t)s * nsp + a) * (int64_t)(kmax + 1) * kSplineRec32; };
-        auto load = [&](int a) {
-            const float* r = base(a) + (size_t)LISA_IDX(iv[a].j, kmax + 1) * kSplineRec32;
-            iv[a].xr = __ldg(r + 0);
-            iv[a].nxo = dup2(-__ldg(r + 1));
-            iv[a].nxo_lo = dup2(-__ldg(r + 8));
-            if (__ldg(r + 7) <= (float)kRobustT) {
-                iv[a].c0 = dup2(__ldg(r + 2));
-                iv[a].c1 = dup2(__ldg(r + 3));
-                iv[a].c2 = dup2(__ldg(r + 4));
-                iv[a].c3 = dup2(__ldg(r + 5));
+        // installs the record of interval j of spline a (its first 36 bytes: A = xr, xo, c0, c1;
+        // B = c2, c3, xl, T; the low part of xo)
+        auto install = [&](int a, int j, float4 A, float4 B, float lo) {
+            iv[a].j = j;
+            iv[a].xr = A.x;
+            iv[a].nxo = dup2(-A.y);
+            iv[a].nxo_lo = dup2(-lo);
+            if (B.w <= (float)kRobustT) {
+                iv[a].c0 = dup2(A.z);
+                iv[a].c1 = dup2(A.w);
+                iv[a].c2 = dup2(B.x);
+                iv[a].c3 = dup2(B.y);
                 hm &= ~(1u << a);
             } else {
                 // ill-conditioned (routed states): the zero cubic keeps the arithmetic benign, and
@@ -181,12 +183,18 @@ __global__ void __launch_bounds__(128, 3)
                 hm |= 1u << a;
             }
         };
+        auto rec4 = [&](int a, int j) {
+            return reinterpret_cast<const float4*>(base(a) + (size_t)LISA_IDX(j, kmax + 1) * kSplineRec32);
+        };
+        auto load = [&](int a, int j) {
+            const float4* r = rec4(a, j);
+            install(a, j, __ldg(r), __ldg(r + 1), __ldg(reinterpret_cast<const float*>(r + 2)));
+        };
         {
             const float x0 = fld(tb, 0, 0);
 #pragma unroll
             for (int a = 0; a < NSP; ++a) {
-                iv[a].j = find_interval<float, kSplineRec32, 6>(base(a), nint_s[a], x0);
-                load(a);
+                load(a, find_interval<float, kSplineRec32, 6>(base(a), nint_s[a], x0));
             }
         }
         // accumulators: chunk sums per lane of the bin pair (registers), running sums in
@@ -239,12 +247,14 @@ __global__ void __launch_bounds__(128, 3)
                 cs[k] = make_float2(0.f, 0.f);
             }
         };
-        auto advance = [&](int a, float x) {
-            while (x >= iv[a].xr && iv[a].j < __ldg(nint_s + a) - 1) {
-                store_mom(a);
-                ++iv[a].j;
-                load(a);
-            }
+        // moves every spline to its interval holding x (the last interval's right end is +inf)
+        auto advance_all = [&](float x) {
+#pragma unroll
+            for (int a = 0; a < NSP; ++a)
+                while (x >= iv[a].xr && iv[a].j < kmax) {
+                    store_mom(a);
+                    load(a, iv[a].j + 1);
+                }
         };
         // one scalar bin (the fields f[0..11] of the table: x, ell, nu, G_oms, G_tm, G_h, and the
         // low part of x), its sums in the first lane of the pair accumulators; the intervals
@@ -464,11 +474,16 @@ __global__ void __launch_bounds__(128, 3)
                     for (int k = 0; k < kPairRec / 4; ++k) q4[k] = reinterpret_cast<const float4*>(T)[ip * (kPairRec / 4) + k];
                     const float2 xl = XL[ip];
                     const float2* F = reinterpret_cast<const float2*>(q4);
-                    bool split = false;
+                    float xmin = iv[0].xr;
 #pragma unroll
-                    for (int a = 0; a < NSP; ++a) {
-                        advance(a, F[0].x);
-                        split |= !(F[0].y < iv[a].xr);
+                    for (int a = 1; a < NSP; ++a) xmin = fminf(xmin, iv[a].xr);
+                    bool split = !(F[0].y < xmin);
+                    if (split) {
+                        advance_all(F[0].x);
+                        xmin = iv[0].xr;
+#pragma unroll
+                        for (int a = 1; a < NSP; ++a) xmin = fminf(xmin, iv[a].xr);
+                        split = !(F[0].y < xmin);
                     }
                     if (split) {
                         // a knot between the two bins: each on its own intervals
@@ -479,8 +494,7 @@ __global__ void __launch_bounds__(128, 3)
                             f1[k] = F[k].y;
                         }
                         bin(f0, xl.x);
-#pragma unroll
-                        for (int a = 0; a < NSP; ++a) advance(a, f1[0]);
+                        advance_all(f1[0]);
                         bin(f1, xl.y);
                     } else {
                         pair(F, xl);
