@@ -311,7 +311,8 @@ lisa_status lisa_averaged_periodogram(const double* d_dev, int32_t n_channels, i
  *    (state, tile) (the fused and the compensated kernels' partial sums) plus 84 bytes per state
  *    (FP32 parameters, work list), each region rounded up to 256 bytes, i.e.
  *    lisa_workspace_bytes(data, kmax, precision, 0) must not exceed it.  The size depends on the
- *    tiling (lisa_data_set_tiling): the paper-scale workload (131,072 bins, 1,024 states) needs
+ *    tiling (lisa_data_set_tiling) and on the split of small problems, which uses more partial sums but
+ *    never takes a problem past the limit: the paper-scale workload (131,072 bins, 1,024 states) needs
  *    about 2.1 MiB at 1,024-bin tiles, which fits, but 4.1 MiB at 512-bin tiles, which does not.
  *    Larger problems get LISA_ERR_WORKSPACE and nothing is launched; use lisa_psd_loglike for
  *    them.
