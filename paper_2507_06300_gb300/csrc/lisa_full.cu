@@ -38,14 +38,15 @@ __device__ __forceinline__ double full_term64(const double pn[3], double ph, con
                                               const double* __restrict__ exptab) {
     double D[3], Cd[3];
     constexpr double kLog10_2 = 0.301029995663981195213739;
-    const double yh = HAS_H ? fma(sl * kLog10_2, q[1], lA + ph) : 0.0;
+    const double yh = HAS_H ? fma(sl * kLog10_2, q[1], ph) : 0.0;
+    const double A = HAS_H ? m64::amplitude(lA, exptab) : 1.0;   // (apart: in the exponent it would round it at its size)
     const bool in_range = m64::small_exponent(pn[0]) && m64::small_exponent(pn[1]) && m64::small_exponent(pn[2]) &&
-                          m64::small_exponent(yh);
+                          m64::small_exponent(yh) && m64::normal_range(A);
     double E[3], eh = 0.0;
     if (in_range) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) E[c] = m64::exp10_fast(pn[c], exptab);
-        if (HAS_H) eh = m64::exp10_fast(yh, exptab);
+        if (HAS_H) eh = A * m64::exp10_fast(yh, exptab);
     } else {
 #pragma unroll 1
         for (int c = 0; c < 3; ++c) E[c] = exp10(pn[c]);

@@ -67,10 +67,10 @@ __device__ __forceinline__ void fb_flag(int32_t* fb, int S, int s) {
     if (atomicExch(fb + s, 1) == 0) fb[S + 1 + atomicAdd(fb + S, 1)] = s;
 }
 
-// A = 10^log10A in FP32 (the library's exp10, about 40 FP64 instructions for every unit, where the table
-// does not reach).
+// A = 10^log10A in FP32 (the library's exp10, about 40 FP64 instructions for every unit, only where the
+// table does not reach).
 __device__ __forceinline__ float amplitude(double v, const double* __restrict__ exptab) {
-    return (float)(m64::small_exponent(v) ? m64::exp10_fast(v, exptab) : exp10(v));
+    return (float)m64::amplitude(v, exptab);
 }
 
 // ---- FP32 adjoint: one warp per (dataset, range, up to 32 states) -----------------------------
@@ -554,11 +554,11 @@ __device__ __noinline__ void adjoint_bin64_wide(const double* P, double ao2, dou
     if (HAS_H) out[4 + C] = H;
 }
 
-// Per state-bin 108 FP64 instructions (about 340 with the library's functions and a division per
+// Per state-bin 110 FP64 instructions (about 340 with the library's functions and a division per
 // channel): the forward pass as loglike_fp64_kernel's, 9 for the channels' reciprocals from one of their
 // product, 21 for the template sums and signals, 24 for the moments.  One unit and warp per CTA: the
 // units of a small problem spread over all SMs and start as registers come free (four units to a CTA,
-// their CTAs half empty: 1.85 against 1.53 ms).  16,384 bins x 400 states with the epilogue: 5.8 -> 1.68 ms.
+// their CTAs half empty: 1.85 against 1.53 ms).  16,384 bins x 400 states with the epilogue: 5.8 -> 1.70 ms.
 constexpr int kLogRun = 64;   // factors of a LogProduct: its mantissa stays below 2^64
 template <int C, bool HAS_H, bool BROKEN>
 __global__ void __launch_bounds__(32)
@@ -579,6 +579,9 @@ __global__ void __launch_bounds__(32)
     const double n2 = BROKEN ? th[4] : n1;
     constexpr double kLog10_2 = 0.301029995663981195213739;
     const double m1 = n1 * kLog10_2, m2 = n2 * kLog10_2;   // slopes in decades per octave
+    // A = 10^log10A once per unit: log10 A inside the bins' exponents would round them at its size
+    const double A = HAS_H ? exp10(lA) : 1.0;
+    const bool A_ok = m64::normal_range(A);
     const int64_t b0 = D.bin0 + (int64_t)U.rho * adj_bins;
     const int nb = (int)min((int64_t)adj_bins, D.bin0 + D.npad - b0);
     const int64_t pre = prefix[s];
@@ -590,7 +593,7 @@ __global__ void __launch_bounds__(32)
         const double* z = srec + (((int64_t)s * nsp + a) * (int64_t)(kmax + 1) + LISA_IDX(j[a], kmax + 1)) * kSplineRec;
         xl[a] = z[0];
         xr[a] = m64::order_key(z[1]);
-        ca[a] = HAS_H && a == C ? z[2] + lA : z[2];
+        ca[a] = z[2];
         cb[a] = z[3];
         cc[a] = z[4];
         cd[a] = z[5];
@@ -653,7 +656,7 @@ __global__ void __launch_bounds__(32)
             nu_run = nu;
         }
         double P[NSP], t[NSP];
-        bool ok = true;
+        bool ok = A_ok;
 #pragma unroll
         for (int a = 0; a < NSP; ++a) {
             t[a] = x - xl[a];
@@ -664,7 +667,7 @@ __global__ void __launch_bounds__(32)
         for (int a = 0; a < NSP; ++a) ok &= m64::small_exponent(P[a]);
         double S[C], E[C], N[C], Eh[C], r[C], qv[NSP];
         double eh = 0.0;
-        if (HAS_H) eh = m64::exp10_fast(P[C], exptab);
+        if (HAS_H) eh = A * m64::exp10_fast(P[C], exptab);
 #pragma unroll
         for (int c = 0; c < C; ++c) {
             N[c] = fma(ao2, go[c], at2 * gt[c]);
@@ -706,9 +709,7 @@ __global__ void __launch_bounds__(32)
             double Pv[NSP], out[4 + NSP];
 #pragma unroll
             for (int a = 0; a < NSP; ++a) {
-                const double c0 = HAS_H && a == C ? __ldg(srec + (((int64_t)s * nsp + a) * (int64_t)(kmax + 1) + j[a]) * kSplineRec + 2)
-                                                  : ca[a];
-                Pv[a] = c0 + t[a] * (cb[a] + t[a] * (cc[a] + t[a] * cd[a]));
+                Pv[a] = ca[a] + t[a] * (cb[a] + t[a] * (cc[a] + t[a] * cd[a]));
             }
             adjoint_bin64_wide<C, HAS_H>(Pv, ao2, at2, lA, BROKEN ? (m64::negative(ell) ? n1 : n2) : n1, q, out);
             acc[0] += nu * (out[0] - (double)C);

@@ -1270,10 +1270,10 @@ __device__ __noinline__ double bin_term64_wide(const double* P, double ao2, doub
 
 // One warp per unit: b64 bins of one dataset x up to 32 of its states (lanes = states, so every lane
 // reads the same bin).  Bound by the FP64 pipe (2 lane operations per clock and SM): per state-bin 16
-// instructions for the four cubics, 17 for their exponentials and the power law, 12 for the PSDs, 4 for
+// instructions for the four cubics, 18 for their exponentials, the power law and A, 12 for the PSDs, 4 for
 // their product and the numerator of sum 1 / S, 4 for the division, 2 for the sums; the logarithm of
 // the channels' product is taken once for up to kLogRun bins of equal nu.  Intervals, range checks and
-// conversions are integer work (lisa_math64.cuh).  65,537 bins x 400 states: 13.7 -> 3.0 ms.
+// conversions are integer work (lisa_math64.cuh).  65,537 bins x 400 states: 13.7 -> 3.08 ms.
 constexpr int kLogRun = 64;   // factors of a LogProduct: its mantissa stays below 2^64
 template <int C, bool HAS_H, bool BROKEN>
 __global__ void __launch_bounds__(64)
@@ -1296,8 +1296,11 @@ __global__ void __launch_bounds__(64)
     const double n2 = BROKEN ? th[4] : n1;
     constexpr double kLog10_2 = 0.301029995663981195213739;
     const double m1 = n1 * kLog10_2, m2 = n2 * kLog10_2;   // slopes in decades per octave
-    // the current interval of each spline: left knot, cubic (the background's with log10 A in its
-    // constant), and its right end as an order key (no FP64 comparison)
+    // A = 10^log10A once per unit: log10 A inside the bins' exponents would round them at its size
+    const double A = HAS_H ? exp10(lA) : 1.0;
+    const bool A_ok = m64::normal_range(A);
+    // the current interval of each spline: left knot, cubic, and its right end as an order key (no
+    // FP64 comparison)
     double xl[NSP], ca[NSP], cb[NSP], cc[NSP], cd[NSP];
     long long xr[NSP];
     int j[NSP];
@@ -1305,7 +1308,7 @@ __global__ void __launch_bounds__(64)
         const double* z = srec + (((int64_t)s * nsp + a) * (int64_t)(kmax + 1) + LISA_IDX(j[a], kmax + 1)) * kSplineRec;
         xl[a] = z[0];
         xr[a] = m64::order_key(z[1]);
-        ca[a] = HAS_H && a == C ? z[2] + lA : z[2];
+        ca[a] = z[2];
         cb[a] = z[3];
         cc[a] = z[4];
         cd[a] = z[5];
@@ -1356,7 +1359,7 @@ __global__ void __launch_bounds__(64)
             nu_run = nu;
         }
         double P[NSP];
-        bool ok = true;
+        bool ok = A_ok;
 #pragma unroll
         for (int a = 0; a < NSP; ++a) {
             const double t = x - xl[a];
@@ -1367,7 +1370,7 @@ __global__ void __launch_bounds__(64)
 #pragma unroll
         for (int a = 0; a < NSP; ++a) ok &= m64::small_exponent(P[a]);
         double S[C], eh = 0.0;
-        if (HAS_H) eh = m64::exp10_fast(P[C], exptab);
+        if (HAS_H) eh = A * m64::exp10_fast(P[C], exptab);
 #pragma unroll
         for (int c = 0; c < C; ++c) {
             const double N = fma(ao2, go[c], at2 * gt[c]);
@@ -1388,9 +1391,7 @@ __global__ void __launch_bounds__(64)
 #pragma unroll
             for (int a = 0; a < NSP; ++a) {
                 const double t = x - xl[a];
-                const double c0 = HAS_H && a == C ? __ldg(srec + (((int64_t)s * nsp + a) * (int64_t)(kmax + 1) + j[a]) * kSplineRec + 2)
-                                                  : ca[a];
-                Pv[a] = c0 + t * (cb[a] + t * (cc[a] + t * cd[a]));
+                Pv[a] = ca[a] + t * (cb[a] + t * (cc[a] + t * cd[a]));
             }
             acc += nu * bin_term64_wide<C, HAS_H>(Pv, ao2, at2, lA, BROKEN ? (m64::negative(ell) ? n1 : n2) : n1, q);
         }
@@ -1436,10 +1437,10 @@ __global__ void finalize_kernel(int S, const int32_t* __restrict__ state_ds, con
     }
 }
 
-// Model PSD in physical units, FP64: one thread per (state, bin).  The FP64 pipe bounds it: 48
-// instructions per state-bin (cubics 16, exponentials and power law 17, PSDs 12, normalisation 3); the
+// Model PSD in physical units, FP64: one thread per (state, bin).  The FP64 pipe bounds it: 49
+// instructions per state-bin (cubics 16, exponentials, power law and A 18, PSDs 12, normalisation 3); the
 // interval searches compare order keys, and the exponentials take the table, on the other pipes (the
-// library's functions: 140).  131,072 bins x 64 states: 2.05 ms -> 0.79 ms.
+// library's functions: 140).  131,072 bins x 64 states: 2.05 ms -> 0.80 ms.
 template <int C>
 __global__ void model_psd_kernel(const int32_t* __restrict__ state_ds, const DatasetDev* __restrict__ ds,
                                  const double* __restrict__ rec64, const double* __restrict__ exptab,
@@ -1450,6 +1451,10 @@ __global__ void model_psd_kernel(const int32_t* __restrict__ state_ds, const Dat
     const int s = blockIdx.y;
     const DatasetDev& D = ds[state_ds[s]];
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    // A = 10^log10A once per CTA (apart: log10 A inside the exponent would round it at its size)
+    __shared__ double s_A;
+    if (threadIdx.x == 0) s_A = has_h ? m64::amplitude(theta[(size_t)s * LISA_N_THETA + 2], exptab) : 1.0;
+    __syncthreads();
     if (i >= D.nbins) return;
     double* o = out + D.psd_base + (int64_t)(s - D.s0) * C * D.nbins;
     if (sstat[s] & kUserBits) {
@@ -1481,13 +1486,13 @@ __global__ void model_psd_kernel(const int32_t* __restrict__ state_ds, const Dat
     }
     const double sl = (broken && !m64::negative(ell)) ? th[4] : th[3];
     constexpr double kLog10_2 = 0.301029995663981195213739;
-    const double yh = has_h ? fma(sl * kLog10_2, ell, th[2] + Pv[C]) : 0.0;
-    ok = m64::small_exponent(yh);
+    const double yh = has_h ? fma(sl * kLog10_2, ell, Pv[C]) : 0.0, A = s_A;
+    ok = m64::small_exponent(yh) && m64::normal_range(A);
 #pragma unroll
     for (int c = 0; c < C; ++c) ok &= m64::small_exponent(Pv[c]);
     double E[C], eh = 0.0;
     if (ok) {
-        if (has_h) eh = m64::exp10_fast(yh, exptab);
+        if (has_h) eh = A * m64::exp10_fast(yh, exptab);
 #pragma unroll
         for (int c = 0; c < C; ++c) E[c] = m64::exp10_fast(Pv[c], exptab);
     } else {

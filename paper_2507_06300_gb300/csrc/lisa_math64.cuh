@@ -6,7 +6,7 @@
 // that need not be rounded to 53 bits runs elsewhere: exponents, table indices, conversions and
 // comparisons on the integer pipe (from the bits of the doubles), reciprocal seeds and the last terms of
 // the series, below 2^-28 of the result, in FP32.  Against the library's exp10, exp2, log and
-// division a state-bin of the likelihood takes 55 FP64 instructions instead of 225.
+// division a state-bin of the likelihood takes 58 FP64 instructions instead of 225.
 #pragma once
 
 #include "lisa_math.cuh"
@@ -46,8 +46,9 @@ __device__ __forceinline__ bool small_exponent(double v) { return (hi32(v) & 0x7
 // 10^v for |v| < 100 from the table T of 2^(j / kExpTab) (the table-driven scheme of Tang, ACM TOMS 15,
 // 1989): 4 FP64 instructions, error within 1 ulp plus the rounding of v.  v = k log10(2) / 8192 + r with
 // k chosen in FP32 (any k near the nearest one does), r exact to twice the precision;
-// 10^r = 1 + r ln10 + q, where q <= 2^-30 is summed in FP32.  The table (64 KB) is read through L1,
-// which the kernels that use it leave free.
+// 10^r = 1 + r ln10 + q with q = (r ln10)^2 / 2 + (r ln10)^3 / 6 <= 2^-30 formed in float-float and rounded
+// once to FP32 (2^-55 of the result; plain FP32 products of a truncated r left 2 ulp).  The table (64 KB)
+// is read through L1, which the kernels that use it leave free.
 __device__ __forceinline__ double exp10_fast(double v, const double* __restrict__ T) {
     constexpr double C_hi = 0x1.34413509f79ffp-15;    // log10(2) / 8192, rounded to FP64
     constexpr double C_lo = -0x1.9dc1da994fd21p-72;   // and the rest
@@ -57,12 +58,25 @@ __device__ __forceinline__ double exp10_fast(double v, const double* __restrict_
     const double kd = to_double(tf - 12582912.f);
     double r = fma(kd, -C_hi, v);
     r = fma(kd, -C_lo, r);
+    // r = rf + rl: its truncation to FP32 and the 29 bits below
     const float rf = to_float(r);
-    const float q = rf * rf * fmaf(rf, 2.03467859f, 2.65094906f);   // ln10^2 / 2, ln10^3 / 6
+    const unsigned hr = hi32(r), er = (hr >> 20) & 0x7ffu;
+    const float sc = er >= 960u ? __uint_as_float((hr & 0x80000000u) | ((er - 948u) << 23)) : 0.f;   // 2^(e - 52)
+    const float rl = (float)(lo32(r) & 0x1fffffffu) * sc;
+    constexpr float K2 = 2.65094906f, K2l = 5.39269431e-08f, K3 = 2.03467859f;   // ln10^2 / 2, ln10^3 / 6
+    const float h = rf * rf;
+    const float l = fmaf(2.f * rf, rl, fmaf(rf, rf, -h));
+    const float q0 = K2 * h;
+    const float q = q0 + (fmaf(K2, h, -q0) + fmaf(K2, l, fmaf(rf, K3, K2l) * h));
     const double p = fma(r, kLn10, to_double(q));
     const double t = __ldg(T + (k & (kExpTab - 1)));
     const double e = fma(t, p, t);
     return __hiloint2double((int)(hi32(e) + (unsigned)((k >> 13) << 20)), (int)lo32(e));
+}
+
+// A = 10^log10A, any value.
+__device__ __forceinline__ double amplitude(double v, const double* __restrict__ T) {
+    return small_exponent(v) ? exp10_fast(v, T) : exp10(v);
 }
 
 // n / d for a normal d well inside the range: an FP32 reciprocal of d's mantissa and one cubic step

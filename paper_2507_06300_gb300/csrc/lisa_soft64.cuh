@@ -17,12 +17,10 @@ __device__ __forceinline__ float rsqrt_seed(float v) {
 }
 __device__ __forceinline__ float bits_float(uint32_t b) { return __uint_as_float(b); }
 __device__ __forceinline__ uint32_t float_bits(float f) { return __float_as_uint(f); }
-__device__ __forceinline__ uint64_t mul_hi(uint64_t a, uint64_t b) { return __umul64hi(a, b); }
 #else
 inline float rsqrt_seed(float v) { return 1.0f / __builtin_sqrtf(v); }
 inline float bits_float(uint32_t b) { float f; __builtin_memcpy(&f, &b, 4); return f; }
 inline uint32_t float_bits(float f) { uint32_t b; __builtin_memcpy(&b, &f, 4); return b; }
-inline uint64_t mul_hi(uint64_t a, uint64_t b) { return (uint64_t)(((unsigned __int128)a * b) >> 64); }
 #endif
 
 constexpr uint64_t kMant = (1ull << 52) - 1, kOne = 1ull << 52;
@@ -71,7 +69,8 @@ LISA_HD bool sqrt_half(uint64_t v, uint64_t& out) {
 // the product is not normal.
 LISA_HD bool mul(int ea, uint64_t A, uint64_t x, uint64_t& out) {
     const uint64_t X = (x & kMant) | kOne;
-    uint64_t hi = mul_hi(A, X), lo = A * X;    // [2^51, 2^53) and the bits below
+    const unsigned __int128 P = (unsigned __int128)A * X;
+    uint64_t hi = (uint64_t)(P >> 64), lo = (uint64_t)P;    // [2^51, 2^53) and the bits below
     int e = ea + exp_of(x) - 1022;
     if (!(hi >> 52)) {
         hi = (hi << 1) | (lo >> 63);

@@ -67,3 +67,26 @@ def test_gradient_split(precision, n_bins, n_states, kind):
     assert np.all(np.isfinite(G1)) and np.all(np.isfinite(L1[St == 0]))
     np.testing.assert_allclose(L1, L2, rtol=1e-13, atol=0)
     assert np.all(np.abs(G1 - G2) <= 1e-9 * np.abs(G2).max(axis=1, keepdims=True))
+
+
+@pytest.mark.parametrize("n_bins,n_states", [(2, 65), (63, 70), (130, 129), (1025, 66)])
+def test_dense_one_warp_ctas(n_bins, n_states):
+    """The dense covariance with more than 64 states (one warp per CTA, staged pieces) at ragged sizes,
+    both precisions against the oracle at the FP32 bound."""
+    from tests._workloads import oracle_dataset_full
+    from tests.test_gpu_full import _check
+    wl = synth.workload("tiny", cov_model=1, n_bins=n_bins, n_states=n_states)
+    _check(wl, oracle_dataset_full(wl), fp64_rtol=None)
+
+
+@pytest.mark.parametrize("run", [1, 2, 63, 64, 65, 130])
+def test_fp64_runs_of_equal_nu(run):
+    """The FP64 kernels take one logarithm per run of bins with equal nu (at most 64): log L of the forward
+    call and of the gradient call with nu changing every `run` bins, some of it zero."""
+    wl = _wl(700, 40)
+    wl.nu = np.array([4.0, 0.0, 7.0, 1.0, 128.0])[(np.arange(700) // run) % 5]
+    P, L_ref, St = oracle_batched(wl)
+    Lg, _, _, L = gpu_grad(wl, P, FP64)
+    ok = St == 0
+    np.testing.assert_allclose(L[ok], L_ref[ok], rtol=1e-12, atol=0)
+    np.testing.assert_allclose(Lg[ok], L_ref[ok], rtol=1e-12, atol=0)
