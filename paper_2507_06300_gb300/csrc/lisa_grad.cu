@@ -769,12 +769,13 @@ __global__ void __launch_bounds__(MODE == kComp ? 128 : 512)
     adjoint_range_kernel(int S, const int32_t* __restrict__ state_ds, const DatasetDev* __restrict__ ds,
                          const float* __restrict__ rec32, const float* __restrict__ xlo32,
                          const float* __restrict__ elllo32, const double* __restrict__ theta,
-                         const int32_t* __restrict__ sstat, const int32_t* __restrict__ list, int R,
-                         int32_t* __restrict__ fb, int32_t* __restrict__ next_item,
+                         const int32_t* __restrict__ sstat, const int32_t* list, int R, int32_t* fb,
+                         int32_t* __restrict__ next_item,
                          const int32_t* __restrict__ nint, const void* __restrict__ srec_v,
                          const float2* __restrict__ hull, int kmax, int nsp, const int64_t* __restrict__ prefix,
-                         double* __restrict__ scal, double* __restrict__ mom, int adj_bins,
-                         const double* __restrict__ exptab) {
+                         double* scal, double* mom, int adj_bins, const double* __restrict__ exptab) {
+    // list (the fallback's), fb, scal and mom are also written by the kernel before, which may still run
+    // when this one starts: not __restrict__, so that no access to them is moved above the wait
     constexpr int NSP = C + (HAS_H ? 1 : 0);
     // this pass's ranges: kComp takes kAdjBins bins whatever the adjoint's range size (its lanes'
     // FP32 template sums then cover the same bins), each holding `sub` of the adjoint's ranges, the
@@ -1334,7 +1335,7 @@ __device__ __noinline__ bool epilogue_spline(int s, int a, int has_h, int broken
                                              const double* __restrict__ theta, const int32_t* __restrict__ count,
                                              const double* __restrict__ kx, const double* __restrict__ kw, int kmax,
                                              int kind, int nsp, const int64_t* __restrict__ prefix,
-                                             const double* __restrict__ scal, const double* __restrict__ mom,
+                                             const double* scal, const double* mom,
                                              const double2* __restrict__ rx32, const double2* __restrict__ rx64,
                                              const void* __restrict__ srec_v, int fp32, double* __restrict__ out_logL,
                                              double* __restrict__ grad, double* sX, double* sY) {
@@ -1651,13 +1652,14 @@ __global__ void __launch_bounds__(128, 4)
                             const DatasetDev* __restrict__ ds, const int32_t* __restrict__ sstat,
                             const double* __restrict__ theta, const int32_t* __restrict__ count,
                             const double* __restrict__ kx, const double* __restrict__ kw, int kmax, int kind, int nsp,
-                            const int64_t* __restrict__ prefix, const double* __restrict__ scal,
-                            const double* __restrict__ mom, const double2* __restrict__ rx32,
+                            const int64_t* __restrict__ prefix, const double* scal, const double* mom,
+                            const double2* __restrict__ rx32,
                             const double2* __restrict__ rx64, const void* __restrict__ srec_v, int fp32,
                             double* __restrict__ out_logL, double* __restrict__ grad,
-                            const int32_t* __restrict__ fb) {
+                            const int32_t* fb) {
     __shared__ double sX[4][64];
     __shared__ double sY[4][64];
+    // scal, mom and fb (not __restrict__) are read only after the kernels that write them have ended
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int warp = threadIdx.x >> 5;
     const int64_t u = (int64_t)blockIdx.x * 4 + warp;

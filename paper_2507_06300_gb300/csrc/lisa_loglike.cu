@@ -1403,11 +1403,12 @@ __global__ void __launch_bounds__(64)
 // Per state (one warp): fixed-order sum of its tiles' partials (lane-strided, then a shuffle
 // tree) plus the dataset constants.
 __global__ void finalize_kernel(int S, const int32_t* __restrict__ state_ds, const DatasetDev* __restrict__ ds,
-                                const int32_t* __restrict__ sstat, const double* __restrict__ partial,
+                                const int32_t* __restrict__ sstat, const double* partial,
                                 const int32_t* __restrict__ rent, const RobustEntry* __restrict__ rlist,
-                                const double* __restrict__ rpart, const int* __restrict__ err, int fp32,
-                                double* __restrict__ out) {
+                                const double* rpart, const int* err, int fp32, double* __restrict__ out) {
     // launched as a programmatic dependent of the likelihood's last kernel, whose end it waits for
+    // (partial, rpart and err are written by kernels that may still run when this one starts: not
+    // __restrict__, so that no load of them is moved above the wait)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int s = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
