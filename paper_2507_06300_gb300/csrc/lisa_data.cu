@@ -292,6 +292,7 @@ lisa_status rebuild_work(lisa_data* d) {
     for (const DatasetDev& D : d->h_ds)
         if (D.ns > 0)
             max_seg = std::max(max_seg, (seg_bins(t.tile_bins, kThreads32 / lanes(D), 1) + kSegBins - 1) / kSegBins);
+    d->n_partials64 = 0;   // (set below; the layout so far is the FP32 path's)
     int64_t n_items = lay_out(1);
     const size_t ws1 = ws_fwd_bytes(d);
     const int64_t enough = (int64_t)(d->cov == LISA_COV_FULL ? kMinItemsPerSmFull : kMinItemsPerSm) * d->n_sm;
@@ -307,7 +308,7 @@ lisa_status rebuild_work(lisa_data* d) {
     // the plain FP64 kernels' units: half a segment of bins x 32 states, one warp each.  (They share
     // the FP64 pipe, so what counts is that the units are many and of one size; half a segment is what
     // the workspace of the FP32 path holds slots for.)
-    for (int64_t b64 = std::max<int64_t>(16, (t.tile_bins / d->nseg + 3) / 4 * 2);; b64 *= 2) {
+    auto units64 = [&](int64_t b64) {
         int64_t units = 0, slots = 0;
         d->b64 = (int32_t)b64;
         for (DatasetDev& D : d->h_ds) {
@@ -318,7 +319,39 @@ lisa_status rebuild_work(lisa_data* d) {
             slots += (int64_t)D.n64 * D.ns;
         }
         d->n_units64 = units;
-        if (ws_bytes64(d, slots) <= ws_fwd_bytes(d)) break;
+        d->n_partials64 = slots;
+    };
+    const size_t ws32 = ws_fwd_bytes(d);
+    int64_t b64 = std::max<int64_t>(16, (t.tile_bins / d->nseg + 3) / 4 * 2);
+    for (;; b64 *= 2) {
+        units64(b64);
+        if (ws_fwd_bytes(d) <= ws32) break;
+    }
+    // Few units are halved, down to 4 bins per lane while some SMs have none and to 16 while an SM has fewer
+    // than kMinUnits64PerSm; their slots, a few hundred kB, may exceed the FP32 path's.  (A unit costs about
+    // 100 FP64 instructions besides its bins' 58 each, and a state's finalize reads its slots 256 at a
+    // time.)  Dense covariance, 16,384 bins x
+    // 16 states: 64 units of 256 bins 1,559 us, 512 of 32 236 us; 65,536 bins x 16 states 332 -> 158 us.  At 8 per SM
+    // the halved units exceeded the 12 warps resident per SM, a second wave: 32 data sets of 8,000 bins x 4 states
+    // 158 -> 231 us.
+    int min_sw = 32;   // lanes side by side in the units of the smallest dataset (unit_of)
+    int64_t max_n = 0;
+    for (const DatasetDev& D : d->h_ds)
+        if (D.ns > 0) {
+            min_sw = std::min(min_sw, pow2ceil(D.ns));
+            max_n = std::max(max_n, D.npad);
+        }
+    while (d->n_units64 > 0 && b64 >= 32 && b64 % 4 == 0) {
+        const int64_t per_lane = b64 / 2 * min_sw / 32;
+        const bool idle = d->n_units64 < d->n_sm && per_lane >= 4;
+        const bool thin = d->n_units64 < (int64_t)kMinUnits64PerSm * d->n_sm && per_lane >= 16;
+        if (!(idle || thin) || 2 * max_n > 1024 * b64) break;
+        units64(b64 / 2);
+        if (ws32 <= LISA_NOALLOC_SCRATCH_BYTES && ws_fwd_bytes(d) > LISA_NOALLOC_SCRATCH_BYTES) {
+            units64(b64);
+            break;
+        }
+        b64 /= 2;
     }
     items.reserve((size_t)n_items);
     for (int k = 0; k < d->n_datasets; ++k) {

@@ -81,7 +81,7 @@ __device__ __forceinline__ double full_term64(const double pn[3], double ph, con
 }
 
 // ---- plain FP64 path --------------------------------------------------------------------------
-// One warp per unit of b64 bins x 32 states, as the diagonal model's (lanes = states).
+// One warp per unit of b64 bins x 32 states, as the diagonal model's (lanes = states, or states x rows of bins).
 template <bool HAS_H, bool BROKEN>
 __global__ void __launch_bounds__(64)
     full_fp64_kernel(int64_t n_units, int n_ds, int b64, const double* __restrict__ rec64,
@@ -93,11 +93,10 @@ __global__ void __launch_bounds__(64)
     constexpr int ZB = 3 + (HAS_H ? 1 : 0);   // first correlation spline
     const int64_t u = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (u >= n_units) return;
-    int slot, s;
-    const DatasetDev& D = m64::unit_of(ds, n_ds, u, slot, s);
-    if (s >= D.s0 + D.ns || sstat[s] != 0) return;
-    const int64_t b0 = D.bin0 + (int64_t)slot * b64;
-    const int nb = (int)min((int64_t)b64, D.bin0 + D.npad - b0);
+    m64::Unit64 w;
+    const DatasetDev& D = m64::unit_of(ds, n_ds, u, b64, sstat, w);
+    const int nb = w.nb, s = nb > 0 ? w.s : D.s0;
+    const int64_t b0 = w.b0;
     const double* th = theta + (size_t)s * LISA_N_THETA;
     const double ao2 = th[0] * th[0], at2 = th[1] * th[1], lA = th[2], n1 = th[3];
     const double n2 = BROKEN ? th[4] : n1;
@@ -113,8 +112,8 @@ __global__ void __launch_bounds__(64)
         cc[a] = z[4];
         cd[a] = z[5];
     };
-    const double x0 = __ldg(rec64 + b0 * kRec);
-    for (int a = 0; a < NSP; ++a) {
+    const double x0 = nb > 0 ? __ldg(rec64 + b0 * kRec) : 0.0;
+    for (int a = 0; a < NSP && nb > 0; ++a) {
         const int64_t sp = (int64_t)s * nsp + a;
         j[a] = find_interval<double, kSplineRec, 0>(srec + sp * (int64_t)(kmax + 1) * kSplineRec, nint[sp], x0);
         load(a);
@@ -146,7 +145,7 @@ __global__ void __launch_bounds__(64)
         const double zv[3] = {P[ZB], P[ZB + 1], P[ZB + 2]};
         acc += qq[2] * full_term64<HAS_H>(pn, HAS_H ? P[3] : 0.0, zv, qq, xcv, ao2, at2, lA, sl, exptab);
     }
-    partial[D.pbase64 + (int64_t)(s - D.s0) * D.n64 + LISA_IDX(slot, D.n64)] = acc;
+    m64::store_unit(D, w, sstat, acc, partial);
 }
 
 // ---- FP32 bulk path ---------------------------------------------------------------------------

@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <vector>
 
@@ -92,6 +93,7 @@ constexpr int kExpTab = 8192;               // entries of the FP64 path's table 
 constexpr int kXsStride = 32;               // bins between the host copies of log10 f
 constexpr int kMinItemsPerSm = 2;            // fewer items per SM than this are split into segments
 constexpr int kMinItemsPerSmFull = 32;       // the same for the dense covariance
+constexpr int kMinUnits64PerSm = 6;          // plain FP64: halve the units of a call with fewer per SM
 constexpr int kBlockItemsPerCta = 16;       // contiguous blocks need this many items per CTA
 constexpr double kBlockThreadBins = 128.0;  // and fewer bins per thread and item than this
 
@@ -199,6 +201,7 @@ struct lisa_data {
     bool chunk_items = false;        // every item is one FP32 chunk of one-row items (loglike_chunk_kernel)
     int32_t b64 = 0;                 // bins per unit of the plain FP64 kernels
     int64_t n_units64 = 0;           // their units
+    int64_t n_partials64 = 0;        // and their partial sums
     double* d_exptab = nullptr;      // [kExpTab] 2^(j / kExpTab)
     // per-kernel timing of lisa_psd_loglike (lisa_data_set_profiling): events around the main,
     // compensated and finalize kernels of the most recent uncaptured call
@@ -290,12 +293,12 @@ inline WsLayout ws_layout(const lisa_data* d) {
     L.off_rlist = L.off_prm + ws_prm_bytes(d);
     L.off_rent = L.off_rlist + ws_rlist_bytes(d);
     L.off_rpart = L.off_rent + ws_rent_bytes(d);
-    L.bytes = L.off_rpart + ws_rpart_bytes(d);
+    // the plain FP64 path keeps its partial sums (256 bytes on) in the same bytes
+    L.bytes = std::max(L.off_rpart + ws_rpart_bytes(d),
+                       (256 + sizeof(double) * (size_t)d->n_partials64 + 255) / 256 * 256);
     return L;
 }
 inline size_t ws_fwd_bytes(const lisa_data* d) { return ws_layout(d).bytes; }
-// The plain FP64 path keeps its partial sums (256 bytes on) in the same bytes.
-inline size_t ws_bytes64(const lisa_data* d, int64_t n_partials64) { return 256 + sizeof(double) * (size_t)n_partials64; }
 
 // Extra workspace of the adjoint entry point (after the forward region); the FP32 call also holds
 // a per-state flag (states redone by the fallback pass).

@@ -1269,11 +1269,12 @@ __device__ __noinline__ double bin_term64_wide(const double* P, double ao2, doub
 }
 
 // One warp per unit: b64 bins of one dataset x up to 32 of its states (lanes = states, so every lane
-// reads the same bin).  Bound by the FP64 pipe (2 lane operations per clock and SM): per state-bin 16
+// reads the same bin; up to 16 states leave room for rows of bins).  Bound by the FP64 pipe (2 lane operations per clock and SM): per state-bin 16
 // instructions for the four cubics, 18 for their exponentials, the power law and A, 12 for the PSDs, 4 for
 // their product and the numerator of sum 1 / S, 4 for the division, 2 for the sums; the logarithm of
 // the channels' product is taken once for up to kLogRun bins of equal nu.  Intervals, range checks and
-// conversions are integer work (lisa_math64.cuh).  65,537 bins x 400 states: 13.7 -> 3.08 ms.
+// conversions are integer work (lisa_math64.cuh).  65,537 bins x 400 states: 13.7 -> 3.08 ms;
+// with the rows 262,144 bins x 4 states 547 -> 156 us, 131,072 bins x 1 state 95 -> 43 us.
 constexpr int kLogRun = 64;   // factors of a LogProduct: its mantissa stays below 2^64
 template <int C, bool HAS_H, bool BROKEN>
 __global__ void __launch_bounds__(64)
@@ -1285,12 +1286,10 @@ __global__ void __launch_bounds__(64)
     constexpr int NSP = C + (HAS_H ? 1 : 0);
     const int64_t u = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (u >= n_units) return;
-    int slot, s;
-    const DatasetDev& D = m64::unit_of(ds, n_ds, u, slot, s);
-    if (s >= D.s0 + D.ns || sstat[s] != 0) return;
-    const int64_t b0 = D.bin0 + (int64_t)slot * b64;
-    const int nb = (int)min((int64_t)b64, D.bin0 + D.npad - b0);
-    const double* q = rec64 + b0 * kRec;
+    m64::Unit64 w;
+    const DatasetDev& D = m64::unit_of(ds, n_ds, u, b64, sstat, w);
+    const int nb = w.nb, s = nb > 0 ? w.s : D.s0;
+    const double* q = rec64 + w.b0 * kRec;
     const double* th = theta + (size_t)s * LISA_N_THETA;
     const double ao2 = th[0] * th[0], at2 = th[1] * th[1], lA = th[2], n1 = th[3];
     const double n2 = BROKEN ? th[4] : n1;
@@ -1319,13 +1318,15 @@ __global__ void __launch_bounds__(64)
 #pragma unroll
         for (int a = 1; a < NSP; ++a) xmin = min(xmin, xr[a]);
     };
+    if (nb > 0) {
 #pragma unroll
-    for (int a = 0; a < NSP; ++a) {
-        const int64_t sp = (int64_t)s * nsp + a;
-        j[a] = find_interval<double, kSplineRec, 0>(srec + sp * (int64_t)(kmax + 1) * kSplineRec, nint[sp], __ldg(q));
-        load(a);
+        for (int a = 0; a < NSP; ++a) {
+            const int64_t sp = (int64_t)s * nsp + a;
+            j[a] = find_interval<double, kSplineRec, 0>(srec + sp * (int64_t)(kmax + 1) * kSplineRec, nint[sp], __ldg(q));
+            load(a);
+        }
+        nearest();
     }
-    nearest();
     double acc = 0.0, run = 0.0;   // the finished runs, and the current run's sum of 1 / S
     m64::LogProduct lp;
     lp.reset();
@@ -1350,7 +1351,7 @@ __global__ void __launch_bounds__(64)
             }
             nearest();
         }
-        // a run of bins with one nu ends (the lanes share the bins)
+        // a run of bins with one nu ends
         if (__double_as_longlong(nu) != __double_as_longlong(nu_run) || len == kLogRun) {
             acc = fma(nu_run, run + lp.log_value(), acc);
             run = 0.0;
@@ -1397,7 +1398,7 @@ __global__ void __launch_bounds__(64)
         }
     }
     acc = fma(nu_run, run + lp.log_value(), acc);
-    partial[D.pbase64 + (int64_t)(s - D.s0) * D.n64 + LISA_IDX(slot, D.n64)] = acc;
+    m64::store_unit(D, w, sstat, acc, partial);
 }
 
 // Per state (one warp): fixed-order sum of its tiles' partials (lane-strided, then a shuffle
@@ -1421,7 +1422,15 @@ __global__ void finalize_kernel(int S, const int32_t* __restrict__ state_ds, con
     const int n = fp32 ? D.nslots : D.n64;
     const double* p = partial + (fp32 ? D.pbase : D.pbase64) + (int64_t)(s - D.s0) * n;
     double sum = 0.0;
-    for (int t = lane; t < n; t += 32) sum += p[t];
+    int t = lane;
+    for (; t + 7 * 32 < n; t += 8 * 32) {   // eight loads in flight, added in the order of one at a time
+        double v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = p[t + 32 * k];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) sum += v[k];
+    }
+    for (; t < n; t += 32) sum += p[t];
     // FP32 mode: the compensated kernel's sums of this state's units, if it has any
     const int e = fp32 ? rent[s] : -1;
     if (e >= 0) {

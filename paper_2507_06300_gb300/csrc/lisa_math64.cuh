@@ -110,10 +110,19 @@ struct LogProduct {
     __device__ __forceinline__ double log_value() const { return fma((double)e, kLn2, log(m)); }
 };
 
-// The calling warp's unit u of a plain FP64 kernel: its dataset (the last one whose first unit is <= u;
-// empty ones share their successor's), its slot of b64 bins, and its lane's state.
-__device__ __forceinline__ const DatasetDev& unit_of(const DatasetDev* __restrict__ ds, int n_ds, int64_t u, int& slot,
-                                                     int& s) {
+// The calling lane's part of unit u of a plain FP64 likelihood kernel: its state s (sw lanes side by side
+// hold different states), and its bins [b0, b0 + nb) of the unit's slot of b64.
+struct Unit64 {
+    int slot, s, sw, nb;
+    int64_t b0;
+};
+
+// The calling warp's unit u: its dataset (the last one whose first unit is <= u; empty ones share their
+// successor's) and its lanes' parts.  A dataset of up to 16 states splits a unit's bins over 32 / sw rows,
+// sw the next power of two of its states: with one lane per state whatever their number, 4 states left 28
+// of a warp's lanes idle, and the pipe takes as long for them (figures at loglike_fp64_kernel).
+__device__ __forceinline__ const DatasetDev& unit_of(const DatasetDev* __restrict__ ds, int n_ds, int64_t u, int b64,
+                                                     const int32_t* __restrict__ sstat, Unit64& w) {
     int lo = 0, hi = n_ds - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
@@ -121,9 +130,25 @@ __device__ __forceinline__ const DatasetDev& unit_of(const DatasetDev* __restric
     }
     const DatasetDev& D = ds[lo];
     const int groups = (D.ns + 31) >> 5;
-    slot = (int)((u - D.ubase64) / groups);
-    s = D.s0 + 32 * (int)((u - D.ubase64) % groups) + (int)(threadIdx.x & 31);
+    const int lane = (int)(threadIdx.x & 31);
+    w.sw = D.ns > 16 ? 32 : 1 << (32 - __clz(D.ns - 1));   // (__clz(0) = 32)
+    w.slot = (int)((u - D.ubase64) / groups);
+    w.s = D.s0 + 32 * (int)((u - D.ubase64) % groups) + (lane & (w.sw - 1));
+    const int64_t first = (int64_t)w.slot * b64;
+    const int n = (int)min((int64_t)b64, D.npad - first);
+    const int rows = 32 / w.sw, r = lane / w.sw;
+    const int a = r * n / rows;
+    w.b0 = D.bin0 + first + a;
+    w.nb = w.s < D.s0 + D.ns && sstat[w.s] == 0 ? (r + 1) * n / rows - a : 0;
     return D;
+}
+
+// The unit's sum of a state over its rows (in a fixed order, by all lanes), stored by the first row.
+__device__ __forceinline__ void store_unit(const DatasetDev& D, const Unit64& w, const int32_t* __restrict__ sstat,
+                                           double acc, double* __restrict__ partial) {
+    for (int o = 16; o >= w.sw; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+    if ((int)(threadIdx.x & 31) < w.sw && w.s < D.s0 + D.ns && sstat[w.s] == 0)
+        partial[D.pbase64 + (int64_t)(w.s - D.s0) * D.n64 + LISA_IDX(w.slot, D.n64)] = acc;
 }
 
 }  // namespace m64

@@ -103,3 +103,28 @@ def test_fp64_runs_of_equal_nu(run):
     ok = St == 0
     np.testing.assert_allclose(L[ok], L_ref[ok], rtol=1e-12, atol=0)
     np.testing.assert_allclose(Lg[ok], L_ref[ok], rtol=1e-12, atol=0)
+
+
+@pytest.mark.parametrize("n_bins,n_states", [(1, 1), (15, 2), (31, 3), (64, 16), (1001, 5), (4097, 1), (700, 17)])
+def test_fp64_rows(n_bins, n_states):
+    """The FP64 likelihood of few states: each warp's lanes split the bins in rows, some of them empty, at
+    the tolerance of many states."""
+    wl = _wl(n_bins, n_states)
+    P, L_ref, St = oracle_batched(wl)
+    L, St_gpu = gpu_eval(wl, P, FP64)
+    np.testing.assert_array_equal(St_gpu, St)
+    ok = St == 0
+    np.testing.assert_allclose(L[ok], L_ref[ok], rtol=1e-12, atol=0)
+
+
+@pytest.mark.parametrize("n_bins,n_states", [(700, 1), (701, 6), (1024, 16)])
+def test_fp64_rows_dense(n_bins, n_states):
+    """The same for the dense covariance."""
+    import oracle
+    from tests._workloads import oracle_dataset_full
+    wl = synth.workload("tiny", cov_model=1, n_bins=n_bins, n_states=n_states)
+    ds = oracle_dataset_full(wl)
+    L_ref, St_ref = oracle.loglike_full(ds, wl.theta, wl.knots.as_dict())
+    L, _ = gpu_eval(wl, ds["P9"], FP64)
+    ok = St_ref == 0
+    np.testing.assert_allclose(L[ok], L_ref[ok], rtol=1e-12, atol=0)
