@@ -328,11 +328,11 @@ lisa_status rebuild_work(lisa_data* d) {
         if (ws_fwd_bytes(d) <= ws32) break;
     }
     // Few units are halved, down to 4 bins per lane while some SMs have none and to 16 while an SM has fewer
-    // than kMinUnits64PerSm; their slots, a few hundred kB, may exceed the FP32 path's.  (A unit costs about
-    // 100 FP64 instructions besides its bins' 58 each, and a state's finalize reads its slots 256 at a
-    // time.)  Dense covariance, 16,384 bins x
-    // 16 states: 64 units of 256 bins 1,559 us, 512 of 32 236 us; 65,536 bins x 16 states 332 -> 158 us.  At 8 per SM
-    // the halved units exceeded the 12 warps resident per SM, a second wave: 32 data sets of 8,000 bins x 4 states
+    // than kMinUnits64PerSm, and to 512 slots per state; the slots may exceed the FP32 path's bytes by a few
+    // hundred kB.  (A unit costs about 100 FP64 instructions besides its bins' 58 each, and a state's
+    // finalize reads its slots 256 at a time.)  Dense covariance, 16,384 bins x 16 states: 64 units of 256
+    // bins 1,559 us, 512 of 32 bins 236 us; 65,536 bins x 16 states 332 -> 158 us.  With 8 per SM the halved
+    // units exceeded the 12 warps resident on an SM, a second wave: 32 data sets of 8,000 bins x 4 states
     // 158 -> 231 us.
     int min_sw = 32;   // lanes side by side in the units of the smallest dataset (unit_of)
     int64_t max_n = 0;
