@@ -520,12 +520,13 @@ def run_ours(args):
                              "scale": float(max(abs(L64[wk] - K_d[ds_of[wk]]), Cnu_d[ds_of[wk]]))},
              "tiling": I["tiling"], "autotune_top": [[t, round(v, 4)] for t, v in I["table"][:5]]}
         r["speedup_fp32_vs_fp64"] = r["value"] / r["fp64_plain"]["value"]
-        fp64_rate = (sb / (ll64 / 1e3)) * FP64_PIPE_PER_STATE_BIN    # FP64-pipe instructions per second
-        r["fp64_plain"]["roofline"] = {
-            "bound": "alu", "pipe": "FP64", "achieved": fp64_rate / 1e9, "peak": rates["dfma"] / 1e9, "unit": "Gop/s",
-            "frac": fp64_rate / rates["dfma"], "ops_per_state_bin": FP64_PIPE_PER_STATE_BIN,
-            "ops_source": "ncu thread-level FP64-pipe instruction count per state-bin (profiles/loglike_fp64_ops.md)",
-            "peak_source": "measured live by lisa_pipe_rates (fma.rn.f64)", "timing": "the likelihood graph only"}
+        if not wl.cov_model:   # the count is the diagonal model's
+            fp64_rate = (sb / (ll64 / 1e3)) * FP64_PIPE_PER_STATE_BIN    # FP64-pipe instructions per second
+            r["fp64_plain"]["roofline"] = {
+                "bound": "alu", "pipe": "FP64", "achieved": fp64_rate / 1e9, "peak": rates["dfma"] / 1e9, "unit": "Gop/s",
+                "frac": fp64_rate / rates["dfma"], "ops_per_state_bin": FP64_PIPE_PER_STATE_BIN,
+                "ops_source": "ncu thread-level FP64-pipe instruction count per state-bin (profiles/loglike_fp64_ops.md)",
+                "peak_source": "measured live by lisa_pipe_rates (fma.rn.f64)", "timing": "the likelihood graph only"}
         return r, ev32, clocks
 
     def roofline_of(I, r):
