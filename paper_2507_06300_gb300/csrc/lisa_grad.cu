@@ -554,11 +554,11 @@ __device__ __noinline__ void adjoint_bin64_wide(const double* P, double ao2, dou
     if (HAS_H) out[4 + C] = H;
 }
 
-// Per state-bin 110 FP64 instructions (about 340 with the library's functions and a division per
+// Per state-bin 113 FP64 instructions (about 340 with the library's functions and a division per
 // channel): the forward pass as loglike_fp64_kernel's, 9 for the channels' reciprocals from one of their
-// product, 21 for the template sums and signals, 24 for the moments.  One unit and warp per CTA: the
+// product, 24 for the template sums and signals, 24 for the moments.  One unit and warp per CTA: the
 // units of a small problem spread over all SMs and start as registers come free (four units to a CTA,
-// their CTAs half empty: 1.85 against 1.53 ms).  16,384 bins x 400 states with the epilogue: 5.8 -> 1.70 ms.
+// their CTAs half empty: 1.85 against 1.53 ms).  16,384 bins x 400 states with the epilogue: 5.8 -> 1.74 ms.
 constexpr int kLogRun = 64;   // factors of a LogProduct: its mantissa stays below 2^64
 template <int C, bool HAS_H, bool BROKEN>
 __global__ void __launch_bounds__(32)
@@ -677,8 +677,8 @@ __global__ void __launch_bounds__(32)
         }
         const double p01 = S[0] * S[1];
         const double prod = C == 3 ? p01 * S[C - 1] : p01;
-        ok &= m64::normal_range(p01) && m64::normal_range(prod) && m64::normal_range(S[0]) && m64::normal_range(S[1]) &&
-              m64::normal_range(S[C - 1]);
+        ok &= m64::normal_range(p01) && m64::normal_range(prod) && m64::square_range(S[0]) && m64::square_range(S[1]) &&
+              m64::square_range(S[C - 1]);
         if (ok) {
             const double rp = m64::divide(1.0, prod);
             if (C == 3) {
@@ -693,7 +693,8 @@ __global__ void __launch_bounds__(32)
             double H = 0.0;
 #pragma unroll
             for (int c = 0; c < C; ++c) {
-                const double g = fma(nu, r[c], -nu) * r[c];   // nu (1 - S) / S^2
+                // nu (1 - S) / S^2, with 1 - S from S: r - 1 cancels to r's own error of 2-3 ulp
+                const double g = nu * r[c] * fma(-S[c], r[c], r[c]);
                 const double gE = g * E[c];
                 run += r[c];
                 acc[1] = fma(gE, go[c], acc[1]);

@@ -40,6 +40,8 @@ __device__ __forceinline__ int exponent(double v) { return (int)((hi32(v) >> 20)
 __device__ __forceinline__ bool negative(double v) { return (int)hi32(v) < 0; }   // (-0 included)
 // Whether |v| lies in [2^-900, 2^900) (false for NaN).
 __device__ __forceinline__ bool normal_range(double v) { return (unsigned)(exponent(v) - 123) < 1800u; }
+// Whether |v| lies in [2^-480, 2^480): the squares of v and 1 / v are finite.
+__device__ __forceinline__ bool square_range(double v) { return (unsigned)(exponent(v) - 543) < 960u; }
 // |v| < 100 (false for NaN): the range of exp10_fast.
 __device__ __forceinline__ bool small_exponent(double v) { return (hi32(v) & 0x7fffffffu) < 0x40590000u; }
 
