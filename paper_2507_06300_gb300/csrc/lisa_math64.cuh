@@ -29,10 +29,11 @@ __device__ __forceinline__ double to_double(float f) {
     const unsigned b = __float_as_uint(f);
     return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
 }
-// The order of doubles on integers (NaN excluded): comparisons without the FP64 pipe.
+// The order of doubles on integers (NaN excluded): comparisons without the FP64 pipe.  -0 and +0 have one
+// key, as they compare equal (a knot at -0 does not lie inside a band that ends at +0).
 __device__ __forceinline__ long long order_key(double v) {
-    const long long b = __double_as_longlong(v);
-    return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
+    const long long b = __double_as_longlong(v), m = b >> 63;
+    return ((b & 0x7fffffffffffffffLL) ^ m) - m;
 }
 // Biased exponent of a double (0: zero or subnormal, 2047: infinite or NaN).
 __device__ __forceinline__ int exponent(double v) { return (int)((hi32(v) >> 20) & 0x7ffu); }
