@@ -749,7 +749,7 @@ __global__ void __launch_bounds__(32)
 // Mode kFallback: the states the FP32 epilogue flagged (their FP32 sums left the FP32 range), all
 // their bins: spline values in float-float from the FP32 records, the PSDs, 1 / S-hat and the
 // sums in FP64; the sums overwrite the slots (every interval from the range's first bin to its
-// last), in the FP32 adjoint's convention (moments about the records' midpoints, q without ln10).
+// last; zeros in the further slots of an interval that several of the adjoint's ranges hold), in the FP32 adjoint's convention (moments about the records' midpoints, q without ln10).
 // A resident grid runs the (state, range) items of a compact list (kComp: the setup's route
 // list; kFallback: the flag area's list), each CTA fetching its next item from a counter.
 // The CTA's warps (4 for kComp, 16 for kFallback) split the range's bins, their lanes 32
@@ -778,11 +778,10 @@ __global__ void __launch_bounds__(MODE == kComp ? 128 : 512)
     // list (the fallback's), fb, scal and mom are also written by the kernel before, which may still run
     // when this one starts: not __restrict__, so that no access to them is moved above the wait
     constexpr int NSP = C + (HAS_H ? 1 : 0);
-    // this pass's ranges: kComp takes kAdjBins bins whatever the adjoint's range size (its lanes'
-    // FP32 template sums then cover the same bins), each holding `sub` of the adjoint's ranges, the
-    // first of which has index rho * sub; kFallback takes the adjoint's ranges
-    const int rbins = MODE == kComp ? kAdjBins : adj_bins;
-    const int sub = rbins / adj_bins;
+    // this pass's ranges hold `sub` of the adjoint's, the first of which has index rho * sub (R: the most
+    // ranges of any dataset, the adjoint's for kFallback).  kComp takes kAdjBins bins whatever the adjoint's
+    // range size (its lanes' FP32 template sums then cover the same bins); kFallback picks below
+    int sub = MODE == kComp ? kAdjBins / adj_bins : 1;
     // per warp, spline and interval (from the range's first) the 4 moment sums: dynamic shared
     // memory of nwarps * NSP * (kmax + 1) * 4 doubles
     extern __shared__ double s_m[];
@@ -799,6 +798,16 @@ __global__ void __launch_bounds__(MODE == kComp ? 128 : 512)
     asm volatile("griddepcontrol.launch_dependents;");
     // kFallback reads what the passes before it wrote; kComp only adds to it, after its own work
     if (MODE == kFallback) asm volatile("griddepcontrol.wait;" ::: "memory");
+    // kFallback: the longest ranges, of kAdjBins bins at most, that give every CTA an item.  A CTA's 16 warps
+    // take 8 bins each from a range of 128 and pay for the search and the merge all the same: with the
+    // adjoint's ranges throughout, the call with every state flagged took 18.2 ms for 131,072 bins x 64
+    // states (2.9 with these; 3.3 with 2,048 bins throughout), 7.6 ms for 8,191 bins x 400 (1.5; 2.2), and with
+    // one state in sixteen flagged 0.69 ms (0.35; 1.1).
+    if (MODE == kFallback) {
+        while (2 * sub * adj_bins <= kAdjBins && (int64_t)list[0] * ((R + 2 * sub - 1) / (2 * sub)) >= gridDim.x) sub *= 2;
+        R = (R + sub - 1) / sub;
+    }
+    const int rbins = sub * adj_bins;
     const int n_items = list[0] * R;
     for (;;) {
     if (threadIdx.x == 0) s_item = atomicAdd(next_item, 1);
@@ -1206,6 +1215,20 @@ __global__ void __launch_bounds__(MODE == kComp ? 128 : 512)
     }
     if (MODE == kComp) asm volatile("griddepcontrol.wait;" ::: "memory");
     __syncthreads();
+    if (MODE == kFallback && sub > 1) {
+        // the slots of the adjoint's ranges (their intervals lie end to end), for the sums to overwrite the
+        // first one of each interval
+        const int n_sub = min(sub, D.nranges - rho * sub);
+#pragma unroll
+        for (int a = 0; a < NSP; ++a) {
+            double* row = mom_row(mom, pre, s, a, nsp, kmax, D.nranges);
+            const int n = n_sub + s_jl[a] - j0[a];
+            for (int e = threadIdx.x; e < 4 * n; e += blockDim.x)
+                row[4 * (int64_t)LISA_IDX(rho * sub + j0[a] + (e >> 2), D.nranges + kmax + 1) + (e & 3)] = 0.0;
+        }
+        for (int e = threadIdx.x; e < 6 * n_sub; e += blockDim.x) scal[6 * (pre + (int64_t)rho * sub) + e] = 0.0;
+        __syncthreads();
+    }
     // the warps' sums in order, to the slots
     for (int e = threadIdx.x; e < NSP * nsl; e += blockDim.x) {
         const int a = e / nsl, jr = e % nsl;
@@ -1216,30 +1239,28 @@ __global__ void __launch_bounds__(MODE == kComp ? 128 : 512)
             v[p] = 0.0;
             for (int w = 0; w < nwarps; ++w) v[p] += sm(w, a, jr, p);
         }
-        double* row = mom_row(mom, pre, s, a, nsp, kmax, D.nranges);
-        if (MODE == kComp) {
-            // the sums go to the slot of the first of the adjoint's ranges that holds a bin of the
-            // interval
-            if (v[0] != 0.0 || v[1] != 0.0 || v[2] != 0.0 || v[3] != 0.0) {
-                int i = 0;
-                if (sub > 1 && j > 0) {
-                    const float left = right_end(a, j - 1);
-                    int hi = nb - 1;
-                    while (i < hi) {
-                        const int mid = (i + hi) >> 1;
-                        if (xbin(mid) >= left) hi = mid; else i = mid + 1;
-                    }
-                }
-                row += 4 * (int64_t)LISA_IDX(rho * sub + i / adj_bins + j, D.nranges + kmax + 1);
-                bool bad = false;
-                for (int p = 0; p < 4; ++p) {
-                    row[p] += v[p];
-                    bad |= !isfinite(row[p]);
-                }
-                if (bad) fb_flag(fb, S, s);
+        // the sums go to the slot of the first of the adjoint's ranges that holds a bin of the interval
+        // (kComp: if there are any)
+        if (MODE == kComp && v[0] == 0.0 && v[1] == 0.0 && v[2] == 0.0 && v[3] == 0.0) continue;
+        int i = 0;
+        if (sub > 1 && j > 0) {
+            const float left = right_end(a, j - 1);
+            int hi = nb - 1;
+            while (i < hi) {
+                const int mid = (i + hi) >> 1;
+                if (xbin(mid) >= left) hi = mid; else i = mid + 1;
             }
+        }
+        double* row = mom_row(mom, pre, s, a, nsp, kmax, D.nranges) +
+                      4 * (int64_t)LISA_IDX(rho * sub + i / adj_bins + j, D.nranges + kmax + 1);
+        if (MODE == kComp) {
+            bool bad = false;
+            for (int p = 0; p < 4; ++p) {
+                row[p] += v[p];
+                bad |= !isfinite(row[p]);
+            }
+            if (bad) fb_flag(fb, S, s);
         } else {
-            row += 4 * (int64_t)LISA_IDX(rho + j, D.nranges + kmax + 1);
             for (int p = 0; p < 4; ++p) row[p] = v[p];
         }
     }
