@@ -29,9 +29,17 @@ __device__ __forceinline__ double to_double(float f) {
     const unsigned b = __float_as_uint(f);
     return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
 }
-// The order of doubles on integers (NaN excluded): comparisons without the FP64 pipe.  -0 and +0 have one
-// key, as they compare equal (a knot at -0 does not lie inside a band that ends at +0).
+// The order of doubles on integers (NaN excluded; -0 lies below +0): comparisons without the FP64 pipe.  For
+// bins against knots: no bin's x is -0 (log10 of 1 Hz is +0), so a knot at a zero of either sign is at or below
+// the bin at 1 Hz, as it compares.
 __device__ __forceinline__ long long order_key(double v) {
+    const long long b = __double_as_longlong(v);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
+}
+// The same with one key for both zeros, for knots against knots and band edges: a knot at -0 does not lie
+// inside a band that ends at +0.  (Its two further instructions in the bins' searches cost the model PSD 0.81
+// -> 0.99 ms, the FP64 likelihood 2 %.)
+__device__ __forceinline__ long long position_key(double v) {
     const long long b = __double_as_longlong(v), m = b >> 63;
     return ((b & 0x7fffffffffffffffLL) ^ m) - m;
 }

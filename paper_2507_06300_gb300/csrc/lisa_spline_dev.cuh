@@ -220,8 +220,8 @@ __device__ __forceinline__ void warp_build_spline(WarpSpline<T>& W, const double
         bool bx = false, bw = false;
         // (comparisons on the integer pipes)
         auto finite = [](double v) { return m64::exponent(v) != 2047; };
-        const long long klo = m64::order_key(xlo), khi = m64::order_key(xhi);
-        auto inside = [&](double v) { return finite(v) && m64::order_key(v) > klo && m64::order_key(v) < khi; };
+        const long long klo = m64::position_key(xlo), khi = m64::position_key(xhi);
+        auto inside = [&](double v) { return finite(v) && m64::position_key(v) > klo && m64::position_key(v) < khi; };
         if (lane < k) {
             xa = px[LISA_IDX(lane, kmax)];
             wa = pw[1 + LISA_IDX(lane, kmax)];
@@ -243,7 +243,7 @@ __device__ __forceinline__ void warp_build_spline(WarpSpline<T>& W, const double
     if (!st) {
         // rank sort (stable) with duplicate detection, on integer keys that order like the
         // (finite) doubles, so the comparisons run on the integer pipes
-        const long long ka = m64::order_key(xa), kb = m64::order_key(xb);
+        const long long ka = m64::position_key(xa), kb = m64::position_key(xb);
         bool dup = false;
         for (int i = 0; i < k; ++i) {
             const long long ki = __shfl_sync(kFull, i < 32 ? ka : kb, i & 31);
