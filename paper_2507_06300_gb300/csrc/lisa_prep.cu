@@ -95,8 +95,8 @@ struct LaneSum {
 // fixed order for a given G), and with G >= 4 its lanes share the epilogue: lane c divides channel
 // c's sum, lane 3 writes the bin's centre and nu.  With FP64 multiply-adds the FP64 pipe bounded this
 // kernel (two of them per complex sample, 81 us for 25.2 M samples at its rate against 60 us of HBM
-// time); the lanes' sums of squares run on the integer pipes (about 40 instructions a sample, exact to
-// 2^-61 of the sum) where a bin has enough samples to pay for the conversion of the sums, which is the
+// time); the lanes' sums of squares run on the integer pipes (about 40 instructions a sample; at most 3 n
+// units of 2^-62 of the largest of a lane's n squares too small) where a bin has enough samples to pay for the conversion of the sums, which is the
 // rule's line at 12 samples per bin.  25.2 M samples in 64-sample bins: 125 us -> 92 us.
 template <int C, int G, bool SOFT>
 __global__ void __launch_bounds__(256)

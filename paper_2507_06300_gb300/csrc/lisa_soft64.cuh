@@ -83,8 +83,10 @@ LISA_HD bool mul(int ea, uint64_t A, uint64_t x, uint64_t& out) {
 }
 
 // Sum of squares in fixed point: (top, acc), 96 bits, times 2^(2 (E - 1023) - 62), E the largest biased
-// exponent met.  Each square is cut at 2^-62 of its own size and at 2^-62 of the largest one: below the
-// rounding of an FP64 accumulation.
+// exponent met.  Each square loses less than two units of its own last bit to its truncation and the sum
+// less than one at each shift, so n squares come out at most 3 n units of 2^-62 of the largest one's binade
+// too small, never too large.  Additions in FP64 may lose more: 2e5 squares of 2^-61 beside one of 1, 3.6e-14
+// here, 7.9e-14 there.
 struct SquareSum {
     uint64_t acc;
     uint32_t top;
