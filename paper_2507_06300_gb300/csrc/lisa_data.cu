@@ -374,7 +374,26 @@ lisa_status rebuild_work(lisa_data* d) {
             }
         }
     }
+    d->fast_knots = false;
     const int occ = t.ctas_per_sm > 0 ? t.ctas_per_sm : fused_ctas_per_sm(d, t);
+    // The fused kernel's form of the knot chunks (at group 4; see loglike_fp32_kernel), FAST or plain:
+    //  - plain up to 384-bin tiles, of which five CTAs' fit into an SM, which is what its registers allow
+    //    (131,072 bins x 4,096 states: 128 bins 1,304 us plain, 1,377 FAST; 384 1,091, 1,106; 448 1,109, 1,100);
+    //  - FAST for split items: their few CTAs wait for the records that it loads together (4,000 bins x 64
+    //    states 78 plain, 68);
+    //  - items of at most two rows: plain while a CTA has fewer than two of them, since the chain of the lowest
+    //    tile, which holds most knots, is the kernel's time (131,072 x 512: 190, 194), then FAST (768 states, 2.5
+    //    items a CTA: 233, 229; 1,024: 293, 288; 2,048: 530, 523);
+    //  - items of more rows, whose warps meet a knot in most blocks: the other way round (32 data sets of 2,000
+    //    bins x 16 states, 0.2 items a CTA: 86, 80; 128 of 24,000, ten: 281, 284).
+    if (d->nseg > 1) {
+        d->fast_knots = true;
+    } else if (d->stage_bins > 384) {
+        const bool many = items.size() >= 2 * (size_t)d->n_sm * (size_t)std::max(occ, 1);
+        bool rows = false;   // more than two
+        for (const DatasetDev& D : d->h_ds) rows |= D.ns > 0 && lanes(D) < kThreads32 / 2;
+        d->fast_knots = many != rows;
+    }
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(d->n_sm * std::max(occ, 1), (int64_t)items.size()));
     // contiguous blocks pay off when a CTA has many items and each thread takes few bins from an
     // item (small state chunks: the per-item interval search dominates); with a few items per CTA

@@ -198,6 +198,7 @@ struct lisa_data {
     int32_t nseg = 1;                // segments per work item
     int32_t stage_bins = 0;          // bins per staging buffer of the fused kernels
     int32_t rt_bins = 0;             // bins per unit of the compensated kernel
+    bool fast_knots = false;         // the fused kernel's form of the knot chunks (group 4)
     bool chunk_items = false;        // every item is one FP32 chunk of one-row items (loglike_chunk_kernel)
     int32_t b64 = 0;                 // bins per unit of the plain FP64 kernels
     int64_t n_units64 = 0;           // their units

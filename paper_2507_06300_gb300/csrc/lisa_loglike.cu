@@ -351,8 +351,15 @@ constexpr int kStages = 2;
 constexpr int kChunkPairs = 32;   // pair blocks per FP32 partial sum (64 bins)
 constexpr int kWarps32 = kThreads32 / 32;
 
-template <int C, bool HAS_H, bool BROKEN, int G>
-__global__ void __launch_bounds__(kThreads32, G == 2 ? 5 : 4)
+// Two forms of the knot chunks.  FAST takes U pair blocks at once between the knots and loads the next
+// records of all splines that pass one together: fewer instructions where knots are few, 112-124 registers at
+// G = 4, four CTAs per SM.  The other takes pair block after pair block, each spline's next record when it is
+// due: the shorter chain in a tile full of knots, 90 registers at G = 4, five CTAs where the staged tiles leave
+// room for five.  rebuild_work has the line between them.  At G = 8 FAST spills 64-88 bytes at four CTAs
+// (131,072 bins x 4,096 states, 128-bin tiles: 1,378 -> 1,414 us), and at G = 2 it takes the sixth CTA (512-bin
+// tiles 1,125 -> 1,288 us): they have the other form alone.
+template <int C, bool HAS_H, bool BROKEN, int G, bool FAST>
+__global__ void __launch_bounds__(kThreads32, FAST || G == 8 ? 4 : (G == 4 ? 5 : 6))
     loglike_fp32_kernel(const WorkItem* __restrict__ items, int n_items, const int32_t* __restrict__ cta_first,
                         const float* __restrict__ rec32,
                         const StateParams* __restrict__ prm, const int32_t* __restrict__ sstat,
@@ -600,7 +607,7 @@ __global__ void __launch_bounds__(kThreads32, G == 2 ? 5 : 4)
                         for (; ip < pcend; ++ip, blk += kPairRec / 4) {
                             // U blocks at once where no lane reaches a knot in them (the same operations
                             // in the same order)
-                            if (ip + U <= pcend &&
+                            if (FAST && ip + U <= pcend &&
                                 !__any_sync(__activemask(), blk[(U - 1) * (kPairRec / 4)].y >= xmin)) {
 #pragma unroll
                                 for (int u = 0; u < U; ++u) {
@@ -614,7 +621,10 @@ __global__ void __launch_bounds__(kThreads32, G == 2 ? 5 : 4)
                                 continue;
                             }
                             const float4 q0 = blk[0];
-                            if (q0.y >= xmin) {
+                            if (!FAST && q0.y >= xmin) {
+                                acc2.x += scalar_bin(2 * ip);
+                                acc2.x += scalar_bin(2 * ip + 1);
+                            } else if (q0.y >= xmin) {
                                 // the next record of every spline that passes a knot by the second
                                 // bin, all loads in flight at once (one spline after the other, each
                                 // load waited for, cost 1.4 % of the paper-scale step: 299 -> 295 us)
@@ -628,8 +638,8 @@ __global__ void __launch_bounds__(kThreads32, G == 2 ? 5 : 4)
                                         NB[a] = __ldg(q + 1);
                                         have |= 1u << a;
                                     }
-#pragma unroll 1
-                                for (int e = 0; e < 2; ++e) {
+#pragma unroll
+                                for (int e = 0; e < 2; ++e) {   // (as a loop 2-7 % of a call of few items per CTA)
                                     const float x = e ? q0.y : q0.x;
                                     if (x >= xmin) {
 #pragma unroll
@@ -1520,11 +1530,19 @@ __global__ void model_psd_kernel(const int32_t* __restrict__ state_ds, const Dat
 }
 
 template <int C, bool H, bool B, int G>
+auto fused_kernel(bool fast_knots) {
+    auto kern = loglike_fp32_kernel<C, H, B, G, false>;
+    if constexpr (G == 4)
+        if (fast_knots) kern = loglike_fp32_kernel<C, H, B, G, true>;
+    return kern;
+}
+
+template <int C, bool H, bool B, int G>
 cudaError_t launch_fp32_g(const lisa_data* d, const StateParams* prm, const int32_t* sstat, const int32_t* nint,
                           const float* kxr, unsigned long long* rcount, const RobustEntry* rlist, const float* srec,
                           int kmax,
                           double* partial, double* rpart, int* err, cudaStream_t sm, bool prof) {
-    auto kern = loglike_fp32_kernel<C, H, B, G>;
+    auto kern = fused_kernel<C, H, B, G>(d->fast_knots);
     const size_t smem = 2 * (size_t)d->stage_bins * kRec * sizeof(float);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -1577,8 +1595,8 @@ int robust_occupancy() {
 }
 
 template <int C, bool H, bool B, int G>
-int occupancy_g(int stage_bins) {
-    auto kern = loglike_fp32_kernel<C, H, B, G>;
+int occupancy_g(int stage_bins, bool fast_knots) {
+    auto kern = fused_kernel<C, H, B, G>(fast_knots);
     const size_t smem = 2 * (size_t)stage_bins * kRec * sizeof(float);
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
         cudaGetLastError();
@@ -1593,19 +1611,19 @@ int occupancy_g(int stage_bins) {
 }
 
 template <int C, bool H, bool B>
-int occupancy_m(const lisa_tiling& t, int stage_bins) {
+int occupancy_m(const lisa_tiling& t, int stage_bins, bool fast_knots) {
     switch (t.group) {
-        case 2: return occupancy_g<C, H, B, 2>(stage_bins);
-        case 8: return occupancy_g<C, H, B, 8>(stage_bins);
-        default: return occupancy_g<C, H, B, 4>(stage_bins);
+        case 2: return occupancy_g<C, H, B, 2>(stage_bins, fast_knots);
+        case 8: return occupancy_g<C, H, B, 8>(stage_bins, fast_knots);
+        default: return occupancy_g<C, H, B, 4>(stage_bins, fast_knots);
     }
 }
 
 template <int C>
-int occupancy_c(int sgwb, const lisa_tiling& t, int stage_bins) {
-    if (sgwb == 0) return occupancy_m<C, false, false>(t, stage_bins);
-    if (sgwb == 1) return occupancy_m<C, true, false>(t, stage_bins);
-    return occupancy_m<C, true, true>(t, stage_bins);
+int occupancy_c(int sgwb, const lisa_tiling& t, int stage_bins, bool fast_knots) {
+    if (sgwb == 0) return occupancy_m<C, false, false>(t, stage_bins, fast_knots);
+    if (sgwb == 1) return occupancy_m<C, true, false>(t, stage_bins, fast_knots);
+    return occupancy_m<C, true, true>(t, stage_bins, fast_knots);
 }
 
 template <int C, bool H, bool B>
@@ -1662,7 +1680,8 @@ cudaError_t dispatch_model(const lisa_data* d, bool fp32, const double* theta, c
 }  // namespace
 
 int fused_ctas_per_sm(const lisa_data* d, const lisa_tiling& t) {
-    return d->C == 3 ? occupancy_c<3>(d->sgwb_model, t, d->stage_bins) : occupancy_c<2>(d->sgwb_model, t, d->stage_bins);
+    return d->C == 3 ? occupancy_c<3>(d->sgwb_model, t, d->stage_bins, d->fast_knots)
+                     : occupancy_c<2>(d->sgwb_model, t, d->stage_bins, d->fast_knots);
 }
 
 template <int C>
