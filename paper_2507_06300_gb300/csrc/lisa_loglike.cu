@@ -1252,9 +1252,12 @@ __global__ void __launch_bounds__(kRobWarps * 32, 2)
                           const float* __restrict__ elllo32, const StateParams* __restrict__ prm,
                           const int32_t* __restrict__ nint, const float* __restrict__ srec, int kmax, int nsp,
                           double* __restrict__ rpart, int* __restrict__ err, unsigned wait_limit) {
-    asm volatile("griddepcontrol.launch_dependents;");   // the finalize kernel (it waits for this one's end)
     robust_units<C, HAS_H, BROKEN>(rcount, rlist, tile_bins, rec32, xlo32, elllo32, prm, nint, srec, kmax, nsp, rpart,
                                    err, wait_limit);
+    // the finalize kernel may start (it waits for this one's end).  Only now: its CTAs, resident from this
+    // kernel's start on, delayed likelihood-only calls (131,072 bins x 1,024 states,
+    // 128-bin tiles, group 2: 330 -> 318 us; 512 and 8: 283 -> 279)
+    asm volatile("griddepcontrol.launch_dependents;");
     // launched as a programmatic dependent of the fused kernel, so that its CTAs can start on SMs
     // the fused kernel's CTAs have left; it reads nothing the fused kernel writes, but it does not
     // complete before the fused kernel has (the finalize kernel after it then sees both)
