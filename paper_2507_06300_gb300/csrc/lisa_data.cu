@@ -303,8 +303,9 @@ lisa_status rebuild_work(lisa_data* d) {
             break;
         }
     }
-    d->chunk_items = d->nseg > 1 && seg_bins(t.tile_bins, 1, d->nseg) == kSegBins;
-    for (const DatasetDev& D : d->h_ds) d->chunk_items &= D.ns == 0 || lanes(D) == kThreads32;
+    bool one_row = true;   // every item's threads hold different states
+    for (const DatasetDev& D : d->h_ds) one_row &= D.ns == 0 || lanes(D) == kThreads32;
+    d->chunk_items = one_row && d->nseg > 1 && seg_bins(t.tile_bins, 1, d->nseg) == kSegBins;
     // the plain FP64 kernels' units: half a segment of bins x 32 states, one warp each.  (They share
     // the FP64 pipe, so what counts is that the units are many and of one size; half a segment is what
     // the workspace of the FP32 path holds slots for.)
@@ -421,9 +422,12 @@ lisa_status rebuild_work(lisa_data* d) {
     };
     std::vector<int32_t> cta_first((size_t)grid + 1, 0);
     if (d->cov == LISA_COV_FULL) {
-        // the dense kernels take the items in order: the low-frequency tiles, which hold most knots and
-        // ill-conditioned intervals, first
-        std::stable_sort(items.begin(), items.end(), [](const WorkItem& a, const WorkItem& b) { return a.slot < b.slot; });
+        // the one-warp dense kernel starts the items in order, as SMs come free: the low-frequency tiles,
+        // which hold most knots and ill-conditioned intervals, first.  The other form's resident CTAs take
+        // every gridDim-th item, and a CTA that starts with the lowest tile would get the lowest of every
+        // further round too: they keep the (dataset, chunk, tile) order (131,072 bins x 256 states: 32
+        // states an item at 64-bin tiles 573 us, 893 sorted; at 512-bin tiles 741, 1,118).
+        if (one_row) std::stable_sort(items.begin(), items.end(), [](const WorkItem& a, const WorkItem& b) { return a.slot < b.slot; });
     } else if (d->fblocks) {
         // contiguous blocks of the (dataset, chunk, tile)-ordered list, cut so that every CTA gets
         // the same cost (item boundaries at cost midpoints)
