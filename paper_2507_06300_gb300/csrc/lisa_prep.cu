@@ -41,27 +41,21 @@ __global__ void __launch_bounds__(256) fd_synth_kernel(const double* __restrict_
     }
 }
 
-// A lane's sum of squares: fixed point on the integer pipes (SOFT), or FP64 multiply-adds.
-template <bool SOFT>
+// A lane's sum of squares in fixed point on the integer pipes.
 struct LaneSum {
-    static constexpr int kBatch = SOFT ? 4 : 1;   // samples added at once
-    double fp;   // SOFT: of batches with an infinity or a NaN only
+    double fp;   // of batches with an infinity or a NaN only
     soft64::SquareSum q;
     __device__ __forceinline__ void reset() {
         fp = 0.0;
-        if (SOFT) q.reset();
+        q.reset();
     }
-    // Adds kBatch samples (absent ones as zeros, which add nothing).
+    // Adds N samples (absent ones as zeros, which add nothing).
+    template <int N>
     __device__ __forceinline__ void add(const double2* v) {
-        if (!SOFT) {
-#pragma unroll
-            for (int u = 0; u < kBatch; ++u) fp = fma(v[u].x, v[u].x, fma(v[u].y, v[u].y, fp));
-            return;
-        }
-        uint64_t b[2 * kBatch];
+        uint64_t b[2 * N];
         int e = 0;
 #pragma unroll
-        for (int u = 0; u < kBatch; ++u) {
+        for (int u = 0; u < N; ++u) {
             b[2 * u] = (uint64_t)__double_as_longlong(v[u].x);
             b[2 * u + 1] = (uint64_t)__double_as_longlong(v[u].y);
             e = max(e, max(soft64::exp_of(b[2 * u]), soft64::exp_of(b[2 * u + 1])));
@@ -69,16 +63,15 @@ struct LaneSum {
         if (e > q.E) {
             if (e == 2047) {   // an infinity or a NaN: the sum is one too
 #pragma unroll
-                for (int u = 0; u < kBatch; ++u) fp = fma(v[u].x, v[u].x, fma(v[u].y, v[u].y, fp));
+                for (int u = 0; u < N; ++u) fp = fma(v[u].x, v[u].x, fma(v[u].y, v[u].y, fp));
                 return;
             }
             q.raise(e);
         }
 #pragma unroll
-        for (int u = 0; u < 2 * kBatch; ++u) q.add(b[u]);
+        for (int u = 0; u < 2 * N; ++u) q.add(b[u]);
     }
     __device__ __forceinline__ double value() const {
-        if (!SOFT) return fp;
         // the 96-bit sum rounded to FP64, scaled by 2^(2 (E - 1023) - 62) in two exact halves
         const double m = fma((double)q.top, 18446744073709551616.0, (double)q.acc);
         const int k = 2 * (q.E - 1023) - 62, k1 = k >> 1, k2 = k - k1;
@@ -90,19 +83,34 @@ struct LaneSum {
     }
 };
 
+constexpr int kFixedMin = 12;           // samples from which a bin's sums run in fixed point
+constexpr int kFixedBatch = 4;          // samples that a lane adds at once there
+constexpr int kSerialThreadsPerSm = 512;
+constexpr int kSerialWidths = 4;
+constexpr int kTogetherMax = 4;         // one lane per bin: bins of fewer samples have no second load of a channel
+
 // Averaged periodogram: a group of G lanes per bin (G divides 32), lanes striding over the bin's
 // samples with 16-byte loads; the group's partial sums are combined by a butterfly of shuffles (a
 // fixed order for a given G), and with G >= 4 its lanes share the epilogue: lane c divides channel
 // c's sum, lane 3 writes the bin's centre and nu.  With FP64 multiply-adds the FP64 pipe bounded this
 // kernel (two of them per complex sample, 81 us for 25.2 M samples at its rate against 60 us of HBM
-// time); the lanes' sums of squares run on the integer pipes (about 40 instructions a sample; at most 3 n
-// units of 2^-62 of the largest of a lane's n squares too small) where a bin has enough samples to pay for the conversion of the sums, which is the
-// rule's line at 12 samples per bin.  25.2 M samples in 64-sample bins: 125 us -> 92 us.
-template <int C, int G, bool SOFT>
+// time); the lanes' sums of squares run on the integer pipes (about 40 instructions a sample; at most
+// 3 n units of 2^-62 of the largest of a lane's n squares too small, less than FP64 additions may lose) where
+// a bin has enough samples to pay for the conversion of the sums, which is the line at kFixedMin.
+// 25.2 M samples in 64-sample bins: 125 us -> 92 us.
+//
+// That takes many bins side by side.  Where the loads of a few lanes are waited for, four of one channel in
+// flight instead of four of every channel cost more than the FP64 pipe.  So a bin of up to `serial_max` samples
+// takes the channels one after the other, in fixed point from kFixedMin samples on, and a wider one all
+// channels together, in FP64; serial_max is kSerialWidths mean widths, or 0 when the bins have fewer than
+// kSerialThreadsPerSm lanes per SM.  Every bin serial (by its mean width in fixed point): 8,000 bins of 1,000
+// samples (64,000 lanes) 115 us, together 104; 12,000 of 300 (96,000) the same; 20,000 bins of 1 to 4,000
+// samples 402, 298 with this rule; 400 bins of 20,000 samples among 20,000 of one or two 1.89 ms, 1.32.
+template <int C, int G>
 __global__ void __launch_bounds__(256)
     avg_periodogram_kernel(const double2* __restrict__ d, int64_t n_freq, double f0, double df,
                            const int64_t* __restrict__ off, int64_t n_bins, double* __restrict__ P,
-                           double* __restrict__ f_out, double* __restrict__ nu_out, int n_ch) {
+                           double* __restrict__ f_out, double* __restrict__ nu_out, int n_ch, int64_t serial_max) {
     const int lane = threadIdx.x & (G - 1);
     const int64_t g0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
     const int64_t ng = ((int64_t)gridDim.x * blockDim.x) / G;
@@ -115,30 +123,54 @@ __global__ void __launch_bounds__(256)
             b0 = min(max(__ldg(off + i), (int64_t)0), n_freq);
             b1 = min(max(__ldg(off + i + 1), b0), n_freq);
         }
+        const int64_t n = b1 - b0;
         double acc[C];
 #pragma unroll
-        for (int c = 0; c < C; ++c) {
-            acc[c] = 0.0;
-            if (c >= n_ch) continue;
-            LaneSum<SOFT> sum;
-            sum.reset();
-            const double2* dc = d + (int64_t)c * n_freq;
-            constexpr int kBatch = LaneSum<SOFT>::kBatch;
-#pragma unroll(SOFT ? 1 : 4)
-            for (int64_t k = b0 + lane; k < b1; k += kBatch * G) {
-                double2 v[kBatch];
+        for (int c = 0; c < C; ++c) acc[c] = 0.0;
+        if (n > serial_max || (G == 1 && n < kTogetherMax)) {
+#pragma unroll 4
+            for (int64_t k = b0 + lane; k < b1; k += G) {
 #pragma unroll
-                for (int u = 0; u < kBatch; ++u)
-                    v[u] = k + u * G < b1 ? __ldg(dc + k + u * G) : make_double2(0.0, 0.0);
-                sum.add(v);
+                for (int c = 0; c < C; ++c) {
+                    if (c < n_ch) {
+                        const double2 v = __ldg(d + (int64_t)c * n_freq + k);
+                        acc[c] = fma(v.x, v.x, fma(v.y, v.y, acc[c]));
+                    }
+                }
             }
-            acc[c] = sum.value();
+        } else if (G == 1 || n < kFixedMin) {
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                if (c >= n_ch) continue;
+                const double2* dc = d + (int64_t)c * n_freq;
+#pragma unroll 4
+                for (int64_t k = b0 + lane; k < b1; k += G) {
+                    const double2 v = __ldg(dc + k);
+                    acc[c] = fma(v.x, v.x, fma(v.y, v.y, acc[c]));
+                }
+            }
+        } else {
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                if (c >= n_ch) continue;
+                LaneSum sum;
+                sum.reset();
+                const double2* dc = d + (int64_t)c * n_freq;
+#pragma unroll 1
+                for (int64_t k = b0 + lane; k < b1; k += kFixedBatch * G) {
+                    double2 v[kFixedBatch];
+#pragma unroll
+                    for (int u = 0; u < kFixedBatch; ++u)
+                        v[u] = k + u * G < b1 ? __ldg(dc + k + u * G) : make_double2(0.0, 0.0);
+                    sum.add<kFixedBatch>(v);
+                }
+                acc[c] = sum.value();
+            }
         }
 #pragma unroll
         for (int o = G / 2; o > 0; o >>= 1)
 #pragma unroll
             for (int c = 0; c < C; ++c) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o, G);
-        const int64_t n = b1 - b0;
         if (G >= 4) {
             double v = acc[0];
 #pragma unroll
@@ -159,7 +191,7 @@ __global__ void __launch_bounds__(256)
     }
 }
 
-template <int C, int G, bool SOFT>
+template <int C, int G>
 cudaError_t launch_avg(const double2* d, int64_t n_freq, double f0, double df, const int64_t* off, int64_t n_bins,
                        double* P, double* f, double* nu, int n_ch, cudaStream_t sm) {
     int dev = 0, n_sm = 1;
@@ -169,7 +201,9 @@ cudaError_t launch_avg(const double2* d, int64_t n_freq, double f0, double df, c
     const int64_t want = (n_bins * G + threads - 1) / threads;
     const int64_t cap = (int64_t)n_sm * 8;   // persistent: 8 blocks of 256 threads per SM
     const unsigned grid = (unsigned)(want < cap ? (want < 1 ? 1 : want) : cap);
-    avg_periodogram_kernel<C, G, SOFT><<<grid, threads, 0, sm>>>(d, n_freq, f0, df, off, n_bins, P, f, nu, n_ch);
+    const bool many = n_bins * G >= (int64_t)kSerialThreadsPerSm * n_sm;
+    const int64_t serial_max = many ? (int64_t)(kSerialWidths * ((double)n_freq / (double)n_bins)) : 0;
+    avg_periodogram_kernel<C, G><<<grid, threads, 0, sm>>>(d, n_freq, f0, df, off, n_bins, P, f, nu, n_ch, serial_max);
     return cudaGetLastError();
 }
 
@@ -211,11 +245,11 @@ extern "C" lisa_status lisa_averaged_periodogram(const double* d, int32_t n_chan
     const double width = (double)n_freq / (double)n_bins;
     cudaError_t e;
     if (width >= 256.0)
-        e = launch_avg<3, 8, true>(dd, n_freq, f0, df, off, n_bins, P, f, nu, n_channels, sm);
+        e = launch_avg<3, 8>(dd, n_freq, f0, df, off, n_bins, P, f, nu, n_channels, sm);
     else if (width >= 12.0)
-        e = launch_avg<3, 4, true>(dd, n_freq, f0, df, off, n_bins, P, f, nu, n_channels, sm);
+        e = launch_avg<3, 4>(dd, n_freq, f0, df, off, n_bins, P, f, nu, n_channels, sm);
     else
-        e = launch_avg<3, 1, false>(dd, n_freq, f0, df, off, n_bins, P, f, nu, n_channels, sm);
+        e = launch_avg<3, 1>(dd, n_freq, f0, df, off, n_bins, P, f, nu, n_channels, sm);
     return check_cuda(e);
 }
 
