@@ -8,6 +8,7 @@
 #include <new>
 
 #include "lisa_internal.cuh"
+#include "lisa_math64.cuh"
 #include "lisa_debug.h"
 #include "lisa_peaks.h"
 
@@ -209,11 +210,11 @@ void release(lisa_data* d) {
     d->d_items = nullptr;
 }
 
-// 2^(j / kExpTab) rounded from long double, computed once per process.
+// The table of the FP64 path's exponential, computed once per process.
 const double* exp_table() {
     static const std::vector<double> T = [] {
-        std::vector<double> v((size_t)kExpTab);
-        for (int j = 0; j < kExpTab; ++j) v[(size_t)j] = (double)std::exp2((long double)j / kExpTab);
+        std::vector<double> v((size_t)kExpTabDoubles);
+        m64::fill_exp_table(v.data());
         return v;
     }();
     return T.data();
@@ -695,14 +696,14 @@ lisa_status lisa_data_create(const lisa_data_desc* desc, lisa_stream_t stream, l
         (st = dev_alloc(&d->d_elllo32, (size_t)NP)) || (st = dev_alloc(&nu_p, (size_t)NP)) ||
         (st = dev_alloc(&f, (size_t)N)) ||
         (st = dev_alloc(&nu, (size_t)N)) || (st = dev_alloc(&lnP, (size_t)NP)) ||
-        (st = dev_alloc(&R, (size_t)C * N)) || (st = dev_alloc(&d->d_exptab, (size_t)kExpTab + 4 * (size_t)rbase)))
+        (st = dev_alloc(&R, (size_t)C * N)) || (st = dev_alloc(&d->d_exptab, (size_t)kExpTabDoubles + 4 * (size_t)rbase)))
         return fail(st);
-    d->d_rx32 = reinterpret_cast<double2*>(d->d_exptab + kExpTab);
+    d->d_rx32 = reinterpret_cast<double2*>(d->d_exptab + kExpTabDoubles);
     d->d_rx64 = d->d_rx32 + rbase;
     cudaStream_t sm = (cudaStream_t)stream;
     bool ok = cudaMemcpyAsync(d->d_ds, d->h_ds.data(), D * sizeof(DatasetDev), cudaMemcpyHostToDevice, sm) == cudaSuccess &&
               cudaMemcpyAsync(d->d_state_ds, state_ds.data(), S * sizeof(int32_t), cudaMemcpyHostToDevice, sm) == cudaSuccess &&
-              cudaMemcpyAsync(d->d_exptab, exp_table(), kExpTab * sizeof(double), cudaMemcpyHostToDevice, sm) == cudaSuccess &&
+              cudaMemcpyAsync(d->d_exptab, exp_table(), kExpTabDoubles * sizeof(double), cudaMemcpyHostToDevice, sm) == cudaSuccess &&
               cudaMemcpyAsync(f, q.freq, N * sizeof(double), cudaMemcpyHostToDevice, sm) == cudaSuccess &&
               cudaMemcpyAsync(nu, q.nu, N * sizeof(double), cudaMemcpyHostToDevice, sm) == cudaSuccess &&
               cudaMemcpyAsync(d->d_P, q.periodogram, C * N * sizeof(double), cudaMemcpyHostToDevice, sm) == cudaSuccess &&

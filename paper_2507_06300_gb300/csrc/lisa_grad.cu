@@ -524,7 +524,7 @@ __global__ void __launch_bounds__(128, 3)
     }
 }
 
-// ---- FP64 adjoint (plain): same decomposition, FP64 throughout ---------------------------------
+// ---- FP64 adjoint (plain): same decomposition, every value and sum in FP64 ---------------------
 // One bin's sums by the library's exp10, exp2 and log and FP64 divisions, for bins whose exponents or
 // products leave the range of the short forms: out[0] = sum_c (1 / S_c + ln S_c), out[1..3] = To, Tt, H,
 // out[4..] = each spline's q / ln10.  g = nu (1 - S) / S^2 is applied as nu (r - 1) (r E) with
@@ -554,9 +554,8 @@ __device__ __noinline__ void adjoint_bin64_wide(const double* P, double ao2, dou
     if (HAS_H) out[4 + C] = H;
 }
 
-// Per state-bin 113 FP64 instructions (about 340 with the library's functions and a division per
-// channel): the forward pass as loglike_fp64_kernel's, 9 for the channels' reciprocals from one of their
-// product, 24 for the template sums and signals, 24 for the moments.  One unit and warp per CTA: the
+// Per state-bin 115 FP64 instructions (about 340 with the library's functions and a division per
+// channel): the forward pass as loglike_fp64_kernel's, 9 for the channels' reciprocals, 24 for the template sums and signals, 24 for the moments.  One unit and warp per CTA: the
 // units of a small problem spread over all SMs and start as registers come free (four units to a CTA,
 // their CTAs half empty: 1.85 against 1.53 ms).  16,384 bins x 400 states with the epilogue: 5.8 -> 1.74 ms.
 constexpr int kLogRun = 64;   // factors of a LogProduct: its mantissa stays below 2^64
@@ -580,7 +579,7 @@ __global__ void __launch_bounds__(32)
     constexpr double kLog10_2 = 0.301029995663981195213739;
     const double m1 = n1 * kLog10_2, m2 = n2 * kLog10_2;   // slopes in decades per octave
     // A = 10^log10A once per unit: log10 A inside the bins' exponents would round them at its size
-    const double A = HAS_H ? exp10(lA) : 1.0;
+    const double A = HAS_H ? m64::amplitude(lA, exptab) : 1.0;
     const bool A_ok = m64::normal_range(A);
     const int64_t b0 = D.bin0 + (int64_t)U.rho * adj_bins;
     const int nb = (int)min((int64_t)adj_bins, D.bin0 + D.npad - b0);
@@ -680,20 +679,14 @@ __global__ void __launch_bounds__(32)
         ok &= m64::normal_range(p01) && m64::normal_range(prod) && m64::square_range(S[0]) && m64::square_range(S[1]) &&
               m64::square_range(S[C - 1]);
         if (ok) {
-            const double rp = m64::divide(1.0, prod);
-            if (C == 3) {
-                const double rp2 = rp * S[C - 1];
-                r[C - 1] = rp * p01;
-                r[0] = rp2 * S[1];
-                r[1] = rp2 * S[0];
-            } else {
-                r[0] = rp * S[1];
-                r[1] = rp * S[0];
-            }
+            // (three reciprocals take two instructions more than one of the channels' product, whose factors'
+            // roundings leave each r 2-3 units off instead of half a one)
+#pragma unroll
+            for (int c = 0; c < C; ++c) r[c] = m64::reciprocal(S[c]);
             double H = 0.0;
 #pragma unroll
             for (int c = 0; c < C; ++c) {
-                // nu (1 - S) / S^2, with 1 - S from S: r - 1 cancels to r's own error of 2-3 ulp
+                // nu (1 - S) / S^2, with 1 - S from S: r - 1 cancels to r's own error
                 const double g = nu * r[c] * fma(-S[c], r[c], r[c]);
                 const double gE = g * E[c];
                 run += r[c];

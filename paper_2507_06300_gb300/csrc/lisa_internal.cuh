@@ -90,6 +90,7 @@ constexpr int kAdjWarpsPerSm = 12;
 // wide in log10 f) hold most of them, and each advance stalls its warp on record loads.
 constexpr double kKnotBinsPerDecade = 2500.0;
 constexpr int kExpTab = 8192;               // entries of the FP64 path's table of 2^(j / kExpTab)
+constexpr int kExpTabDoubles = kExpTab + kExpTab / 2;   // with their rounding errors (floats) behind them
 constexpr int kXsStride = 32;               // bins between the host copies of log10 f
 constexpr int kMinItemsPerSm = 2;            // fewer items per SM than this are split into segments
 constexpr int kMinItemsPerSmFull = 32;       // the same for the dense covariance
@@ -203,7 +204,7 @@ struct lisa_data {
     int32_t b64 = 0;                 // bins per unit of the plain FP64 kernels
     int64_t n_units64 = 0;           // their units
     int64_t n_partials64 = 0;        // and their partial sums
-    double* d_exptab = nullptr;      // [kExpTab] 2^(j / kExpTab)
+    double* d_exptab = nullptr;      // [kExpTabDoubles] 2^(j / kExpTab) (m64::fill_exp_table)
     // per-kernel timing of lisa_psd_loglike (lisa_data_set_profiling): events around the main,
     // compensated and finalize kernels of the most recent uncaptured call
     cudaEvent_t prof_ev[4] = {nullptr, nullptr, nullptr, nullptr};

@@ -1265,7 +1265,7 @@ __global__ void __launch_bounds__(kRobWarps * 32, 2)
 }
 
 
-// ---- plain FP64 path: FP64 throughout ------------------------------------------------------
+// ---- plain FP64 path -----------------------------------------------------------------------
 
 // One bin's sum_c (1 / S_c + ln S_c) by the library's exp10, exp2 and log and FP64 divisions, for
 // bins whose exponents or products leave the range of the short forms (any value, NaN included).
@@ -1284,7 +1284,7 @@ __device__ __noinline__ double bin_term64_wide(const double* P, double ao2, doub
 // One warp per unit: b64 bins of one dataset x up to 32 of its states (lanes = states, so every lane
 // reads the same bin; up to 16 states leave room for rows of bins).  Bound by the FP64 pipe (2 lane operations per clock and SM): per state-bin 16
 // instructions for the four cubics, 18 for their exponentials, the power law and A, 12 for the PSDs, 4 for
-// their product and the numerator of sum 1 / S, 4 for the division, 2 for the sums; the logarithm of
+// their product and the numerator of sum 1 / S, 5 for the division, 2 for the sums; the logarithm of
 // the channels' product is taken once for up to kLogRun bins of equal nu.  Intervals, range checks and
 // conversions are integer work (lisa_math64.cuh).  65,537 bins x 400 states: 13.7 -> 3.08 ms;
 // with the rows 262,144 bins x 4 states 547 -> 156 us, 131,072 bins x 1 state 95 -> 43 us.
@@ -1309,7 +1309,7 @@ __global__ void __launch_bounds__(64)
     constexpr double kLog10_2 = 0.301029995663981195213739;
     const double m1 = n1 * kLog10_2, m2 = n2 * kLog10_2;   // slopes in decades per octave
     // A = 10^log10A once per unit: log10 A inside the bins' exponents would round them at its size
-    const double A = HAS_H ? exp10(lA) : 1.0;
+    const double A = HAS_H ? m64::amplitude(lA, exptab) : 1.0;
     const bool A_ok = m64::normal_range(A);
     // the current interval of each spline: left knot, cubic, and its right end as an order key (no
     // FP64 comparison)

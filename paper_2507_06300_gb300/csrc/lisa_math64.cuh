@@ -5,14 +5,29 @@
 // instruction of a warp takes the pipe as long as 64 other instructions take to issue.  So everything
 // that need not be rounded to 53 bits runs elsewhere: exponents, table indices, conversions and
 // comparisons on the integer pipe (from the bits of the doubles), reciprocal seeds and the last terms of
-// the series, below 2^-28 of the result, in FP32.  Against the library's exp10, exp2, log and
+// the series, below 2^-28 of the result, in FP32 pairs of 46 bits.  Against the library's exp10, exp2, log and
 // division a state-bin of the likelihood takes 58 FP64 instructions instead of 225.
 #pragma once
+
+#include <cmath>
+#include <cstring>
 
 #include "lisa_math.cuh"
 
 namespace lisa {
 namespace m64 {
+
+// Host: the table of exp10_fast, kExpTabDoubles doubles: 2^(j / kExpTab) rounded to FP64, then the
+// relative errors of these roundings (what is missing of each, over it) as floats.
+inline void fill_exp_table(double* T) {
+    float* c = reinterpret_cast<float*>(T + kExpTab);
+    for (int j = 0; j < kExpTab; ++j) {
+        const long double v = std::exp2((long double)j / kExpTab);
+        T[j] = (double)v;
+        const float e = (float)((v - (long double)T[j]) / v);
+        std::memcpy(c + j, &e, sizeof e);
+    }
+}
 
 __device__ __forceinline__ unsigned hi32(double v) { return (unsigned)__double2hiint(v); }
 __device__ __forceinline__ unsigned lo32(double v) { return (unsigned)__double2loint(v); }
@@ -55,11 +70,13 @@ __device__ __forceinline__ bool square_range(double v) { return (unsigned)(expon
 __device__ __forceinline__ bool small_exponent(double v) { return (hi32(v) & 0x7fffffffu) < 0x40590000u; }
 
 // 10^v for |v| < 100 from the table T of 2^(j / kExpTab) (the table-driven scheme of Tang, ACM TOMS 15,
-// 1989): 4 FP64 instructions, error within 1 ulp plus the rounding of v.  v = k log10(2) / 8192 + r with
-// k chosen in FP32 (any k near the nearest one does), r exact to twice the precision;
-// 10^r = 1 + r ln10 + q with q = (r ln10)^2 / 2 + (r ln10)^3 / 6 <= 2^-30 formed in float-float and rounded
-// once to FP32 (2^-55 of the result; plain FP32 products of a truncated r left 2 ulp).  The table (64 KB)
-// is read through L1, which the kernels that use it leave free.
+// 1989): 4 FP64 instructions.  v = k log10(2) / 8192 + r with k chosen in FP32 (|r| <= 0.85 of a step), r
+// exact to twice the precision; 10^r = 1 + r ln10 + q with q = (r ln10)^2 / 2 + (r ln10)^3 / 6 <= 2^-28.6,
+// which with the table entry's rounding error is formed in float-float and taken into p to 2^-45 of q: one
+// rounding is left.  Error at most 0.51 units of the last place, rms 0.29 (the library's exp10 takes about 40
+// instructions).  With q rounded to FP32 and T[j] as it is, it was up to 1.7 units, rms 0.41, and the
+// model PSD's error against 64 bits half a percent above that of the library's functions.  The table
+// (96 KB) is read through L1, which the kernels that use it leave free.
 __device__ __forceinline__ double exp10_fast(double v, const double* __restrict__ T) {
     constexpr double C_hi = 0x1.34413509f79ffp-15;    // log10(2) / 8192, rounded to FP64
     constexpr double C_lo = -0x1.9dc1da994fd21p-72;   // and the rest
@@ -78,9 +95,17 @@ __device__ __forceinline__ double exp10_fast(double v, const double* __restrict_
     const float h = rf * rf;
     const float l = fmaf(2.f * rf, rl, fmaf(rf, rf, -h));
     const float q0 = K2 * h;
-    const float q = q0 + (fmaf(K2, h, -q0) + fmaf(K2, l, fmaf(rf, K3, K2l) * h));
-    const double p = fma(r, kLn10, to_double(q));
-    const double t = __ldg(T + (k & (kExpTab - 1)));
+    const int j = k & (kExpTab - 1);
+    const float c = __ldg(reinterpret_cast<const float*>(T + kExpTab) + j);
+    const dm::ff q = dm::two_sum(q0, fmaf(K2, h, -q0) + fmaf(K2, l, fmaf(rf, K3, K2l) * h) + c);
+    // q as a double: its low part, below 2^-23 of the high one, rounded to 2^-45 of the high one's exponent
+    // and added to that one's bits
+    const unsigned qb = __float_as_uint(q.hi), eq = (qb >> 23) & 0xffu;
+    const float lo_scale = eq >= 64u ? __uint_as_float((qb & 0x80000000u) | ((299u - eq) << 23)) : 0.f;
+    const int lo = __float_as_int(fmaf(q.lo, lo_scale, 12582912.f)) - 0x4b400000;
+    const double qd = __longlong_as_double(__double_as_longlong(to_double(q.hi)) + ((long long)lo << 7));
+    const double p = fma(r, kLn10, qd);
+    const double t = __ldg(T + j);
     const double e = fma(t, p, t);
     return __hiloint2double((int)(hi32(e) + (unsigned)((k >> 13) << 20)), (int)lo32(e));
 }
@@ -90,18 +115,28 @@ __device__ __forceinline__ double amplitude(double v, const double* __restrict__
     return small_exponent(v) ? exp10_fast(v, T) : exp10(v);
 }
 
-// n / d for a normal d well inside the range: an FP32 reciprocal of d's mantissa and one cubic step
-// (4 FP64 instructions, error within 1 ulp).
-__device__ __forceinline__ double divide(double n, double d) {
+// 1 / d to 2^-21 for a normal positive d of exponent within +-900, as a double: an FP32 reciprocal of d's
+// mantissa, in (1/2, 1], times 2^-(exponent of d).
+__device__ __forceinline__ double reciprocal_seed(double d) {
     const unsigned h = hi32(d);
     const float m = __uint_as_float(0x3f800000u | ((h & 0xfffffu) << 3) | (lo32(d) >> 29));
     const unsigned b = __float_as_uint(dm::rcp_approx(m));
-    // 1 / m in (1/2, 1] as a double, times 2^-(exponent of d)
-    const double r = __hiloint2double((int)((b >> 3) + (896u << 20) + (1023u << 20) - (h & 0x7ff00000u)), (int)(b << 29));
-    const double e = fma(-d, r, 1.0);
-    const double e2 = fma(e, e, e);
+    return __hiloint2double((int)((b >> 3) + (896u << 20) + (1023u << 20) - (h & 0x7ff00000u)), (int)(b << 29));
+}
+// 1 / d by one cubic step: 3 FP64 instructions, rounded once (error up to half a unit of the last place
+// and 2^-64 of the result).
+__device__ __forceinline__ double reciprocal(double d) {
+    const double r = reciprocal_seed(d), e = fma(-d, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
+// n / d: a reciprocal to 2^-42, the quotient by it and one correction by the remainder: 5 FP64
+// instructions, rounded once.  (n r (1 + e + e^2), 4 instructions, rounds twice: up to 1 unit, 1.2 with a
+// seed one unit off.)
+__device__ __forceinline__ double divide(double n, double d) {
+    const double r0 = reciprocal_seed(d);
+    const double r = fma(r0, fma(-d, r0, 1.0), r0);
     const double w = n * r;
-    return fma(w, e2, w);
+    return fma(fma(-d, w, n), r, w);
 }
 
 // Running product of normal positive doubles as mantissa and exponent: one FP64 instruction a factor.
