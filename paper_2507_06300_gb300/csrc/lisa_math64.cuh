@@ -24,7 +24,7 @@ inline void fill_exp_table(double* T) {
     for (int j = 0; j < kExpTab; ++j) {
         const long double v = std::exp2((long double)j / kExpTab);
         T[j] = (double)v;
-        const float e = (float)((v - (long double)T[j]) / v);
+        const float e = (float)(v - (long double)T[j]) / (float)T[j];
         std::memcpy(c + j, &e, sizeof e);
     }
 }
