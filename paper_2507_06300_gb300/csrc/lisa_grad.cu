@@ -525,21 +525,22 @@ __global__ void __launch_bounds__(128, 3)
 }
 
 // ---- FP64 adjoint (plain): same decomposition, every value and sum in FP64 ---------------------
-// One bin's sums by the library's exp10, exp2 and log and FP64 divisions, for bins whose exponents or
-// products leave the range of the short forms: out[0] = sum_c (1 / S_c + ln S_c), out[1..3] = To, Tt, H,
+// One bin's sums with a logarithm per channel, and the library's functions for the factors out of the short
+// forms' range (as bin_term64_wide), for bins with an exponent or a product out of it: out[0] = sum_c (1 / S_c + ln S_c), out[1..3] = To, Tt, H,
 // out[4..] = each spline's q / ln10.  g = nu (1 - S) / S^2 is applied as nu (r - 1) (r E) with
 // r = 1 / S: no intermediate overflows where S^2 would (S beyond 1e154).
 template <int C, bool HAS_H>
 __device__ __noinline__ void adjoint_bin64_wide(const double* P, double ao2, double at2, double lA, double slope,
-                                                const double* __restrict__ q, double* out) {
-    const double eh = HAS_H ? exp10(lA + P[C]) * exp2(slope * q[1]) : 0.0;
+                                                const double* __restrict__ q, const double* __restrict__ exptab,
+                                                double* out) {
+    const double eh = HAS_H ? m64::background_wide(lA, P[C], slope * q[1], exptab) : 0.0;
     double fwd = 0.0, To = 0.0, Tt = 0.0, H = 0.0;
     for (int c = 0; c < C; ++c) {
-        const double E = exp10(P[c]);
+        const double E = m64::amplitude(P[c], exptab);
         const double N = ao2 * q[3 + c] + at2 * q[6 + c];
         const double Eh = HAS_H ? eh * q[9 + c] : 0.0;
         const double Sc = E * N + Eh;
-        const double r = 1.0 / Sc;
+        const double r = m64::reciprocal_wide(Sc);
         const double gr = q[2] * (r - 1.0), rE = r * E;
         fwd += r + log(Sc);
         To += gr * rE * q[3 + c];
@@ -664,48 +665,52 @@ __global__ void __launch_bounds__(32)
         if (HAS_H) P[C] = fma(BROKEN ? (m64::negative(ell) ? m1 : m2) : m1, ell, P[C]);
 #pragma unroll
         for (int a = 0; a < NSP; ++a) ok &= m64::small_exponent(P[a]);
-        double S[C], E[C], N[C], Eh[C], r[C], qv[NSP];
-        double eh = 0.0;
-        if (HAS_H) eh = A * m64::exp10_fast(P[C], exptab);
-#pragma unroll
-        for (int c = 0; c < C; ++c) {
-            N[c] = fma(ao2, go[c], at2 * gt[c]);
-            E[c] = m64::exp10_fast(P[c], exptab);
-            Eh[c] = HAS_H ? eh * gh[c] : 0.0;
-            S[c] = HAS_H ? fma(N[c], E[c], Eh[c]) : N[c] * E[c];
-        }
-        const double p01 = S[0] * S[1];
-        const double prod = C == 3 ? p01 * S[C - 1] : p01;
-        ok &= m64::normal_range(p01) && m64::normal_range(prod) && m64::square_range(S[0]) && m64::square_range(S[1]) &&
-              m64::square_range(S[C - 1]);
+        double qv[NSP];
         if (ok) {
-            // (three reciprocals take two instructions more than one of the channels' product, whose factors'
-            // roundings leave each r 2-3 units off instead of half a one)
-#pragma unroll
-            for (int c = 0; c < C; ++c) r[c] = m64::reciprocal(S[c]);
-            double H = 0.0;
+            double S[C], E[C], N[C], Eh[C], r[C], eh = 0.0;
+            if (HAS_H) eh = A * m64::exp10_fast(P[C], exptab);
 #pragma unroll
             for (int c = 0; c < C; ++c) {
-                // nu (1 - S) / S^2, with 1 - S from S: r - 1 cancels to r's own error
-                const double g = nu * r[c] * fma(-S[c], r[c], r[c]);
-                const double gE = g * E[c];
-                run += r[c];
-                acc[1] = fma(gE, go[c], acc[1]);
-                acc[2] = fma(gE, gt[c], acc[2]);
-                qv[c] = gE * N[c];
-                if (HAS_H) H = c == 0 ? g * Eh[c] : fma(g, Eh[c], H);
+                N[c] = fma(ao2, go[c], at2 * gt[c]);
+                E[c] = m64::exp10_fast(P[c], exptab);
+                Eh[c] = HAS_H ? eh * gh[c] : 0.0;
+                S[c] = HAS_H ? fma(N[c], E[c], Eh[c]) : N[c] * E[c];
             }
-            if (HAS_H) qv[C] = H;
-            run -= (double)C;
-            lp.mul(prod);
-            ++len;
-        } else {
+            const double p01 = S[0] * S[1];
+            const double prod = C == 3 ? p01 * S[C - 1] : p01;
+            ok = m64::normal_range(p01) && m64::normal_range(prod) && m64::square_range(S[0]) && m64::square_range(S[1]) &&
+                  m64::square_range(S[C - 1]);
+            if (ok) {
+                // (three reciprocals take two instructions more than one of the channels' product, whose factors'
+                // roundings leave each r 2-3 units off instead of half a one)
+#pragma unroll
+                for (int c = 0; c < C; ++c) r[c] = m64::reciprocal(S[c]);
+                double H = 0.0;
+#pragma unroll
+                for (int c = 0; c < C; ++c) {
+                    // nu (1 - S) / S^2, with 1 - S from S: r - 1 cancels to r's own error
+                    const double g = nu * r[c] * fma(-S[c], r[c], r[c]);
+                    const double gE = g * E[c];
+                    run += r[c];
+                    acc[1] = fma(gE, go[c], acc[1]);
+                    acc[2] = fma(gE, gt[c], acc[2]);
+                    qv[c] = gE * N[c];
+                    if (HAS_H) H = c == 0 ? g * Eh[c] : fma(g, Eh[c], H);
+                }
+                if (HAS_H) qv[C] = H;
+                run -= (double)C;
+                lp.mul(prod);
+                ++len;
+            }
+        }
+        if (!ok) {
             double Pv[NSP], out[4 + NSP];
 #pragma unroll
             for (int a = 0; a < NSP; ++a) {
                 Pv[a] = ca[a] + t[a] * (cb[a] + t[a] * (cc[a] + t[a] * cd[a]));
             }
-            adjoint_bin64_wide<C, HAS_H>(Pv, ao2, at2, lA, BROKEN ? (m64::negative(ell) ? n1 : n2) : n1, q, out);
+            adjoint_bin64_wide<C, HAS_H>(Pv, ao2, at2, lA, BROKEN ? (m64::negative(ell) ? n1 : n2) : n1, q, exptab,
+                                         out);
             acc[0] += nu * (out[0] - (double)C);
             acc[1] += out[1];
             acc[2] += out[2];

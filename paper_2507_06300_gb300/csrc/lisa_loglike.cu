@@ -1267,16 +1267,19 @@ __global__ void __launch_bounds__(kRobWarps * 32, 2)
 
 // ---- plain FP64 path -----------------------------------------------------------------------
 
-// One bin's sum_c (1 / S_c + ln S_c) by the library's exp10, exp2 and log and FP64 divisions, for
-// bins whose exponents or products leave the range of the short forms (any value, NaN included).
+// One bin's sum_c (1 / S_c + ln S_c) with a logarithm per channel, and the library's functions for the factors
+// out of the short forms' range: for bins with an exponent or a product out of it (any value, NaN included).
+// A warp with lanes of both kinds runs both forms, so each factor within the range takes the short one here
+// too: 65,536 bins x 16 states, a noise spline of every other state at 120 decades, 632 -> 507 us
 template <int C, bool HAS_H>
 __device__ __noinline__ double bin_term64_wide(const double* P, double ao2, double at2, double lA, double slope,
-                                               const double* __restrict__ q) {
-    const double eh = HAS_H ? exp10(lA + P[C]) * exp2(slope * q[1]) : 0.0;
+                                               const double* __restrict__ q, const double* __restrict__ exptab) {
+    const double eh = HAS_H ? m64::background_wide(lA, P[C], slope * q[1], exptab) : 0.0;
     double term = 0.0;
     for (int c = 0; c < C; ++c) {
-        const double Sc = (ao2 * q[3 + c] + at2 * q[6 + c]) * exp10(P[c]) + (HAS_H ? eh * q[9 + c] : 0.0);
-        term += 1.0 / Sc + log(Sc);
+        const double Sc =
+            (ao2 * q[3 + c] + at2 * q[6 + c]) * m64::amplitude(P[c], exptab) + (HAS_H ? eh * q[9 + c] : 0.0);
+        term += m64::reciprocal_wide(Sc) + log(Sc);
     }
     return term;
 }
@@ -1383,31 +1386,35 @@ __global__ void __launch_bounds__(64)
         if (HAS_H) P[C] = fma(slope, ell, P[C]);
 #pragma unroll
         for (int a = 0; a < NSP; ++a) ok &= m64::small_exponent(P[a]);
-        double S[C], eh = 0.0;
-        if (HAS_H) eh = A * m64::exp10_fast(P[C], exptab);
-#pragma unroll
-        for (int c = 0; c < C; ++c) {
-            const double N = fma(ao2, go[c], at2 * gt[c]);
-            const double E = m64::exp10_fast(P[c], exptab);
-            S[c] = HAS_H ? fma(N, E, eh * gh[c]) : N * E;
-        }
-        const double p01 = S[0] * S[1];
-        const double prod = C == 3 ? p01 * S[C - 1] : p01;
-        const double num = C == 3 ? fma(S[C - 1], S[0] + S[1], p01) : S[0] + S[1];
-        // products of normal size: nothing over- or underflowed on the way
-        ok &= m64::normal_range(p01) && m64::normal_range(prod) && m64::normal_range(num);
         if (ok) {
-            run += m64::divide(num, prod);
-            lp.mul(prod);
-            ++len;
-        } else {
+            double S[C], eh = 0.0;
+            if (HAS_H) eh = A * m64::exp10_fast(P[C], exptab);
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                const double N = fma(ao2, go[c], at2 * gt[c]);
+                const double E = m64::exp10_fast(P[c], exptab);
+                S[c] = HAS_H ? fma(N, E, eh * gh[c]) : N * E;
+            }
+            const double p01 = S[0] * S[1];
+            const double prod = C == 3 ? p01 * S[C - 1] : p01;
+            const double num = C == 3 ? fma(S[C - 1], S[0] + S[1], p01) : S[0] + S[1];
+            // products of normal size: nothing over- or underflowed on the way
+            ok = m64::normal_range(p01) && m64::normal_range(prod) && m64::normal_range(num);
+            if (ok) {
+                run += m64::divide(num, prod);
+                lp.mul(prod);
+                ++len;
+            }
+        }
+        if (!ok) {
             double Pv[NSP];
 #pragma unroll
             for (int a = 0; a < NSP; ++a) {
                 const double t = x - xl[a];
                 Pv[a] = ca[a] + t * (cb[a] + t * (cc[a] + t * cd[a]));
             }
-            acc += nu * bin_term64_wide<C, HAS_H>(Pv, ao2, at2, lA, BROKEN ? (m64::negative(ell) ? n1 : n2) : n1, q);
+            acc += nu * bin_term64_wide<C, HAS_H>(Pv, ao2, at2, lA, BROKEN ? (m64::negative(ell) ? n1 : n2) : n1, q,
+                                                   exptab);
         }
     }
     acc = fma(nu_run, run + lp.log_value(), acc);

@@ -110,9 +110,15 @@ __device__ __forceinline__ double exp10_fast(double v, const double* __restrict_
     return __hiloint2double((int)(hi32(e) + (unsigned)((k >> 13) << 20)), (int)lo32(e));
 }
 
-// A = 10^log10A, any value.
+// 10^v, any value (A = 10^log10A, and a spline's factor in the wide forms).
 __device__ __forceinline__ double amplitude(double v, const double* __restrict__ T) {
     return small_exponent(v) ? exp10_fast(v, T) : exp10(v);
+}
+// 10^lA 10^p 2^y (the background's factor), any values.
+__device__ __forceinline__ double background_wide(double lA, double p, double y, const double* __restrict__ T) {
+    constexpr double kLog10_2 = 0.301029995663981195213739;
+    const double v = fma(y, kLog10_2, p), A = amplitude(lA, T);
+    return small_exponent(v) && normal_range(A) ? A * exp10_fast(v, T) : exp10(lA + p) * exp2(y);
 }
 
 // 1 / d to 2^-21 for a normal positive d of exponent within +-900, as a double: an FP32 reciprocal of d's
@@ -129,6 +135,8 @@ __device__ __forceinline__ double reciprocal(double d) {
     const double r = reciprocal_seed(d), e = fma(-d, r, 1.0);
     return fma(r, fma(e, e, e), r);
 }
+// 1 / d for any d >= 0 (NaN included).
+__device__ __forceinline__ double reciprocal_wide(double d) { return normal_range(d) ? reciprocal(d) : 1.0 / d; }
 // n / d: a reciprocal to 2^-42, the quotient by it and one correction by the remainder: 5 FP64
 // instructions, rounded once.  (n r (1 + e + e^2), 4 instructions, rounds twice: up to 1 unit, 1.2 with a
 // seed one unit off.)
