@@ -464,6 +464,9 @@ __global__ void __launch_bounds__(kThreads32, FAST || G == 8 ? 4 : (G == 4 ? 5 :
             const WorkItem pw = items[it - step];
             carry = w.ds == pw.ds && w.s0 == pw.s0 && w.slot == pw.slot + 1;
         }
+        // (a segment past the end of a thread's run locates nothing: without this the next slot's item would
+        // carry over the intervals of the states of an item before it)
+        if (!carry) s_hm[tid] = 0u;
         const int sc = w.sc;
         const int R = kThreads32 / sc;
         const int ls = tid & (sc - 1);
