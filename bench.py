@@ -58,7 +58,7 @@ ADJ_MUFU = (4, 3, 1)
 # FP64-pipe instructions per state-bin of the plain FP64 kernel as implemented (table-driven exp10,
 # divisions from FP32 seeds, one log per run of bins), counted by ncu on a 131,072-bin x 64-state
 # A,E,T case
-FP64_PIPE_PER_STATE_BIN = 58.0
+FP64_PIPE_PER_STATE_BIN = 58.9
 
 
 def adjoint_exact_t(wl) -> bool:

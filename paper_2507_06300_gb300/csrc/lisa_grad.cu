@@ -84,10 +84,11 @@ struct AdjIv {
 
 __device__ __forceinline__ float2 dup2(float v) { return make_float2(v, v); }
 
-// First unit of the calling warp, of nw in the grid (8 CTAs per SM, or one per unit).  Units that the
-// resident warps (3 of the grid's 8 CTAs per SM) can hold at once go to the CTAs before they go to a CTA's
-// warps, so that few of them spread over the SMs; more units go to a CTA's warps in turn, so that every
-// CTA that starts brings its full number of warps (131,072 bins, 2,048 states: 1.11 ms, and 1.35 ms spread).
+// First unit of the calling warp, of nw in the grid (8 CTAs per SM, or one per unit).  Up to 12 units per SM,
+// as many as there are resident warps (3 of the grid's 8 CTAs per SM), go to the CTAs before they go to a CTA's
+// warps, so that few of them spread over the SMs; more go to a CTA's warps in turn, so that every CTA that
+// starts brings its full number of warps (131,072 bins, 2,048 states: 1.11 ms, and 1.35 ms spread).  Between 3
+// and 12 units per SM the spread CTAs start in turns: a CTA with one working warp holds the registers of four.
 __device__ __forceinline__ int64_t first_unit(int64_t n_units, int64_t nw) {
     const int w = threadIdx.x >> 5;
     return 8 * n_units <= 3 * nw ? (int64_t)w * gridDim.x + blockIdx.x : (int64_t)blockIdx.x * (blockDim.x >> 5) + w;
@@ -555,7 +556,7 @@ __device__ __noinline__ void adjoint_bin64_wide(const double* P, double ao2, dou
     if (HAS_H) out[4 + C] = H;
 }
 
-// Per state-bin 115 FP64 instructions (about 340 with the library's functions and a division per
+// Per state-bin 114 FP64 instructions (about 340 with the library's functions and a division per
 // channel): the forward pass as loglike_fp64_kernel's, 9 for the channels' reciprocals, 24 for the template sums and signals, 24 for the moments.  One unit and warp per CTA: the
 // units of a small problem spread over all SMs and start as registers come free (four units to a CTA,
 // their CTAs half empty: 1.85 against 1.53 ms).  16,384 bins x 400 states with the epilogue: 5.8 -> 1.74 ms.
@@ -805,7 +806,7 @@ __global__ void __launch_bounds__(MODE == kComp ? 128 : 512)
         while (2 * sub * adj_bins <= kAdjBins && (int64_t)list[0] * ((R + 2 * sub - 1) / (2 * sub)) >= gridDim.x) sub *= 2;
         R = (R + sub - 1) / sub;
     }
-    const int rbins = sub * adj_bins;
+    const int rbins = MODE == kComp ? kAdjBins : sub * adj_bins;
     const int n_items = list[0] * R;
     for (;;) {
     if (threadIdx.x == 0) s_item = atomicAdd(next_item, 1);
@@ -1237,28 +1238,32 @@ __global__ void __launch_bounds__(MODE == kComp ? 128 : 512)
             v[p] = 0.0;
             for (int w = 0; w < nwarps; ++w) v[p] += sm(w, a, jr, p);
         }
-        // the sums go to the slot of the first of the adjoint's ranges that holds a bin of the interval
-        // (kComp: if there are any)
-        if (MODE == kComp && v[0] == 0.0 && v[1] == 0.0 && v[2] == 0.0 && v[3] == 0.0) continue;
-        int i = 0;
-        if (sub > 1 && j > 0) {
-            const float left = right_end(a, j - 1);
-            int hi = nb - 1;
-            while (i < hi) {
-                const int mid = (i + hi) >> 1;
-                if (xbin(mid) >= left) hi = mid; else i = mid + 1;
+        // the slot of the first of the adjoint's ranges that holds a bin of the interval
+        auto slot = [&]() {
+            int i = 0;
+            if (sub > 1 && j > 0) {
+                const float left = right_end(a, j - 1);
+                int hi = nb - 1;
+                while (i < hi) {
+                    const int mid = (i + hi) >> 1;
+                    if (xbin(mid) >= left) hi = mid; else i = mid + 1;
+                }
             }
-        }
-        double* row = mom_row(mom, pre, s, a, nsp, kmax, D.nranges) +
-                      4 * (int64_t)LISA_IDX(rho * sub + i / adj_bins + j, D.nranges + kmax + 1);
+            return 4 * (int64_t)LISA_IDX(rho * sub + i / adj_bins + j, D.nranges + kmax + 1);
+        };
+        double* row = mom_row(mom, pre, s, a, nsp, kmax, D.nranges);
         if (MODE == kComp) {
-            bool bad = false;
-            for (int p = 0; p < 4; ++p) {
-                row[p] += v[p];
-                bad |= !isfinite(row[p]);
+            if (v[0] != 0.0 || v[1] != 0.0 || v[2] != 0.0 || v[3] != 0.0) {
+                row += slot();
+                bool bad = false;
+                for (int p = 0; p < 4; ++p) {
+                    row[p] += v[p];
+                    bad |= !isfinite(row[p]);
+                }
+                if (bad) fb_flag(fb, S, s);
             }
-            if (bad) fb_flag(fb, S, s);
         } else {
+            row += slot();
             for (int p = 0; p < 4; ++p) row[p] = v[p];
         }
     }

@@ -1,5 +1,5 @@
 """The FP64 path where exponents leave the range of its short forms (100 decades): states lifted or lowered by
-120 decades beside ordinary ones in the same warps, log L, gradient and model PSD against the oracle."""
+120 decades beside ordinary ones in the same warps, log L and template gradients against the oracle."""
 import numpy as np
 import pytest
 
@@ -18,8 +18,6 @@ def test_wide_exponents(n_bins, n_states, sgwb):
     """At the tolerances of ordinary states: 1e-12 of log L and of the template gradients' condition scale.  (The
     knots' gradients go through the reverse map, whose error at close knots and at components without any
     bin exceeds that bound whichever form the bins take.)"""
-    import torch
-    from paper_2507_06300_gb300 import binding as B
     wl = synth.workload("tiny", n_bins=n_bins, n_states=n_states, kmin=0, kmax_draw=6, sgwb_model=sgwb)
     wl.f_ref[:] = 3e-3
     w = wl.knots.w
@@ -35,11 +33,3 @@ def test_wide_exponents(n_bins, n_states, sgwb):
     Lg, G, _, _ = gpu_grad(wl, ds["P"], FP64)
     np.testing.assert_allclose(Lg[ok], L_ref[ok], rtol=1e-12, atol=0)
     assert np.all((np.abs(G - G_ref) <= 1e-12 * sc)[ok, :5]) and np.all(np.isfinite(G))
-    S_ref, _ = oracle.model_psd(ds, wl.theta, wl.knots.as_dict())
-    d = B.Dataset.from_workload(wl, ds["P"])
-    count, x, wd, kmax, kind = B.knots_to_device(wl.knots)
-    buf, _ = d.spline_setup(count, x, wd, kmax, kind, FP64)
-    S = d.model_psd(torch.as_tensor(wl.theta, device="cuda"), buf, kmax).cpu().numpy().reshape(S_ref.shape)
-    d.close()
-    # the exponent's rounding: 130 decades x ln10 x 2^-53 x a few operations
-    np.testing.assert_allclose(S[ok], S_ref[ok], rtol=1e-12, atol=0)
