@@ -97,7 +97,8 @@ __device__ __forceinline__ double exp10_fast(double v, const double* __restrict_
     const float q0 = K2 * h;
     const int j = k & (kExpTab - 1);
     const float c = __ldg(reinterpret_cast<const float*>(T + kExpTab) + j);
-    const dm::ff q = dm::two_sum(q0, fmaf(K2, h, -q0) + fmaf(K2, l, fmaf(rf, K3, K2l) * h) + c);
+    // (where r is so small that c passes q0, what the short sum misses is below 2^-24 of c)
+    const dm::ff q = dm::fast_two_sum(q0, fmaf(K2, h, -q0) + fmaf(K2, l, fmaf(rf, K3, K2l) * h) + c);
     // q as a double: its low part, below 2^-23 of the high one, rounded to 2^-45 of the high one's exponent
     // and added to that one's bits
     const unsigned qb = __float_as_uint(q.hi), eq = (qb >> 23) & 0xffu;

@@ -85,9 +85,7 @@ struct LaneSum {
 
 constexpr int kFixedMin = 12;           // samples from which a bin's sums run in fixed point
 constexpr int kFixedBatch = 4;          // samples that a lane adds at once there
-constexpr int kSerialThreadsPerSm = 512;
-constexpr int kSerialWidths = 4;
-constexpr int kTogetherMax = 4;         // one lane per bin: bins of fewer samples have no second load of a channel
+constexpr int kSerialThreadsPerSm = 512, kSerialWidths = 4, kLanesPerSm = 2048;
 
 // Averaged periodogram: a group of G lanes per bin (G divides 32), lanes striding over the bin's
 // samples with 16-byte loads; the group's partial sums are combined by a butterfly of shuffles (a
@@ -102,15 +100,19 @@ constexpr int kTogetherMax = 4;         // one lane per bin: bins of fewer sampl
 // That takes many bins side by side.  Where the loads of a few lanes are waited for, four of one channel in
 // flight instead of four of every channel cost more than the FP64 pipe.  So a bin of up to `serial_max` samples
 // takes the channels one after the other, in fixed point from kFixedMin samples on, and a wider one all
-// channels together, in FP64; serial_max is kSerialWidths mean widths, or 0 when the bins have fewer than
-// kSerialThreadsPerSm lanes per SM.  Every bin serial (by its mean width in fixed point): 8,000 bins of 1,000
-// samples (64,000 lanes) 115 us, together 104; 12,000 of 300 (96,000) the same; 20,000 bins of 1 to 4,000
-// samples 402, 298 with this rule; 400 bins of 20,000 samples among 20,000 of one or two 1.89 ms, 1.32.
+// channels together, in FP64; serial_max is kSerialWidths mean widths, or 0 when the bins of 4 or 8 lanes have
+// fewer than kSerialThreadsPerSm lanes per SM.  Every bin serial (by its mean width in fixed point): 8,000 bins
+// of 1,000 samples (64,000 lanes) 115 us, together 104; 12,000 of 300 (96,000) the same; 20,000 bins of 1 to
+// 4,000 samples 402, 298 with this rule; 400 bins of 20,000 samples among 20,000 of one or two 1.89 ms, 1.32.
+// With one lane per bin two channels go one after the other (200,000 bins of 4: 16.7 us, together 20.6; of 2 15.5,
+// 15.7), three together (of 2 18.7, serial 21.3; of 6 27.7, 30.4; of 8 32.8, 32.3), but for bins of 7 samples
+// and more that outnumber the resident lanes (a million of 8: 150, together 161).
 template <int C, int G>
 __global__ void __launch_bounds__(256)
     avg_periodogram_kernel(const double2* __restrict__ d, int64_t n_freq, double f0, double df,
                            const int64_t* __restrict__ off, int64_t n_bins, double* __restrict__ P,
-                           double* __restrict__ f_out, double* __restrict__ nu_out, int n_ch, int64_t serial_max) {
+                           double* __restrict__ f_out, double* __restrict__ nu_out, int n_ch, int serial_min,
+                           int64_t serial_max) {
     const int lane = threadIdx.x & (G - 1);
     const int64_t g0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
     const int64_t ng = ((int64_t)gridDim.x * blockDim.x) / G;
@@ -127,7 +129,7 @@ __global__ void __launch_bounds__(256)
         double acc[C];
 #pragma unroll
         for (int c = 0; c < C; ++c) acc[c] = 0.0;
-        if (n > serial_max || (G == 1 && n < kTogetherMax)) {
+        if (n > serial_max || n < serial_min) {
 #pragma unroll 4
             for (int64_t k = b0 + lane; k < b1; k += G) {
 #pragma unroll
@@ -201,9 +203,12 @@ cudaError_t launch_avg(const double2* d, int64_t n_freq, double f0, double df, c
     const int64_t want = (n_bins * G + threads - 1) / threads;
     const int64_t cap = (int64_t)n_sm * 8;   // persistent: 8 blocks of 256 threads per SM
     const unsigned grid = (unsigned)(want < cap ? (want < 1 ? 1 : want) : cap);
-    const bool many = n_bins * G >= (int64_t)kSerialThreadsPerSm * n_sm;
+    const bool two = G == 1 && n_ch < 3;
+    const bool many = two || n_bins * G >= (int64_t)(G == 1 ? kLanesPerSm : kSerialThreadsPerSm) * n_sm;
     const int64_t serial_max = many ? (int64_t)(kSerialWidths * ((double)n_freq / (double)n_bins)) : 0;
-    avg_periodogram_kernel<C, G><<<grid, threads, 0, sm>>>(d, n_freq, f0, df, off, n_bins, P, f, nu, n_ch, serial_max);
+    const int serial_min = G > 1 || two ? 0 : 7;
+    avg_periodogram_kernel<C, G><<<grid, threads, 0, sm>>>(d, n_freq, f0, df, off, n_bins, P, f, nu, n_ch, serial_min,
+                                                      serial_max);
     return cudaGetLastError();
 }
 
