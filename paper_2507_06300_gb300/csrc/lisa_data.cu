@@ -703,10 +703,7 @@ lisa_status lisa_data_create(const lisa_data_desc* desc, lisa_stream_t stream, l
     cudaStream_t sm = (cudaStream_t)stream;
     bool ok = cudaMemcpyAsync(d->d_ds, d->h_ds.data(), D * sizeof(DatasetDev), cudaMemcpyHostToDevice, sm) == cudaSuccess &&
               cudaMemcpyAsync(d->d_state_ds, state_ds.data(), S * sizeof(int32_t), cudaMemcpyHostToDevice, sm) == cudaSuccess &&
-              // (two copies: pageable copies of up to 64 KB are staged without a wait)
-              cudaMemcpyAsync(d->d_exptab, exp_table(), kExpTab * sizeof(double), cudaMemcpyHostToDevice, sm) == cudaSuccess &&
-              cudaMemcpyAsync(d->d_exptab + kExpTab, exp_table() + kExpTab, (kExpTabDoubles - kExpTab) * sizeof(double),
-                              cudaMemcpyHostToDevice, sm) == cudaSuccess &&
+              cudaMemcpyAsync(d->d_exptab, exp_table(), kExpTabDoubles * sizeof(double), cudaMemcpyHostToDevice, sm) == cudaSuccess &&
               cudaMemcpyAsync(f, q.freq, N * sizeof(double), cudaMemcpyHostToDevice, sm) == cudaSuccess &&
               cudaMemcpyAsync(nu, q.nu, N * sizeof(double), cudaMemcpyHostToDevice, sm) == cudaSuccess &&
               cudaMemcpyAsync(d->d_P, q.periodogram, C * N * sizeof(double), cudaMemcpyHostToDevice, sm) == cudaSuccess &&

@@ -89,7 +89,7 @@ constexpr int kAdjWarpsPerSm = 12;
 // interval advances: knots are drawn uniformly in log10 f, so the low-frequency tiles (few bins,
 // wide in log10 f) hold most of them, and each advance stalls its warp on record loads.
 constexpr double kKnotBinsPerDecade = 2500.0;
-constexpr int kExpTab = 8192;               // entries of the FP64 path's table of 2^(j / kExpTab)
+constexpr int kExpTab = 4096;               // entries of the FP64 path's table of 2^(j / kExpTab)
 constexpr int kExpTabDoubles = kExpTab + kExpTab / 2;   // with their rounding errors (floats) behind them
 constexpr int kXsStride = 32;               // bins between the host copies of log10 f
 constexpr int kMinItemsPerSm = 2;            // fewer items per SM than this are split into segments

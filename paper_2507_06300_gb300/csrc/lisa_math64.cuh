@@ -17,8 +17,8 @@
 namespace lisa {
 namespace m64 {
 
-// Host: the table of exp10_fast, kExpTabDoubles doubles: 2^(j / kExpTab) rounded to FP64, then the
-// relative errors of these roundings (what is missing of each, over it) as floats.
+// Host: the table of exp10_fast, kExpTabDoubles doubles: 2^(j / kExpTab) rounded to FP64, then the relative
+// errors of these roundings (what is missing, over the entry) as floats.
 inline void fill_exp_table(double* T) {
     float* c = reinterpret_cast<float*>(T + kExpTab);
     for (int j = 0; j < kExpTab; ++j) {
@@ -52,11 +52,11 @@ __device__ __forceinline__ long long order_key(double v) {
     return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
 }
 // The same with one key for both zeros, for knots against knots and band edges: a knot at -0 does not lie
-// inside a band that ends at +0.  (Its two further instructions in the bins' searches cost the model PSD 0.81
-// -> 0.99 ms, the FP64 likelihood 2 %.)
+// inside a band that ends at +0.  (In the bins' searches too, the further instructions cost the model PSD 0.81 ->
+// 0.99 ms, the FP64 likelihood 2 %.)
 __device__ __forceinline__ long long position_key(double v) {
-    const long long b = __double_as_longlong(v), m = b >> 63;
-    return ((b & 0x7fffffffffffffffLL) ^ m) - m;
+    const long long k = order_key(v);
+    return k == -1 ? 0 : k;   // (-1 is -0's key alone)
 }
 // Biased exponent of a double (0: zero or subnormal, 2047: infinite or NaN).
 __device__ __forceinline__ int exponent(double v) { return (int)((hi32(v) >> 20) & 0x7ffu); }
@@ -70,45 +70,37 @@ __device__ __forceinline__ bool square_range(double v) { return (unsigned)(expon
 __device__ __forceinline__ bool small_exponent(double v) { return (hi32(v) & 0x7fffffffu) < 0x40590000u; }
 
 // 10^v for |v| < 100 from the table T of 2^(j / kExpTab) (the table-driven scheme of Tang, ACM TOMS 15,
-// 1989): 4 FP64 instructions.  v = k log10(2) / 8192 + r with k chosen in FP32 (|r| <= 0.85 of a step), r
-// exact to twice the precision; 10^r = 1 + r ln10 + q with q = (r ln10)^2 / 2 + (r ln10)^3 / 6 <= 2^-28.6,
-// which with the table entry's rounding error is formed in float-float and taken into p to 2^-45 of q: one
-// rounding is left.  Error at most 0.51 units of the last place, rms 0.29 (the library's exp10 takes about 40
-// instructions).  With q rounded to FP32 and T[j] as it is, it was up to 1.7 units, rms 0.41, and the
-// model PSD's error against 64 bits half a percent above that of the library's functions.  The table
-// (96 KB) is read through L1, which the kernels that use it leave free.
+// 1989): 4 FP64 instructions.  v = k log10(2) / 4096 + r with k chosen in FP32 (|r| <= 0.7 of a step);
+// 10^r = 1 + r ln10 + q with q = sum_(n = 2..4) (r ln10)^n / n! <= 2^-27, formed in float-float.  What is
+// missing besides is below 2^-50 and collected in one FP32 number: q's low part, k times what log10(2) / 4096
+// rounded off, and the table entry's rounding error.  Added to q and r ln10 in FP64, so one rounding is left:
+// error at most 0.51 units of the last place, rms 0.29 (the library's exp10 takes about 40 instructions).  With q
+// rounded to FP32 and the entries as they are, it was up to 1.7 units, rms 0.41, and the model PSD's error
+// against 64 bits half a percent above that of the library's functions.  The tables (48 KB) are read through
+// L1, which the kernels that use them leave free (8,192 entries, 96 KB, cost the dense covariance's careful bins
+// 2-4 %, entry and error in one 16-byte load small FP64 calls 10 %).
 __device__ __forceinline__ double exp10_fast(double v, const double* __restrict__ T) {
-    constexpr double C_hi = 0x1.34413509f79ffp-15;    // log10(2) / 8192, rounded to FP64
-    constexpr double C_lo = -0x1.9dc1da994fd21p-72;   // and the rest
-    static_assert(kExpTab == 8192, "constants");
-    const float tf = fmaf(to_float(v), 27213.2350f, 12582912.f);   // 8192 / log10(2): k in the low bits
-    const int k = __float_as_int(tf) - 0x4b400000;
-    const double kd = to_double(tf - 12582912.f);
-    double r = fma(kd, -C_hi, v);
-    r = fma(kd, -C_lo, r);
+    constexpr double C_hi = 0x1.34413509f79ffp-14;    // log10(2) / 4096, rounded to FP64
+    constexpr float C_lo = 0x1.9dc1da994fd21p-71 * 2.302585092994045684;   // what that is too large, times ln10
+    static_assert(kExpTab == 4096, "constants");
+    const float tf = fmaf(to_float(v), 13606.6175f, 12582912.f);   // 4096 / log10(2): k in the low bits
+    const int k = __float_as_int(tf) - 0x4b400000, j = k & (kExpTab - 1);
+    const double t = __ldg(T + j);
+    const float kf = tf - 12582912.f, c = __ldg(reinterpret_cast<const float*>(T + kExpTab) + j);
+    const double r = fma(to_double(kf), -C_hi, v);
     // r = rf + rl: its truncation to FP32 and the 29 bits below
     const float rf = to_float(r);
     const unsigned hr = hi32(r), er = (hr >> 20) & 0x7ffu;
     const float sc = er >= 960u ? __uint_as_float((hr & 0x80000000u) | ((er - 948u) << 23)) : 0.f;   // 2^(e - 52)
     const float rl = (float)(lo32(r) & 0x1fffffffu) * sc;
-    constexpr float K2 = 2.65094906f, K2l = 5.39269431e-08f, K3 = 2.03467859f;   // ln10^2 / 2, ln10^3 / 6
+    constexpr float K2 = 2.65094906f, K2l = 5.39269431e-08f, K3 = 2.03467859f, K4 = 1.17125515f;   // ln10^n / n!
     const float h = rf * rf;
     const float l = fmaf(2.f * rf, rl, fmaf(rf, rf, -h));
     const float q0 = K2 * h;
-    const int j = k & (kExpTab - 1);
-    const float c = __ldg(reinterpret_cast<const float*>(T + kExpTab) + j);
-    // (where r is so small that c passes q0, what the short sum misses is below 2^-24 of c)
-    const dm::ff q = dm::fast_two_sum(q0, fmaf(K2, h, -q0) + fmaf(K2, l, fmaf(rf, K3, K2l) * h) + c);
-    // q as a double: its low part, below 2^-23 of the high one, rounded to 2^-45 of the high one's exponent
-    // and added to that one's bits
-    const unsigned qb = __float_as_uint(q.hi), eq = (qb >> 23) & 0xffu;
-    const float lo_scale = eq >= 64u ? __uint_as_float((qb & 0x80000000u) | ((299u - eq) << 23)) : 0.f;
-    const int lo = __float_as_int(fmaf(q.lo, lo_scale, 12582912.f)) - 0x4b400000;
-    const double qd = __longlong_as_double(__double_as_longlong(to_double(q.hi)) + ((long long)lo << 7));
-    const double p = fma(r, kLn10, qd);
-    const double t = __ldg(T + j);
+    const dm::ff q = dm::fast_two_sum(q0, fmaf(K2, h, -q0) + fmaf(K2, l, fmaf(rf, fmaf(rf, K4, K3), K2l) * h));
+    const double p = fma(r, kLn10, to_double(q.hi) + to_double(fmaf(kf, C_lo, q.lo + c)));
     const double e = fma(t, p, t);
-    return __hiloint2double((int)(hi32(e) + (unsigned)((k >> 13) << 20)), (int)lo32(e));
+    return __hiloint2double((int)(hi32(e) + (unsigned)((k >> 12) << 20)), (int)lo32(e));
 }
 
 // 10^v, any value (A = 10^log10A, and a spline's factor in the wide forms).

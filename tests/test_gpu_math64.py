@@ -2,8 +2,8 @@
 precision (numpy's longdouble, 64 bits or more), in units of the result's last place.
 
 Bounds, from the arithmetic: the result is rounded once, after a correction that is exact to 2^-60 of it, so
-half a unit; the exponential adds the neglected fourth-order term, (0.85 ln2 / 8192)^4 / 24 = 1.1e-18, 0.01
-units, and the rounding of its linear term (2^-67)."""
+half a unit; the exponential's series may neglect up to (0.85 ln2 / 8192)^4 / 24 = 1.1e-18, 0.01 units, and its
+linear term is rounded to 2^-66."""
 import ctypes
 import os
 import subprocess
