@@ -559,7 +559,7 @@ __device__ __noinline__ void adjoint_bin64_wide(const double* P, double ao2, dou
 // Per state-bin 114 FP64 instructions (about 340 with the library's functions and a division per
 // channel): the forward pass as loglike_fp64_kernel's, 9 for the channels' reciprocals, 24 for the template sums and signals, 24 for the moments.  One unit and warp per CTA: the
 // units of a small problem spread over all SMs and start as registers come free (four units to a CTA,
-// their CTAs half empty: 1.85 against 1.53 ms).  16,384 bins x 400 states with the epilogue: 5.8 -> 1.74 ms.
+// their CTAs half empty: 1.85 against 1.53 ms).  16,384 bins x 400 states with the epilogue: 5.8 -> 1.75 ms.
 constexpr int kLogRun = 64;   // factors of a LogProduct: its mantissa stays below 2^64
 template <int C, bool HAS_H, bool BROKEN>
 __global__ void __launch_bounds__(32)

@@ -1293,7 +1293,7 @@ __device__ __noinline__ double bin_term64_wide(const double* P, double ao2, doub
 // their product and the numerator of sum 1 / S, 5 for the division, 2 for the sums; the logarithm of
 // the channels' product is taken once for up to kLogRun bins of equal nu.  Intervals, range checks and
 // conversions are integer work (lisa_math64.cuh).  65,537 bins x 400 states: 13.7 -> 3.12 ms;
-// with the rows 262,144 bins x 4 states 547 -> 156 us, 131,072 bins x 1 state 95 -> 43 us.
+// with the rows 262,144 bins x 4 states 547 -> 158 us, 131,072 bins x 1 state 95 -> 45 us.
 constexpr int kLogRun = 64;   // factors of a LogProduct: its mantissa stays below 2^64
 template <int C, bool HAS_H, bool BROKEN>
 __global__ void __launch_bounds__(64)

@@ -5,7 +5,7 @@
 // instruction of a warp takes the pipe as long as 64 other instructions take to issue.  So everything
 // that need not be rounded to 53 bits runs elsewhere: exponents, table indices, conversions and
 // comparisons on the integer pipe (from the bits of the doubles), reciprocal seeds and the last terms of
-// the series, below 2^-28 of the result, in FP32 pairs of 46 bits.  Against the library's exp10, exp2, log and
+// the series, below 2^-27 of the result, in FP32 pairs.  Against the library's exp10, exp2, log and
 // division a state-bin of the likelihood takes 59 FP64 instructions instead of 225.
 #pragma once
 
